@@ -30,6 +30,7 @@
 //               keep the issue slots busy
 //   warps 18-19 one elected lane each issues the TMA stores of one 64-feature
 //               half's staging tiles and recycles them
+// (INT8 output: warps 2-13 are the epilogue, each works by itself; see EpiI8.)
 // Everything is handed over with mbarriers (full/empty per smem stage,
 // full/empty per accumulator buffer, full/free per staging tile), so no warp
 // waits for another one's instruction stream; two accumulator buffers let the
@@ -70,6 +71,11 @@ constexpr int kMetaCol = 224;       // metadata slots: 4 columns per stage from 
 constexpr int kMaxEpiGroups = 2 * kMaxPhases;   // groups of four epilogue warps: 64 features x chunk phase
 constexpr int kMaxEpiBufs = 3;                  // staging tiles per group, at most
 constexpr int kEpiBufBytes = kChunkT * 128;           // [32 tokens][64 features] f16
+// INT8 output has an epilogue of its own shape (EpiI8) and no store warps
+constexpr int kI8Turns = 3;                           // warps per 32 features, taking turns at the chunks
+constexpr int kI8Warps = 4 * kI8Turns;
+constexpr int kI8ChunkT = 16;                         // tokens per chunk
+constexpr int kI8BufBytes = kI8ChunkT * 32;           // [16 tokens][32 features] i8, two per warp
 
 // kHalf: the FP16 2:4 sparse model (binary16 operands, FP32 accumulators) instead of INT8.  A stage
 // still covers 128 columns of W: 128 bytes of kept values per feature row, and two 128-byte-swizzled
@@ -91,7 +97,6 @@ struct Cfg {
     static constexpr int kThreads = 32 * (kStoreWarp0 + 2);
     static constexpr int kEpiGroups = 2 * kPhases;             // 64 features x chunk phase: four warps share a staging tile
     static constexpr int kEpiBufs = kPhases == 3 ? 2 : kPhases == 1 ? 6 : kHalf ? 2 : 3;      // staging tiles per group
-    static constexpr int kI8Bufs = 2 * kEpiBufs;               // INT8 output: one ring per phase over the same shared memory
     static constexpr int kEpiBytes = kEpiGroups * kEpiBufs * kEpiBufBytes;
     static constexpr int kCtlBytes = 1024;
     static constexpr int kSmemBytes = kStages * kStageBytes + kEpiBytes + kCtlBytes + 1024 /* alignment slack */;
@@ -103,6 +108,8 @@ struct Cfg {
     static_assert(kStageBytes % 1024 == 0, "stages keep the 1024-byte alignment of the swizzled tiles");
     static_assert(kStages <= 8, "eight metadata slots below the second accumulator");
     static_assert(kSmemBytes <= 232448, "shared memory per CTA");
+    static_assert(kI8Warps * 2 * kI8BufBytes <= kEpiBytes, "staging buffers of the INT8 epilogue");
+    static constexpr int threads(int out_type) { return out_type == GPUSQ_OUT_I8 ? 32 * (2 + kI8Warps) : kThreads; }
 };
 
 struct Ctl {
@@ -441,25 +448,33 @@ struct EpiF16 {
     }
 };
 
-// INT8 epilogue of one worker warp (requantised output): the FP16 epilogue's structure with bytes.
-// The warp owns 16 tensor-memory lanes (features) and every other 32-token chunk; tcgen05.ld in the
-// 16x256b shape gives a thread, per block of eight tokens, two neighbouring tokens of features f and
-// f + 8.  Their four codes, packed into one word, are exactly the fragment of the 8-bit matrix store
-// (stmatrix m16n8 b8, transposed): one instruction per chunk writes the warp's 32 tokens x 16 features
-// as 16-byte row pieces into a 128-byte-swizzled [32 tokens][128 features] staging tile that the
-// eight warps of the same chunk parity fill together; a TMA store writes full 128-byte rows of Y.
-template <int kI8Bufs, int kPhases, bool kTwin>
+// INT8 epilogue of one worker warp (requantised output).  The warp owns 32 tensor-memory lanes
+// (features) and every third 16-token chunk, and works by itself from the accumulator to global memory:
+// two loads of 16 lanes x 16 columns in the accumulator-fragment shape (the next chunk's are in flight
+// during the arithmetic), after which a thread holds, for feature f = lane / 4 and f + 8, f + 16, f + 24,
+// the tokens 8 i + 2 (lane % 4) and the next one, i = 0, 1; the four codes of two tokens and two features
+// (f and f + 8) packed into one word are exactly the fragment of the 8-bit matrix store (stmatrix m16n8
+// b8, transposed), so one instruction puts the chunk, as 16 rows of 32 bytes, into one of the warp's two
+// staging buffers; a chunk later it is read back in 16-byte pieces and stored.  The 16-byte columns of a
+// row are permuted so that neither access has bank conflicts.  The __syncwarp behind a chunk's matrix
+// store also orders the reads of the chunk before against the matrix store of the chunk after.
+// What bounds it: instruction issue (~6 dispatch cycles per value, 14 with GELU).  No hand-over between
+// warps: the eight warps that filled a 128-feature tile together for a store warp's bulk stores needed,
+// per tile of 256 x 224 at K = 768, 5015 cycles of a loaded GPU (7371 with GELU); this needs 4014 (6170).
+// Twelve warps: eight (6505 with GELU) are short of latency hiding with GELU, sixteen of registers (8360).
+template <bool kTwin>
 struct EpiI8 {
     const GemmParams *p;
     Ctl *ctl;
-    uint8_t *epi_smem;
-    uint32_t tmem_base, tmem_empty0, tmem_empty1;
+    uint32_t buf0, tmem_base, tmem_empty0, tmem_empty1;
     float x_scale, out_scale;
-    int warp, lane, rank, cluster_id, num_clusters, tiles_n, num_tiles;
+    int warp, lane, rank, cluster_id, num_clusters;
 
-    uint32_t buf_addr, full_bar, free_bar, buf_idx, free_parity, ring0, full0, free0;
-    uint32_t stm_off;
-    float2 sc2[2], bi2[2];
+    uint32_t stm_addr, lds_addr;   // this lane's matrix-store and read address in the current buffer
+    float2 sc2[4], bi2[4];         // scale and bias of this thread's four features, duplicated for packed math
+    uint8_t *y;                    // where this lane stores its 16 bytes of the chunk
+    int64_t y_step;
+    int rows;                      // rows of Y from y's on that exist (<= 0: this lane stores nothing)
     QuantScale qs;
 
     __device__ __forceinline__ void release(int acc)
@@ -469,89 +484,86 @@ struct EpiI8 {
         if (lane == 0) ptx::mbar_arrive_cluster(acc ? tmem_empty1 : tmem_empty0);
     }
 
-    template <bool kGelu>
-    __device__ __forceinline__ bool step(uint32_t (&v)[16], uint32_t (&vn)[16], uint32_t next_taddr, int acc, int tile)
+    __device__ __forceinline__ static void load(uint32_t taddr, uint32_t (&v)[16])
+    {
+        ptx::tmem_ld_16x256b_x2(taddr, v, 0);
+        ptx::tmem_ld_16x256b_x2(taddr + (16u << 16), v, 8);
+    }
+
+    // the chunk whose matrix store was issued last: read it back and store it to Y
+    __device__ __forceinline__ void flush()
+    {
+        const uint4 w = ptx::ld_shared_v4(lds_addr);
+        if (rows > 0) *reinterpret_cast<uint4 *>(y) = w;
+        y += y_step;
+        rows -= kI8Turns * kI8ChunkT;
+        lds_addr ^= (uint32_t)kI8BufBytes;
+    }
+
+    // One chunk held in v (its loads were issued earlier).  next_taddr != 0: issue this warp's next loads
+    // into vn; otherwise v was the warp's last chunk of the tile and the accumulator is released.  kFlush:
+    // the chunk before this one is stored to Y in the shadow of this one's arithmetic.
+    template <bool kGelu, bool kFlush>
+    __device__ __forceinline__ void step(uint32_t (&v)[16], uint32_t (&vn)[16], uint32_t next_taddr, int acc)
     {
         ptx::tmem_ld_wait_regs(v);
         if (next_taddr)
-            ptx::tmem_ld_16x256b_x4(next_taddr, vn);
+            load(next_taddr, vn);
         else
             release(acc);
-        uint32_t pk[4];
+        if (kFlush) flush();
+        float2 f[8], m[8];
+        float big = 0.0f;
+        uint32_t differ = 0, pk[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            // feature f: tokens 8i + 2(t%4), +1; feature f + 8: the same tokens
-            float2 ya = __ffma2_rn(make_float2(__int2float_rn((int32_t)v[4 * i]), __int2float_rn((int32_t)v[4 * i + 1])), sc2[0], bi2[0]);
-            float2 yb = __ffma2_rn(make_float2(__int2float_rn((int32_t)v[4 * i + 2]), __int2float_rn((int32_t)v[4 * i + 3])), sc2[1], bi2[1]);
-            if (kGelu) {
-                ya = gelu_pair(ya);
-                yb = gelu_pair(yb);
-            }
-            // values beyond +-127 out_scale saturate: rare, so they are only detected here (one
-            // compare per four values) and handled, clamp included, by the exact branch
-            const bool beyond = fmaxf(fmaxf(fabsf(ya.x), fabsf(ya.y)), fmaxf(fabsf(yb.x), fabsf(yb.y))) > qs.x_max;
-            uint32_t differ = 0;
-            float2 ma = quant2_sums<false>(ya, qs, differ), mb = quant2_sums<false>(yb, qs, differ);
-            if (differ != 0u || beyond || qs.always_divide) {
-                ma = quant2_exact<true>(ya, qs);
-                mb = quant2_exact<true>(yb, qs);
-            }
-            pk[i] = pack4_low_bytes(ma, mb);
+        for (int e = 0; e < 8; ++e) {
+            const int j = 2 * (e >> 2) + (e & 1);          // which of the four features
+            f[e] = __ffma2_rn(make_float2(__int2float_rn((int32_t)v[2 * e]), __int2float_rn((int32_t)v[2 * e + 1])), sc2[j], bi2[j]);
+            if (kGelu) f[e] = gelu_pair(f[e]);
+            big = ptx::max3_abs(big, f[e].x, f[e].y);
+            m[e] = quant2_sums<false>(f[e], qs, differ);
         }
-        bool to;
-        if (!ptx::mbar_wait_bounded(free_bar, free_parity, &ctl->abort_flag, to)) {
-            if (to && lane == 0) report_timeout(*p, ctl, tile, 2, 200 + (int)buf_idx);
-            return false;
+        // values beyond +-127 out_scale saturate, and products next to a rounding tie do not decide: both
+        // are rare, only detected here and redone by the exact branch, clamp included
+        if (differ != 0u || big > qs.x_max || qs.always_divide) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) m[e] = quant2_exact<true>(f[e], qs);
         }
-        ptx::stmatrix_x4_trans_b8(buf_addr + stm_off, pk[0], pk[1], pk[2], pk[3]);
-        ptx::fence_proxy_async_smem();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) pk[i] = pack4_low_bytes(m[2 * i], m[2 * i + 1]);
+        ptx::stmatrix_x4_trans_b8(stm_addr, pk[0], pk[1], pk[2], pk[3]);
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(full_bar);
-        if (++buf_idx == (uint32_t)kI8Bufs) {
-            buf_idx = 0;
-            free_parity ^= 1u;
-            buf_addr = ring0;
-            full_bar = full0;
-            free_bar = free0;
-        } else {
-            buf_addr += kEpiBufBytes;
-            full_bar += 8;
-            free_bar += 8;
-        }
-        return true;
+        stm_addr ^= (uint32_t)kI8BufBytes;
     }
 
     template <bool kGelu>
     __device__ __forceinline__ void run()
     {
         const int quarter = warp & 3;                      // tensor-memory lanes [32q, 32q+32) are this warp's to read
-        const int half = ((warp - 2) >> 2) & 1;            // which 16 of them
-        const int par = (warp - 2) >> 3;                   // which chunks: every kPhases-th one
-        const int nofs = quarter * 32 + 16 * half + (lane >> 2);
-        // this lane's address in the matrix store: row = token `lane` of the chunk, the warp's 16-byte column
-        stm_off = (uint32_t)(lane * 128 + (((2 * quarter + half) ^ (lane & 7)) << 4));
-        // the barriers of the staging tiles, taken as one array: ring `par` uses entries par * kI8Bufs ...
-        ring0 = ptx::smem_u32(epi_smem + par * kI8Bufs * kEpiBufBytes);
-        full0 = ptx::smem_u32(&ctl->stg_full[0]) + (uint32_t)(par * kI8Bufs * 8);
-        free0 = ptx::smem_u32(&ctl->stg_free[0]) + (uint32_t)(par * kI8Bufs * 8);
-        buf_addr = ring0;
-        full_bar = full0;
-        free_bar = free0;
-        buf_idx = 0;
-        free_parity = 1;                                   // first round: the tiles are free
+        const int turn = (warp - 2) >> 2;                  // which chunks: every kI8Turns-th one
+        const int nofs = quarter * 32 + (lane >> 2);       // this thread's first feature in the CTA's 128
+        const int row_l = lane >> 1, col_l = quarter * 32 + (lane & 1) * 16;      // this lane's row and feature when storing
+        {
+            // this lane addresses memory row lane % 8 of matrix lane / 8: token t, features 16 (matrix / 2) ...
+            const int t = 8 * ((lane >> 3) & 1) + (lane & 7);
+            stm_addr = buf0 + (uint32_t)(t * 32 + (((lane >> 4) ^ ((t >> 2) & 1)) << 4));
+            lds_addr = buf0 + (uint32_t)(row_l * 32 + (((lane & 1) ^ ((row_l >> 2) & 1)) << 4));
+        }
         const int64_t M = p->M;
         const int N = p->N;
         const float *w_scale = p->w_scale, *bias = p->bias;
+        y_step = (int64_t)kI8Turns * kI8ChunkT * N;
         qs = make_quant_scale(out_scale);
 
-        float ws_next[2], bi_next[2];
+        // scale and bias of a tile are fetched one tile ahead: the loads are in flight during a whole tile
+        float ws_next[4], bi_next[4];
         auto fetch = [&](const TileWalk<kTwin> &w) {
             int n0, unused_h;
             int64_t unused;
             w.origin(*p, rank, n0, unused, unused_h);
-            const bool in = w.tile < num_tiles && n0 < N;
+            const bool in = w.tile < p->num_tiles;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < 4; ++j) {
                 const int n = n0 + nofs + 8 * j;
                 ws_next[j] = (in && n < N) ? __ldg(w_scale + n) : 0.0f;
                 bi_next[j] = (in && n < N && bias) ? __ldg(bias + n) : 0.0f;
@@ -559,8 +571,8 @@ struct EpiI8 {
         };
         TileWalk<kTwin> walk(*p, cluster_id, num_clusters);
         fetch(walk);
-        int local = 0;
-        for (; walk.tile < num_tiles; ++local) {
+        int local = 0, done = 0;                           // tiles; chunks so far modulo kI8Turns
+        for (; walk.tile < p->num_tiles; ++local) {
             const int tile = walk.tile;
             int n0, h;
             int64_t m0;
@@ -568,43 +580,46 @@ struct EpiI8 {
             walk.next(*p, num_clusters);
             const int acc = local & 1;
             const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
-            const bool n_valid = n0 < N;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < 4; ++j) {
                 const float sc = __fmul_rn(ws_next[j], x_scale);
                 sc2[j] = make_float2(sc, sc);
                 bi2[j] = make_float2(bi_next[j], bi_next[j]);
             }
             fetch(walk);
+            // tokens of the tile that exist (none: a twin tile's second half); the warps of a quarter take
+            // the chunks in turn, across tiles
+            const int64_t ahead = M - m0;
+            const int left = ahead < h ? (ahead > 0 ? (int)ahead : 0) : h;
+            const int all = (left + kI8ChunkT - 1) / kI8ChunkT;
+            const int first = turn >= done ? turn - done : turn - done + kI8Turns;
+            done = (done + all) % kI8Turns;
+            int chunks = n0 + quarter * 32 < N ? (all - first + kI8Turns - 1) / kI8Turns : 0;    // none past the last feature
+            rows = n0 + col_l < N ? left - first * kI8ChunkT - row_l : 0;
+            y = reinterpret_cast<uint8_t *>(p->Y) + (m0 + first * kI8ChunkT + row_l) * N + n0 + col_l;
             bool to;
             if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, &ctl->abort_flag, to)) {
                 if (to && lane == 0) report_timeout(*p, ctl, tile, 2, 100 + acc);
                 return;
             }
             ptx::tc_fence_after();
-            int nchunks = 0;
-            if (n_valid) {
-                const int64_t left = M - m0;
-                nchunks = left >= h ? h / kChunkT : (int)((left + kChunkT - 1) / kChunkT);
-            }
-            const int c0 = (par + local) % kPhases;
-            int mine = (nchunks - c0 + kPhases - 1) / kPhases;
-            if (mine <= 0) {
+            if (chunks <= 0) {
                 release(acc);
                 continue;
             }
-            uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32 + half * 16) << 16) +
-                             (uint32_t)(acc * kAccStride + c0 * kChunkT);
+            uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccStride + first * kI8ChunkT);
             uint32_t v0[16], v1[16];
-            ptx::tmem_ld_16x256b_x4(taddr, v0);
-            for (;;) {
-                taddr += kPhases * kChunkT;
-                if (!step<kGelu>(v0, v1, --mine ? taddr : 0u, acc, tile)) return;
-                if (!mine) break;
-                taddr += kPhases * kChunkT;
-                if (!step<kGelu>(v1, v0, --mine ? taddr : 0u, acc, tile)) return;
-                if (!mine) break;
+            load(taddr, v0);
+            taddr += kI8Turns * kI8ChunkT;
+            step<kGelu, false>(v0, v1, --chunks ? taddr : 0u, acc);
+            while (chunks) {
+                taddr += kI8Turns * kI8ChunkT;
+                step<kGelu, true>(v1, v0, --chunks ? taddr : 0u, acc);
+                if (!chunks) break;
+                taddr += kI8Turns * kI8ChunkT;
+                step<kGelu, true>(v0, v1, --chunks ? taddr : 0u, acc);
             }
+            flush();
         }
     }
 };
@@ -614,7 +629,7 @@ struct EpiI8 {
 // kAmax: the FP16 epilogue also merges max |Y| into a device word (its own instantiation, so that the
 // ordinary kernel's register allocation is untouched)
 template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((Cfg<kSparse, kHalf>::kThreads), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((Cfg<kSparse, kHalf>::threads(kOut)), 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_e,
                const __grid_constant__ CUtensorMap map_y, const GemmParams p)
@@ -626,7 +641,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     uint8_t *epi_smem = smem + C::kStages * C::kStageBytes;
     Ctl *ctl = reinterpret_cast<Ctl *>(epi_smem + C::kEpiBytes);
     constexpr int kBufs = C::kEpiBufs;      // staging tiles per group in the FP16-output path
-    constexpr int kPhases = C::kPhases, kEpiWarps = C::kEpiWarps, kStoreWarp0 = C::kStoreWarp0, kI8Bufs = C::kI8Bufs;
+    constexpr int kPhases = C::kPhases, kEpiWarps = kOut == GPUSQ_OUT_I8 ? kI8Warps : C::kEpiWarps, kStoreWarp0 = 2 + kEpiWarps;
     volatile uint32_t *abort_flag = &ctl->abort_flag;
 
     const int warp = threadIdx.x >> 5;
@@ -653,7 +668,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
         for (int g = 0; g < C::kEpiGroups * kBufs; ++g) {
-            ptx::mbar_init(ptx::smem_u32(&ctl->stg_full[g]), kOut == GPUSQ_OUT_I8 ? 8 : 4);
+            ptx::mbar_init(ptx::smem_u32(&ctl->stg_full[g]), 4);
             ptx::mbar_init(ptx::smem_u32(&ctl->stg_free[g]), 1);
         }
         ctl->abort_flag = 0;
@@ -663,7 +678,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ptx::prefetch_tensormap(&map_b);
         if (p.n_big * p.pair_cols < p.pair_tiles) ptx::prefetch_tensormap(&map_b2);
         if (kSparse) ptx::prefetch_tensormap(&map_e);
-        if (kOut != GPUSQ_OUT_I32) ptx::prefetch_tensormap(&map_y);
+        if (kOut == GPUSQ_OUT_F16) ptx::prefetch_tensormap(&map_y);
     }
     if (warp == 1) {
         ptx::tmem_alloc_pair(ptx::smem_u32(&ctl->tmem_base), kTmemCols);
@@ -878,46 +893,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             // the staging tiles must stay valid until the bulk stores have read them, and the
             // stores must be complete before the kernel ends
             ptx::tma_store_wait_all<0>();
-        } else if (kOut == GPUSQ_OUT_I8 && ptx::elect_one()) {
-            // INT8 output: a staging tile holds all 128 features of a chunk; every chunk phase has its
-            // ring; this lane serves the rings of even (first store warp) or odd phases
-            const int odd = warp - kStoreWarp0;
-            const uint32_t full0 = ptx::smem_u32(&ctl->stg_full[0]), free0 = ptx::smem_u32(&ctl->stg_free[0]);
-            uint32_t filled[kMaxPhases] = {};              // staging tiles stored so far, per ring
-            uint32_t prev1 = 0, prev2 = 0;
-            int local = 0;
-            bool ok = true;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles;
-                 walk.next(p, num_clusters), ++local) {
-                const int tile = walk.tile;
-                int n0, h;
-                int64_t m0;
-                walk.origin(p, (int)rank, n0, m0, h);
-                if (n0 >= p.N) continue;
-                const int64_t left = p.M - m0;
-                const int nchunks = left >= h ? h / kChunkT : (int)((left + kChunkT - 1) / kChunkT);
-                for (int c = 0; c < nchunks; ++c) {
-                    const int ring = (c + kPhases - local % kPhases) % kPhases;
-                    if ((ring & 1) != odd) continue;
-                    const uint32_t count = filled[ring];
-                    const uint32_t slot = (uint32_t)(ring * kI8Bufs) + count % kI8Bufs;
-                    bool to;
-                    if (!ptx::mbar_wait_bounded(full0 + 8u * slot, (count / kI8Bufs) & 1u, abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, tile, 3, (int)slot);
-                        ok = false;
-                        break;
-                    }
-                    ptx::tma_store_2d(&map_y, ptx::smem_u32(epi_smem + (int)slot * kEpiBufBytes), n0,
-                                      (int32_t)(m0 + c * kChunkT));
-                    ptx::tma_store_commit();
-                    ptx::tma_store_wait_read<2>();
-                    if (prev2) ptx::mbar_arrive(prev2);
-                    prev2 = prev1;
-                    prev1 = free0 + 8u * slot;
-                    ++filled[ring];
-                }
-            }
-            ptx::tma_store_wait_all<0>();
         }
     } else {
         // ------------------------------------------------------------ epilogue
@@ -955,10 +930,10 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             else
                 e.template run<false, kAmax>();
         } else if (kOut == GPUSQ_OUT_I8) {
-            EpiI8<kI8Bufs, kPhases, kTwin> e;
+            EpiI8<kTwin> e;
             e.p = &p;
             e.ctl = ctl;
-            e.epi_smem = epi_smem;
+            e.buf0 = ptx::smem_u32(epi_smem + (warp - 2) * 2 * kI8BufBytes);
             e.tmem_base = tmem_base;
             e.tmem_empty0 = tmem_empty0;
             e.tmem_empty1 = tmem_empty1;
@@ -969,8 +944,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             e.rank = (int)rank;
             e.cluster_id = cluster_id;
             e.num_clusters = num_clusters;
-            e.tiles_n = tiles_n;
-            e.num_tiles = num_tiles;
             if (p.act == GPUSQ_ACT_GELU)
                 e.template run<true>();
             else
@@ -1319,7 +1292,7 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
     if (out_type != GPUSQ_OUT_I32 && (!w_scale || !x_scale)) return GPUSQ_ERR_NULL;
     if (out_type == GPUSQ_OUT_I8 && !out_scale) return GPUSQ_ERR_NULL;
     if (M <= 0 || N <= 0 || K <= 0 || K % 16 || M > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
-    // rows of Y are written by bulk tensor stores, whose row pitch is a multiple of 16 bytes
+    // rows of Y are written by bulk tensor stores (FP16) or in 16-byte pieces (INT8)
     if ((out_type == GPUSQ_OUT_F16 && N % 8) || (out_type == GPUSQ_OUT_I8 && N % 16)) return GPUSQ_ERR_SHAPE;
     if (!aligned(Xq, 16) || !aligned(Wsrc, 16) || !aligned(Y, 16)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
@@ -1368,9 +1341,6 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
     }
     CUtensorMap map_y = map_b;      // placeholder unless the output is FP16
     if (out_type == GPUSQ_OUT_F16) ok = ok && make_map_y_f16(&map_y, Y, (uint64_t)M, (uint64_t)N);
-    // INT8 output: box = 128 features x 32 tokens, 128-byte swizzle (the INT8 staging-tile layout)
-    if (out_type == GPUSQ_OUT_I8)
-        ok = ok && make_map_u8(&map_y, Y, (uint64_t)M, (uint64_t)N, 128, (uint32_t)kChunkT, CU_TENSOR_MAP_SWIZZLE_128B);
     if (!ok) return GPUSQ_ERR_CUDA;
 
     // launches without a twin column run the instantiation that has no trace of it
@@ -1382,8 +1352,8 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
         return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
                         : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
     if (out_type == GPUSQ_OUT_I8)
-        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
+        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8, false, true>, C::threads(GPUSQ_OUT_I8), smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
+                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8>, C::threads(GPUSQ_OUT_I8), smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
     return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
                     : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
 }

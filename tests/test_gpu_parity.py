@@ -321,6 +321,22 @@ def test_epilogue_gelu_wide_range(B):
     assert f16_ulp_distance(Y, Y_o).max() <= F16_ULP_TOL
 
 
+@pytest.mark.parametrize("M", [1, 15, 16, 17, 47, 49, 225])     # edges of the 16-token chunks and of a tile
+@pytest.mark.parametrize("N", [16, 48, 144, 272])               # features that end inside a warp's 32 and inside a pair's 256
+def test_int8_output_writes_its_rows_and_nothing_else(B, M, N):
+    d, prep, Xq, xs = _prep(17 + M + N, M, N, 64)
+    acc_o = oracle.spgemm_acc(Xq, prep["vals"], prep["meta"])
+    out_scale = np.float32(0.02)
+    Q_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=0, out_type=1, out_scale=out_scale)
+    buf = torch.full((M * N + 4096,), 77, dtype=torch.int8, device="cuda")
+    Y = buf[2048:2048 + M * N].view(M, N)
+    B.spgemm_i8(cu(Xq), B.pack24(cu(prep["vals"]), cu(prep["meta"])), N, w_scale=cu(prep["w_scale"]),
+                x_scale=cu(np.array([xs], np.float32)), bias=cu(d["bias"]), out_type=B.OUT_I8,
+                out_scale=cu(np.array([out_scale], np.float32)), Y=Y)
+    assert np.array_equal(Y.cpu().numpy(), Q_o)          # integer decisions of a fixed IEEE sequence
+    assert (buf[:2048] == 77).all() and (buf[2048 + M * N:] == 77).all()
+
+
 @pytest.mark.parametrize("M,N,K,block_t", [(514, 256, 1280, 0), (197, 128, 192, 0), (1000, 384, 256, 96),
                                            (33, 128, 64, 32), (1576, 768, 192, 224), (394, 96, 48, 0),
                                            (500, 288, 96, 64), (333, 576, 192, 0), (70, 16, 16, 0)])
