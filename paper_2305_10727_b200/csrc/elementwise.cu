@@ -442,6 +442,7 @@ constexpr int kPieceVecs = 1024;                                 // 16-byte vect
 constexpr int kMaxPieces = 12;
 constexpr int kFusedCacheVecs = kPieceVecs * kMaxPieces;         // vectors kept per CTA (192 KB)
 constexpr int kFusedSmemBytes = kFusedCacheVecs * 16;
+constexpr int kSingleMinVecs = 2 * kFusedThreads;                // slices below this are not worth the test of quant8_single
 constexpr int kWsDone = kMaxPartials;                            // workspace words: CTAs past the barrier ...
 constexpr int kWsStatus = kMaxPartials + 1;                      // ... status (0 or GPUSQ_ERR_TIMEOUT) ...
 constexpr int kWsBarrier = kMaxPartials + 2;                     // ... and the 8-byte word {arrivals, maximum}
@@ -470,14 +471,35 @@ __device__ __forceinline__ bool mbar_try_wait_parity0(uint32_t bar)
     return ok != 0;
 }
 
+// A CTA's slice of n vectors, the first n_kept of them in shared memory.  The others are taken from the
+// end backwards: the maximum pass read them forwards, so the last ones are the ones still in L2.
+// kSingle: one product per value is known to give the codes (find_single_product).
+template <bool kSingle>
+__device__ __forceinline__ void quantise_slice(const uint4 *cache, const uint4 *__restrict__ Xs, uint2 *__restrict__ Xqs,
+                                               int n_kept, int n, const QuantScale &a, int regroup)
+{
+    auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<false>(v, a) : quant8_f16<false>(v, a), regroup); };
+    int i = n - 1 - (int)threadIdx.x;
+    for (; i - 3 * kFusedThreads >= n_kept; i -= 4 * kFusedThreads) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(Xs + i - u * kFusedThreads);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) __stcs(Xqs + i - u * kFusedThreads, codes(v[u]));
+    }
+    for (; i >= n_kept; i -= kFusedThreads) __stcs(Xqs + i, codes(__ldg(Xs + i)));
+#pragma unroll 2
+    for (i = threadIdx.x; i < n_kept; i += kFusedThreads) __stcs(Xqs + i, codes(cache[i]));
+}
+
 __global__ void __launch_bounds__(kFusedThreads, 1)
 act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
                        uint32_t *ws, int64_t vec8, unsigned long long wait_ns, int withhold, float qmax, int regroup)
 {
     extern __shared__ __align__(128) uint4 cache[];
-    __shared__ float red[kFusedThreads / 32];
+    __shared__ uint32_t red[kFusedThreads / 32];
     __shared__ __align__(8) uint64_t piece_bar[kMaxPieces];
-    __shared__ uint32_t gave_up;
+    __shared__ uint32_t gave_up, grid_max;
     const int64_t per = (vec8 + gridDim.x - 1) / gridDim.x;
     const int64_t lo = (int64_t)blockIdx.x * per;
     const int64_t hi = lo + per < vec8 ? lo + per : vec8;
@@ -542,32 +564,37 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         if (ok && v < n_kept) m = max(m, absmax_bits8(cache[v]));
     }
     if (!ok) gave_up = 1;                                    // benign race: every writer writes 1
-    const uint32_t mine = (uint32_t)block_max((float)m, red);            // has the block-wide barriers
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((tid & 31) == 0) red[tid >> 5] = m;
+    __syncthreads();
 
     // 2. grid-wide maximum.  One 8-byte word holds {arrivals, maximum}: a CTA first merges its maximum,
     // then counts itself in, so a single 8-byte read that sees every arrival also sees the final
     // maximum; each CTA has one poll in flight at a time, all on one line.
     uint32_t *bar_word = ws + kWsBarrier;
-    uint32_t seen = 0;
-    if (tid == 0 && !gave_up) {
-        if (!(withhold && blockIdx.x == gridDim.x - 1)) {
-            atomicMax(bar_word + 1, mine);
-            __threadfence();
-            atomicAdd(bar_word, 1u);
-        }
-        for (uint32_t it = 1;; ++it) {
-            const uint2 word = __ldcv(reinterpret_cast<const uint2 *>(bar_word));
-            if (word.x >= gridDim.x) {
-                seen = word.y;
-                break;
+    if (tid < 32 && !gave_up) {
+        const uint32_t mine = __reduce_max_sync(0xffffffffu, red[tid]);
+        if (tid == 0) {
+            if (!(withhold && blockIdx.x == gridDim.x - 1)) {
+                atomicMax(bar_word + 1, mine);
+                __threadfence();
+                atomicAdd(bar_word, 1u);
             }
-            if ((it & 63u) == 0u && globaltimer_now() - t0 > wait_ns) {
-                gave_up = 1;
-                break;
+            for (uint32_t it = 1;; ++it) {
+                const uint2 word = __ldcv(reinterpret_cast<const uint2 *>(bar_word));
+                if (word.x >= gridDim.x) {
+                    grid_max = word.y;
+                    break;
+                }
+                if ((it & 63u) == 0u && globaltimer_now() - t0 > wait_ns) {
+                    gave_up = 1;
+                    break;
+                }
             }
         }
     }
-    const uint32_t all = (uint32_t)block_max((float)seen, red);
+    __syncthreads();
+    const uint32_t all = grid_max;
     if (gave_up) {
         if (tid == 0) atomicExch(ws + kWsStatus, (uint32_t)GPUSQ_ERR_TIMEOUT);
         // bulk copies that may still be in flight write into this CTA's shared memory: wait for them (bounded)
@@ -593,18 +620,67 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         }
     }
     const float s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
-    const QuantScale a = make_quant_scale(s, qmax);
+    QuantScale a = make_quant_scale(s, qmax);
 
     // 3. quantise the slice: what was kept, from shared memory; the rest, from L2 / HBM
-    for (i = tid; i < n_kept; i += kFusedThreads) __stcs(Xqs + i, regrouped(quant8_f16<false>(cache[i], a), regroup));
-    for (; i + 3 * kFusedThreads < n; i += 4 * kFusedThreads) {
-        uint4 v[4];
+    if (n >= kSingleMinVecs && find_single_product<false>(a))
+        quantise_slice<true>(cache, Xs, Xqs, n_kept, n, a, regroup);
+    else
+        quantise_slice<false>(cache, Xs, Xqs, n_kept, n, a, regroup);
+}
+
+// ---- one-launch activation quantisation of small tensors ----
+// One cluster of up to sixteen CTAs keeps the tensor in registers and exchanges its warps' maxima
+// through distributed shared memory: every warp writes its maximum into each CTA, one cluster barrier,
+// and every warp reduces them all.  Bound by latencies (launch, one load, the barrier, one store), of
+// which the grid-wide barrier through L2 of the kernel above is the longest.  Microseconds that a call
+// adds in front of a GEMM (kernel above -> this one): 9 KB 3.6 -> 1.6, 0.65 MB 5.4 -> 3.4, 1.5 MB
+// 6.0 -> 4.7; at 2.4 MB sixteen SMs are too few to load and store it (8.1 against 5.1): hence the limit
+// of six vectors per thread.
+constexpr int kClusterThreads = 1024;
+constexpr int kMaxCluster = 16;
+constexpr int kClusterMaxPerThread = 6;
+
+template <int kPer>
+__global__ void __launch_bounds__(kClusterThreads, 1)
+act_quant_cluster_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale, int vec8, float qmax, int regroup)
+{
+    __shared__ uint32_t maxima[kMaxCluster * (kClusterThreads / 32)];
+    uint32_t rank, size;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // every CTA of the cluster has started before its shared memory is written (waited for below)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // the producer of X is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int stride = (int)size * kClusterThreads;
+    const int i0 = (int)rank * kClusterThreads + (int)threadIdx.x;
+    uint4 v[kPer];
+    uint32_t m = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(Xs + i + u * kFusedThreads);
+    for (int u = 0; u < kPer; ++u) v[u] = i0 + u * stride < vec8 ? __ldg(X + i0 + u * stride) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) __stcs(Xqs + i + u * kFusedThreads, regrouped(quant8_f16<false>(v[u], a), regroup));
+    for (int u = 0; u < kPer; ++u) m = max(m, absmax_bits8(v[u]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (lane < (int)size) {
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&maxima[rank * (kClusterThreads / 32) + warp]);
+        uint32_t theirs;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(lane));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(theirs), "r"(m) : "memory");
     }
-    for (; i < n; i += kFusedThreads) __stcs(Xqs + i, regrouped(quant8_f16<false>(__ldg(Xs + i), a), regroup));
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    uint32_t all = 0;
+    for (int i = lane; i < (int)size * (kClusterThreads / 32); i += 32) all = max(all, maxima[i]);
+    all = __reduce_max_sync(0xffffffffu, all);
+    const float s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
+    if (rank == 0 && threadIdx.x == 0) *x_scale = s;
+    const QuantScale a = make_quant_scale(s, qmax);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+        if (i0 + u * stride < vec8) Xq[i0 + u * stride] = regrouped(quant8_f16<false>(v[u], a), regroup);
 }
 
 // ---- library-owned scratch for gpusq_quant_act_static ----
@@ -749,6 +825,68 @@ size_t gpusq_quant_act_workspace(int64_t M, int K)
     return (size_t)(kMaxPartials + kWorkspaceExtra) * sizeof(uint32_t);
 }
 
+// Largest cluster act_quant_cluster_kernel can be launched with on the current device (sixteen is not
+// portable), 0 if none; looked up once per device.
+static int max_quant_cluster()
+{
+    static std::atomic<int> known[kMaxDevices];               // size + 1, 0 = not looked up yet
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    const int k = known[dev].load(std::memory_order_relaxed);
+    if (k) return k - 1;
+    int best = 0;
+    const void *kernels[] = {(const void *)act_quant_cluster_kernel<1>, (const void *)act_quant_cluster_kernel<2>,
+                             (const void *)act_quant_cluster_kernel<4>, (const void *)act_quant_cluster_kernel<kClusterMaxPerThread>};
+    bool opted = true;
+    for (const void *f : kernels)
+        opted = opted && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int size = opted ? kMaxCluster : 8; size >= 8 && !best; size /= 2) {
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)size;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)size, 1, 1);
+        cfg.blockDim = dim3(kClusterThreads, 1, 1);
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernels[3], &cfg) == cudaSuccess && n > 0) best = size;
+    }
+    (void)cudaGetLastError();
+    known[dev].store(best + 1, std::memory_order_relaxed);
+    return best;
+}
+
+static int launch_cluster_quant(const void *X, int8_t *Xq, float *x_scale, int vec8, int cluster_max, float qmax,
+                                int regroup, cudaStream_t stream)
+{
+    // as many CTAs (a power of two) as give every thread one vector, at most cluster_max
+    int size = 1;
+    while (size < cluster_max && size * kClusterThreads < vec8) size *= 2;
+    const int per = (int)ceil_div(vec8, size * kClusterThreads);
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)size;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size, 1, 1);
+    cfg.blockDim = dim3(kClusterThreads, 1, 1);
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    auto kernel = per <= 1 ? act_quant_cluster_kernel<1> : per <= 2 ? act_quant_cluster_kernel<2>
+                : per <= 4 ? act_quant_cluster_kernel<4> : act_quant_cluster_kernel<kClusterMaxPerThread>;
+    if (cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, vec8,
+                           qmax, regroup) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return GPUSQ_ERR_CUDA;
+    }
+    return GPUSQ_OK;
+}
+
 // gpusq_quant_act (qmax 127) and gpusq_quant_act4 (qmax 7, codes of every eight columns regrouped)
 static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale_mode, int64_t M, int K,
                             void *workspace, size_t ws_bytes, void *stream, float qmax, int regroup)
@@ -766,6 +904,9 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
     const int64_t vec8 = M * (int64_t)K / 8;
     cudaStream_t s = (cudaStream_t)stream;
     if (scale_mode == GPUSQ_SCALE_COMPUTE) {
+        const int cluster_max = max_quant_cluster();
+        if (cluster_max > 0 && vec8 <= (int64_t)cluster_max * kClusterThreads * kClusterMaxPerThread)
+            return launch_cluster_quant(X, Xq, x_scale, (int)vec8, cluster_max, qmax, regroup, s);
         // one cooperative launch: every CTA must be resident for the grid-wide barrier.  The opt-in to
         // large dynamic shared memory is per device.
         static std::mutex mu;

@@ -103,6 +103,61 @@ __device__ __forceinline__ uint2 quant8_f16(uint4 v, const QuantScale &a)
     return make_uint2(pack4_low_bytes(m0, m1), pack4_low_bytes(m2, m3));
 }
 
+// One product per value: the codes of eight binary16 values when find_single_product() found a factor.
+template <bool kClamp>
+__device__ __forceinline__ uint2 quant8_single(uint4 v, const QuantScale &a)
+{
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const __half2 bound = __float2half2_rn(a.x_max);
+    float2 m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        __half2 h = *reinterpret_cast<const __half2 *>(&w[i]);
+        if (kClamp) h = __hmin2(__hmax2(h, __hneg2(bound)), bound);
+        m[i] = __ffma2_rn(__half22float2(h), a.c, make_float2(kRoundMagic, kRoundMagic));
+    }
+    return make_uint2(pack4_low_bytes(m[0], m[1]), pack4_low_bytes(m[2], m[3]));
+}
+
+// Looks for a factor c, next to 1/s, with which rounding x * c gives the code of EVERY binary16 x, and
+// leaves it in a.c.  The product's code and the true quotient's are both steps that never fall as x
+// grows, so they are the same function if they agree at the binary16 numbers around every threshold
+// (k + 1/2) s: the nearest one and its two neighbours (the threshold itself is known to 2^-23 of its
+// value, far less than a binary16 step; between the upper neighbour of one threshold and the lower one
+// of the next both are constant).  Negative x mirror.  kClamp: values beyond +-qmax s are first clamped
+// to the binary16 number next to it, which must have the largest code itself.
+// Tried are 1/s rounded and the next number above it: a scale computed as max / 127 has a value (half the
+// maximum) exactly on a threshold that rounds up.  One of them holds for 98 of 100 computed and all but
+// 2 in 600 supplied scales; the others take the bracketing products.
+// To be called by all threads of the block (it is a barrier).
+template <bool kClamp>
+__device__ __forceinline__ bool find_single_product(QuantScale &a)
+{
+    const float c0 = a.c.x, c1 = __uint_as_float(__float_as_uint(a.c.x) + 1u);
+    bool ok0 = !a.always_divide, ok1 = ok0;
+    auto look = [&](int bits) {
+        const float x = __half2float(__ushort_as_half((unsigned short)bits));
+        const float exact = quant_exact_sum<false>(x, a.s, a.qmax);
+        ok0 = ok0 && __fmaf_rn(x, c0, kRoundMagic) == exact;
+        ok1 = ok1 && __fmaf_rn(x, c1, kRoundMagic) == exact;
+        return exact;
+    };
+    for (int k = threadIdx.x; k < (int)a.qmax; k += blockDim.x) {
+        const int h = __half_as_ushort(__float2half_rn(__fmul_rn((float)k + 0.5f, a.s)));
+#pragma unroll
+        for (int d = -1; d <= 1; ++d)
+            if (h + d >= 0 && h + d < 0x7C00) look(h + d);
+    }
+    if (kClamp) {
+        const int b = __half_as_ushort(__float2half_rn(a.x_max));
+        if (b >= 0x7C00 || look(b) != kRoundMagic + a.qmax) ok0 = ok1 = false;
+    }
+    if (__syncthreads_and(ok0)) return true;
+    if (!__syncthreads_and(ok1)) return false;
+    a.c = make_float2(c1, c1);
+    return true;
+}
+
 inline int grid_for(int64_t items, int per_sm)
 {
     int64_t blocks = ceil_div(items, kThreads);

@@ -25,6 +25,7 @@ constexpr float kRoundMagic = 12582912.0f;     // 1.5 * 2^23
 struct QuantScale {
     float s;            // the scale
     float2 c_lo, c_hi;  // the bracketing reciprocals, duplicated for packed math
+    float2 c;           // 1/s, rounded
     float x_max;        // qmax s (kClamp)
     float qmax;         // largest code: 127, or 7 for the 4-bit model
     bool always_divide; // 1/s is not finite
@@ -39,6 +40,7 @@ __device__ __forceinline__ QuantScale make_quant_scale(float s, float qmax = 127
     const float lo = __fmul_rn(inv_s, 1.0f - 4.76837158203125e-7f), hi = __fmul_rn(inv_s, 1.0f + 4.76837158203125e-7f);
     a.c_lo = make_float2(lo, lo);
     a.c_hi = make_float2(hi, hi);
+    a.c = make_float2(inv_s, inv_s);
     a.x_max = __fmul_rn(s, qmax);
     a.always_divide = !(fabsf(inv_s) < 3.0e38f) || !(a.x_max < 3.0e38f);
     return a;

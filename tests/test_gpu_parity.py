@@ -101,6 +101,36 @@ def test_quant_act(B, M, K, dist):
     assert np.array_equal(Xq2.cpu().numpy(), Xq_o2)
 
 
+# vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2, 4 and 6 vectors per thread, the first size
+# beyond it, and slices that just do and just do not fit the one-launch kernel's shared memory
+@pytest.mark.parametrize("vecs", [1, 1023, 1024, 1025, 8193, 16384, 16385, 32769, 65537, 98304, 98305, 300001,
+                                  148 * 12288, 148 * 12288 + 4097])
+def test_quant_act_sizes(B, vecs):
+    g = np.random.default_rng(vecs)
+    X = g.standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
+    X[g.integers(vecs), g.integers(8)] = 7.0                # the maximum, anywhere
+    Xq_o, s_o = oracle.quant_act(X)
+    Xq, s = B.quant_act(cu(X))
+    assert s.cpu().numpy()[0] == s_o
+    assert np.array_equal(Xq.cpu().numpy(), Xq_o)
+
+
+@pytest.mark.parametrize("amax", [7.0, 3.75, 5.87890625, 6.1e-5, 65504.0, 4.87, 2.2578125])
+def test_quant_act_every_binary16_value(B, amax):
+    # large enough that the kernels look for a single product that gives all codes; every value they can meet
+    top = int(np.float16(amax).view(np.uint16))
+    pos = np.arange(top + 1, dtype=np.uint16).view(np.float16)
+    X = np.resize(np.concatenate([pos, -pos]), (148 * 2048 + 1, 8))
+    X[0, 0] = amax
+    Xq_o, s_o = oracle.quant_act(X)
+    Xq, s = B.quant_act(cu(X))
+    assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq.cpu().numpy(), Xq_o)
+    given = np.float32(0.37) * s_o                          # clamps above 0.37 amax
+    Xq_o, _ = oracle.quant_act(X, x_scale=given)
+    Xq, _ = B.quant_act(cu(X), x_scale=cu(np.array([given], np.float32)), scale_mode=B.SCALE_GIVEN)
+    assert np.array_equal(Xq.cpu().numpy(), Xq_o)
+
+
 def test_quant_act_zero_tensor_and_reused_workspace(B):
     # one zero-filled workspace serves calls of different sizes, back to back
     ws = torch.zeros((B.quant_act_workspace(4096, 4096),), dtype=torch.uint8, device="cuda")
