@@ -273,15 +273,40 @@ __device__ __forceinline__ uint2 regrouped(uint2 q, int regroup)
     return regroup ? make_uint2(__byte_perm(q.x, q.y, 0x6420), __byte_perm(q.x, q.y, 0x7531)) : q;
 }
 
+// One pass over a tensor whose scale is known, four vectors in flight per thread.
+// kSingle: one product per value is known to give the codes (find_single_product).
+template <bool kSingle>
+__device__ __forceinline__ void quantise_strided(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, int64_t vec8,
+                                                 const QuantScale &a, int regroup)
+{
+    auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<true>(v, a) : quant8_f16<true>(v, a), regroup); };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; i + 3 * stride < vec8; i += 4 * stride) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(X + i + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) Xq[i + u * stride] = codes(v[u]);
+    }
+    for (; i < vec8; i += stride) Xq[i] = codes(__ldg(X + i));
+}
+
 // n_partials > 0: the scale is derived from the partial maxima and written to
 // *x_scale by block 0; absmax != NULL: it is derived from *absmax (the tensor's maximum magnitude,
 // left there by the kernel that produced X) and written; otherwise *x_scale is read.
-__global__ void __launch_bounds__(kThreads)
+// Bound by HBM: back to back on cold tensors 51.6 MB take 14.6 us (17.1 with two loads in flight, two
+// waves of blocks and the bracketing products), 11.8 being what the bytes need; in front of a GEMM
+// 19.4 MB add 7.3 us (8.3), 0.65 MB 1.6 (2.7).
+constexpr int kQuantBlocksPerSm = 4;      // what 64 registers a thread leave room for: one wave
+__global__ void __launch_bounds__(kThreads, kQuantBlocksPerSm)
 act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
                  const uint32_t *__restrict__ partial, int n_partials, int64_t vec8,
-                 const float *__restrict__ absmax = nullptr, float qmax = 127.0f, int regroup = 0)
+                 const float *__restrict__ absmax, float qmax, int regroup)
 {
     __shared__ float red[kThreads / 32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float s;
     if (absmax) {
         s = scale_from_amax(__ldg(absmax), qmax);
@@ -296,15 +321,20 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
     } else {
         s = *x_scale;
     }
-    const QuantScale a = make_quant_scale(s, qmax);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + stride < vec8; i += 2 * stride) {
-        const uint4 v0 = __ldg(X + i), v1 = __ldg(X + i + stride);
-        Xq[i] = regrouped(quant8_f16<true>(v0, a), regroup);
-        Xq[i + stride] = regrouped(quant8_f16<true>(v1, a), regroup);
-    }
-    for (; i < vec8; i += stride) Xq[i] = regrouped(quant8_f16<true>(__ldg(X + i), a), regroup);
+    QuantScale a = make_quant_scale(s, qmax);
+    // the test of the single product pays from four vectors per thread on
+    if (vec8 >= 4 * (int64_t)gridDim.x * blockDim.x && find_single_product<true>(a))
+        quantise_strided<true>(X, Xq, vec8, a, regroup);
+    else
+        quantise_strided<false>(X, Xq, vec8, a, regroup);
+}
+
+static int launch_act_quant(const void *X, int8_t *Xq, float *x_scale, const uint32_t *partial, int n_partials, int64_t vec8,
+                            const float *absmax, float qmax, int regroup, cudaStream_t stream)
+{
+    return launch_behind(act_quant_kernel, grid_for(vec8, kQuantBlocksPerSm), kThreads, stream,
+                         reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, partial, n_partials,
+                         vec8, absmax, qmax, regroup);
 }
 
 // ---- patch embedding (Sec. 3.3): quantise an image batch and lay it out as the GEMM's rows ----
@@ -345,23 +375,10 @@ struct PatchGeom {
     FastDiv by_row, by_pp, by_p, by_t, by_tx;   // divisors Kp / kVec, P P, P, T, Tx
 };
 
-template <int kVec>
-__global__ void __launch_bounds__(kThreads)
-patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, float *x_scale,
-                   const uint32_t *__restrict__ partial, int n_partials, const PatchGeom g, uint32_t items)
+template <int kVec, bool kSingle>
+__device__ __forceinline__ void patch_quantise(const __half *__restrict__ img, int8_t *__restrict__ Xq, const PatchGeom &g,
+                                               uint32_t items, const QuantScale &a)
 {
-    __shared__ float red[kThreads / 32];
-    float s;
-    if (n_partials > 0) {
-        uint32_t m = 0;
-        for (int i = threadIdx.x; i < n_partials; i += blockDim.x) m = max(m, __ldg(partial + i));
-        const uint32_t bits = (uint32_t)block_max((float)m, red);
-        s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)bits)));
-        if (blockIdx.x == 0 && threadIdx.x == 0) *x_scale = s;
-    } else {
-        s = *x_scale;
-    }
-    const QuantScale a = make_quant_scale(s);
     // item i -> where its codes go, and where its pixels are (nullptr in the padding columns);
     // every dividend is below `items` < 2^31
     auto locate = [&](uint32_t i, int8_t *&dst) -> const __half * {
@@ -392,7 +409,7 @@ patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, floa
     };
     auto emit = [&](uint4 v, int8_t *dst) {                // code(0) = 0: the padding needs no special case
         if (kVec == 8) {
-            *reinterpret_cast<uint2 *>(dst) = quant8_f16<true>(v, a);
+            *reinterpret_cast<uint2 *>(dst) = kSingle ? quant8_single<true>(v, a) : quant8_f16<true>(v, a);
         } else {
             uint32_t differ = 0;
             const float2 f0 = h2f(v.x), f1 = h2f(v.y);
@@ -408,18 +425,44 @@ patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, floa
     };
     const uint32_t stride = gridDim.x * blockDim.x;
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i < items && stride < items - i; i += 2 * stride) {       // two items in flight per thread
-        int8_t *d0, *d1;
-        const __half *s0 = locate(i, d0), *s1 = locate(i + stride, d1);
-        const uint4 v0 = fetch(s0), v1 = fetch(s1);
-        emit(v0, d0);
-        emit(v1, d1);
+    for (; i < items && 3 * stride < items - i; i += 4 * stride) {   // four items in flight per thread
+        int8_t *d[4];
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = fetch(locate(i + u * stride, d[u]));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) emit(v[u], d[u]);
     }
-    if (i < items) {
+    for (; i < items; i = stride < items - i ? i + stride : items) {
         int8_t *d0;
         const __half *s0 = locate(i, d0);
         emit(fetch(s0), d0);
     }
+}
+
+template <int kVec>
+__global__ void __launch_bounds__(kThreads, kQuantBlocksPerSm)
+patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, float *x_scale,
+                   const uint32_t *__restrict__ partial, int n_partials, const PatchGeom g, uint32_t items)
+{
+    __shared__ float red[kThreads / 32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float s;
+    if (n_partials > 0) {
+        uint32_t m = 0;
+        for (int i = threadIdx.x; i < n_partials; i += blockDim.x) m = max(m, __ldg(partial + i));
+        const uint32_t bits = (uint32_t)block_max((float)m, red);
+        s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)bits)));
+        if (blockIdx.x == 0 && threadIdx.x == 0) *x_scale = s;
+    } else {
+        s = *x_scale;
+    }
+    QuantScale a = make_quant_scale(s);
+    if (kVec == 8 && items / 4 >= gridDim.x * blockDim.x && find_single_product<true>(a))
+        patch_quantise<kVec, true>(img, Xq, g, items, a);
+    else
+        patch_quantise<kVec, false>(img, Xq, g, items, a);
 }
 
 // ---- one-launch activation quantisation (scale computed from the tensor) ----
@@ -951,10 +994,7 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         }
         return GPUSQ_OK;
     }
-    act_quant_kernel<<<grid_for(ceil_div(vec8, 2), 8), kThreads, 0, s>>>(
-        reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, nullptr, 0, vec8, nullptr, qmax,
-        regroup);
-    return launch_status();
+    return launch_act_quant(X, Xq, x_scale, nullptr, 0, vec8, nullptr, qmax, regroup, s);
 }
 
 int gpusq_quant_act(const void *X, int8_t *Xq, float *x_scale, int scale_mode, int64_t M, int K,
@@ -978,9 +1018,7 @@ int gpusq_quant_act_absmax(const void *X, int8_t *Xq, float *x_scale, const floa
     if (!aligned(X, 16) || !aligned(Xq, 16)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t vec8 = M * (int64_t)K / 8;
-    act_quant_kernel<<<grid_for(ceil_div(vec8, 2), 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, nullptr, 0, vec8, absmax);
-    return launch_status();
+    return launch_act_quant(X, Xq, x_scale, nullptr, 0, vec8, absmax, 127.0f, 0, (cudaStream_t)stream);
 }
 
 int gpusq_set_quant_act_wait(unsigned long long limit_ns, int withhold_last_cta)
@@ -1007,14 +1045,12 @@ int gpusq_quant_act_static(const void *X, int8_t *Xq, float *x_scale, int scale_
     int n_partials = 0;
     if (scale_mode == GPUSQ_SCALE_COMPUTE) {
         // every slot that is read below is written here first, so stale contents do not matter
-        n_partials = grid_for(ceil_div(vec8, 4), 8);
-        if (n_partials > kMaxPartials) n_partials = kMaxPartials;
-        act_absmax_kernel<<<n_partials, kThreads, 0, s>>>(reinterpret_cast<const uint4 *>(X), scratch, vec8);
-        if (int st = launch_status()) return st;
+        n_partials = absmax_blocks(vec8);
+        if (int st = launch_behind(act_absmax_kernel, n_partials, kAbsmaxThreads, s, reinterpret_cast<const uint4 *>(X),
+                                   scratch, vec8))
+            return st;
     }
-    act_quant_kernel<<<grid_for(ceil_div(vec8, 2), 8), kThreads, 0, s>>>(
-        reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, scratch, n_partials, vec8);
-    return launch_status();
+    return launch_act_quant(X, Xq, x_scale, scratch, n_partials, vec8, nullptr, 127.0f, 0, s);
 }
 
 int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mode, int B, int C, int H, int W,
@@ -1044,10 +1080,10 @@ int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mod
         // the partial maxima use the first words of the workspace, every one written before it is
         // read; the words behind them (gpusq_quant_act's barrier) are not touched
         const int64_t vec8 = elems / 8;
-        n_partials = grid_for(ceil_div(vec8, 4), 8);
-        if (n_partials > kMaxPartials) n_partials = kMaxPartials;
-        act_absmax_kernel<<<n_partials, kThreads, 0, s>>>(reinterpret_cast<const uint4 *>(img), partial, vec8);
-        if (int st = launch_status()) return st;
+        n_partials = absmax_blocks(vec8);
+        if (int st = launch_behind(act_absmax_kernel, n_partials, kAbsmaxThreads, s, reinterpret_cast<const uint4 *>(img),
+                                   partial, vec8))
+            return st;
     }
     PatchGeom g;
     g.C = C; g.H = H; g.W = W; g.P = P;
@@ -1058,15 +1094,9 @@ int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mod
     g.by_p = make_fast_div((uint32_t)P);
     g.by_t = make_fast_div((uint32_t)g.T);
     g.by_tx = make_fast_div((uint32_t)g.Tx);
-    const int grid = grid_for(items, 8);
-    const __half *src = reinterpret_cast<const __half *>(img);
-    if (vec == 8)
-        patch_quant_kernel<8><<<grid, kThreads, 0, s>>>(src, Xq, x_scale, partial, n_partials, g, (uint32_t)items);
-    else if (vec == 4)
-        patch_quant_kernel<4><<<grid, kThreads, 0, s>>>(src, Xq, x_scale, partial, n_partials, g, (uint32_t)items);
-    else
-        patch_quant_kernel<2><<<grid, kThreads, 0, s>>>(src, Xq, x_scale, partial, n_partials, g, (uint32_t)items);
-    return launch_status();
+    const auto kernel = vec == 8 ? patch_quant_kernel<8> : vec == 4 ? patch_quant_kernel<4> : patch_quant_kernel<2>;
+    return launch_behind(kernel, grid_for(items, kQuantBlocksPerSm), kThreads, s, reinterpret_cast<const __half *>(img), Xq,
+                         x_scale, (const uint32_t *)partial, n_partials, g, (uint32_t)items);
 }
 
 const char *gpusq_status_string(int status)

@@ -66,22 +66,36 @@ __device__ __forceinline__ uint32_t absmax_bits8(uint4 v)
     return max(a & 0xFFFFu, a >> 16);
 }
 
-static __global__ void __launch_bounds__(kThreads)
+// Partial maxima, one per block of at most two per SM: eight 16-byte loads in flight per thread.
+constexpr int kAbsmaxThreads = 512;
+static __global__ void __launch_bounds__(kAbsmaxThreads)
 act_absmax_kernel(const uint4 *__restrict__ X, uint32_t *__restrict__ partial, int64_t vec8)
 {
-    __shared__ float red[kThreads / 32];
+    __shared__ uint32_t red[kAbsmaxThreads / 32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t m = 0;
-    for (; i + 3 * stride < vec8; i += 4 * stride) {
-        uint4 v0 = __ldg(X + i), v1 = __ldg(X + i + stride), v2 = __ldg(X + i + 2 * stride),
-              v3 = __ldg(X + i + 3 * stride);
-        m = max(max(m, absmax_bits8(v0)), max(absmax_bits8(v1), max(absmax_bits8(v2), absmax_bits8(v3))));
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vec8; i += 8 * stride) {
+        uint4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i + u * stride < vec8 ? __ldg(X + i + u * stride) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m = max(m, absmax_bits8(v[u]));
     }
-    for (; i < vec8; i += stride) m = max(m, absmax_bits8(__ldg(X + i)));
-    // binary16 bit patterns below 0x8000 are exact small integers in binary32: reuse the float reduction
-    const float r = block_max((float)m, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = (uint32_t)r;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xffffffffu, threadIdx.x < kAbsmaxThreads / 32 ? red[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) partial[blockIdx.x] = m;
+    }
+}
+
+inline int absmax_blocks(int64_t vec8)
+{
+    const int64_t want = ceil_div(vec8, kAbsmaxThreads), most = 2 * (int64_t)num_sms();
+    return (int)(want < most ? want : most < kMaxPartials ? most : kMaxPartials);
 }
 
 // eight binary16 values (16 bytes) -> eight INT8 codes (8 bytes); one exactness test for all eight
@@ -165,5 +179,25 @@ inline int grid_for(int64_t items, int per_sm)
     return (int)(blocks < cap ? (blocks < 1 ? 1 : blocks) : cap);
 }
 
+// Launch that may be set up while the previous kernel of the stream drains; the kernel itself waits
+// (griddepcontrol.wait) before it touches memory.
+template <typename... P, typename... A>
+inline int launch_behind(void (*kernel)(P...), int grid, int threads, cudaStream_t stream, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.stream = stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return GPUSQ_ERR_CUDA;
+    }
+    return GPUSQ_OK;
+}
 
 }  // namespace gpusq

@@ -120,7 +120,7 @@ def test_quant_act_every_binary16_value(B, amax):
     # large enough that the kernels look for a single product that gives all codes; every value they can meet
     top = int(np.float16(amax).view(np.uint16))
     pos = np.arange(top + 1, dtype=np.uint16).view(np.float16)
-    X = np.resize(np.concatenate([pos, -pos]), (148 * 2048 + 1, 8))
+    X = np.resize(np.concatenate([pos, -pos]), (16 * 148 * 256 + 1, 8))
     X[0, 0] = amax
     Xq_o, s_o = oracle.quant_act(X)
     Xq, s = B.quant_act(cu(X))
