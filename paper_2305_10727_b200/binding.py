@@ -31,6 +31,7 @@ EXPORTS = (
 )
 
 _lib = None
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 class GpusqError(RuntimeError):
@@ -101,12 +102,15 @@ def _check(status: int, where: str) -> None:
         raise GpusqError(status, where)
 
 
+# Addresses are passed as plain integers (the argument types convert them) and the stream is asked for as
+# its handle: a pointer object per argument and a Stream object per call cost 5 of the 10 us that a call
+# took on the host, more than most kernels of a small batch run.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    return _raw_stream(_current_device())
 
 
 def _dev(t: torch.Tensor, dtype, what: str) -> torch.Tensor:
