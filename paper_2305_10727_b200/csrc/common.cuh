@@ -31,11 +31,6 @@ inline int num_sms()
     return n;
 }
 
-inline int launch_status()
-{
-    return cudaGetLastError() == cudaSuccess ? GPUSQ_OK : GPUSQ_ERR_CUDA;
-}
-
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 

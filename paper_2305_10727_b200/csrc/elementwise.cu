@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(kThreads)
 prune24_kernel(const float4 *__restrict__ W, float4 *Wp, uint8_t *mask, int64_t groups)
 {
     // W and Wp may be the same buffer: every thread reads a group before it writes it.
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (; i + (UNROLL - 1) * stride < groups; i += UNROLL * stride) {
@@ -49,13 +50,60 @@ prune24_kernel(const float4 *__restrict__ W, float4 *Wp, uint8_t *mask, int64_t 
     }
 }
 
-// One block per output channel (row): pass 1 finds max|w|, pass 2 re-reads the
-// row (L1/L2 resident: a row is at most 20 KB) and writes four codes per store.
+// ------------------------------------------------------------- quant_weight
+// Symmetric per-row quantisation.  A row sits in the registers of one warp (kBlockRow = false, rows of
+// up to 1024) or of one block (up to 8192), kPer float4 per thread: one pass over the weights, no barrier
+// in the warp form, and the codes by the bracketing products instead of a division per weight.  Bound by
+// launch and latency below some 20 MB; a block per row, two reads and a division per weight against this:
+// 3072 x 1024 10.4 -> 3.7 us, 1024 x 4096 11.6 -> 4.4 us.
+template <int kPer, bool kBlockRow>
 __global__ void __launch_bounds__(kThreads)
-quant_weight_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq,
-                    float *__restrict__ w_scale, int N, int K4)
+quant_weight_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq, float *__restrict__ w_scale, int N, int K4,
+                    float qmax)
+{
+    __shared__ uint32_t red[kThreads / 32];
+    constexpr int T = kBlockRow ? kThreads : 32;           // threads per row
+    const int n = kBlockRow ? (int)blockIdx.x : (int)(blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5));
+    const int t = kBlockRow ? (int)threadIdx.x : (int)(threadIdx.x & 31);
+    begin_behind();
+    if (n >= N) return;                                    // whole warps only
+    const float4 *row = Wp + (int64_t)n * K4;
+    float4 v[kPer];
+    float m = 0.0f;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) v[u] = t + u * T < K4 ? __ldg(row + t + u * T) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) m = fmaxf(m, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
+    uint32_t bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));      // non-negative floats order like their patterns
+    if (kBlockRow) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = bits;
+        __syncthreads();
+        bits = __reduce_max_sync(0xffffffffu, red[threadIdx.x & (kThreads / 32 - 1)]);
+    }
+    const float s = scale_from_amax(__uint_as_float(bits), qmax);
+    if (t == 0) w_scale[n] = s;
+    const QuantScale a = make_quant_scale(s, qmax);
+    uint32_t *out = Wq + (int64_t)n * K4;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const float2 f0 = make_float2(v[u].x, v[u].y), f1 = make_float2(v[u].z, v[u].w);
+        uint32_t differ = 0;
+        float2 m0 = quant2_sums<false>(f0, a, differ), m1 = quant2_sums<false>(f1, a, differ);
+        if (differ != 0u || a.always_divide) {
+            m0 = quant2_exact<true>(f0, a);
+            m1 = quant2_exact<true>(f1, a);
+        }
+        if (t + u * T < K4) out[t + u * T] = pack4_low_bytes(m0, m1);
+    }
+}
+
+// Rows longer than the registers of a block: the row is read twice (the second time out of L1 / L2).
+__global__ void __launch_bounds__(kThreads)
+quant_weight_long_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq,
+                         float *__restrict__ w_scale, int N, int K4, float qmax)
 {
     __shared__ float red[kThreads / 32];
+    begin_behind();
     for (int n = blockIdx.x; n < N; n += gridDim.x) {
         const float4 *row = Wp + (int64_t)n * K4;
         float m = 0.0f;
@@ -63,17 +111,40 @@ quant_weight_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq,
             float4 v = __ldg(row + k);
             m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
-        const float s = scale_from_amax(block_max(m, red));
+        const float s = scale_from_amax(block_max(m, red), qmax);
         if (threadIdx.x == 0) w_scale[n] = s;
         uint32_t *out = Wq + (int64_t)n * K4;
+        const int q = (int)qmax;
         for (int k = threadIdx.x; k < K4; k += blockDim.x) {
-            float4 v = __ldg(row + k);
-            uint32_t c = (uint32_t)(quant_code(v.x, s) & 0xFF) | ((uint32_t)(quant_code(v.y, s) & 0xFF) << 8) |
-                         ((uint32_t)(quant_code(v.z, s) & 0xFF) << 16) |
-                         ((uint32_t)(quant_code(v.w, s) & 0xFF) << 24);
-            out[k] = c;
+            const float4 v = __ldg(row + k);
+            out[k] = (uint32_t)(quant_code(v.x, s, q) & 0xFF) | ((uint32_t)(quant_code(v.y, s, q) & 0xFF) << 8) |
+                     ((uint32_t)(quant_code(v.z, s, q) & 0xFF) << 16) | ((uint32_t)(quant_code(v.w, s, q) & 0xFF) << 24);
         }
     }
+}
+
+// gpusq_quant_weight (qmax 127) and gpusq_quant_weight4 (7)
+int quant_weight_common(const float *Wp, int8_t *Wq, float *w_scale, int N, int K, void *stream, float qmax)
+{
+    if (!Wp || !Wq || !w_scale) return GPUSQ_ERR_NULL;
+    if (N <= 0 || K <= 0 || K % 4) return GPUSQ_ERR_SHAPE;
+    if (!aligned(Wp, 16) || !aligned(Wq, 4)) return GPUSQ_ERR_ALIGN;
+    if (int st = check_arch()) return st;
+    const float4 *src = reinterpret_cast<const float4 *>(Wp);
+    uint32_t *dst = reinterpret_cast<uint32_t *>(Wq);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int K4 = K / 4;
+    if (K4 > 8 * kThreads)
+        return launch_behind(quant_weight_long_kernel, N < num_sms() * 8 ? N : num_sms() * 8, kThreads, s, src, dst, w_scale,
+                             N, K4, qmax);
+    if (K4 > 8 * 32) {
+        auto kernel = K4 <= 2 * kThreads ? quant_weight_kernel<2, true>
+                    : K4 <= 4 * kThreads ? quant_weight_kernel<4, true> : quant_weight_kernel<8, true>;
+        return launch_behind(kernel, N, kThreads, s, src, dst, w_scale, N, K4, qmax);
+    }
+    auto kernel = K4 <= 32 ? quant_weight_kernel<1, false> : K4 <= 2 * 32 ? quant_weight_kernel<2, false>
+                : K4 <= 4 * 32 ? quant_weight_kernel<4, false> : quant_weight_kernel<8, false>;
+    return launch_behind(kernel, (int)ceil_div(N, kThreads / 32), kThreads, s, src, dst, w_scale, N, K4, qmax);
 }
 
 // ---------------------------------------------------------------- compress
@@ -95,6 +166,7 @@ __global__ void __launch_bounds__(kThreads)
 compress24_x4_kernel(const uint4 *__restrict__ Wq, uint2 *__restrict__ vals,
                      uint16_t *__restrict__ meta, int64_t quads)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += stride) {
         const uint4 w = __ldg(Wq + i);
@@ -113,6 +185,7 @@ __global__ void __launch_bounds__(kThreads)
 compress24_x2_kernel(const uint2 *__restrict__ Wq, uint32_t *__restrict__ vals,
                      uint8_t *__restrict__ meta, int64_t pairs)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += stride) {
         const uint2 w = __ldg(Wq + i);
@@ -136,6 +209,7 @@ __global__ void __launch_bounds__(kThreads)
 decompress24_kernel(const uint32_t *__restrict__ vals, const uint8_t *__restrict__ meta,
                     uint2 *__restrict__ Wq, int64_t pairs)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += stride) {
         const uint32_t v = __ldg(vals + i);
@@ -151,46 +225,57 @@ decompress24_kernel(const uint32_t *__restrict__ vals, const uint8_t *__restrict
 // are contiguous and rows follow each other: the 2 KB block is what one
 // tcgen05.cp 128x128b instruction moves into tensor memory.  Padding groups
 // get the well-formed nibble 0x4 (positions 0 and 1); their values are zero.
+// kWide: rows of vals and meta can be read in 16-byte pieces (K % 128 == 0, aligned pointers); otherwise
+// vals in words and meta in bytes.  3072 x 1024: 2.2 us (6.5 with metadata bytes and 64-bit divisions).
+template <bool kWide>
 __global__ void __launch_bounds__(kThreads)
 pack24_kernel(const int8_t *__restrict__ vals, const uint8_t *__restrict__ meta,
               uint8_t *__restrict__ packed, int N, int K, int Np, int Kp)
 {
-    const int row_chunks = Kp / 32;                       // 16-byte chunks per padded value row
-    const int64_t val_chunks = (int64_t)Np * row_chunks;
-    const int kt = Kp / 128;
-    const int64_t meta_chunks = (int64_t)Np * kt;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    begin_behind();
+    const uint32_t row_chunks = Kp / 32;                  // 16-byte chunks per padded value row
+    const uint32_t kt = Kp / 128;                         // k blocks, one metadata chunk per row each
     uint8_t *meta_out = packed + (int64_t)Np * (Kp / 2);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < val_chunks + meta_chunks;
-         i += stride) {
-        uint32_t w[4];
-        if (i < val_chunks) {
-            const int n = (int)(i / row_chunks), c = (int)(i % row_chunks);
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(vals + (int64_t)n * (K / 2));
+    // grid: x over the chunks of a row (values, then metadata), y over the rows
+    for (int n = blockIdx.y * blockDim.y + threadIdx.y; n < Np; n += gridDim.y * blockDim.y) {
+        for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < row_chunks + kt; c += gridDim.x * blockDim.x) {
+            uint4 w;
+            if (c < row_chunks) {
+                if (kWide) {
+                    w = n < N ? __ldg(reinterpret_cast<const uint4 *>(vals + (int64_t)n * (K / 2)) + c) : make_uint4(0u, 0u, 0u, 0u);
+                } else {
+                    const uint32_t *src = reinterpret_cast<const uint32_t *>(vals + (int64_t)n * (K / 2));
+                    uint32_t q[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int byte = 16 * c + 4 * j;          // K/2 is a multiple of 4
-                w[j] = (n < N && byte < K / 2) ? __ldg(src + byte / 4) : 0u;
-            }
-            *reinterpret_cast<uint4 *>(packed + i * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-            const int64_t j = i - val_chunks;             // (tile_n, tile_k, r)
-            const int r = (int)(j % 128);
-            const int tk = (int)((j / 128) % kt);
-            const int tn = (int)(j / (128 * (int64_t)kt));
-            const int n = tn * 128 + r;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t word = 0;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const int byte = 16 * tk + 4 * q + b;
-                    const uint32_t v = (n < N && byte < K / 8) ? meta[(int64_t)n * (K / 8) + byte] : 0x44u;
-                    word |= v << (8 * b);
+                    for (int j = 0; j < 4; ++j) {
+                        const int byte = 16 * (int)c + 4 * j;         // K/2 is a multiple of 4
+                        q[j] = (n < N && byte < K / 2) ? __ldg(src + byte / 4) : 0u;
+                    }
+                    w = make_uint4(q[0], q[1], q[2], q[3]);
                 }
-                w[q] = word;
+                *reinterpret_cast<uint4 *>(packed + ((int64_t)n * row_chunks + c) * 16) = w;
+            } else {
+                const uint32_t tk = c - row_chunks;
+                if (kWide) {
+                    w = n < N ? __ldg(reinterpret_cast<const uint4 *>(meta + (int64_t)n * (K / 8)) + tk)
+                              : make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
+                } else {
+                    uint32_t q[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        q[j] = 0;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            const int byte = 16 * (int)tk + 4 * j + b;
+                            const uint32_t v = (n < N && byte < K / 8) ? __ldg(meta + (int64_t)n * (K / 8) + byte) : 0x44u;
+                            q[j] |= v << (8 * b);
+                        }
+                    }
+                    w = make_uint4(q[0], q[1], q[2], q[3]);
+                }
+                // (feature tile, k block, row of the tile)
+                *reinterpret_cast<uint4 *>(meta_out + (((int64_t)(n / 128) * kt + tk) * 128 + n % 128) * 16) = w;
             }
-            *reinterpret_cast<uint4 *>(meta_out + j * 16) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 }
@@ -203,6 +288,7 @@ __global__ void __launch_bounds__(kThreads)
 compress24_f16_kernel(const float4 *__restrict__ Wp, uint2 *__restrict__ vals, uint8_t *__restrict__ meta,
                       int64_t pairs)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += stride) {
         uint32_t kept[2], nib[2];
@@ -236,32 +322,40 @@ __global__ void __launch_bounds__(kThreads)
 pack24_f16_kernel(const uint16_t *__restrict__ vals, const uint8_t *__restrict__ meta,
                   uint8_t *__restrict__ packed, int N, int K, int Np, int Kp)
 {
-    const int row_chunks = Kp / 16;                       // 16-byte chunks (8 values) per padded value row
-    const int64_t val_chunks = (int64_t)Np * row_chunks;
-    const int kt = Kp / 128;
-    const int64_t meta_bytes = (int64_t)Np * (Kp / 8);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    begin_behind();
+    const uint32_t row_chunks = Kp / 16;                  // 16-byte chunks (8 values) per padded value row
+    const uint32_t kt = Kp / 128;
+    const uint32_t row_words = Kp / 32;                   // 4-byte words of metadata per row
     uint8_t *meta_out = packed + (int64_t)Np * Kp;        // Kp / 2 values of two bytes per row
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < val_chunks + meta_bytes; i += stride) {
-        if (i < val_chunks) {
-            const int n = (int)(i / row_chunks), c = (int)(i % row_chunks);
-            uint32_t w[4];
+    // grid: x over the chunks and metadata words of a row, y over the rows
+    for (int n = blockIdx.y * blockDim.y + threadIdx.y; n < Np; n += gridDim.y * blockDim.y) {
+        for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < row_chunks + row_words; c += gridDim.x * blockDim.x) {
+            if (c < row_chunks) {
+                uint32_t w[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int v = 8 * c + 2 * j;              // K / 2 is a multiple of 4: pairs do not straddle the end
-                w[j] = (n < N && v < K / 2)
-                           ? __ldg(reinterpret_cast<const uint32_t *>(vals + (int64_t)n * (K / 2)) + v / 2) : 0u;
+                for (int j = 0; j < 4; ++j) {
+                    const int v = 8 * (int)c + 2 * j;     // K / 2 is a multiple of 4: pairs do not straddle the end
+                    w[j] = (n < N && v < K / 2)
+                               ? __ldg(reinterpret_cast<const uint32_t *>(vals + (int64_t)n * (K / 2)) + v / 2) : 0u;
+                }
+                *reinterpret_cast<uint4 *>(packed + ((int64_t)n * row_chunks + c) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+            } else {
+                // source bytes kb = 4 j .. 4 j + 3 of k block tk: two pairs (kb % 2 = 0, 1), 128 bytes apart
+                const uint32_t q = c - row_chunks, tk = q / 4, j = q % 4;
+                const int m = n % 128;
+                uint8_t *dst = meta_out + ((int64_t)(n / 128) * kt + tk) * 2048 + 256 * (m / 16) + 16 * (m % 8) + 4 * j + 2 * ((m / 8) % 2);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t pair = 0;
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const int byte = 16 * (int)tk + 4 * (int)j + 2 * h + b;
+                        const uint32_t v = (n < N && byte < K / 8) ? __ldg(meta + (int64_t)n * (K / 8) + byte) : 0x44u;
+                        pair |= v << (8 * b);
+                    }
+                    *reinterpret_cast<uint16_t *>(dst + 128 * h) = (uint16_t)pair;
+                }
             }
-            *reinterpret_cast<uint4 *>(packed + i * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-            const int64_t j = i - val_chunks;             // one destination byte: (tile_n, tile_k, offset)
-            const int off = (int)(j % 2048);
-            const int tk = (int)((j / 2048) % kt);
-            const int tn = (int)(j / (2048 * (int64_t)kt));
-            const int m = 16 * (off >> 8) + 8 * ((off >> 1) & 1) + ((off >> 4) & 7);
-            const int kb = 4 * ((off >> 2) & 3) + 2 * ((off >> 7) & 1) + (off & 1);
-            const int n = tn * 128 + m, byte = 16 * tk + kb;
-            meta_out[j] = (n < N && byte < K / 8) ? __ldg(meta + (int64_t)n * (K / 8) + byte) : (uint8_t)0x44;
         }
     }
 }
@@ -305,8 +399,7 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
                  const float *__restrict__ absmax, float qmax, int regroup)
 {
     __shared__ float red[kThreads / 32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    begin_behind();
     float s;
     if (absmax) {
         s = scale_from_amax(__ldg(absmax), qmax);
@@ -446,8 +539,7 @@ patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, floa
                    const uint32_t *__restrict__ partial, int n_partials, const PatchGeom g, uint32_t items)
 {
     __shared__ float red[kThreads / 32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    begin_behind();
     float s;
     if (n_partials > 0) {
         uint32_t m = 0;
@@ -762,21 +854,13 @@ int gpusq_prune24(const float *W, float *Wp, uint8_t *mask, int N, int K, void *
     if (!aligned(W, 16) || !aligned(Wp, 16)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t groups = (int64_t)N * (K / 4);
-    prune24_kernel<4><<<grid_for(ceil_div(groups, 4), 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(W), reinterpret_cast<float4 *>(Wp), mask, groups);
-    return launch_status();
+    return launch_behind(prune24_kernel<4>, grid_for(ceil_div(groups, 4), 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const float4 *>(W), reinterpret_cast<float4 *>(Wp), mask, groups);
 }
 
 int gpusq_quant_weight(const float *Wp, int8_t *Wq, float *w_scale, int N, int K, void *stream)
 {
-    if (!Wp || !Wq || !w_scale) return GPUSQ_ERR_NULL;
-    if (N <= 0 || K <= 0 || K % 4) return GPUSQ_ERR_SHAPE;
-    if (!aligned(Wp, 16) || !aligned(Wq, 4)) return GPUSQ_ERR_ALIGN;
-    if (int st = check_arch()) return st;
-    const int grid = N < num_sms() * 8 ? N : num_sms() * 8;
-    quant_weight_kernel<<<grid, kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(Wp), reinterpret_cast<uint32_t *>(Wq), w_scale, N, K / 4);
-    return launch_status();
+    return quant_weight_common(Wp, Wq, w_scale, N, K, stream, 127.0f);
 }
 
 int gpusq_compress24(const int8_t *Wq, int8_t *vals, uint8_t *meta, int N, int K, void *stream)
@@ -787,14 +871,12 @@ int gpusq_compress24(const int8_t *Wq, int8_t *vals, uint8_t *meta, int N, int K
     if (int st = check_arch()) return st;
     const int64_t groups = (int64_t)N * (K / 4);
     if (K % 16 == 0 && aligned(Wq, 16) && aligned(vals, 8) && aligned(meta, 2)) {
-        compress24_x4_kernel<<<grid_for(groups / 4, 8), kThreads, 0, (cudaStream_t)stream>>>(
-            reinterpret_cast<const uint4 *>(Wq), reinterpret_cast<uint2 *>(vals),
-            reinterpret_cast<uint16_t *>(meta), groups / 4);
-    } else {
-        compress24_x2_kernel<<<grid_for(groups / 2, 8), kThreads, 0, (cudaStream_t)stream>>>(
-            reinterpret_cast<const uint2 *>(Wq), reinterpret_cast<uint32_t *>(vals), meta, groups / 2);
+        return launch_behind(compress24_x4_kernel, grid_for(groups / 4, 8), kThreads, (cudaStream_t)stream,
+                             reinterpret_cast<const uint4 *>(Wq), reinterpret_cast<uint2 *>(vals),
+                             reinterpret_cast<uint16_t *>(meta), groups / 4);
     }
-    return launch_status();
+    return launch_behind(compress24_x2_kernel, grid_for(groups / 2, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const uint2 *>(Wq), reinterpret_cast<uint32_t *>(vals), meta, groups / 2);
 }
 
 int gpusq_decompress24(const int8_t *vals, const uint8_t *meta, int8_t *Wq, int N, int K, void *stream)
@@ -804,9 +886,8 @@ int gpusq_decompress24(const int8_t *vals, const uint8_t *meta, int8_t *Wq, int 
     if (!aligned(Wq, 8) || !aligned(vals, 4)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t pairs = (int64_t)N * (K / 8);
-    decompress24_kernel<<<grid_for(pairs, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const uint32_t *>(vals), meta, reinterpret_cast<uint2 *>(Wq), pairs);
-    return launch_status();
+    return launch_behind(decompress24_kernel, grid_for(pairs, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const uint32_t *>(vals), meta, reinterpret_cast<uint2 *>(Wq), pairs);
 }
 
 size_t gpusq_packed_bytes(int N, int K)
@@ -823,10 +904,12 @@ int gpusq_pack24(const int8_t *vals, const uint8_t *meta, void *Wpacked, int N, 
     if (!aligned(vals, 4) || !aligned(Wpacked, 256)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int Np = round_up(N, 256), Kp = round_up(K, 128);
-    const int64_t chunks = (int64_t)Np * (Kp / 32) + (int64_t)Np * (Kp / 128);
-    pack24_kernel<<<grid_for(chunks, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        vals, meta, reinterpret_cast<uint8_t *>(Wpacked), N, K, Np, Kp);
-    return launch_status();
+    const bool wide = K % 128 == 0 && aligned(vals, 16) && aligned(meta, 16);
+    // blocks of 32 chunks x 8 rows
+    const dim3 block(32, kThreads / 32, 1);
+    const dim3 grid((unsigned)ceil_div(Kp / 32 + Kp / 128, 32), (unsigned)(Np / 8 < 65535 ? Np / 8 : 65535), 1);
+    return launch_behind(wide ? pack24_kernel<true> : pack24_kernel<false>, grid, block, (cudaStream_t)stream, vals, meta,
+                         reinterpret_cast<uint8_t *>(Wpacked), N, K, Np, Kp);
 }
 
 int gpusq_compress24_f16(const float *Wp, void *vals, uint8_t *meta, int N, int K, void *stream)
@@ -836,9 +919,8 @@ int gpusq_compress24_f16(const float *Wp, void *vals, uint8_t *meta, int N, int 
     if (!aligned(Wp, 16) || !aligned(vals, 8)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t pairs = (int64_t)N * (K / 8);
-    compress24_f16_kernel<<<grid_for(pairs, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(Wp), reinterpret_cast<uint2 *>(vals), meta, pairs);
-    return launch_status();
+    return launch_behind(compress24_f16_kernel, grid_for(pairs, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const float4 *>(Wp), reinterpret_cast<uint2 *>(vals), meta, pairs);
 }
 
 size_t gpusq_packed_bytes_f16(int N, int K)
@@ -855,10 +937,10 @@ int gpusq_pack24_f16(const void *vals, const uint8_t *meta, void *Wpacked, int N
     if (!aligned(vals, 4) || !aligned(Wpacked, 256)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int Np = round_up(N, 256), Kp = round_up(K, 128);
-    const int64_t items = (int64_t)Np * (Kp / 16) + (int64_t)Np * (Kp / 8);
-    pack24_f16_kernel<<<grid_for(items, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const uint16_t *>(vals), meta, reinterpret_cast<uint8_t *>(Wpacked), N, K, Np, Kp);
-    return launch_status();
+    const dim3 block(32, kThreads / 32, 1);
+    const dim3 grid((unsigned)ceil_div(Kp / 16 + Kp / 32, 32), (unsigned)(Np / 8 < 65535 ? Np / 8 : 65535), 1);
+    return launch_behind(pack24_f16_kernel, grid, block, (cudaStream_t)stream, reinterpret_cast<const uint16_t *>(vals), meta,
+                         reinterpret_cast<uint8_t *>(Wpacked), N, K, Np, Kp);
 }
 
 size_t gpusq_quant_act_workspace(int64_t M, int K)

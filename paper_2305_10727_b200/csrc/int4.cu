@@ -20,6 +20,7 @@ namespace gpusq {
 __global__ void __launch_bounds__(kThreads)
 prune48_kernel(const float4 *__restrict__ W, float4 *Wp, uint8_t *mask, int64_t chunks)
 {
+    begin_behind();
     // W and Wp may be the same buffer: every thread reads its chunk before it writes it.
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < chunks; i += stride) {
@@ -33,31 +34,6 @@ prune48_kernel(const float4 *__restrict__ W, float4 *Wp, uint8_t *mask, int64_t 
         __stcs(Wp + 2 * i, a);
         __stcs(Wp + 2 * i + 1, b);
         if (mask) mask[i] = (uint8_t)mk;
-    }
-}
-
-// ------------------------------------------------------------ quant_weight4
-// One block per output channel: max |w|, scale = max / 7, codes in [-7, 7] (INT8 containers).
-__global__ void __launch_bounds__(kThreads)
-quant_weight4_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq, float *__restrict__ w_scale, int N,
-                     int K4)
-{
-    __shared__ float red[kThreads / 32];
-    for (int n = blockIdx.x; n < N; n += gridDim.x) {
-        const float4 *row = Wp + (int64_t)n * K4;
-        float m = 0.0f;
-        for (int k = threadIdx.x; k < K4; k += blockDim.x) {
-            const float4 v = __ldg(row + k);
-            m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-        }
-        const float s = scale_from_amax(block_max(m, red), 7.0f);
-        if (threadIdx.x == 0) w_scale[n] = s;
-        uint32_t *out = Wq + (int64_t)n * K4;
-        for (int k = threadIdx.x; k < K4; k += blockDim.x) {
-            const float4 v = __ldg(row + k);
-            out[k] = (uint32_t)(quant_code(v.x, s, 7) & 0xFF) | ((uint32_t)(quant_code(v.y, s, 7) & 0xFF) << 8) |
-                     ((uint32_t)(quant_code(v.z, s, 7) & 0xFF) << 16) | ((uint32_t)(quant_code(v.w, s, 7) & 0xFF) << 24);
-        }
     }
 }
 
@@ -79,6 +55,7 @@ __device__ __forceinline__ void compress_chunk(uint32_t lo, uint32_t hi, uint32_
 __global__ void __launch_bounds__(kThreads)
 compress48_kernel(const uint4 *__restrict__ Wq, uint32_t *__restrict__ vals, uint8_t *__restrict__ meta, int64_t pairs)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += stride) {
         const uint4 w = __ldg(Wq + i);
@@ -99,6 +76,7 @@ __global__ void __launch_bounds__(kThreads)
 expand48_kernel(const uint32_t *__restrict__ vals4, const uint8_t *__restrict__ meta4, uint2 *__restrict__ vals,
                 uint16_t *__restrict__ meta, int64_t pairs)
 {
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += stride) {
         const uint32_t v = __ldg(vals4 + i), m = __ldg(meta4 + i);
@@ -126,21 +104,13 @@ int gpusq_prune48(const float *W, float *Wp, uint8_t *mask, int N, int K, void *
     if (!aligned(W, 16) || !aligned(Wp, 16)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t chunks = (int64_t)N * (K / 8);
-    prune48_kernel<<<grid_for(chunks, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(W), reinterpret_cast<float4 *>(Wp), mask, chunks);
-    return launch_status();
+    return launch_behind(prune48_kernel, grid_for(chunks, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const float4 *>(W), reinterpret_cast<float4 *>(Wp), mask, chunks);
 }
 
 int gpusq_quant_weight4(const float *Wp, int8_t *Wq, float *w_scale, int N, int K, void *stream)
 {
-    if (!Wp || !Wq || !w_scale) return GPUSQ_ERR_NULL;
-    if (N <= 0 || K <= 0 || K % 4) return GPUSQ_ERR_SHAPE;
-    if (!aligned(Wp, 16) || !aligned(Wq, 4)) return GPUSQ_ERR_ALIGN;
-    if (int st = check_arch()) return st;
-    const int grid = N < num_sms() * 8 ? N : num_sms() * 8;
-    quant_weight4_kernel<<<grid, kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const float4 *>(Wp), reinterpret_cast<uint32_t *>(Wq), w_scale, N, K / 4);
-    return launch_status();
+    return quant_weight_common(Wp, Wq, w_scale, N, K, stream, 7.0f);
 }
 
 int gpusq_compress48(const int8_t *Wq, uint8_t *vals4, uint8_t *meta4, int N, int K, void *stream)
@@ -150,9 +120,8 @@ int gpusq_compress48(const int8_t *Wq, uint8_t *vals4, uint8_t *meta4, int N, in
     if (!aligned(Wq, 16) || !aligned(vals4, 4)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t pairs = (int64_t)N * (K / 16);
-    compress48_kernel<<<grid_for(pairs, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const uint4 *>(Wq), reinterpret_cast<uint32_t *>(vals4), meta4, pairs);
-    return launch_status();
+    return launch_behind(compress48_kernel, grid_for(pairs, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const uint4 *>(Wq), reinterpret_cast<uint32_t *>(vals4), meta4, pairs);
 }
 
 int gpusq_expand48(const uint8_t *vals4, const uint8_t *meta4, int8_t *vals, uint8_t *meta, int N, int K, void *stream)
@@ -162,10 +131,8 @@ int gpusq_expand48(const uint8_t *vals4, const uint8_t *meta4, int8_t *vals, uin
     if (!aligned(vals4, 4) || !aligned(vals, 8) || !aligned(meta, 2)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
     const int64_t pairs = (int64_t)N * (K / 16);
-    expand48_kernel<<<grid_for(pairs, 8), kThreads, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const uint32_t *>(vals4), meta4, reinterpret_cast<uint2 *>(vals),
-        reinterpret_cast<uint16_t *>(meta), pairs);
-    return launch_status();
+    return launch_behind(expand48_kernel, grid_for(pairs, 8), kThreads, (cudaStream_t)stream,
+                         reinterpret_cast<const uint32_t *>(vals4), meta4, reinterpret_cast<uint2 *>(vals), reinterpret_cast<uint16_t *>(meta), pairs);
 }
 
 }  // extern "C"

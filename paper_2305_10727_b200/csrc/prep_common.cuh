@@ -53,6 +53,16 @@ __device__ __forceinline__ float block_max(float v, float *red)
     return r;
 }
 
+// First statement of a kernel launched with launch_behind(): what was launched before is complete from
+// here on, and what is launched next may be set up.
+__device__ __forceinline__ void begin_behind()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+int quant_weight_common(const float *Wp, int8_t *Wq, float *w_scale, int N, int K, void *stream, float qmax);
+
 constexpr int kMaxDevices = 64;
 constexpr int kMaxPartials = 2048;   // workspace: one 32-bit partial maximum per block ...
 constexpr int kWorkspaceExtra = 64;  // ... and, behind them, the control words of the one-launch kernel
@@ -72,8 +82,7 @@ static __global__ void __launch_bounds__(kAbsmaxThreads)
 act_absmax_kernel(const uint4 *__restrict__ X, uint32_t *__restrict__ partial, int64_t vec8)
 {
     __shared__ uint32_t red[kAbsmaxThreads / 32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");                  // what was launched before is complete
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    begin_behind();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     uint32_t m = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vec8; i += 8 * stride) {
@@ -182,14 +191,14 @@ inline int grid_for(int64_t items, int per_sm)
 // Launch that may be set up while the previous kernel of the stream drains; the kernel itself waits
 // (griddepcontrol.wait) before it touches memory.
 template <typename... P, typename... A>
-inline int launch_behind(void (*kernel)(P...), int grid, int threads, cudaStream_t stream, A... args)
+inline int launch_behind(void (*kernel)(P...), dim3 grid, dim3 threads, cudaStream_t stream, A... args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = 1;

@@ -101,6 +101,22 @@ def test_quant_act(B, M, K, dist):
     assert np.array_equal(Xq2.cpu().numpy(), Xq_o2)
 
 
+# rows in the registers of a warp (up to 1024) and of a block (up to 8192), and longer ones
+@pytest.mark.parametrize("K", [4, 128, 132, 256, 512, 516, 1024, 1028, 2048, 2052, 4096, 4100, 8192, 8196])
+@pytest.mark.parametrize("N", [1, 9])
+def test_quant_weight_row_lengths(B, N, K):
+    W = (np.random.default_rng(N + K).standard_normal((N, K)) * 0.02).astype(np.float32)
+    W[0, K - 1] = -0.25                                     # the maximum in the last lane
+    if N > 1:
+        W[1] = 0.0
+    Wq_o, ws_o = oracle.quant_weight(W)
+    Wq, ws = B.quant_weight(cu(W))
+    assert np.array_equal(ws.cpu().numpy(), ws_o) and np.array_equal(Wq.cpu().numpy(), Wq_o)
+    Wq_o, ws_o = oracle.quant_weight4(W)
+    Wq, ws = B.quant_weight4(cu(W))
+    assert np.array_equal(ws.cpu().numpy(), ws_o) and np.array_equal(Wq.cpu().numpy(), Wq_o)
+
+
 # vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2, 4 and 6 vectors per thread, the first size
 # beyond it, and slices that just do and just do not fit the one-launch kernel's shared memory
 @pytest.mark.parametrize("vecs", [1, 1023, 1024, 1025, 8193, 16384, 16385, 32769, 65537, 98304, 98305, 300001,
