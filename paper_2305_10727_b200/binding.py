@@ -4,7 +4,10 @@ Every function has the name of the C entry point it calls (without the
 ``gpusq_`` prefix), takes CUDA ``torch`` tensors, allocates the outputs with
 torch when the caller does not pass them, enqueues on torch's current stream
 and returns without synchronising.  All arithmetic runs in the CUDA kernels.
-A missing library or a non-zero status raises; there is no fallback.
+A missing library or a non-zero status raises; there is no fallback.  The
+functions that run per inference or per weight do their checks, allocations
+and the call in ``_gpusq_torch.so`` (csrc/torch_binding.cpp); the rest goes
+through ctypes.
 """
 from __future__ import annotations
 
@@ -93,6 +96,20 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+_native = None
+
+
+def _n():
+    """The native part of this binding; raises if it or libgpusq.so is missing."""
+    global _native
+    if _native is None:
+        load()
+        from . import _gpusq_torch
+        _gpusq_torch.set_errors(GpusqError, torch.OutOfMemoryError)
+        _native = _gpusq_torch
+    return _native
+
+
 def status_string(status: int) -> str:
     return load().gpusq_status_string(int(status)).decode()
 
@@ -102,9 +119,9 @@ def _check(status: int, where: str) -> None:
         raise GpusqError(status, where)
 
 
-# Addresses are passed as plain integers (the argument types convert them) and the stream is asked for as
-# its handle: a pointer object per argument and a Stream object per call cost 5 of the 10 us that a call
-# took on the host, more than most kernels of a small batch run.
+# For the calls that go through ctypes.  Addresses are passed as plain integers (the argument types convert
+# them) and the stream is asked for as its handle: a pointer object per argument and a Stream object per
+# call cost 5 us.
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
@@ -121,36 +138,15 @@ def _dev(t: torch.Tensor, dtype, what: str) -> torch.Tensor:
 
 def prune24(W: torch.Tensor, Wp: Optional[torch.Tensor] = None, mask: Optional[torch.Tensor] = None,
             want_mask: bool = False):
-    _dev(W, torch.float32, "W")
-    N, K = W.shape
-    if Wp is None:
-        Wp = torch.empty_like(W)
-    if mask is None and want_mask:
-        mask = torch.empty((N, K // 4), dtype=torch.uint8, device=W.device)
-    _check(load().gpusq_prune24(_ptr(W), _ptr(Wp), _ptr(mask), N, K, _stream()), "gpusq_prune24")
-    return (Wp, mask) if want_mask else Wp
+    return _n().prune24(W, Wp, mask, bool(want_mask))
 
 
 def quant_weight(Wp: torch.Tensor, Wq: Optional[torch.Tensor] = None, w_scale: Optional[torch.Tensor] = None):
-    _dev(Wp, torch.float32, "Wp")
-    N, K = Wp.shape
-    if Wq is None:
-        Wq = torch.empty((N, K), dtype=torch.int8, device=Wp.device)
-    if w_scale is None:
-        w_scale = torch.empty((N,), dtype=torch.float32, device=Wp.device)
-    _check(load().gpusq_quant_weight(_ptr(Wp), _ptr(Wq), _ptr(w_scale), N, K, _stream()), "gpusq_quant_weight")
-    return Wq, w_scale
+    return _n().quant_weight(Wp, Wq, w_scale)
 
 
 def compress24(Wq: torch.Tensor, vals: Optional[torch.Tensor] = None, meta: Optional[torch.Tensor] = None):
-    _dev(Wq, torch.int8, "Wq")
-    N, K = Wq.shape
-    if vals is None:
-        vals = torch.empty((N, K // 2), dtype=torch.int8, device=Wq.device)
-    if meta is None:
-        meta = torch.empty((N, K // 8), dtype=torch.uint8, device=Wq.device)
-    _check(load().gpusq_compress24(_ptr(Wq), _ptr(vals), _ptr(meta), N, K, _stream()), "gpusq_compress24")
-    return vals, meta
+    return _n().compress24(Wq, vals, meta)
 
 
 def decompress24(vals: torch.Tensor, meta: torch.Tensor, Wq: Optional[torch.Tensor] = None):
@@ -168,13 +164,7 @@ def packed_bytes(N: int, K: int) -> int:
 
 
 def pack24(vals: torch.Tensor, meta: torch.Tensor, Wpacked: Optional[torch.Tensor] = None):
-    _dev(vals, torch.int8, "vals")
-    _dev(meta, torch.uint8, "meta")
-    N, K = vals.shape[0], vals.shape[1] * 2
-    if Wpacked is None:
-        Wpacked = torch.empty((packed_bytes(N, K),), dtype=torch.uint8, device=vals.device)
-    _check(load().gpusq_pack24(_ptr(vals), _ptr(meta), _ptr(Wpacked), N, K, _stream()), "gpusq_pack24")
-    return Wpacked
+    return _n().pack24(vals, meta, Wpacked)
 
 
 def quant_act_workspace(M: int, K: int) -> int:
@@ -183,20 +173,7 @@ def quant_act_workspace(M: int, K: int) -> int:
 
 def quant_act(X: torch.Tensor, Xq: Optional[torch.Tensor] = None, x_scale: Optional[torch.Tensor] = None,
               scale_mode: int = SCALE_COMPUTE, workspace: Optional[torch.Tensor] = None):
-    _dev(X, torch.float16, "X")
-    M, K = X.shape
-    if Xq is None:
-        Xq = torch.empty((M, K), dtype=torch.int8, device=X.device)
-    if x_scale is None:
-        if scale_mode == SCALE_GIVEN:
-            raise ValueError("scale_mode GIVEN needs x_scale")
-        x_scale = torch.empty((1,), dtype=torch.float32, device=X.device)
-    if workspace is None and scale_mode == SCALE_COMPUTE:
-        workspace = torch.zeros((quant_act_workspace(M, K),), dtype=torch.uint8, device=X.device)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().gpusq_quant_act(_ptr(X), _ptr(Xq), _ptr(x_scale), scale_mode, M, K, _ptr(workspace),
-                                  ws_bytes, _stream()), "gpusq_quant_act")
-    return Xq, x_scale
+    return _n().quant_act(X, Xq, x_scale, scale_mode, workspace)
 
 
 QUANT_ACT_STATUS_OFFSET = 8196       # GPUSQ_QUANT_ACT_STATUS_OFFSET of gpusq.h
@@ -268,60 +245,29 @@ def flatten_conv_weight(W4: torch.Tensor, Kp: Optional[int] = None) -> torch.Ten
     return Wf
 
 
-_OUT_DTYPE = {OUT_F16: torch.float16, OUT_I8: torch.int8, OUT_I32: torch.int32}
-
-
-def _gemm(fn_name, Xq, Wop, w_scale, x_scale, bias, act, out_type, out_scale, Y, N, status_buf):
-    _dev(Xq, torch.int8, "Xq")
-    M, K = Xq.shape
-    if Y is None:
-        Y = torch.empty((M, N), dtype=_OUT_DTYPE[out_type], device=Xq.device)
-    fn = getattr(load(), fn_name)
-    _check(fn(_ptr(Xq), _ptr(Wop), _ptr(w_scale), _ptr(x_scale), _ptr(bias), act, out_type, _ptr(out_scale),
-              _ptr(Y), M, N, K, _ptr(status_buf), _stream()), fn_name)
-    return Y
-
-
 def spgemm_i8(Xq: torch.Tensor, Wpacked: torch.Tensor, N: int, w_scale=None, x_scale=None, bias=None,
               act: int = ACT_NONE, out_type: int = OUT_F16, out_scale=None, Y=None, status_buf=None):
-    return _gemm("gpusq_spgemm_i8", Xq, Wpacked, w_scale, x_scale, bias, act, out_type, out_scale, Y, N,
-                 status_buf)
+    return _n().spgemm_i8(Xq, Wpacked, N, w_scale, x_scale, bias, act, out_type, out_scale, Y, status_buf)
 
 
 def spgemm_i8_absmax(Xq: torch.Tensor, Wpacked: torch.Tensor, N: int, w_scale, x_scale, bias=None,
                      act: int = ACT_NONE, Y=None, y_absmax=None, status_buf=None):
     """gpusq_spgemm_i8_absmax: FP16 output plus max |Y| merged into y_absmax (float32[1], zeroed here if not given)."""
-    _dev(Xq, torch.int8, "Xq")
-    M, K = Xq.shape
-    if Y is None:
-        Y = torch.empty((M, N), dtype=torch.float16, device=Xq.device)
     if y_absmax is None:
         y_absmax = torch.zeros((1,), dtype=torch.float32, device=Xq.device)
-    _check(load().gpusq_spgemm_i8_absmax(_ptr(Xq), _ptr(Wpacked), _ptr(w_scale), _ptr(x_scale), _ptr(bias), act,
-                                         _ptr(Y), _ptr(y_absmax), M, N, K, _ptr(status_buf), _stream()),
-           "gpusq_spgemm_i8_absmax")
-    return Y, y_absmax
+    return _n().spgemm_i8_absmax(Xq, Wpacked, N, w_scale, x_scale, bias, act, Y, y_absmax, status_buf)
 
 
 def quant_act_absmax(X: torch.Tensor, absmax: torch.Tensor, Xq: Optional[torch.Tensor] = None,
                      x_scale: Optional[torch.Tensor] = None):
     """gpusq_quant_act_absmax: one-pass quantisation with the scale derived from a known max |X|."""
-    _dev(X, torch.float16, "X")
-    M, K = X.shape
-    if Xq is None:
-        Xq = torch.empty((M, K), dtype=torch.int8, device=X.device)
-    if x_scale is None:
-        x_scale = torch.empty((1,), dtype=torch.float32, device=X.device)
-    _check(load().gpusq_quant_act_absmax(_ptr(X), _ptr(Xq), _ptr(x_scale), _ptr(absmax), M, K, _stream()),
-           "gpusq_quant_act_absmax")
-    return Xq, x_scale
+    return _n().quant_act_absmax(X, absmax, Xq, x_scale)
 
 
 def gemm_i8_dense(Xq: torch.Tensor, Wq: torch.Tensor, w_scale=None, x_scale=None, bias=None,
                   act: int = ACT_NONE, out_type: int = OUT_F16, out_scale=None, Y=None, status_buf=None):
     _dev(Wq, torch.int8, "Wq")
-    return _gemm("gpusq_gemm_i8_dense", Xq, Wq, w_scale, x_scale, bias, act, out_type, out_scale, Y,
-                 Wq.shape[0], status_buf)
+    return _n().gemm_i8_dense(Xq, Wq, Wq.shape[0], w_scale, x_scale, bias, act, out_type, out_scale, Y, status_buf)
 
 
 def set_block_tokens(block_t: int) -> None:
@@ -344,12 +290,7 @@ OUT_F32 = 2
 
 
 def compress24_f16(Wp: torch.Tensor):
-    _dev(Wp, torch.float32, "Wp")
-    N, K = Wp.shape
-    vals = torch.empty((N, K // 2), dtype=torch.float16, device=Wp.device)
-    meta = torch.empty((N, K // 8), dtype=torch.uint8, device=Wp.device)
-    _check(load().gpusq_compress24_f16(_ptr(Wp), _ptr(vals), _ptr(meta), N, K, _stream()), "gpusq_compress24_f16")
-    return vals, meta
+    return _n().compress24_f16(Wp)
 
 
 def packed_bytes_f16(N: int, K: int) -> int:
@@ -357,80 +298,34 @@ def packed_bytes_f16(N: int, K: int) -> int:
 
 
 def pack24_f16(vals: torch.Tensor, meta: torch.Tensor, Wpacked: Optional[torch.Tensor] = None):
-    _dev(vals, torch.float16, "vals")
-    _dev(meta, torch.uint8, "meta")
-    N, K = vals.shape[0], vals.shape[1] * 2
-    if Wpacked is None:
-        Wpacked = torch.empty((packed_bytes_f16(N, K),), dtype=torch.uint8, device=vals.device)
-    _check(load().gpusq_pack24_f16(_ptr(vals), _ptr(meta), _ptr(Wpacked), N, K, _stream()), "gpusq_pack24_f16")
-    return Wpacked
+    return _n().pack24_f16(vals, meta, Wpacked)
 
 
 def spgemm_f16(X: torch.Tensor, Wpacked: torch.Tensor, N: int, bias=None, act: int = ACT_NONE,
                out_type: int = OUT_F16, Y=None, status_buf=None):
-    _dev(X, torch.float16, "X")
-    M, K = X.shape
-    if Y is None:
-        Y = torch.empty((M, N), dtype=torch.float16 if out_type == OUT_F16 else torch.float32, device=X.device)
-    _check(load().gpusq_spgemm_f16(_ptr(X), _ptr(Wpacked), _ptr(bias), act, out_type, _ptr(Y), M, N, K,
-                                   _ptr(status_buf), _stream()), "gpusq_spgemm_f16")
-    return Y
+    return _n().spgemm_f16(X, Wpacked, N, bias, act, out_type, Y, status_buf)
 
 
 # ---- INT4 model (pair-wise 4:8 sparsity) ----
 
 def prune48(W: torch.Tensor, want_mask: bool = False):
-    _dev(W, torch.float32, "W")
-    N, K = W.shape
-    Wp = torch.empty_like(W)
-    mask = torch.empty((N, K // 8), dtype=torch.uint8, device=W.device) if want_mask else None
-    _check(load().gpusq_prune48(_ptr(W), _ptr(Wp), _ptr(mask), N, K, _stream()), "gpusq_prune48")
-    return (Wp, mask) if want_mask else Wp
+    return _n().prune48(W, bool(want_mask))
 
 
 def quant_weight4(Wp: torch.Tensor):
-    _dev(Wp, torch.float32, "Wp")
-    N, K = Wp.shape
-    Wq = torch.empty((N, K), dtype=torch.int8, device=Wp.device)
-    w_scale = torch.empty((N,), dtype=torch.float32, device=Wp.device)
-    _check(load().gpusq_quant_weight4(_ptr(Wp), _ptr(Wq), _ptr(w_scale), N, K, _stream()), "gpusq_quant_weight4")
-    return Wq, w_scale
+    return _n().quant_weight4(Wp, None, None)
 
 
 def compress48(Wq: torch.Tensor):
-    _dev(Wq, torch.int8, "Wq")
-    N, K = Wq.shape
-    vals4 = torch.empty((N, K // 4), dtype=torch.uint8, device=Wq.device)
-    meta4 = torch.empty((N, K // 16), dtype=torch.uint8, device=Wq.device)
-    _check(load().gpusq_compress48(_ptr(Wq), _ptr(vals4), _ptr(meta4), N, K, _stream()), "gpusq_compress48")
-    return vals4, meta4
+    return _n().compress48(Wq)
 
 
 def expand48(vals4: torch.Tensor, meta4: torch.Tensor):
     """(vals4, meta4) of the 4-bit format -> (vals, meta) of the 2:4 INT8 format, columns regrouped."""
-    _dev(vals4, torch.uint8, "vals4")
-    _dev(meta4, torch.uint8, "meta4")
-    N, K = vals4.shape[0], vals4.shape[1] * 4
-    vals = torch.empty((N, K // 2), dtype=torch.int8, device=vals4.device)
-    meta = torch.empty((N, K // 8), dtype=torch.uint8, device=vals4.device)
-    _check(load().gpusq_expand48(_ptr(vals4), _ptr(meta4), _ptr(vals), _ptr(meta), N, K, _stream()), "gpusq_expand48")
-    return vals, meta
+    return _n().expand48(vals4, meta4)
 
 
 def quant_act4(X: torch.Tensor, Xq: Optional[torch.Tensor] = None, x_scale: Optional[torch.Tensor] = None,
                scale_mode: int = SCALE_COMPUTE, workspace: Optional[torch.Tensor] = None):
     """gpusq_quant_act4: 4-bit activation codes (INT8 containers) in the regrouped column order."""
-    _dev(X, torch.float16, "X")
-    M, K = X.shape
-    if Xq is None:
-        Xq = torch.empty((M, K), dtype=torch.int8, device=X.device)
-    if x_scale is None:
-        if scale_mode == SCALE_GIVEN:
-            raise ValueError("scale_mode GIVEN needs x_scale")
-        x_scale = torch.empty((1,), dtype=torch.float32, device=X.device)
-    if workspace is None and scale_mode == SCALE_COMPUTE:
-        workspace = torch.zeros((quant_act_workspace(M, K),), dtype=torch.uint8, device=X.device)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().gpusq_quant_act4(_ptr(X), _ptr(Xq), _ptr(x_scale), scale_mode, M, K, _ptr(workspace), ws_bytes,
-                                   _stream()), "gpusq_quant_act4")
-    return Xq, x_scale
+    return _n().quant_act4(X, Xq, x_scale, scale_mode, workspace)

@@ -1,15 +1,18 @@
-"""Build libgpusq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Build libgpusq.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the native part of the
+torch binding, _gpusq_torch.so, with the host compiler."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgpusq.so")
+BINDING = os.path.join(HERE, "_gpusq_torch.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -25,6 +28,32 @@ def _deps():
     return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
 
 
+def _binding_is_stale() -> bool:
+    deps = [os.path.join(CSRC, "torch_binding.cpp"), os.path.join(ROOT, "include", "gpusq.h")]
+    return not os.path.exists(BINDING) or any(os.path.getmtime(f) > os.path.getmtime(BINDING) for f in deps)
+
+
+def build_binding(force: bool = False) -> str:
+    """Needs libgpusq.so beside it (found there at run time as well)."""
+    if not force and not _binding_is_stale():
+        return BINDING
+    import torch
+
+    t = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = BINDING + ".%d.tmp" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(t, "include"),
+           "-I" + os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(cuda, "include"),
+           "-o", tmp, os.path.join(CSRC, "torch_binding.cpp"), "-L" + HERE, "-l:libgpusq.so",
+           "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, BINDING)
+    return BINDING
+
+
 def is_stale() -> bool:
     if not os.path.exists(LIB):
         return True
@@ -33,13 +62,13 @@ def is_stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not is_stale():
-        return LIB
-    nvcc = os.environ.get("NVCC", "nvcc")
-    tmp = LIB + ".%d.tmp" % os.getpid()
-    cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources()
-    subprocess.run(cmd, check=True)
-    os.replace(tmp, LIB)
+    if force or is_stale():
+        nvcc = os.environ.get("NVCC", "nvcc")
+        tmp = LIB + ".%d.tmp" % os.getpid()
+        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources()
+        subprocess.run(cmd, check=True)
+        os.replace(tmp, LIB)
+    build_binding(force)
     return LIB
 
 
