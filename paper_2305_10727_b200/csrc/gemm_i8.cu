@@ -18,29 +18,18 @@
 // output and keeps the sparse instruction's operand reads within the
 // shared-memory bandwidth of one SM.
 //
-// Persistent clusters (one per SM pair), twenty warps per CTA:
+// Persistent clusters (one per SM pair), fourteen warps per CTA:
 //   warp 0      TMA producer (one elected lane), in both CTAs; every load of a
 //               stage counts its bytes on the full barrier of the pair's CTA 0
 //   warp 1      tensor-memory owner (both CTAs); in CTA 0 one elected lane
 //               issues the MMAs for the pair and signals barriers in both CTAs
-//   warps 2-17  epilogue: each warp owns 16 tensor-memory lanes (features) and
-//               every other 32-token chunk; four warps (64 features) fill one
-//               staging tile per chunk.  The work on a chunk is short and
-//               latency-bound, so several warps per scheduler are needed to
-//               keep the issue slots busy
-//   warps 18-19 one elected lane each issues the TMA stores of one 64-feature
-//               half's staging tiles and recycles them
-// (INT8 output: warps 2-13 are the epilogue, each works by itself; see EpiI8.)
-// Everything is handed over with mbarriers (full/empty per smem stage,
-// full/empty per accumulator buffer, full/free per staging tile), so no warp
-// waits for another one's instruction stream; two accumulator buffers let the
-// epilogue of tile i overlap the main loop of tile i+1.
-//
-// FP16 epilogue: tcgen05.ld in the 16x256b (accumulator-fragment) shape with
-// the next chunk's load in flight during the arithmetic, FP32 math, pairs of
-// tokens packed to f16x2, stmatrix.trans into a 128-byte-swizzled
-// [32 tokens][64 features] staging tile, TMA store to Y (full 128-byte row
-// segments; rows beyond M and features beyond N clipped by the tensor map).
+//   warps 2-13  epilogue: each warp owns 32 tensor-memory lanes (features) and
+//               every third 16-token chunk, and works by itself from the
+//               accumulator to global memory
+// Stages and accumulators are handed over with mbarriers (full/empty per smem
+// stage, full/empty per accumulator buffer); two accumulator buffers let the
+// epilogue of tile i overlap the main loop of tile i+1.  Nothing is handed over
+// between epilogue warps.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -57,25 +46,18 @@ constexpr int kBlockF = 128;        // features per CTA and tile
 constexpr int kPairF = 2 * kBlockF; // features per CTA pair and tile
 constexpr int kBlockK = 128;        // K per stage
 constexpr int kMaxBlockT = 224;     // tokens per tile (runtime value, multiple of 32)
-constexpr int kChunkT = 32;         // tokens per epilogue chunk
-// Chunk phases of the epilogue: eight epilogue warps per phase.  Two (16 warps of 96 registers) is
-// what is built; one (8 warps) is as fast without GELU and slower with it or with INT8 output, three
-// (24 warps of 72 registers, two staging tiles per group) is 1.5x slower on every layer.
-#ifndef GPUSQ_PHASES
-#define GPUSQ_PHASES 2
-#endif
-constexpr int kMaxPhases = 3;       // chunk phases: eight epilogue warps (128 features) per phase
+constexpr int kChunkT = 16;         // tokens per epilogue chunk
+// Epilogue warps per 32 features, taking turns at the chunks.  Three (twelve warps of up to 128 registers)
+// is the best of two to four: with two the latencies of a chunk show, with four (96 registers) INT8 output
+// with GELU spills, and the set-up of a tile, which every warp does, is paid once more.
+constexpr int kTurns = 3;
+constexpr int kEpiWarps = 4 * kTurns;
+constexpr int kThreadsGemm = 32 * (2 + kEpiWarps);
 constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;     // column offset of the second accumulator
 constexpr int kMetaCol = 224;       // metadata slots: 4 columns per stage from here (below the second accumulator)
-constexpr int kMaxEpiGroups = 2 * kMaxPhases;   // groups of four epilogue warps: 64 features x chunk phase
-constexpr int kMaxEpiBufs = 3;                  // staging tiles per group, at most
-constexpr int kEpiBufBytes = kChunkT * 128;           // [32 tokens][64 features] f16
-// INT8 output has an epilogue of its own shape (EpiI8) and no store warps
-constexpr int kI8Turns = 3;                           // warps per 32 features, taking turns at the chunks
-constexpr int kI8Warps = 4 * kI8Turns;
-constexpr int kI8ChunkT = 16;                         // tokens per chunk
-constexpr int kI8BufBytes = kI8ChunkT * 32;           // [16 tokens][32 features] i8, two per warp
+constexpr int kEpiBufBytes = kChunkT * 64;            // [16 tokens][32 features] f16 (INT8 output uses half of it)
+constexpr int kEpiBytes = kEpiWarps * 2 * kEpiBufBytes;     // two buffers per epilogue warp
 
 // kHalf: the FP16 2:4 sparse model (binary16 operands, FP32 accumulators) instead of INT8.  A stage
 // still covers 128 columns of W: 128 bytes of kept values per feature row, and two 128-byte-swizzled
@@ -88,28 +70,18 @@ struct Cfg {
     static constexpr int kBBytes = kBAtoms * (kMaxBlockT / 2) * 128;   // this CTA's half of the token rows
     static constexpr int kMetaBytes = kSparse ? 2048 : 0;
     static constexpr int kStageBytes = kABytes + kBBytes + kMetaBytes;
-    static constexpr int kStages = kHalf ? 4 : kSparse ? 7 : 5;
-    // Epilogue warps: eight per chunk phase (the warps of phase p take the chunks c of a tile with
-    // (p + tile count) mod kPhases == c mod kPhases).
-    static constexpr int kPhases = kHalf ? 2 : GPUSQ_PHASES;
-    static constexpr int kEpiWarps = 8 * kPhases;
-    static constexpr int kStoreWarp0 = 2 + kEpiWarps;          // first of the two store warps
-    static constexpr int kThreads = 32 * (kStoreWarp0 + 2);
-    static constexpr int kEpiGroups = 2 * kPhases;             // 64 features x chunk phase: four warps share a staging tile
-    static constexpr int kEpiBufs = kPhases == 3 ? 2 : kPhases == 1 ? 6 : kHalf ? 2 : 3;      // staging tiles per group
-    static constexpr int kEpiBytes = kEpiGroups * kEpiBufs * kEpiBufBytes;
+    static constexpr int kStages = kHalf ? 4 : kSparse ? 8 : 6;
     static constexpr int kCtlBytes = 1024;
-    static constexpr int kSmemBytes = kStages * kStageBytes + kEpiBytes + kCtlBytes + 1024 /* alignment slack */;
+    static constexpr int kSmemBytes = kStages * kStageBytes + kEpiBytes + kCtlBytes + 2048 /* alignment slack */;
     static constexpr int kMmasPerStage = kHalf ? 4 : kSparse ? 2 : 4;
     static constexpr int kAStepBytes = 32;                    // per MMA along K, all variants
     static constexpr int kBStepBytes = kHalf ? 64 : kSparse ? 64 : 32;
     static constexpr int kASwizzle = kHalf ? 128 : kSparse ? 64 : 128;
     static constexpr int kMetaColsPerMma = kHalf ? 1 : 2;     // 32-bit tensor-memory columns of metadata per MMA
     static_assert(kStageBytes % 1024 == 0, "stages keep the 1024-byte alignment of the swizzled tiles");
+    static_assert((kStages * kStageBytes) % 2048 == 0, "staging buffers");
     static_assert(kStages <= 8, "eight metadata slots below the second accumulator");
     static_assert(kSmemBytes <= 232448, "shared memory per CTA");
-    static_assert(kI8Warps * 2 * kI8BufBytes <= kEpiBytes, "staging buffers of the INT8 epilogue");
-    static constexpr int threads(int out_type) { return out_type == GPUSQ_OUT_I8 ? 32 * (2 + kI8Warps) : kThreads; }
 };
 
 struct Ctl {
@@ -118,8 +90,6 @@ struct Ctl {
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
     uint64_t drain;
-    uint64_t stg_full[kMaxEpiGroups * kMaxEpiBufs];     // staging tile written by its four warps (flat: group * bufs + tile)
-    uint64_t stg_free[kMaxEpiGroups * kMaxEpiBufs];     // staging tile read by its TMA store
     uint32_t tmem_base;
     uint32_t abort_flag;
     uint32_t wait_us;       // directly behind the flag: the bounded waits read their limit from here
@@ -190,18 +160,18 @@ struct TileWalk {
     // the tile is one of the lower ones (token tiles from n_big on)
     __device__ __forceinline__ bool low(const GemmParams &p) const { return !twin(p) && tm >= p.n_big; }
     // first feature and first token of CTA `rank`'s part, and the tile's height in tokens
-    __device__ __forceinline__ void origin(const GemmParams &p, int rank, int &n0, int64_t &m0, int &h) const
+    __device__ __forceinline__ void origin(const GemmParams &p, int rank, int &n0, int &m0, int &h) const
     {
         if (twin(p)) {
             n0 = p.twin_n0;
-            m0 = ((int64_t)(tile - p.pair_tiles) * 2 + rank) * p.block_t;
+            m0 = ((tile - p.pair_tiles) * 2 + rank) * p.block_t;      // fits: see set_tiling
             h = p.block_t;
             return;
         }
         n0 = tn * kPairF + rank * kBlockF;
         const int below = tm - p.n_big;                 // > 0: that many lower tiles precede this one
         h = below >= 0 ? p.block_t - 32 : p.block_t;
-        m0 = (int64_t)tm * p.block_t - (below > 0 ? (int64_t)below * 32 : 0);
+        m0 = tm * p.block_t - (below > 0 ? below * 32 : 0);         // < M
     }
 };
 
@@ -254,216 +224,25 @@ __device__ __forceinline__ float2 gelu_pair(float2 y)
                       make_float2(fmaxf(y.x, 0.0f), fmaxf(y.y, 0.0f)));
 }
 
-// FP16 epilogue of one worker warp.  The warp owns 16 tensor-memory lanes (features) and every
-// other 32-token chunk of each tile.  Per chunk: wait for the chunk's tcgen05.ld (issued one chunk
-// ahead), issue the next one, convert / scale / activate 16 values per thread, wait for a free
-// staging tile, two stmatrix, proxy fence, arrive on the tile's full barrier.  The loop is written
-// for few instructions per chunk: whatever can be precomputed or advanced incrementally is.
-template <bool kAccFloat, int kBufs, int kPhases, bool kTwin>
-struct EpiF16 {
-    const GemmParams *p;
-    Ctl *ctl;
-    uint32_t tmem_base, stage0, stg_full0, stg_free0, tmem_empty0, tmem_empty1;
-    float x_scale;
-    int warp, lane, rank, cluster_id, num_clusters, tiles_n, num_tiles;
-
-    // staging-tile ring of this warp's group
-    uint32_t buf_addr, full_bar, free_bar, buf_idx, free_parity;
-    uint32_t stm_off;          // this lane's stmatrix row address inside a staging tile (second one: + 2048)
-    float2 sc2[2], bi2[2];     // scale and bias of this thread's two features, duplicated for packed math
-    float amax;                // kAmax: largest |y| this thread has produced for a token that exists
-
-    __device__ __forceinline__ void release(int acc)
-    {
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(acc ? tmem_empty1 : tmem_empty0);
-    }
-
-    // One chunk held in v (its load was issued earlier).  next_taddr != 0: issue this warp's next
-    // load into vn; otherwise v was the warp's last chunk of the tile and the accumulator is released.
-    // rows: tokens of the chunk that exist (32 except at the end of the tensor); only kAmax looks at
-    // it, the stores clip by themselves.
-    template <bool kGelu, bool kAmax>
-    __device__ __forceinline__ bool step(uint32_t (&v)[16], uint32_t (&vn)[16], uint32_t next_taddr, int acc,
-                                         int tile, int rows)
-    {
-        ptx::tmem_ld_wait_regs(v);
-        if (next_taddr)
-            ptx::tmem_ld_16x256b_x4(next_taddr, vn);
-        else
-            release(acc);
-        uint32_t pk[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                // INT32 sums are converted; the FP16 model's FP32 sums are taken as they are (scale 1)
-                const float2 a = kAccFloat ? make_float2(__uint_as_float(v[4 * i + 2 * j]), __uint_as_float(v[4 * i + 2 * j + 1]))
-                                           : make_float2(__int2float_rn((int32_t)v[4 * i + 2 * j]),
-                                                         __int2float_rn((int32_t)v[4 * i + 2 * j + 1]));
-                float2 y = __ffma2_rn(a, sc2[j], bi2[j]);
-                if (kGelu) y = gelu_pair(y);
-                const __half2 hh = __floats2half2_rn(y.x, y.y);   // low = token 2(t%4), high = +1
-                pk[2 * i + j] = *reinterpret_cast<const uint32_t *>(&hh);
-                if (kAmax) {
-                    // rounding is monotonic: the maximum of the rounded outputs is the rounded maximum.
-                    // Rows past the end of the tensor hold the bias only and do not count.
-                    const int tok = 8 * i + 2 * (lane & 3);
-                    if (rows >= kChunkT) {
-                        amax = fmaxf(amax, fmaxf(fabsf(y.x), fabsf(y.y)));
-                    } else {
-                        if (tok < rows) amax = fmaxf(amax, fabsf(y.x));
-                        if (tok + 1 < rows) amax = fmaxf(amax, fabsf(y.y));
-                    }
-                }
-            }
-        // the staging tile's previous contents have been stored
-        bool to;
-        if (!ptx::mbar_wait_bounded(free_bar, free_parity, &ctl->abort_flag, to)) {
-            if (to && lane == 0) report_timeout(*p, ctl, tile, 2, 200 + (int)buf_idx);
-            return false;
-        }
-        // matrices of one stmatrix: (tokens 0-7, feat 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15)
-        ptx::stmatrix_x4_trans(buf_addr + stm_off, pk[0], pk[1], pk[2], pk[3]);
-        ptx::stmatrix_x4_trans(buf_addr + stm_off + 2048u, pk[4], pk[5], pk[6], pk[7]);
-        ptx::fence_proxy_async_smem();                     // this lane's writes, for the TMA store
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(full_bar);
-        if (++buf_idx == (uint32_t)kBufs) {
-            buf_idx = 0;
-            free_parity ^= 1u;
-            buf_addr = stage0;
-            full_bar = stg_full0;
-            free_bar = stg_free0;
-        } else {
-            buf_addr += kEpiBufBytes;
-            full_bar += 8;
-            free_bar += 8;
-        }
-        return true;
-    }
-
-    template <bool kGelu, bool kAmax>
-    __device__ __forceinline__ void run()
-    {
-        const int quarter = warp & 3;                      // tensor-memory lanes [32q, 32q+32) are this warp's to read
-        const int half = ((warp - 2) >> 2) & 1;            // which 16 of them
-        const int par = (warp - 2) >> 3;                   // which chunks: every kPhases-th one
-        const int nofs = quarter * 32 + 16 * half + (lane >> 2);       // this thread's first feature in the CTA's 128
-        amax = 0.0f;
-        {
-            // stmatrix row of this lane: token 8 (mid / 2) + r of the tile, 16-byte column c16 (128-byte swizzle)
-            const int mid = lane >> 3, r = lane & 7;
-            const int tok = 8 * (mid >> 1) + r;
-            const int c16 = 4 * (quarter & 1) + 2 * half + (mid & 1);
-            stm_off = (uint32_t)(tok * 128 + ((c16 ^ r) << 4));
-        }
-        buf_addr = stage0;
-        full_bar = stg_full0;
-        free_bar = stg_free0;
-        buf_idx = 0;
-        free_parity = 1;                                   // first round: the tiles are free
-        const int64_t M = p->M;
-        const int N = p->N;
-        const float *w_scale = p->w_scale, *bias = p->bias;
-
-        // scale and bias of a tile are fetched one tile ahead: the loads are in flight during a whole tile
-        float ws_next[2], bi_next[2];
-        auto fetch = [&](const TileWalk<kTwin> &w) {
-            int n0, unused_h;
-            int64_t unused;
-            w.origin(*p, rank, n0, unused, unused_h);
-            const bool in = w.tile < num_tiles && n0 < N;
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int n = n0 + nofs + 8 * j;           // N need not fill the last 128-feature block
-                ws_next[j] = (in && n < N) ? (w_scale ? __ldg(w_scale + n) : 1.0f) : 0.0f;
-                bi_next[j] = (in && n < N && bias) ? __ldg(bias + n) : 0.0f;
-            }
-        };
-        TileWalk<kTwin> walk(*p, cluster_id, num_clusters);
-        fetch(walk);
-        int local = 0;
-        for (; walk.tile < num_tiles; ++local) {
-            const int tile = walk.tile;
-            int n0, h;
-            int64_t m0;
-            walk.origin(*p, rank, n0, m0, h);
-            walk.next(*p, num_clusters);
-            const int acc = local & 1;
-            const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
-            const bool n_valid = n0 < N;                   // the pair's second CTA may lie past the last feature
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float sc = __fmul_rn(ws_next[j], x_scale);
-                sc2[j] = make_float2(sc, sc);
-                bi2[j] = make_float2(bi_next[j], bi_next[j]);
-            }
-            fetch(walk);
-            bool to;
-            if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, &ctl->abort_flag, to)) {
-                if (to && lane == 0) report_timeout(*p, ctl, tile, 2, 100 + acc);
-                return;
-            }
-            ptx::tc_fence_after();
-            int nchunks = 0;
-            if (n_valid) {
-                const int64_t left = M - m0;               // > 0
-                nchunks = left >= h ? h / kChunkT : (int)((left + kChunkT - 1) / kChunkT);
-            }
-            // this warp's chunks of the tile: c0, c0 + kPhases, ...; the phases rotate every tile
-            const int c0 = (par + local) % kPhases;
-            int mine = (nchunks - c0 + kPhases - 1) / kPhases;         // how many of them
-            if (mine <= 0) {
-                release(acc);
-                continue;
-            }
-            uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32 + half * 16) << 16) +
-                             (uint32_t)(acc * kAccStride + c0 * kChunkT);
-            uint32_t v0[16], v1[16];
-            ptx::tmem_ld_16x256b_x4(taddr, v0);
-            // tokens that exist from this warp's chunk on (at least 32 everywhere but at the end of the tensor)
-            const int64_t ahead = M - m0 - (int64_t)c0 * kChunkT;
-            int rows = ahead > 4 * kMaxBlockT ? 4 * kMaxBlockT : (int)ahead;
-            for (;;) {
-                taddr += kPhases * kChunkT;
-                if (!step<kGelu, kAmax>(v0, v1, --mine ? taddr : 0u, acc, tile, rows)) return;
-                if (!mine) break;
-                rows -= kPhases * kChunkT;
-                taddr += kPhases * kChunkT;
-                if (!step<kGelu, kAmax>(v1, v0, --mine ? taddr : 0u, acc, tile, rows)) return;
-                if (!mine) break;
-                rows -= kPhases * kChunkT;
-            }
-        }
-        if (kAmax) {
-            // largest |Y| of this warp as the binary16 value that was stored, merged as a bit pattern
-            // (non-negative binary32 values order like their patterns)
-            float m = __half2float(__float2half_rn(amax));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == 0 && m > 0.0f) atomicMax(reinterpret_cast<unsigned int *>(p->y_absmax), __float_as_uint(m));
-        }
-    }
-};
-
-// INT8 epilogue of one worker warp (requantised output).  The warp owns 32 tensor-memory lanes
-// (features) and every third 16-token chunk, and works by itself from the accumulator to global memory:
-// two loads of 16 lanes x 16 columns in the accumulator-fragment shape (the next chunk's are in flight
-// during the arithmetic), after which a thread holds, for feature f = lane / 4 and f + 8, f + 16, f + 24,
-// the tokens 8 i + 2 (lane % 4) and the next one, i = 0, 1; the four codes of two tokens and two features
-// (f and f + 8) packed into one word are exactly the fragment of the 8-bit matrix store (stmatrix m16n8
-// b8, transposed), so one instruction puts the chunk, as 16 rows of 32 bytes, into one of the warp's two
-// staging buffers; a chunk later it is read back in 16-byte pieces and stored.  The 16-byte columns of a
-// row are permuted so that neither access has bank conflicts.  The __syncwarp behind a chunk's matrix
-// store also orders the reads of the chunk before against the matrix store of the chunk after.
-// What bounds it: instruction issue (~6 dispatch cycles per value, 14 with GELU).  No hand-over between
-// warps: the eight warps that filled a 128-feature tile together for a store warp's bulk stores needed,
-// per tile of 256 x 224 at K = 768, 5015 cycles of a loaded GPU (7371 with GELU); this needs 4014 (6170).
-// Twelve warps: eight (6505 with GELU) are short of latency hiding with GELU, sixteen of registers (8360).
-template <bool kTwin>
-struct EpiI8 {
+// Epilogue of one warp, FP16 (kI8 = false) or requantised INT8 output.  A chunk is 32 features x 16
+// tokens: two loads of 16 lanes x 16 columns in the accumulator-fragment shape, after which a thread
+// holds, for feature f = lane / 4 and f + 8, f + 16, f + 24, the tokens 8 i + 2 (lane % 4) and the next
+// one, i = 0, 1.  Transposing matrix stores put them, as rows of one token, into one of the warp's two
+// staging buffers (INT8: the four codes of two tokens and two features packed into one word are exactly
+// the fragment of the 8-bit matrix store); the buffer is read back in 16-byte pieces of rows, which are
+// stored to Y.  The 16-byte columns of a row are permuted so that neither access has bank conflicts.  The
+// __syncwarp behind a chunk's matrix stores also orders the reads of the chunk before against the matrix
+// stores of the chunk after.
+// What bounds it: the instructions issued.  The arithmetic takes 3 dispatch cycles per value (convert,
+// scale and half a pack; a packed FP32 instruction takes two), 13 with GELU, 6 to 16 with INT8 output;
+// everything else was made short: 32-bit tile arithmetic, one buffer of accumulators (the load of the next
+// chunk is issued as soon as this one is converted), scale and bias asked for before the wait for the
+// tile.  Sixteen warps that filled staging tiles together for two warps issuing bulk stores, as FP16
+// output had it, took for DeiT-Base at batch 64 (M = 12608): 768 -> 2304 19.7 us, 768 -> 3072 with GELU
+// 32.5, 3072 -> 768 21.5; this takes 19.0, 29.6, 20.0, part of it by the eighth pipeline stage for which
+// the staging tiles left no room.  Per-warp bulk stores instead of the plain ones: 19.3, 31.0, 19.8.
+template <bool kAccFloat, bool kI8, bool kTwin>
+struct Epilogue {
     const GemmParams *p;
     Ctl *ctl;
     uint32_t buf0, tmem_base, tmem_empty0, tmem_empty1;
@@ -471,10 +250,12 @@ struct EpiI8 {
     int warp, lane, rank, cluster_id, num_clusters;
 
     uint32_t stm_addr, lds_addr;   // this lane's matrix-store and read address in the current buffer
-    float2 sc2[4], bi2[4];         // scale and bias of this thread's four features, duplicated for packed math
-    uint8_t *y;                    // where this lane stores its 16 bytes of the chunk
-    int64_t y_step;
-    int rows;                      // rows of Y from y's on that exist (<= 0: this lane stores nothing)
+    uint8_t *y0, *y1;              // where this lane stores the first and (FP16) second eight tokens of the chunk
+    uint32_t row_bytes;            // of Y
+    int rows;                      // rows of Y from y0's on that exist (<= 0: this lane stores nothing)
+    float sc[4], bi[4];            // scale and bias of this thread's four features
+    int left;                      // tokens of the tile, from the chunk on, that exist
+    __half2 amax2;                 // kAmax: largest |y| this thread has produced for a token that exists
     QuantScale qs;
 
     __device__ __forceinline__ void release(int acc)
@@ -490,136 +271,178 @@ struct EpiI8 {
         ptx::tmem_ld_16x256b_x2(taddr + (16u << 16), v, 8);
     }
 
-    // the chunk whose matrix store was issued last: read it back and store it to Y
-    __device__ __forceinline__ void flush()
-    {
-        const uint4 w = ptx::ld_shared_v4(lds_addr);
-        if (rows > 0) *reinterpret_cast<uint4 *>(y) = w;
-        y += y_step;
-        rows -= kI8Turns * kI8ChunkT;
-        lds_addr ^= (uint32_t)kI8BufBytes;
-    }
-
-    // One chunk held in v (its loads were issued earlier).  next_taddr != 0: issue this warp's next loads
-    // into vn; otherwise v was the warp's last chunk of the tile and the accumulator is released.  kFlush:
-    // the chunk before this one is stored to Y in the shadow of this one's arithmetic.
-    template <bool kGelu, bool kFlush>
-    __device__ __forceinline__ void step(uint32_t (&v)[16], uint32_t (&vn)[16], uint32_t next_taddr, int acc)
-    {
-        ptx::tmem_ld_wait_regs(v);
-        if (next_taddr)
-            load(next_taddr, vn);
-        else
-            release(acc);
-        if (kFlush) flush();
-        float2 f[8], m[8];
-        float big = 0.0f;
-        uint32_t differ = 0, pk[4];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int j = 2 * (e >> 2) + (e & 1);          // which of the four features
-            f[e] = __ffma2_rn(make_float2(__int2float_rn((int32_t)v[2 * e]), __int2float_rn((int32_t)v[2 * e + 1])), sc2[j], bi2[j]);
-            if (kGelu) f[e] = gelu_pair(f[e]);
-            big = ptx::max3_abs(big, f[e].x, f[e].y);
-            m[e] = quant2_sums<false>(f[e], qs, differ);
-        }
-        // values beyond +-127 out_scale saturate, and products next to a rounding tie do not decide: both
-        // are rare, only detected here and redone by the exact branch, clamp included
-        if (differ != 0u || big > qs.x_max || qs.always_divide) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) m[e] = quant2_exact<true>(f[e], qs);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) pk[i] = pack4_low_bytes(m[2 * i], m[2 * i + 1]);
-        ptx::stmatrix_x4_trans_b8(stm_addr, pk[0], pk[1], pk[2], pk[3]);
-        __syncwarp();
-        stm_addr ^= (uint32_t)kI8BufBytes;
-    }
-
+    // value pair e of the chunk: features f + 8 (e % 2) + 16 (e / 4), tokens 8 (e / 2 % 2) + 2 (lane % 4), + 1
     template <bool kGelu>
+    __device__ __forceinline__ float2 value(const uint32_t (&v)[16], int e) const
+    {
+        const int j = 2 * (e >> 2) + (e & 1);
+        // INT32 sums are converted; the FP16 model's FP32 sums are taken as they are (scale 1)
+        const float2 a = kAccFloat ? make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]))
+                                   : make_float2(__int2float_rn((int32_t)v[2 * e]), __int2float_rn((int32_t)v[2 * e + 1]));
+        const float2 y = __ffma2_rn(a, make_float2(sc[j], sc[j]), make_float2(bi[j], bi[j]));
+        return kGelu ? gelu_pair(y) : y;
+    }
+
+    template <bool kGelu, bool kAmax>
+    __device__ __forceinline__ void convert(const uint32_t (&v)[16], uint32_t (&pk)[8])
+    {
+        if (kI8) {
+            float2 y[8], m[8];
+            float big = 0.0f;
+            uint32_t differ = 0;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                y[e] = value<kGelu>(v, e);
+                big = ptx::max3_abs(big, y[e].x, y[e].y);
+                m[e] = quant2_sums<false>(y[e], qs, differ);
+            }
+            // values beyond +-127 out_scale saturate, and products next to a rounding tie do not decide: both
+            // are rare, only detected here and redone by the exact branch, clamp included
+            if (differ != 0u || big > qs.x_max || qs.always_divide) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) m[e] = quant2_exact<true>(y[e], qs);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) pk[i] = pack4_low_bytes(m[2 * i], m[2 * i + 1]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float2 y = value<kGelu>(v, e);
+                const __half2 hh = __floats2half2_rn(y.x, y.y);   // low = token 2(t%4), high = +1
+                pk[e] = *reinterpret_cast<const uint32_t *>(&hh);
+                if (kAmax) {
+                    __half2 a = hh;
+                    if (left < kChunkT) {                          // tokens past the end hold the bias only
+                        const int tok = 8 * ((e >> 1) & 1) + 2 * (lane & 3);
+                        a = make_half2(tok < left ? __low2half(hh) : __ushort_as_half(0),
+                                       tok + 1 < left ? __high2half(hh) : __ushort_as_half(0));
+                    }
+                    amax2 = __hmax2(amax2, __habs2(a));
+                }
+            }
+        }
+    }
+
+    __device__ __forceinline__ void put(const uint32_t (&pk)[8])
+    {
+        if (kI8) {
+            ptx::stmatrix_x4_trans_b8(stm_addr, pk[0], pk[1], pk[2], pk[3]);
+        } else {
+            // matrices of one store: (tokens 0-7, feat 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15)
+            ptx::stmatrix_x4_trans(stm_addr, pk[0], pk[1], pk[2], pk[3]);
+            ptx::stmatrix_x4_trans(stm_addr ^ 32u, pk[4], pk[5], pk[6], pk[7]);
+        }
+        __syncwarp();
+        const uint4 w0 = ptx::ld_shared_v4(lds_addr);
+        if (rows > 0) *reinterpret_cast<uint4 *>(y0) = w0;
+        if (!kI8) {
+            const uint4 w1 = ptx::ld_shared_v4(lds_addr + 512u);
+            if (rows > 8) *reinterpret_cast<uint4 *>(y1) = w1;
+            y1 += (uint64_t)(kTurns * kChunkT * row_bytes);
+        }
+        y0 += (uint64_t)(kTurns * kChunkT * row_bytes);
+        rows -= kTurns * kChunkT;
+        lds_addr ^= (uint32_t)kEpiBufBytes;
+        stm_addr ^= (uint32_t)kEpiBufBytes;
+        left -= kTurns * kChunkT;
+    }
+
+    template <bool kGelu, bool kAmax>
     __device__ __forceinline__ void run()
     {
         const int quarter = warp & 3;                      // tensor-memory lanes [32q, 32q+32) are this warp's to read
-        const int turn = (warp - 2) >> 2;                  // which chunks: every kI8Turns-th one
-        const int nofs = quarter * 32 + (lane >> 2);       // this thread's first feature in the CTA's 128
-        const int row_l = lane >> 1, col_l = quarter * 32 + (lane & 1) * 16;      // this lane's row and feature when storing
+        const int turn = (warp - 2) >> 2;                  // which chunks: every kTurns-th one
         {
-            // this lane addresses memory row lane % 8 of matrix lane / 8: token t, features 16 (matrix / 2) ...
-            const int t = 8 * ((lane >> 3) & 1) + (lane & 7);
-            stm_addr = buf0 + (uint32_t)(t * 32 + (((lane >> 4) ^ ((t >> 2) & 1)) << 4));
-            lds_addr = buf0 + (uint32_t)(row_l * 32 + (((lane & 1) ^ ((row_l >> 2) & 1)) << 4));
+            const int mid = lane >> 3, rr = lane & 7;      // this lane addresses memory row rr of matrix mid
+            if (kI8) {
+                const int t = 8 * (mid & 1) + rr;
+                stm_addr = buf0 + (uint32_t)(t * 32 + (((mid >> 1) ^ ((t >> 2) & 1)) << 4));
+            } else {
+                const int t = 8 * (mid >> 1) + rr;
+                stm_addr = buf0 + (uint32_t)(t * 64 + (((mid & 1) ^ ((t >> 1) & 3)) << 4));
+            }
         }
-        const int64_t M = p->M;
-        const int N = p->N;
-        const float *w_scale = p->w_scale, *bias = p->bias;
-        y_step = (int64_t)kI8Turns * kI8ChunkT * N;
-        qs = make_quant_scale(out_scale);
+        const int M = (int)p->M, N = p->N;
+        const int row_l = kI8 ? lane >> 1 : lane >> 2, col_l = kI8 ? (lane & 1) * 16 : (lane & 3) * 8;
+        lds_addr = kI8 ? buf0 + (uint32_t)(row_l * 32 + (((lane & 1) ^ ((row_l >> 2) & 1)) << 4))
+                       : buf0 + (uint32_t)(row_l * 64 + (((lane & 3) ^ ((row_l >> 1) & 3)) << 4));
+        row_bytes = (uint32_t)N * (kI8 ? 1u : 2u);
+        // this thread's first feature, relative to the CTA's 128
+        const int nofs = quarter * 32 + (lane >> 2);
+        const float *w_scale = p->w_scale + nofs, *bias = p->bias + nofs;
+        const bool has_scale = p->w_scale != nullptr, has_bias = p->bias != nullptr;
+        amax2 = __half2half2(__ushort_as_half(0));
+        if (kI8) qs = make_quant_scale(out_scale);
+        const uint32_t full0 = ptx::smem_u32(&ctl->tmem_full[0]);
+        const uint32_t lane_taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
 
-        // scale and bias of a tile are fetched one tile ahead: the loads are in flight during a whole tile
-        float ws_next[4], bi_next[4];
-        auto fetch = [&](const TileWalk<kTwin> &w) {
-            int n0, unused_h;
-            int64_t unused;
-            w.origin(*p, rank, n0, unused, unused_h);
-            const bool in = w.tile < p->num_tiles;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int n = n0 + nofs + 8 * j;
-                ws_next[j] = (in && n < N) ? __ldg(w_scale + n) : 0.0f;
-                bi_next[j] = (in && n < N && bias) ? __ldg(bias + n) : 0.0f;
-            }
-        };
         TileWalk<kTwin> walk(*p, cluster_id, num_clusters);
-        fetch(walk);
-        int local = 0, done = 0;                           // tiles; chunks so far modulo kI8Turns
-        for (; walk.tile < p->num_tiles; ++local) {
-            const int tile = walk.tile;
-            int n0, h;
-            int64_t m0;
+        int acc = 0, done = 0;                             // accumulator; chunks so far modulo kTurns
+        uint32_t acc_phase = 0;
+        while (walk.tile < p->num_tiles) {
+            int n0, m0, h;
             walk.origin(*p, rank, n0, m0, h);
-            walk.next(*p, num_clusters);
-            const int acc = local & 1;
-            const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
+            // asked for now, needed after the first chunk has come in; N need not fill the last 128 features
+            const bool whole = n0 + kBlockF <= N;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float sc = __fmul_rn(ws_next[j], x_scale);
-                sc2[j] = make_float2(sc, sc);
-                bi2[j] = make_float2(bi_next[j], bi_next[j]);
+                const bool in = whole || n0 + nofs + 8 * j < N;
+                sc[j] = in && has_scale ? __ldg(w_scale + n0 + 8 * j) : 1.0f;
+                bi[j] = in && has_bias ? __ldg(bias + n0 + 8 * j) : 0.0f;
             }
-            fetch(walk);
             // tokens of the tile that exist (none: a twin tile's second half); the warps of a quarter take
             // the chunks in turn, across tiles
-            const int64_t ahead = M - m0;
-            const int left = ahead < h ? (ahead > 0 ? (int)ahead : 0) : h;
-            const int all = (left + kI8ChunkT - 1) / kI8ChunkT;
-            const int first = turn >= done ? turn - done : turn - done + kI8Turns;
-            done = (done + all) % kI8Turns;
-            int chunks = n0 + quarter * 32 < N ? (all - first + kI8Turns - 1) / kI8Turns : 0;    // none past the last feature
-            rows = n0 + col_l < N ? left - first * kI8ChunkT - row_l : 0;
-            y = reinterpret_cast<uint8_t *>(p->Y) + (m0 + first * kI8ChunkT + row_l) * N + n0 + col_l;
+            left = min(M - m0, h);
+            if (kTwin) left = max(left, 0);
+            const int all = (left + kChunkT - 1) / kChunkT;
+            int first = turn - done;
+            if (first < 0) first += kTurns;
+            done = (done + all) % kTurns;
+            int chunks = n0 + quarter * 32 < N ? (all - first + kTurns - 1) / kTurns : 0;    // none past the last feature
+            left -= first * kChunkT;
+            const int col = n0 + quarter * 32 + col_l;
+            rows = col < N ? left - row_l : 0;
+            y0 = reinterpret_cast<uint8_t *>(p->Y) + (uint64_t)((uint32_t)m0 + (uint32_t)(first * kChunkT + row_l)) * row_bytes +
+                 (uint32_t)col * (kI8 ? 1u : 2u);
+            y1 = y0 + (uint64_t)(8u * row_bytes);
+            uint32_t taddr = lane_taddr + (uint32_t)(acc * kAccStride + first * kChunkT);
             bool to;
-            if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, &ctl->abort_flag, to)) {
-                if (to && lane == 0) report_timeout(*p, ctl, tile, 2, 100 + acc);
-                return;
+            if (!ptx::mbar_wait_bounded(full0 + 8u * acc, acc_phase, &ctl->abort_flag, to)) {
+                if (to && lane == 0) report_timeout(*p, ctl, walk.tile, 2, 100 + acc);
+                break;
             }
             ptx::tc_fence_after();
             if (chunks <= 0) {
                 release(acc);
-                continue;
+            } else {
+                uint32_t v[16];
+                load(taddr, v);
+                if (!kAccFloat) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) sc[j] = __fmul_rn(sc[j], x_scale);
+                }
+                for (;;) {
+                    uint32_t pk[8];
+                    ptx::tmem_ld_wait_regs(v);
+                    if (--chunks == 0) release(acc);
+                    convert<kGelu, kAmax>(v, pk);
+                    if (chunks) {
+                        taddr += kTurns * kChunkT;
+                        load(taddr, v);
+                    }
+                    put(pk);
+                    if (!chunks) break;
+                }
             }
-            uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccStride + first * kI8ChunkT);
-            uint32_t v0[16], v1[16];
-            load(taddr, v0);
-            taddr += kI8Turns * kI8ChunkT;
-            step<kGelu, false>(v0, v1, --chunks ? taddr : 0u, acc);
-            while (chunks) {
-                taddr += kI8Turns * kI8ChunkT;
-                step<kGelu, true>(v1, v0, --chunks ? taddr : 0u, acc);
-                if (!chunks) break;
-                taddr += kI8Turns * kI8ChunkT;
-                step<kGelu, true>(v0, v1, --chunks ? taddr : 0u, acc);
-            }
-            flush();
+            walk.next(*p, num_clusters);
+            acc ^= 1;
+            acc_phase ^= acc == 0 ? 1u : 0u;
+        }
+        if (kAmax) {
+            float m = fmaxf(__low2float(amax2), __high2float(amax2));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0 && m > 0.0f) atomicMax(reinterpret_cast<unsigned int *>(p->y_absmax), __float_as_uint(m));
         }
     }
 };
@@ -629,19 +452,17 @@ struct EpiI8 {
 // kAmax: the FP16 epilogue also merges max |Y| into a device word (its own instantiation, so that the
 // ordinary kernel's register allocation is untouched)
 template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((Cfg<kSparse, kHalf>::threads(kOut)), 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsGemm, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_e,
-               const __grid_constant__ CUtensorMap map_y, const GemmParams p)
+               const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_e, const GemmParams p)
 {
     using C = Cfg<kSparse, kHalf>;
     extern __shared__ uint8_t smem_raw[];
-    // operand tiles need 1024-byte alignment for the 128-byte swizzle; both CTAs of a pair get the same offsets
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // operand tiles need 1024-byte alignment for the 128-byte swizzle, the pairs of staging buffers 2048 (the
+    // second is reached by flipping an address bit); both CTAs of a pair get the same offsets
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 2047) & ~uintptr_t(2047));
     uint8_t *epi_smem = smem + C::kStages * C::kStageBytes;
-    Ctl *ctl = reinterpret_cast<Ctl *>(epi_smem + C::kEpiBytes);
-    constexpr int kBufs = C::kEpiBufs;      // staging tiles per group in the FP16-output path
-    constexpr int kPhases = C::kPhases, kEpiWarps = kOut == GPUSQ_OUT_I8 ? kI8Warps : C::kEpiWarps, kStoreWarp0 = 2 + kEpiWarps;
+    Ctl *ctl = reinterpret_cast<Ctl *>(epi_smem + kEpiBytes);
     volatile uint32_t *abort_flag = &ctl->abort_flag;
 
     const int warp = threadIdx.x >> 5;
@@ -649,13 +470,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t rank = ptx::cluster_ctarank();            // 0 issues the MMAs of the pair
     const int cluster_id = blockIdx.x >> 1;
     const int num_clusters = gridDim.x >> 1;
-    const int tiles_n = (p.N + kPairF - 1) / kPairF;
     const int num_tiles = p.num_tiles;
     const int k_blocks = (p.K + kBlockK - 1) / kBlockK;        // k blocks of the layer; a twin tile takes them twice
-
-    auto a_smem = [&](int s) { return smem + s * C::kStageBytes; };
-    auto b_smem = [&](int s) { return smem + s * C::kStageBytes + C::kABytes; };
-    auto m_smem = [&](int s) { return smem + s * C::kStageBytes + C::kABytes + C::kBBytes; };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
@@ -667,10 +483,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             ptx::mbar_init(ptx::smem_u32(&ctl->tmem_empty[a]), 2 * kEpiWarps);   // the epilogue warps of both CTAs
         }
         ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
-        for (int g = 0; g < C::kEpiGroups * kBufs; ++g) {
-            ptx::mbar_init(ptx::smem_u32(&ctl->stg_full[g]), 4);
-            ptx::mbar_init(ptx::smem_u32(&ctl->stg_free[g]), 1);
-        }
         ctl->abort_flag = 0;
         ctl->wait_us = p.wait_us;
         ptx::fence_barrier_init();
@@ -678,7 +490,6 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ptx::prefetch_tensormap(&map_b);
         if (p.n_big * p.pair_cols < p.pair_tiles) ptx::prefetch_tensormap(&map_b2);
         if (kSparse) ptx::prefetch_tensormap(&map_e);
-        if (kOut == GPUSQ_OUT_F16) ptx::prefetch_tensormap(&map_y);
     }
     if (warp == 1) {
         ptx::tmem_alloc_pair(ptx::smem_u32(&ctl->tmem_base), kTmemCols);
@@ -698,67 +509,63 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (ptx::elect_one()) {
+            const uint32_t smem0 = ptx::smem_u32(smem);
+            const uint32_t empty0 = ptx::smem_u32(&ctl->empty[0]), full_own = ptx::smem_u32(&ctl->full[0]);
+            const uint32_t full0 = ptx::map_to_cta(full_own, 0);    // all bytes of a stage are counted on CTA 0's barrier
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued = 0;            // bit s: a load into stage s was issued
             uint32_t last_parity = 0;       // bit s: parity of the last phase issued into stage s
             bool ok = true;
             for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles; walk.next(p, num_clusters)) {
-                const int tile = walk.tile;
                 const bool twin = walk.twin(p);
-                const int tw = tile - p.pair_tiles;                               // index among the twin tiles
-                const int tn = twin ? 0 : walk.tn;
-                const int num_kb = twin ? 2 * k_blocks : k_blocks;
-                int n0_unused, h;
-                int64_t m0;
-                walk.origin(p, 0, n0_unused, m0, h);                               // token origin of the pair's tile
-                const int half_t = h >> 1;
-                const CUtensorMap *mb = h == p.block_t ? &map_b : &map_b2;         // box height = half the tile's tokens
+                int n0, m0, h;
+                walk.origin(p, (int)rank, n0, m0, h);
+                if (!twin) m0 += (int)rank * (h >> 1);                            // this CTA's half of the tile's tokens
+                else m0 += (int)rank * ((h >> 1) - p.block_t);                    // of CTA 0's tile first
+                const CUtensorMap *mb = h == p.block_t ? &map_b : &map_b2;        // box height = half the tile's tokens
+                const uint32_t half_bytes = (uint32_t)((h >> 1) * 128);
                 // bytes both CTAs together bring in per stage
-                const uint32_t stage_tx = 2u * (uint32_t)(C::kABytes + C::kBAtoms * half_t * 128 + C::kMetaBytes);
-                for (int ks = 0; ks < num_kb; ++ks) {
-                    if (p.withhold && tile == 0 && ks == num_kb - 1) {
-                        // planted failure (test hook): these loads never come, the MMA issuer's wait runs out
-                        ok = false;
-                        break;
+                const uint32_t stage_tx = 2u * (uint32_t)(C::kABytes + C::kMetaBytes) + 2u * C::kBAtoms * half_bytes;
+                // twin tiles: the first pass of the k blocks runs against the token tile of CTA 0, whose weights
+                // sit in that CTA only (the other one loads zeros from beyond the tensor), the second against CTA 1's
+                int f0 = twin && rank == 1 ? p.oob_row : n0;                      // first weight row loaded
+                int e_row = (n0 / kBlockF) * k_blocks * 8;                        // 2 KB metadata block = 8 rows of 256 bytes
+                const int passes = twin ? 2 : 1;
+                for (int pass = 0; ok && pass < passes; ++pass) {
+                    for (int kb = 0; kb < k_blocks; ++kb) {
+                        if (p.withhold && walk.tile == 0 && pass == passes - 1 && kb == k_blocks - 1) {
+                            // planted failure (test hook): these loads never come, the MMA issuer's wait runs out
+                            ok = false;
+                            break;
+                        }
+                        bool to;
+                        if (!ptx::mbar_wait_bounded(empty0 + 8u * stage, phase ^ 1u, abort_flag, to)) {
+                            if (to) report_timeout(p, ctl, walk.tile, 0, stage);
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t bar = full0 + 8u * stage;
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full_own + 8u * stage, stage_tx);
+                        const uint32_t a = smem0 + (uint32_t)(stage * C::kStageBytes), b = a + C::kABytes;
+                        ptx::tma_load_2d_pair(a, &map_a, bar, kb * (kHalf ? 128 : kSparse ? 64 : 128), f0);
+                        if (kHalf) {
+                            // 128 binary16 columns = two tiles of 128 bytes per token row
+                            ptx::tma_load_2d_pair(b, mb, bar, kb * 256, m0);
+                            ptx::tma_load_2d_pair(b + half_bytes, mb, bar, kb * 256 + 128, m0);
+                        } else {
+                            ptx::tma_load_2d_pair(b, mb, bar, kb * kBlockK, m0);
+                        }
+                        if (kSparse) ptx::tma_load_2d_pair(b + C::kBBytes, &map_e, bar, 0, e_row + kb * 8);
+                        issued |= 1u << stage;
+                        last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
+                        if (++stage == C::kStages) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
                     }
-                    // twin tiles: pass `seg` of the k blocks runs against the token tile of CTA `seg`, whose
-                    // weights sit in that CTA only (the other one loads zeros from beyond the tensor)
-                    const int seg = twin ? ks / k_blocks : 0;
-                    const int kb = ks - seg * k_blocks;
-                    const int w0 = twin ? p.twin_n0 : tn * kPairF + (int)rank * kBlockF;   // first weight row wanted
-                    const int f0 = (twin && seg != (int)rank) ? p.oob_row : w0;          // first weight row loaded
-                    const int t0 = (twin ? (2 * tw + seg) * p.block_t : (int)m0) + (int)rank * half_t;
-                    bool to;
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, tile, 0, stage);
-                        ok = false;
-                        break;
-                    }
-                    // all bytes of the stage, from both CTAs, are counted on CTA 0's barrier
-                    const uint32_t bar = ptx::map_to_cta(ptx::smem_u32(&ctl->full[stage]), 0);
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(ptx::smem_u32(&ctl->full[stage]), stage_tx);
-                    ptx::tma_load_2d_pair(ptx::smem_u32(a_smem(stage)), &map_a, bar,
-                                          kb * (kHalf ? 128 : kSparse ? 64 : 128), f0);
-                    if (kHalf) {
-                        // 128 binary16 columns = two tiles of 128 bytes per token row
-                        ptx::tma_load_2d_pair(ptx::smem_u32(b_smem(stage)), mb, bar, kb * 256, t0);
-                        ptx::tma_load_2d_pair(ptx::smem_u32(b_smem(stage)) + (uint32_t)(half_t * 128), mb, bar,
-                                              kb * 256 + 128, t0);
-                    } else {
-                        ptx::tma_load_2d_pair(ptx::smem_u32(b_smem(stage)), mb, bar, kb * kBlockK, t0);
-                    }
-                    if (kSparse) {
-                        // 2 KB metadata block of (feature tile, k block) = 8 rows of 256 bytes
-                        ptx::tma_load_2d_pair(ptx::smem_u32(m_smem(stage)), &map_e, bar, 0,
-                                              ((w0 / kBlockF) * k_blocks + kb) * 8);
-                    }
-                    issued |= 1u << stage;
-                    last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == C::kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                    m0 += p.block_t;
+                    f0 = rank == 1 ? n0 : p.oob_row;
                 }
             }
             if (*abort_flag && rank == 0) {
@@ -779,18 +586,20 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                              : ptx::make_idesc_i8(kPairF, p.block_t, kSparse);
             const uint32_t idesc_low = kHalf ? ptx::make_idesc_f16_sparse(kPairF, p.block_t - 32)
                                              : ptx::make_idesc_i8(kPairF, p.block_t - 32, kSparse);
+            const uint32_t full0 = ptx::smem_u32(&ctl->full[0]), empty0 = ptx::smem_u32(&ctl->empty[0]);
+            const uint32_t tfull0 = ptx::smem_u32(&ctl->tmem_full[0]), tempty0 = ptx::smem_u32(&ctl->tmem_empty[0]);
+            const uint64_t adesc0 = ptx::make_smem_desc(ptx::smem_u32(smem), C::kASwizzle * 8, C::kASwizzle);
+            const uint64_t bdesc0 = ptx::make_smem_desc(ptx::smem_u32(smem) + C::kABytes, 1024, 128);
+            const uint64_t edesc0 = ptx::make_smem_desc(ptx::smem_u32(smem) + C::kABytes + C::kBBytes, 128, 0);
             int stage = 0;
             uint32_t phase = 0;
-            int local = 0;
+            int acc = 0;
+            uint32_t acc_phase = 0;
             bool ok = true;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles;
-                 walk.next(p, num_clusters), ++local) {
-                const int tile = walk.tile;
-                const int acc = local & 1;
-                const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
+            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles; walk.next(p, num_clusters)) {
                 bool to;
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag, to)) {
-                    if (to) report_timeout(p, ctl, tile, 1, 100 + acc);
+                if (!ptx::mbar_wait_bounded(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, to)) {
+                    if (to) report_timeout(p, ctl, walk.tile, 1, 100 + acc);
                     ok = false;
                     break;
                 }
@@ -800,25 +609,23 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 // a tile of lower height (the token tiles from n_big on) takes the narrower instruction
                 const bool low = walk.low(p);
                 const uint32_t idesc = low ? idesc_low : idesc_big;
-                const int half_t = (low ? p.block_t - 32 : p.block_t) >> 1;
+                const uint32_t half_units = (uint32_t)(((low ? p.block_t - 32 : p.block_t) >> 1) * 128) >> 4;
                 for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, tile, 1, stage);
+                    if (!ptx::mbar_wait_bounded(full0 + 8u * stage, phase, abort_flag, to)) {
+                        if (to) report_timeout(p, ctl, walk.tile, 1, stage);
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
+                    const uint64_t off = (uint64_t)((uint32_t)(stage * C::kStageBytes) >> 4);
                     const uint32_t meta_t = tmem_base + (uint32_t)(kMetaCol + 4 * stage);
-                    if (kSparse) {
-                        ptx::tc_cp_128x128b_pair(meta_t, ptx::make_smem_desc(ptx::smem_u32(m_smem(stage)), 128, 0));
-                    }
-                    const uint64_t adesc = ptx::make_smem_desc(ptx::smem_u32(a_smem(stage)), C::kASwizzle * 8, C::kASwizzle);
-                    const uint64_t bdesc = ptx::make_smem_desc(ptx::smem_u32(b_smem(stage)), 1024, 128);
+                    if (kSparse) ptx::tc_cp_128x128b_pair(meta_t, edesc0 + off);
+                    const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
 #pragma unroll
                     for (int k = 0; k < C::kMmasPerStage; ++k) {
                         const uint64_t ad = adesc + (uint64_t)((k * C::kAStepBytes) >> 4);
                         // FP16 model: MMAs 0, 1 read the first activation tile of the stage, 2, 3 the second
-                        const uint64_t bd = kHalf ? bdesc + (uint64_t)(((k & 1) * 64 + (k >> 1) * half_t * 128) >> 4)
+                        const uint64_t bd = kHalf ? bdesc + (uint64_t)(((k & 1) * 64) >> 4) + (uint64_t)((k >> 1) * half_units)
                                                   : bdesc + (uint64_t)((k * C::kBStepBytes) >> 4);
                         const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
                         // 16-bit operands: one metadata column per MMA, addressed as an even column plus
@@ -832,13 +639,15 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             ptx::tc_mma_i8_pair(d_tmem, ad, bd, idesc, accum);
                     }
                     // the stage is reusable in both CTAs once these MMAs are done
-                    ptx::tc_commit_pair(ptx::smem_u32(&ctl->empty[stage]), 3);
+                    ptx::tc_commit_pair(empty0 + 8u * stage, 3);
                     if (++stage == C::kStages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (ok) ptx::tc_commit_pair(ptx::smem_u32(&ctl->tmem_full[acc]), 3);
+                if (ok) ptx::tc_commit_pair(tfull0 + 8u * acc, 3);
+                acc ^= 1;
+                acc_phase ^= acc == 0 ? 1u : 0u;
             }
             if (*abort_flag) {
                 // let every MMA issued so far retire before tensor memory is released
@@ -848,92 +657,19 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 (void)ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->drain), 0, none, to);
             }
         }
-    } else if (warp >= kStoreWarp0) {
-        // --------------------------------------------------------- TMA stores
-        // One lane per 64-feature half: waits for a staging tile to be filled, stores it, and hands
-        // tiles back to the epilogue warps once the stores have read them.
-        if (kOut == GPUSQ_OUT_F16 && ptx::elect_one()) {
-            const int fgroup = warp - kStoreWarp0;         // features [64 fgroup, 64 fgroup + 64) of the CTA's 128
-            uint32_t filled[kMaxPhases] = {};              // staging tiles stored so far, per chunk phase
-            uint32_t prev1 = 0, prev2 = 0;                 // free barriers of the last two stores (0 = none)
-            int local = 0;
-            bool ok = true;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles;
-                 walk.next(p, num_clusters), ++local) {
-                const int tile = walk.tile;
-                int n0, h;
-                int64_t m0;
-                walk.origin(p, (int)rank, n0, m0, h);
-                if (n0 >= p.N) continue;
-                const int64_t left = p.M - m0;
-                const int nchunks = left >= h ? h / kChunkT : (int)((left + kChunkT - 1) / kChunkT);
-                for (int c = 0; c < nchunks; ++c) {
-                    const int par = (c + kPhases - local % kPhases) % kPhases;     // the warps with (par + local) % kPhases == c % kPhases fill this chunk
-                    const int gi = fgroup * kPhases + par;
-                    const uint32_t count = filled[par];
-                    const uint32_t b = count % kBufs;
-                    bool to;
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->stg_full[gi * kBufs + (int)b]), (count / kBufs) & 1u,
-                                                abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, tile, 3, gi * 8 + (int)b);
-                        ok = false;
-                        break;
-                    }
-                    ptx::tma_store_2d(&map_y, ptx::smem_u32(epi_smem + (gi * kBufs + (int)b) * kEpiBufBytes),
-                                      n0 + fgroup * 64, (int32_t)(m0 + c * kChunkT));
-                    ptx::tma_store_commit();
-                    // all but the two newest stores have read their tiles: hand the third newest back
-                    ptx::tma_store_wait_read<2>();
-                    if (prev2) ptx::mbar_arrive(prev2);
-                    prev2 = prev1;
-                    prev1 = ptx::smem_u32(&ctl->stg_free[gi * kBufs + (int)b]);
-                    ++filled[par];
-                }
-            }
-            // the staging tiles must stay valid until the bulk stores have read them, and the
-            // stores must be complete before the kernel ends
-            ptx::tma_store_wait_all<0>();
-        }
     } else {
         // ------------------------------------------------------------ epilogue
         const int quarter = warp & 3;                      // tensor-memory lanes [32q, 32q+32) are this warp's to read
-        const int par = (warp - 2) >> 3;                   // FP16 path: which chunks, every other one
         const float x_scale = (kOut == GPUSQ_OUT_I32 || kHalf) ? 1.0f : __ldg(p.x_scale);
         const float out_scale = (kOut == GPUSQ_OUT_I8) ? __ldg(p.out_scale) : 1.0f;
         // the accumulators of both CTAs are released on CTA 0's barrier, where the MMA issuer waits
         const uint32_t tmem_empty0 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[0]), 0);
         const uint32_t tmem_empty1 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[1]), 0);
-        const int group = (quarter >> 1) * kPhases + par;  // 64 features x chunk phase: the warps sharing staging tiles
-        const uint32_t stage0 = ptx::smem_u32(epi_smem + group * kBufs * kEpiBufBytes);
-        int local = 0;
-
-        if (kOut == GPUSQ_OUT_F16) {
-            EpiF16<kHalf, kBufs, kPhases, kTwin> e;
+        if (kOut == GPUSQ_OUT_F16 || kOut == GPUSQ_OUT_I8) {
+            Epilogue<kHalf, kOut == GPUSQ_OUT_I8, kTwin> e;
             e.p = &p;
             e.ctl = ctl;
-            e.tmem_base = tmem_base;
-            e.stage0 = stage0;
-            e.stg_full0 = ptx::smem_u32(&ctl->stg_full[group * kBufs]);
-            e.stg_free0 = ptx::smem_u32(&ctl->stg_free[group * kBufs]);
-            e.tmem_empty0 = tmem_empty0;
-            e.tmem_empty1 = tmem_empty1;
-            e.x_scale = x_scale;
-            e.warp = warp;
-            e.lane = lane;
-            e.rank = (int)rank;
-            e.cluster_id = cluster_id;
-            e.num_clusters = num_clusters;
-            e.tiles_n = tiles_n;
-            e.num_tiles = num_tiles;
-            if (p.act == GPUSQ_ACT_GELU)
-                e.template run<true, kAmax>();
-            else
-                e.template run<false, kAmax>();
-        } else if (kOut == GPUSQ_OUT_I8) {
-            EpiI8<kTwin> e;
-            e.p = &p;
-            e.ctl = ctl;
-            e.buf0 = ptx::smem_u32(epi_smem + (warp - 2) * 2 * kI8BufBytes);
+            e.buf0 = ptx::smem_u32(epi_smem + (warp - 2) * 2 * kEpiBufBytes);
             e.tmem_base = tmem_base;
             e.tmem_empty0 = tmem_empty0;
             e.tmem_empty1 = tmem_empty1;
@@ -945,16 +681,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             e.cluster_id = cluster_id;
             e.num_clusters = num_clusters;
             if (p.act == GPUSQ_ACT_GELU)
-                e.template run<true>();
+                e.template run<true, kAmax>();
             else
-                e.template run<false>();
+                e.template run<false, kAmax>();
         } else {
-            // raw INT32 accumulators (for bit-exact comparison): plain coalesced stores; the four warps
-            // of a quarter take every fourth 16-token chunk
+            // raw INT32 accumulators (for bit-exact comparison): plain coalesced stores; the warps
+            // of a quarter take every kTurns-th 16-token chunk
+            int local = 0;
             for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); walk.tile < num_tiles; walk.next(p, num_clusters), ++local) {
                 const int tile = walk.tile;
-                int n0, h;
-                int64_t m0;
+                int n0, m0, h;
                 walk.origin(p, (int)rank, n0, m0, h);
                 const int acc = local & 1;
                 const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
@@ -967,14 +703,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 }
                 ptx::tc_fence_after();
                 const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccStride);
-                for (int c = (warp - 2) >> 2; c < h / 16 && n_valid; c += kEpiWarps / 4) {
+                for (int c = (warp - 2) >> 2; c < h / 16 && n_valid; c += kTurns) {
                     if (m0 + c * 16 >= p.M) break;
                     uint32_t r[16];
                     ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(c * 16), r);
                     ptx::tmem_ld_wait_regs(r);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const int64_t m = m0 + c * 16 + j;
+                        const int64_t m = (int64_t)m0 + c * 16 + j;
                         if (m < p.M && n < p.N) reinterpret_cast<int32_t *>(p.Y)[m * p.N + n] = (int32_t)r[j];
                     }
                 }
@@ -1028,20 +764,6 @@ static bool make_map_u8(CUtensorMap *map, const void *base, uint64_t rows, uint6
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Y [M, N] f16 row-major; box = 64 features x 32 tokens, 128-byte swizzle (the staging-tile layout)
-static bool make_map_y_f16(CUtensorMap *map, void *base, uint64_t M, uint64_t N)
-{
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {N, M};
-    cuuint64_t strides[1] = {N * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)kChunkT};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
 }
 
 // testing hooks (gpusq_testing.h): a forced tile height, and a forced number of full-height token tiles
@@ -1194,7 +916,7 @@ static int max_clusters(int sms)
     if (cached[dev] == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(sms & ~1), 1, 1);
-        cfg.blockDim = dim3(Cfg<kSparse, kHalf>::kThreads, 1, 1);
+        cfg.blockDim = dim3(kThreadsGemm, 1, 1);
         cfg.dynamicSmemBytes = Cfg<kSparse, kHalf>::kSmemBytes;
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, kHalf>, &cfg) != cudaSuccess || n <= 0) {
@@ -1259,14 +981,13 @@ static bool prepare_device(int kind)
 }
 
 template <typename Kernel>
-static int launch_on(Kernel kernel, int threads, int smem_bytes, const CUtensorMap &map_a, const CUtensorMap &map_b,
-                     const CUtensorMap &map_b2, const CUtensorMap &map_e, const CUtensorMap &map_y,
-                     const GemmParams &p, int clusters, void *stream)
+static int launch_on(Kernel kernel, int smem_bytes, const CUtensorMap &map_a, const CUtensorMap &map_b,
+                     const CUtensorMap &map_b2, const CUtensorMap &map_e, const GemmParams &p, int clusters, void *stream)
 {
     const int grid = 2 * (p.num_tiles < clusters ? p.num_tiles : clusters);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.blockDim = dim3(kThreadsGemm, 1, 1);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[1];
@@ -1274,7 +995,7 @@ static int launch_on(Kernel kernel, int threads, int smem_bytes, const CUtensorM
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, map_b2, map_e, map_y, p) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, map_b2, map_e, p) != cudaSuccess) {
         (void)cudaGetLastError();
         return GPUSQ_ERR_CUDA;
     }
@@ -1292,7 +1013,7 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
     if (out_type != GPUSQ_OUT_I32 && (!w_scale || !x_scale)) return GPUSQ_ERR_NULL;
     if (out_type == GPUSQ_OUT_I8 && !out_scale) return GPUSQ_ERR_NULL;
     if (M <= 0 || N <= 0 || K <= 0 || K % 16 || M > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
-    // rows of Y are written by bulk tensor stores (FP16) or in 16-byte pieces (INT8)
+    // rows of Y are written in 16-byte pieces
     if ((out_type == GPUSQ_OUT_F16 && N % 8) || (out_type == GPUSQ_OUT_I8 && N % 16)) return GPUSQ_ERR_SHAPE;
     if (!aligned(Xq, 16) || !aligned(Wsrc, 16) || !aligned(Y, 16)) return GPUSQ_ERR_ALIGN;
     if (int st = check_arch()) return st;
@@ -1339,23 +1060,21 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
         ok = ok && make_map_u8(&map_e, meta, (uint64_t)(Np / 128) * (Kp / 128) * 8, 256, 256, 8,
                                CU_TENSOR_MAP_SWIZZLE_NONE);
     }
-    CUtensorMap map_y = map_b;      // placeholder unless the output is FP16
-    if (out_type == GPUSQ_OUT_F16) ok = ok && make_map_y_f16(&map_y, Y, (uint64_t)M, (uint64_t)N);
     if (!ok) return GPUSQ_ERR_CUDA;
 
     // launches without a twin column run the instantiation that has no trace of it
     const int smem = C::kSmemBytes;
     if (out_type == GPUSQ_OUT_F16 && y_absmax && kSparse)
-        return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                        : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
+        return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                        : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
     if (out_type == GPUSQ_OUT_F16)
-        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
+        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
     if (out_type == GPUSQ_OUT_I8)
-        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8, false, true>, C::threads(GPUSQ_OUT_I8), smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8>, C::threads(GPUSQ_OUT_I8), smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
-    return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32, false, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                    : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
+        return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                        : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+    return twin_col ? launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                    : launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I32>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
 }
 
 // The FP16 2:4 sparse layer: binary16 activations as they are, FP32 accumulation, bias, optional GELU.
@@ -1406,16 +1125,14 @@ static int launch_gemm_f16(const void *X, const void *Wpacked, const float *bias
     const uint8_t *meta = reinterpret_cast<const uint8_t *>(Wpacked) + (size_t)Np * Kp;
     ok = ok && make_map_u8(&map_e, meta, (uint64_t)(Np / 128) * (Kp / 128) * 8, 256, 256, 8,
                            CU_TENSOR_MAP_SWIZZLE_NONE);
-    CUtensorMap map_y = map_b;      // placeholder unless the output is FP16
-    if (out_type == GPUSQ_OUT_F16) ok = ok && make_map_y_f16(&map_y, Y, (uint64_t)M, (uint64_t)N);
     if (!ok) return GPUSQ_ERR_CUDA;
 
     const int smem = C::kSmemBytes;
     if (out_type == GPUSQ_OUT_F16)
-        return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                        : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
-    return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_I32, true, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream)
-                    : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_I32, true>, C::kThreads, smem, map_a, map_b, map_b2, map_e, map_y, p, clusters, stream);
+        return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                        : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+    return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_I32, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                    : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_I32, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
 }
 
 }  // namespace gpusq
