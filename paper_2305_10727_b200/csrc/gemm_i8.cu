@@ -54,8 +54,11 @@ constexpr int kTurns = 3;
 constexpr int kEpiWarps = 4 * kTurns;
 constexpr int kThreadsGemm = 32 * (2 + kEpiWarps);
 constexpr int kTmemCols = 512;
-constexpr int kAccStride = 256;     // column offset of the second accumulator
-constexpr int kMetaCol = 224;       // metadata slots: 4 columns per stage from here (below the second accumulator)
+constexpr int kAccStride = kMaxBlockT;      // column of the second accumulator
+constexpr int kMetaCol = 2 * kMaxBlockT;    // metadata: 4 columns per weight block from here
+constexpr int kMaxWeightBlocks = (kTmemCols - kMetaCol) / 4;
+constexpr int kMaxStages = 8;
+constexpr int kMaxSmem = 232448;            // dynamic shared memory that a CTA may have
 constexpr int kEpiBufBytes = kChunkT * 64;            // [16 tokens][32 features] f16 (INT8 output uses half of it)
 constexpr int kEpiBytes = kEpiWarps * 2 * kEpiBufBytes;     // two buffers per epilogue warp
 
@@ -69,24 +72,27 @@ struct Cfg {
     static constexpr int kBAtoms = kHalf ? 2 : 1;                // 128-byte-wide activation tiles per stage
     static constexpr int kBBytes = kBAtoms * (kMaxBlockT / 2) * 128;   // this CTA's half of the token rows
     static constexpr int kMetaBytes = kSparse ? 2048 : 0;
-    static constexpr int kStageBytes = kABytes + kBBytes + kMetaBytes;
-    static constexpr int kStages = kHalf ? 4 : kSparse ? 8 : 6;
     static constexpr int kCtlBytes = 1024;
-    static constexpr int kSmemBytes = kStages * kStageBytes + kEpiBytes + kCtlBytes + 2048 /* alignment slack */;
+    // Shared memory for operands: weight blocks (values and metadata of 128 features x one k block) and
+    // activation stages.  Streaming, every stage has a weight block of its own; resident, all k blocks of a
+    // feature column stay for a run of tiles and the rest of the room holds activation stages.
+    static constexpr int kWBytes = kABytes + kMetaBytes;
+    static constexpr int kRoom = kMaxSmem - kEpiBytes - kCtlBytes - 2048 /* alignment slack */;
+    static constexpr int kStreamStages = kRoom / (kWBytes + kBBytes) < kMaxStages ? kRoom / (kWBytes + kBBytes) : kMaxStages;
+    static constexpr bool kMayStay = kSparse && !kHalf;     // instantiations with resident weights exist
+    static constexpr int kMinResidentStages = 5;
     static constexpr int kMmasPerStage = kHalf ? 4 : kSparse ? 2 : 4;
     static constexpr int kAStepBytes = 32;                    // per MMA along K, all variants
     static constexpr int kBStepBytes = kHalf ? 64 : kSparse ? 64 : 32;
     static constexpr int kASwizzle = kHalf ? 128 : kSparse ? 64 : 128;
     static constexpr int kMetaColsPerMma = kHalf ? 1 : 2;     // 32-bit tensor-memory columns of metadata per MMA
-    static_assert(kStageBytes % 1024 == 0, "stages keep the 1024-byte alignment of the swizzled tiles");
-    static_assert((kStages * kStageBytes) % 2048 == 0, "staging buffers");
-    static_assert(kStages <= 8, "eight metadata slots below the second accumulator");
-    static_assert(kSmemBytes <= 232448, "shared memory per CTA");
+    static_assert(kABytes % 1024 == 0 && kMetaBytes % 1024 == 0 && kBBytes % 1024 == 0, "alignment of the swizzled tiles");
+    static_assert(kStreamStages <= kMaxWeightBlocks, "metadata columns");
 };
 
 struct Ctl {
-    uint64_t full[8];
-    uint64_t empty[8];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
     uint64_t drain;
@@ -106,41 +112,48 @@ struct GemmParams {
     int64_t M;
     int N;
     int K;
-    int block_t;    // tokens per tile, a multiple of 32: the height of the first n_big token tiles
-    int n_big;      // token tiles of full height; the token tiles after them are 32 tokens lower
+    int block_t;    // tokens per tile, a multiple of 32: the height of the tiles of the first n_big token runs
+    int n_big;      // token runs of full height; the tiles of the runs after them are 32 tokens lower
+    int run_tiles;  // token tiles per run (1 unless kRuns)
     int act;
     int out_type;
     int pair_cols;  // feature columns of 256 that are worked on as ordinary pair tiles
-    int pair_tiles; // pair_cols x token tiles: tiles from here on are twin tiles of the last 128 features
-    int num_tiles;
+    int pair_runs;  // pair_cols x token runs: runs from here on are twin tiles of the last 128 features
+    int num_runs;
+    int stages;     // kRuns: activation stages
+    int w_blocks;   // kRuns: weight blocks in shared memory, one per k block
     int twin_n0;    // first feature of the twin column (256 pair_cols)
     int oob_row;    // a row coordinate beyond the weight tensor: loads from there fill with zeros
     uint32_t wait_us;   // limit of every device-side wait, microseconds
     int withhold;       // test hook: the first cluster's producers stop before the last k block of their first tile
 };
 
-// Where a tile sits.  Normally a pair shares `h` tokens and CTA `rank` owns 128 of the pair's 256
-// features.  Token tiles come in two heights so that the number of tiles can be made to fit the
-// number of CTA pairs (the last wave of a persistent launch is otherwise partly empty): the first
-// n_big token tiles are block_t tokens high, the ones after them block_t - 32.
+// Where the work sits.  It is cut into runs: run_tiles consecutive token tiles (fewer at the end) of one
+// feature column, worked on by one CTA pair, with the column's weights loaded once (resident) or by every
+// tile anew (streaming).  Runs are ordered feature column fastest, and pair c takes runs c, c + pairs, ...:
+// the pairs running at one time cover all columns of the same tokens, so the activations come out of L2.
+// Normally a pair shares a tile's `h` tokens and CTA `rank` owns 128 of its 256 features.  Token runs come
+// in two tile heights so that the number of runs can be made to fit the number of CTA pairs (the last wave
+// of a persistent launch is otherwise partly empty): the tiles of the first n_big token runs are block_t
+// tokens high, those of the runs after them block_t - 32.
 // When the last column of features is at most 128 wide (N mod 256 in 1..128: every
 // layer of at most 128 features, and e.g. N = 384) that would leave the second CTA without output,
 // so that column is worked on in "twin" tiles: each CTA owns the column's features of its OWN
 // `block_t` tokens, and the pair's MMA runs over the k blocks twice, first against the token tile of
 // CTA 0 with the weight block in CTA 0's shared memory and zeros in CTA 1's, then against CTA 1's
 // tokens the other way round, so each CTA's accumulator ends up with W times its own tokens.
-// Ordinary tiles come first (feature column fastest), twin tiles after them.
+// Ordinary runs come first, twin tiles (runs of one, always streaming) after them.
 // kTwin = false (no twin column in this launch) compiles the test away.
-template <bool kTwin>
-struct TileWalk {
-    int tile;       // cluster_id, cluster_id + num_clusters, ...
-    int tn, tm;     // feature column and token tile of an ordinary tile, kept incrementally (no division per tile)
+template <bool kTwin, bool kRuns>
+struct RunWalk {
+    int run;        // cluster_id, cluster_id + num_clusters, ...
+    int tn, tm;     // feature column and token run of an ordinary run, kept incrementally (no division per run)
     int step_n, step_m;
 
-    __device__ __forceinline__ TileWalk(const GemmParams &p, int cluster_id, int num_clusters)
+    __device__ __forceinline__ RunWalk(const GemmParams &p, int cluster_id, int num_clusters)
     {
         const int cols = p.pair_cols > 0 ? p.pair_cols : 1;
-        tile = cluster_id;
+        run = cluster_id;
         tn = cluster_id % cols;
         tm = cluster_id / cols;
         step_n = num_clusters % cols;
@@ -148,7 +161,7 @@ struct TileWalk {
     }
     __device__ __forceinline__ void next(const GemmParams &p, int num_clusters)
     {
-        tile += num_clusters;
+        run += num_clusters;
         tn += step_n;
         tm += step_m;
         if (tn >= p.pair_cols) {
@@ -156,22 +169,28 @@ struct TileWalk {
             ++tm;
         }
     }
-    __device__ __forceinline__ bool twin(const GemmParams &p) const { return kTwin && tile >= p.pair_tiles; }
-    // the tile is one of the lower ones (token tiles from n_big on)
+    __device__ __forceinline__ bool twin(const GemmParams &p) const { return kTwin && run >= p.pair_runs; }
+    // the tiles of the run are the lower ones (token runs from n_big on)
     __device__ __forceinline__ bool low(const GemmParams &p) const { return !twin(p) && tm >= p.n_big; }
-    // first feature and first token of CTA `rank`'s part, and the tile's height in tokens
-    __device__ __forceinline__ void origin(const GemmParams &p, int rank, int &n0, int &m0, int &h) const
+    // first feature and first token of CTA `rank`'s part, the tiles' height in tokens and their number
+    __device__ __forceinline__ void origin(const GemmParams &p, int rank, int &n0, int &m0, int &h, int &tiles) const
     {
         if (twin(p)) {
             n0 = p.twin_n0;
-            m0 = ((tile - p.pair_tiles) * 2 + rank) * p.block_t;      // fits: see set_tiling
+            m0 = ((run - p.pair_runs) * 2 + rank) * p.block_t;          // fits: see set_tiling
             h = p.block_t;
+            tiles = 1;
             return;
         }
         n0 = tn * kPairF + rank * kBlockF;
-        const int below = tm - p.n_big;                 // > 0: that many lower tiles precede this one
+        const int below = tm - p.n_big;                 // > 0: that many runs of lower tiles precede this one
         h = below >= 0 ? p.block_t - 32 : p.block_t;
         m0 = tm * p.block_t - (below > 0 ? below * 32 : 0);         // < M
+        tiles = 1;
+        if (kRuns) {
+            m0 *= p.run_tiles;
+            tiles = min(p.run_tiles, ((int)p.M - m0 - 1) / h + 1);
+        }
     }
 };
 
@@ -241,7 +260,7 @@ __device__ __forceinline__ float2 gelu_pair(float2 y)
 // output had it, took for DeiT-Base at batch 64 (M = 12608): 768 -> 2304 19.7 us, 768 -> 3072 with GELU
 // 32.5, 3072 -> 768 21.5; this takes 19.0, 29.6, 20.0, part of it by the eighth pipeline stage for which
 // the staging tiles left no room.  Per-warp bulk stores instead of the plain ones: 19.3, 31.0, 19.8.
-template <bool kAccFloat, bool kI8, bool kTwin>
+template <bool kAccFloat, bool kI8, bool kTwin, bool kRuns>
 struct Epilogue {
     const GemmParams *p;
     Ctl *ctl;
@@ -376,13 +395,14 @@ struct Epilogue {
         const uint32_t full0 = ptx::smem_u32(&ctl->tmem_full[0]);
         const uint32_t lane_taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
 
-        TileWalk<kTwin> walk(*p, cluster_id, num_clusters);
+        RunWalk<kTwin, kRuns> walk(*p, cluster_id, num_clusters);
         int acc = 0, done = 0;                             // accumulator; chunks so far modulo kTurns
         uint32_t acc_phase = 0;
-        while (walk.tile < p->num_tiles) {
-            int n0, m0, h;
-            walk.origin(*p, rank, n0, m0, h);
-            // asked for now, needed after the first chunk has come in; N need not fill the last 128 features
+        bool ok = true;
+        while (ok && walk.run < p->num_runs) {
+            int n0, m0, h, tiles;
+            walk.origin(*p, rank, n0, m0, h, tiles);
+            // scale and bias of the run, needed after its first chunk has come in; N need not fill the last 128 features
             const bool whole = n0 + kBlockF <= N;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -390,53 +410,62 @@ struct Epilogue {
                 sc[j] = in && has_scale ? __ldg(w_scale + n0 + 8 * j) : 1.0f;
                 bi[j] = in && has_bias ? __ldg(bias + n0 + 8 * j) : 0.0f;
             }
-            // tokens of the tile that exist (none: a twin tile's second half); the warps of a quarter take
-            // the chunks in turn, across tiles
-            left = min(M - m0, h);
-            if (kTwin) left = max(left, 0);
-            const int all = (left + kChunkT - 1) / kChunkT;
-            int first = turn - done;
-            if (first < 0) first += kTurns;
-            done = (done + all) % kTurns;
-            int chunks = n0 + quarter * 32 < N ? (all - first + kTurns - 1) / kTurns : 0;    // none past the last feature
-            left -= first * kChunkT;
             const int col = n0 + quarter * 32 + col_l;
-            rows = col < N ? left - row_l : 0;
-            y0 = reinterpret_cast<uint8_t *>(p->Y) + (uint64_t)((uint32_t)m0 + (uint32_t)(first * kChunkT + row_l)) * row_bytes +
-                 (uint32_t)col * (kI8 ? 1u : 2u);
-            y1 = y0 + (uint64_t)(8u * row_bytes);
-            uint32_t taddr = lane_taddr + (uint32_t)(acc * kAccStride + first * kChunkT);
-            bool to;
-            if (!ptx::mbar_wait_bounded(full0 + 8u * acc, acc_phase, &ctl->abort_flag, to)) {
-                if (to && lane == 0) report_timeout(*p, ctl, walk.tile, 2, 100 + acc);
-                break;
-            }
-            ptx::tc_fence_after();
-            if (chunks <= 0) {
-                release(acc);
-            } else {
-                uint32_t v[16];
-                load(taddr, v);
-                if (!kAccFloat) {
+            const bool any = n0 + quarter * 32 < N;        // this warp's features exist
+            const int row_first = col < N ? row_l : 0x40000000;
+            uint8_t *y_tile = reinterpret_cast<uint8_t *>(p->Y) + (uint64_t)((uint32_t)m0 + (uint32_t)row_l) * row_bytes +
+                              (uint32_t)col * (kI8 ? 1u : 2u);
+            int run_left = M - m0;                         // tokens of the tensor from the tile on
+            for (int t = 0; t < tiles; ++t) {
+                // tokens of the tile that exist (none: a twin tile's second half); the warps of a quarter take
+                // the chunks in turn, across tiles
+                left = min(run_left, h);
+                if (kTwin) left = max(left, 0);
+                run_left -= h;
+                const int all = (left + kChunkT - 1) / kChunkT;
+                int first = turn - done;
+                if (first < 0) first += kTurns;
+                done = (done + all) % kTurns;
+                int chunks = any ? (all - first + kTurns - 1) / kTurns : 0;
+                left -= first * kChunkT;
+                rows = left - row_first;
+                y0 = y_tile + (uint64_t)((uint32_t)(first * kChunkT) * row_bytes);
+                y1 = y0 + (uint64_t)(8u * row_bytes);
+                y_tile += (uint64_t)((uint32_t)h * row_bytes);
+                uint32_t taddr = lane_taddr + (uint32_t)(acc * kAccStride + first * kChunkT);
+                bool to;
+                if (!ptx::mbar_wait_bounded(full0 + 8u * acc, acc_phase, &ctl->abort_flag, to)) {
+                    if (to && lane == 0) report_timeout(*p, ctl, walk.run, 2, 100 + acc);
+                    ok = false;
+                    break;
+                }
+                ptx::tc_fence_after();
+                if (t == 0 && !kAccFloat) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) sc[j] = __fmul_rn(sc[j], x_scale);
                 }
-                for (;;) {
-                    uint32_t pk[8];
-                    ptx::tmem_ld_wait_regs(v);
-                    if (--chunks == 0) release(acc);
-                    convert<kGelu, kAmax>(v, pk);
-                    if (chunks) {
-                        taddr += kTurns * kChunkT;
-                        load(taddr, v);
+                if (chunks <= 0) {
+                    release(acc);
+                } else {
+                    uint32_t v[16];
+                    load(taddr, v);
+                    for (;;) {
+                        uint32_t pk[8];
+                        ptx::tmem_ld_wait_regs(v);
+                        if (--chunks == 0) release(acc);
+                        convert<kGelu, kAmax>(v, pk);
+                        if (chunks) {
+                            taddr += kTurns * kChunkT;
+                            load(taddr, v);
+                        }
+                        put(pk);
+                        if (!chunks) break;
                     }
-                    put(pk);
-                    if (!chunks) break;
                 }
+                acc ^= 1;
+                acc_phase ^= acc == 0 ? 1u : 0u;
             }
             walk.next(*p, num_clusters);
-            acc ^= 1;
-            acc_phase ^= acc == 0 ? 1u : 0u;
         }
         if (kAmax) {
             float m = fmaxf(__low2float(amax2), __high2float(amax2));
@@ -451,7 +480,7 @@ struct Epilogue {
 // own register allocation
 // kAmax: the FP16 epilogue also merges max |Y| into a device word (its own instantiation, so that the
 // ordinary kernel's register allocation is untouched)
-template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false>
+template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false, bool kRuns = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsGemm, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_e, const GemmParams p)
@@ -461,8 +490,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // operand tiles need 1024-byte alignment for the 128-byte swizzle, the pairs of staging buffers 2048 (the
     // second is reached by flipping an address bit); both CTAs of a pair get the same offsets
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 2047) & ~uintptr_t(2047));
-    uint8_t *epi_smem = smem + C::kStages * C::kStageBytes;
-    Ctl *ctl = reinterpret_cast<Ctl *>(epi_smem + kEpiBytes);
+    // staging buffers, weight values, weight metadata, activation stages, control block
+    uint8_t *a_smem = smem + kEpiBytes;
+    const int stages = kRuns ? p.stages : C::kStreamStages, w_blocks = kRuns ? p.w_blocks : C::kStreamStages;
+    uint8_t *m_smem = a_smem + w_blocks * C::kABytes;
+    uint8_t *b_smem = m_smem + w_blocks * C::kMetaBytes;
+    Ctl *ctl = reinterpret_cast<Ctl *>(b_smem + stages * C::kBBytes);
     volatile uint32_t *abort_flag = &ctl->abort_flag;
 
     const int warp = threadIdx.x >> 5;
@@ -470,11 +503,11 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t rank = ptx::cluster_ctarank();            // 0 issues the MMAs of the pair
     const int cluster_id = blockIdx.x >> 1;
     const int num_clusters = gridDim.x >> 1;
-    const int num_tiles = p.num_tiles;
+    const int num_runs = p.num_runs;
     const int k_blocks = (p.K + kBlockK - 1) / kBlockK;        // k blocks of the layer; a twin tile takes them twice
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < C::kStages; ++s) {
+        for (int s = 0; s < stages; ++s) {
             ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1);
             ptx::mbar_init(ptx::smem_u32(&ctl->empty[s]), 1);
         }
@@ -488,7 +521,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ptx::fence_barrier_init();
         ptx::prefetch_tensormap(&map_a);
         ptx::prefetch_tensormap(&map_b);
-        if (p.n_big * p.pair_cols < p.pair_tiles) ptx::prefetch_tensormap(&map_b2);
+        if (p.n_big * p.pair_cols < p.pair_runs) ptx::prefetch_tensormap(&map_b2);
         if (kSparse) ptx::prefetch_tensormap(&map_e);
     }
     if (warp == 1) {
@@ -509,46 +542,56 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (ptx::elect_one()) {
-            const uint32_t smem0 = ptx::smem_u32(smem);
+            const uint32_t a0 = ptx::smem_u32(a_smem), e0 = ptx::smem_u32(m_smem), b0 = ptx::smem_u32(b_smem);
             const uint32_t empty0 = ptx::smem_u32(&ctl->empty[0]), full_own = ptx::smem_u32(&ctl->full[0]);
             const uint32_t full0 = ptx::map_to_cta(full_own, 0);    // all bytes of a stage are counted on CTA 0's barrier
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued = 0;            // bit s: a load into stage s was issued
             uint32_t last_parity = 0;       // bit s: parity of the last phase issued into stage s
-            bool ok = true;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles; walk.next(p, num_clusters)) {
+            bool ok = true, first_run = true;
+            for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); ok && walk.run < num_runs; walk.next(p, num_clusters)) {
                 const bool twin = walk.twin(p);
-                int n0, m0, h;
-                walk.origin(p, (int)rank, n0, m0, h);
+                int n0, m0, h, tiles;
+                walk.origin(p, (int)rank, n0, m0, h, tiles);
                 if (!twin) m0 += (int)rank * (h >> 1);                            // this CTA's half of the tile's tokens
                 else m0 += (int)rank * ((h >> 1) - p.block_t);                    // of CTA 0's tile first
                 const CUtensorMap *mb = h == p.block_t ? &map_b : &map_b2;        // box height = half the tile's tokens
                 const uint32_t half_bytes = (uint32_t)((h >> 1) * 128);
-                // bytes both CTAs together bring in per stage
-                const uint32_t stage_tx = 2u * (uint32_t)(C::kABytes + C::kMetaBytes) + 2u * C::kBAtoms * half_bytes;
+                // bytes both CTAs together bring in per stage, without and with a weight block
+                const uint32_t tx_x = 2u * C::kBAtoms * half_bytes, tx_wx = tx_x + 2u * (uint32_t)C::kWBytes;
                 // twin tiles: the first pass of the k blocks runs against the token tile of CTA 0, whose weights
                 // sit in that CTA only (the other one loads zeros from beyond the tensor), the second against CTA 1's
                 int f0 = twin && rank == 1 ? p.oob_row : n0;                      // first weight row loaded
-                int e_row = (n0 / kBlockF) * k_blocks * 8;                        // 2 KB metadata block = 8 rows of 256 bytes
-                const int passes = twin ? 2 : 1;
+                const int e_row = (n0 / kBlockF) * k_blocks * 8;                  // 2 KB metadata block = 8 rows of 256 bytes
+                const int passes = twin ? 2 : tiles;                              // over the k blocks
+                bool weights = true;                                              // this pass brings the weight blocks
                 for (int pass = 0; ok && pass < passes; ++pass) {
                     for (int kb = 0; kb < k_blocks; ++kb) {
-                        if (p.withhold && walk.tile == 0 && pass == passes - 1 && kb == k_blocks - 1) {
+                        if (p.withhold && walk.run == 0 && pass == passes - 1 && kb == k_blocks - 1) {
                             // planted failure (test hook): these loads never come, the MMA issuer's wait runs out
                             ok = false;
                             break;
                         }
                         bool to;
                         if (!ptx::mbar_wait_bounded(empty0 + 8u * stage, phase ^ 1u, abort_flag, to)) {
-                            if (to) report_timeout(p, ctl, walk.tile, 0, stage);
+                            if (to) report_timeout(p, ctl, walk.run, 0, stage);
                             ok = false;
                             break;
                         }
+                        if (kRuns && weights && !first_run && stages > k_blocks) {
+                            // the weight block's previous contents (k block kb of the run before, k_blocks uses of the
+                            // ring ago) have been multiplied; with fewer stages the wait above says so already
+                            const int st = stage >= k_blocks ? stage - k_blocks : stage - k_blocks + stages;
+                            if (!ptx::mbar_wait_bounded(empty0 + 8u * st, stage >= k_blocks ? phase : phase ^ 1u, abort_flag, to)) {
+                                if (to) report_timeout(p, ctl, walk.run, 0, 32 + st);
+                                ok = false;
+                                break;
+                            }
+                        }
                         const uint32_t bar = full0 + 8u * stage;
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(full_own + 8u * stage, stage_tx);
-                        const uint32_t a = smem0 + (uint32_t)(stage * C::kStageBytes), b = a + C::kABytes;
-                        ptx::tma_load_2d_pair(a, &map_a, bar, kb * (kHalf ? 128 : kSparse ? 64 : 128), f0);
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full_own + 8u * stage, weights ? tx_wx : tx_x);
+                        const uint32_t b = b0 + (uint32_t)(stage * C::kBBytes);
                         if (kHalf) {
                             // 128 binary16 columns = two tiles of 128 bytes per token row
                             ptx::tma_load_2d_pair(b, mb, bar, kb * 256, m0);
@@ -556,21 +599,27 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         } else {
                             ptx::tma_load_2d_pair(b, mb, bar, kb * kBlockK, m0);
                         }
-                        if (kSparse) ptx::tma_load_2d_pair(b + C::kBBytes, &map_e, bar, 0, e_row + kb * 8);
+                        if (weights) {
+                            const int blk = kRuns ? kb : stage;
+                            ptx::tma_load_2d_pair(a0 + (uint32_t)(blk * C::kABytes), &map_a, bar, kb * (kHalf ? 128 : kSparse ? 64 : 128), f0);
+                            if (kSparse) ptx::tma_load_2d_pair(e0 + (uint32_t)(blk * C::kMetaBytes), &map_e, bar, 0, e_row + kb * 8);
+                        }
                         issued |= 1u << stage;
                         last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-                        if (++stage == C::kStages) {
+                        if (++stage == stages) {
                             stage = 0;
                             phase ^= 1u;
                         }
                     }
-                    m0 += p.block_t;
-                    f0 = rank == 1 ? n0 : p.oob_row;
+                    m0 += h;
+                    f0 = twin && rank == 0 ? p.oob_row : n0;
+                    weights = !kRuns;
                 }
+                first_run = false;
             }
             if (*abort_flag && rank == 0) {
                 // do not leave while bulk copies may still land in the pair's shared memory
-                for (int s = 0; s < C::kStages; ++s) {
+                for (int s = 0; s < stages; ++s) {
                     if (issued & (1u << s)) {
                         uint32_t none[2] = {0u, p.wait_us};
                         bool to;
@@ -588,66 +637,72 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                              : ptx::make_idesc_i8(kPairF, p.block_t - 32, kSparse);
             const uint32_t full0 = ptx::smem_u32(&ctl->full[0]), empty0 = ptx::smem_u32(&ctl->empty[0]);
             const uint32_t tfull0 = ptx::smem_u32(&ctl->tmem_full[0]), tempty0 = ptx::smem_u32(&ctl->tmem_empty[0]);
-            const uint64_t adesc0 = ptx::make_smem_desc(ptx::smem_u32(smem), C::kASwizzle * 8, C::kASwizzle);
-            const uint64_t bdesc0 = ptx::make_smem_desc(ptx::smem_u32(smem) + C::kABytes, 1024, 128);
-            const uint64_t edesc0 = ptx::make_smem_desc(ptx::smem_u32(smem) + C::kABytes + C::kBBytes, 128, 0);
+            const uint64_t adesc0 = ptx::make_smem_desc(ptx::smem_u32(a_smem), C::kASwizzle * 8, C::kASwizzle);
+            const uint64_t bdesc0 = ptx::make_smem_desc(ptx::smem_u32(b_smem), 1024, 128);
+            const uint64_t edesc0 = ptx::make_smem_desc(ptx::smem_u32(m_smem), 128, 0);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); ok && walk.tile < num_tiles; walk.next(p, num_clusters)) {
-                bool to;
-                if (!ptx::mbar_wait_bounded(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, to)) {
-                    if (to) report_timeout(p, ctl, walk.tile, 1, 100 + acc);
-                    ok = false;
-                    break;
-                }
-                ptx::tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccStride);
+            for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); ok && walk.run < num_runs; walk.next(p, num_clusters)) {
+                int n0_unused, m0_unused, h, tiles;
+                walk.origin(p, 0, n0_unused, m0_unused, h, tiles);
                 const int num_kb = walk.twin(p) ? 2 * k_blocks : k_blocks;
-                // a tile of lower height (the token tiles from n_big on) takes the narrower instruction
-                const bool low = walk.low(p);
-                const uint32_t idesc = low ? idesc_low : idesc_big;
-                const uint32_t half_units = (uint32_t)(((low ? p.block_t - 32 : p.block_t) >> 1) * 128) >> 4;
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!ptx::mbar_wait_bounded(full0 + 8u * stage, phase, abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, walk.tile, 1, stage);
+                // a run of lower tiles takes the narrower instruction
+                const uint32_t idesc = walk.low(p) ? idesc_low : idesc_big;
+                const uint32_t half_units = (uint32_t)((h >> 1) * 128) >> 4;
+                bool weights = true;                                   // this tile's stages bring weight blocks
+                for (; ok && tiles > 0; --tiles) {
+                    bool to;
+                    if (!ptx::mbar_wait_bounded(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, to)) {
+                        if (to) report_timeout(p, ctl, walk.run, 1, 100 + acc);
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
-                    const uint64_t off = (uint64_t)((uint32_t)(stage * C::kStageBytes) >> 4);
-                    const uint32_t meta_t = tmem_base + (uint32_t)(kMetaCol + 4 * stage);
-                    if (kSparse) ptx::tc_cp_128x128b_pair(meta_t, edesc0 + off);
-                    const uint64_t adesc = adesc0 + off, bdesc = bdesc0 + off;
+                    const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccStride);
+                    for (int kb = 0; kb < num_kb; ++kb) {
+                        if (!ptx::mbar_wait_bounded(full0 + 8u * stage, phase, abort_flag, to)) {
+                            if (to) report_timeout(p, ctl, walk.run, 1, stage);
+                            ok = false;
+                            break;
+                        }
+                        ptx::tc_fence_after();
+                        const int blk = kRuns ? kb : stage;
+                        const uint32_t meta_t = tmem_base + (uint32_t)(kMetaCol + 4 * blk);
+                        if (kSparse && weights) ptx::tc_cp_128x128b_pair(meta_t, edesc0 + (uint64_t)((uint32_t)(blk * C::kMetaBytes) >> 4));
+                        const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)(blk * C::kABytes) >> 4);
+                        const uint64_t bdesc = bdesc0 + (uint64_t)((uint32_t)(stage * C::kBBytes) >> 4);
 #pragma unroll
-                    for (int k = 0; k < C::kMmasPerStage; ++k) {
-                        const uint64_t ad = adesc + (uint64_t)((k * C::kAStepBytes) >> 4);
-                        // FP16 model: MMAs 0, 1 read the first activation tile of the stage, 2, 3 the second
-                        const uint64_t bd = kHalf ? bdesc + (uint64_t)(((k & 1) * 64) >> 4) + (uint64_t)((k >> 1) * half_units)
-                                                  : bdesc + (uint64_t)((k * C::kBStepBytes) >> 4);
-                        const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
-                        // 16-bit operands: one metadata column per MMA, addressed as an even column plus
-                        // the selector bit of the instruction descriptor for the odd one
-                        if (kHalf)
-                            ptx::tc_mma_sp_f16_pair(d_tmem, ad, bd, meta_t + (uint32_t)(k & ~1), idesc | (uint32_t)(k & 1),
-                                                    accum);
-                        else if (kSparse)
-                            ptx::tc_mma_sp_i8_pair(d_tmem, ad, bd, meta_t + 2u * k, idesc, accum);
-                        else
-                            ptx::tc_mma_i8_pair(d_tmem, ad, bd, idesc, accum);
+                        for (int k = 0; k < C::kMmasPerStage; ++k) {
+                            const uint64_t ad = adesc + (uint64_t)((k * C::kAStepBytes) >> 4);
+                            // FP16 model: MMAs 0, 1 read the first activation tile of the stage, 2, 3 the second
+                            const uint64_t bd = kHalf ? bdesc + (uint64_t)(((k & 1) * 64) >> 4) + (uint64_t)((k >> 1) * half_units)
+                                                      : bdesc + (uint64_t)((k * C::kBStepBytes) >> 4);
+                            const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
+                            // 16-bit operands: one metadata column per MMA, addressed as an even column plus
+                            // the selector bit of the instruction descriptor for the odd one
+                            if (kHalf)
+                                ptx::tc_mma_sp_f16_pair(d_tmem, ad, bd, meta_t + (uint32_t)(k & ~1), idesc | (uint32_t)(k & 1),
+                                                        accum);
+                            else if (kSparse)
+                                ptx::tc_mma_sp_i8_pair(d_tmem, ad, bd, meta_t + 2u * k, idesc, accum);
+                            else
+                                ptx::tc_mma_i8_pair(d_tmem, ad, bd, idesc, accum);
+                        }
+                        // the stage is reusable in both CTAs once these MMAs are done
+                        ptx::tc_commit_pair(empty0 + 8u * stage, 3);
+                        if (++stage == stages) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
                     }
-                    // the stage is reusable in both CTAs once these MMAs are done
-                    ptx::tc_commit_pair(empty0 + 8u * stage, 3);
-                    if (++stage == C::kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                    if (ok) ptx::tc_commit_pair(tfull0 + 8u * acc, 3);
+                    weights = !kRuns;
+                    acc ^= 1;
+                    acc_phase ^= acc == 0 ? 1u : 0u;
                 }
-                if (ok) ptx::tc_commit_pair(tfull0 + 8u * acc, 3);
-                acc ^= 1;
-                acc_phase ^= acc == 0 ? 1u : 0u;
             }
             if (*abort_flag) {
                 // let every MMA issued so far retire before tensor memory is released
@@ -666,10 +721,10 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t tmem_empty0 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[0]), 0);
         const uint32_t tmem_empty1 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[1]), 0);
         if (kOut == GPUSQ_OUT_F16 || kOut == GPUSQ_OUT_I8) {
-            Epilogue<kHalf, kOut == GPUSQ_OUT_I8, kTwin> e;
+            Epilogue<kHalf, kOut == GPUSQ_OUT_I8, kTwin, kRuns> e;
             e.p = &p;
             e.ctl = ctl;
-            e.buf0 = ptx::smem_u32(epi_smem + (warp - 2) * 2 * kEpiBufBytes);
+            e.buf0 = ptx::smem_u32(smem + (warp - 2) * 2 * kEpiBufBytes);
             e.tmem_base = tmem_base;
             e.tmem_empty0 = tmem_empty0;
             e.tmem_empty1 = tmem_empty1;
@@ -687,36 +742,39 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         } else {
             // raw INT32 accumulators (for bit-exact comparison): plain coalesced stores; the warps
             // of a quarter take every kTurns-th 16-token chunk
-            int local = 0;
-            for (TileWalk<kTwin> walk(p, cluster_id, num_clusters); walk.tile < num_tiles; walk.next(p, num_clusters), ++local) {
-                const int tile = walk.tile;
-                int n0, m0, h;
-                walk.origin(p, (int)rank, n0, m0, h);
-                const int acc = local & 1;
-                const uint32_t acc_phase = (uint32_t)(local >> 1) & 1u;
-                const bool n_valid = n0 < p.N;
+            int acc = 0;
+            uint32_t acc_phase = 0;
+            bool ok = true;
+            for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); ok && walk.run < num_runs; walk.next(p, num_clusters)) {
+                int n0, m0, h, tiles;
+                walk.origin(p, (int)rank, n0, m0, h, tiles);
                 const int n = n0 + quarter * 32 + lane;                // this thread's output feature
-                bool to;
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, to)) {
-                    if (to && lane == 0) report_timeout(p, ctl, tile, 2, 100 + acc);
-                    break;
-                }
-                ptx::tc_fence_after();
-                const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccStride);
-                for (int c = (warp - 2) >> 2; c < h / 16 && n_valid; c += kTurns) {
-                    if (m0 + c * 16 >= p.M) break;
-                    uint32_t r[16];
-                    ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(c * 16), r);
-                    ptx::tmem_ld_wait_regs(r);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int64_t m = (int64_t)m0 + c * 16 + j;
-                        if (m < p.M && n < p.N) reinterpret_cast<int32_t *>(p.Y)[m * p.N + n] = (int32_t)r[j];
+                for (; tiles > 0; --tiles, m0 += h) {
+                    bool to;
+                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, to)) {
+                        if (to && lane == 0) report_timeout(p, ctl, walk.run, 2, 100 + acc);
+                        ok = false;
+                        break;
                     }
+                    ptx::tc_fence_after();
+                    const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kAccStride);
+                    for (int c = (warp - 2) >> 2; c < h / 16 && n0 < p.N; c += kTurns) {
+                        if (m0 + c * 16 >= p.M) break;
+                        uint32_t r[16];
+                        ptx::tmem_ld_32x32b_x16(tbase + (uint32_t)(c * 16), r);
+                        ptx::tmem_ld_wait_regs(r);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const int64_t m = (int64_t)m0 + c * 16 + j;
+                            if (m < p.M && n < p.N) reinterpret_cast<int32_t *>(p.Y)[m * p.N + n] = (int32_t)r[j];
+                        }
+                    }
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive_cluster(acc ? tmem_empty1 : tmem_empty0);
+                    acc ^= 1;
+                    acc_phase ^= acc == 0 ? 1u : 0u;
                 }
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_cluster(acc ? tmem_empty1 : tmem_empty0);
             }
         }
     }
@@ -773,10 +831,10 @@ static std::atomic<unsigned> g_wait_us{ptx::kDefaultWaitUs};
 static std::atomic<int> g_withhold_loads{0};
 static std::atomic<int> g_cluster_cap{0};           // CTA pairs a launch may use (0 = as many as fit)
 
-// How the token axis is cut into tiles: tok_tiles token tiles, the first n_big of them block_t tokens
-// high, the others block_t - 32.
+// How the token axis of a launch is cut: `runs` token runs of run_tiles tiles each, the tiles of the first
+// n_big runs block_t tokens high, those of the others block_t - 32.
 struct TilePlan {
-    int block_t, n_big, tok_tiles;
+    int block_t, n_big, runs, run_tiles;
 };
 
 // Relative time of one tile of h tokens over kb 128-wide k blocks.  Per tile and CTA the shared memory
@@ -785,54 +843,69 @@ struct TilePlan {
 // token: time per tile ~ (kb + 4) * h + 160 * kb.
 static double tile_cost(double kb, int64_t h) { return (kb + 4.0) * (double)h + 160.0 * kb; }
 
-// Time until the last cluster is done when cluster c works on tiles c, c + clusters, ...: the pair
-// tiles (token tile major, pair_cols feature columns each) first, then the twin tiles of a last
-// narrow feature column (two token tiles of block_t each, the k blocks taken twice).
+// The same for a run of `tiles` tiles whose weights stay: a tile is 8 % shorter, and a change of run,
+// where the new weights wait for the last products with the old ones, costs three tenths of a tile.
+// Measured for FP16 output, streaming -> resident (run length), us: 65792 tokens 1280 -> 3840 193 -> 177
+// (6 tiles), 1280 -> 5120 with GELU 276 -> 257 (8); 25216 tokens 1024 -> 3072 53.2 -> 50.0 (10); at 12608
+// tokens and K = 768 equal.
+static double run_cost(double kb, int64_t h, int tiles)
+{
+    return tiles == 1 ? tile_cost(kb, h) : (0.92 * tiles + 0.3) * tile_cost(kb, h);
+}
+
+// Time until the last cluster is done when cluster c works on runs c, c + clusters, ...: the pair runs
+// (token run major, pair_cols feature columns each) first, then the twin tiles of a last narrow feature
+// column (two token tiles of block_t each, the k blocks taken twice).
 static double makespan(const TilePlan &t, int64_t M, int pair_cols, bool twin_col, int clusters, double kb)
 {
-    double load[148] = {};
-    const int C = clusters < 148 ? clusters : 148;
-    int64_t i = 0;
-    for (int tm = 0; tm < t.tok_tiles; ++tm) {
-        const int low = tm - t.n_big;
-        const int64_t h = low >= 0 ? t.block_t - 32 : t.block_t;
-        const int64_t m0 = (int64_t)tm * t.block_t - (low > 0 ? (int64_t)low * 32 : 0);
-        const double c = tile_cost(kb, M - m0 < h ? M - m0 : h);
-        for (int tn = 0; tn < pair_cols; ++tn, ++i) load[i % C] += c;
+    const int h_low = t.block_t - 32;
+    const double big_cost = run_cost(kb, t.block_t, t.run_tiles);
+    const double low_cost = t.n_big < t.runs ? run_cost(kb, h_low, t.run_tiles) : 0.0;
+    // the last token run may have fewer tiles, and its last tile fewer tokens
+    double last_cost = 0.0;
+    if (t.runs > 0) {
+        const bool low = t.n_big < t.runs;
+        const int h = low ? h_low : t.block_t;
+        const int64_t before = ((int64_t)(t.runs - 1) * t.block_t - (low ? (int64_t)(t.runs - 1 - t.n_big) * 32 : 0)) * t.run_tiles;
+        const int64_t left = M - before;
+        last_cost = t.run_tiles == 1 ? tile_cost(kb, left) : (double)left / (double)((int64_t)h * t.run_tiles) * (low ? low_cost : big_cost);
     }
-    if (twin_col) {
-        const int64_t twins = ceil_div(M, 2 * (int64_t)t.block_t);
-        for (int64_t w = 0; w < twins; ++w, ++i) load[i % C] += tile_cost(2.0 * kb, t.block_t);
-    }
+    const int64_t pair_runs = (int64_t)t.runs * pair_cols, big = (int64_t)t.n_big * pair_cols;
+    const int64_t twins = twin_col ? ceil_div(M, 2 * (int64_t)t.block_t) : 0;
+    const double twin_cost = twin_col ? tile_cost(2.0 * kb, t.block_t) : 0.0;
     double worst = 0.0;
-    for (int c = 0; c < C; ++c) worst = load[c] > worst ? load[c] : worst;
+    for (int c = 0; c < clusters; ++c) {
+        // how many of the first n runs are cluster c's
+        auto of = [&](int64_t n) { return n > c ? (n - c - 1) / clusters + 1 : (int64_t)0; };
+        const int64_t mine = of(pair_runs), full = of(pair_runs - pair_cols), full_big = of(big < pair_runs - pair_cols ? big : pair_runs - pair_cols);
+        const double load = (double)full_big * big_cost + (double)(full - full_big) * low_cost +
+                            (double)(mine - full) * last_cost + (double)(of(pair_runs + twins) - mine) * twin_cost;
+        worst = load > worst ? load : worst;
+    }
     return worst;
 }
 
-// Tile heights for a launch.  Uniform tiles leave the last wave of the persistent launch partly
-// empty whenever the tile count is not close to a multiple of the number of clusters (171 tiles on
-// 74 clusters: three waves for 2.3 waves of work); mixing two heights 32 tokens apart gives a tile
-// count that fits.  Searched only while the launch has few waves (beyond that the last wave weighs
-// little and uniform tiles of the best height are taken); the result is remembered per shape.
-static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters, int K)
+// Tile heights and run lengths of a launch.  Uniform tiles leave the last wave of the persistent launch
+// partly empty whenever the number of runs is not close to a multiple of the number of clusters (171
+// tiles on 74 clusters: three waves for 2.3 waves of work); mixing two heights 32 tokens apart gives a
+// count that fits.  Mixed only while the launch has few waves (beyond that the last wave weighs little);
+// the result is remembered per shape.  Runs of several tiles need the weights of a column to fit into
+// shared memory (may_stay).
+static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters, int K, bool may_stay)
 {
     const double kb = (double)ceil_div(K, kBlockK);
+    static const int kRunTiles[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16};
     const int forced = g_block_t_override.load(std::memory_order_relaxed);
     const int forced_big = g_n_big_override.load(std::memory_order_relaxed);
-    if (forced) {
-        TilePlan t = {forced, (int)ceil_div(M, forced), (int)ceil_div(M, forced)};
-        if (forced_big >= 0 && forced >= 64 && pair_cols > 0) {
-            // as many full-height tiles as asked for (at most what covers M), lower ones for the rest
-            const int64_t nb = forced_big < ceil_div(M, forced) ? forced_big : ceil_div(M, forced);
-            const int64_t rest = M - nb * forced;
-            t.n_big = (int)nb;
-            t.tok_tiles = (int)(nb + (rest > 0 ? ceil_div(rest, forced - 32) : 0));
-        }
-        return t;
+    if (forced && forced_big >= 0 && forced >= 64 && pair_cols > 0) {
+        // as many full-height tiles as asked for (at most what covers M), lower ones for the rest
+        const int64_t nb = forced_big < ceil_div(M, forced) ? forced_big : ceil_div(M, forced);
+        const int64_t rest = M - nb * forced;
+        return {forced, (int)nb, (int)(nb + (rest > 0 ? ceil_div(rest, forced - 32) : 0)), 1};
     }
     struct Entry {
         int64_t M;
-        int pair_cols, twin, clusters, K;
+        int pair_cols, twin, clusters, K, may_stay, forced;
         TilePlan plan;
     };
     static std::mutex mu;
@@ -840,12 +913,14 @@ static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters
     static int used = 0, next = 0;
     {
         std::lock_guard<std::mutex> lock(mu);
-        for (int i = 0; i < used; ++i)
-            if (cache[i].M == M && cache[i].pair_cols == pair_cols && cache[i].twin == (int)twin_col &&
-                cache[i].clusters == clusters && cache[i].K == K)
-                return cache[i].plan;
+        for (int i = 0; i < used; ++i) {
+            const Entry &e = cache[i];
+            if (e.M == M && e.pair_cols == pair_cols && e.twin == (int)twin_col && e.clusters == clusters &&
+                e.K == K && e.may_stay == (int)may_stay && e.forced == forced)
+                return e.plan;
+        }
     }
-    TilePlan best = {kMaxBlockT, 0, 0};
+    TilePlan best = {kMaxBlockT, 0, 0, 1};
     double best_cost = 1e300;
     auto consider = [&](const TilePlan &t) {
         const double c = makespan(t, M, pair_cols, twin_col, clusters, kb);
@@ -854,54 +929,76 @@ static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters
             best = t;
         }
     };
-    for (int bt = kMaxBlockT; bt >= 32; bt -= 32) {
-        const int64_t t_min = ceil_div(M, bt);
-        if (t_min > 0x7FFFFFF) continue;
-        consider({bt, (int)t_min, (int)t_min});                            // uniform
-        if (bt < 64 || pair_cols == 0 || t_min * pair_cols > 16 * (int64_t)clusters) continue;
-        const int64_t t_max = ceil_div(M, bt - 32);
-        for (int64_t T = t_min; T < t_max; ++T) {
-            // fewest full-height tiles with which T tiles cover M
-            const int64_t need = M - T * (bt - 32);
-            const int64_t nb = need > 0 ? ceil_div(need, 32) : 0;
-            if (nb > T) continue;
-            consider({bt, (int)nb, (int)T});
+    for (int R : kRunTiles) {
+        if (R > 1 && !may_stay) break;
+        for (int bt = forced ? forced : kMaxBlockT; bt >= (forced ? forced : 32); bt -= 32) {
+            const int64_t t_min = ceil_div(M, (int64_t)bt * R);
+            if (t_min > 0x7FFFFFF) continue;
+            consider({bt, (int)t_min, (int)t_min, R});                         // uniform
+            if (forced || bt < 64 || pair_cols == 0 || t_min * pair_cols > 16 * (int64_t)clusters) continue;
+            const int64_t t_max = ceil_div(M, (int64_t)(bt - 32) * R);
+            for (int64_t T = t_min; T < t_max; ++T) {
+                // fewest full-height runs with which T runs cover M
+                const int64_t need = M - T * (bt - 32) * R;
+                const int64_t nb = need > 0 ? ceil_div(need, 32 * (int64_t)R) : 0;
+                if (nb > T) continue;
+                consider({bt, (int)nb, (int)T, R});
+            }
         }
     }
     std::lock_guard<std::mutex> lock(mu);
-    cache[next] = {M, pair_cols, (int)twin_col, clusters, K, best};
+    cache[next] = {M, pair_cols, (int)twin_col, clusters, K, (int)may_stay, forced, best};
     next = (next + 1) % 64;
     used = used < 64 ? used + 1 : 64;
     return best;
 }
 
-// Fills the tiling fields of the parameters; false when the tile count does not fit 31 bits.
-static bool set_tiling(GemmParams &p, int64_t M, int N, int K_cost, int clusters)
+// Fills the tiling fields of the parameters; false when the number of runs does not fit 31 bits.
+template <typename C>
+static bool set_tiling(GemmParams &p, int K_cost, int clusters)
 {
-    const int tiles_n = (N + kPairF - 1) / kPairF;
-    // a last feature column of at most 128 features is worked on in twin tiles (see TileWalk)
-    const bool twin_col = N - (tiles_n - 1) * kPairF <= kBlockF && M < 0x7FFFFFFF - 4 * kMaxBlockT;
+    const int tiles_n = (p.N + kPairF - 1) / kPairF;
+    // a last feature column of at most 128 features is worked on in twin tiles (see RunWalk)
+    const bool twin_col = p.N - (tiles_n - 1) * kPairF <= kBlockF && p.M < 0x7FFFFFFF - 4 * kMaxBlockT;
     p.pair_cols = twin_col ? tiles_n - 1 : tiles_n;
+    // The weights of a column can stay when they leave room for kMinResidentStages activation stages.  (The
+    // FP16 model's leave three at K = 768, with which it is slower: 27.5 us streaming, 31.7 resident.)  The
+    // raw sums and the dense variant have no such instantiation, and twin tiles stream.
+    const int kb = (p.K + kBlockK - 1) / kBlockK;
+    const int stages = kb <= kMaxWeightBlocks ? (C::kRoom - kb * C::kWBytes) / C::kBBytes : 0;
+    // With fewer than three waves of tiles there is nothing to keep them for.
+    const bool may_stay = C::kMayStay && p.out_type != GPUSQ_OUT_I32 && !twin_col && stages >= C::kMinResidentStages &&
+                          ceil_div(p.M, kMaxBlockT) * p.pair_cols >= 3 * (int64_t)clusters;
     TilePlan t;
     if (p.pair_cols == 0) {
         // twin tiles only: each cluster takes two token tiles and the k blocks twice
-        t = plan_tiles(ceil_div(M, 2), 1, false, clusters, 2 * K_cost);
-        t = {t.block_t, 0, 0};
+        t = plan_tiles(ceil_div(p.M, 2), 1, false, clusters, 2 * K_cost, false);
+        t = {t.block_t, 0, 0, 1};
     } else {
-        t = plan_tiles(M, p.pair_cols, twin_col, clusters, K_cost);
+        t = plan_tiles(p.M, p.pair_cols, twin_col, clusters, K_cost, may_stay);
     }
     p.block_t = t.block_t;
     p.n_big = t.n_big;
-    const int64_t pair_tiles = (int64_t)p.pair_cols * t.tok_tiles;
-    const int64_t tiles = pair_tiles + (twin_col ? ceil_div(M, 2 * (int64_t)t.block_t) : 0);
-    if (tiles > 0x7FFFFFFF) return false;
-    p.pair_tiles = (int)pair_tiles;
-    p.num_tiles = (int)tiles;
+    p.run_tiles = t.run_tiles;
+    p.stages = t.run_tiles > 1 ? (stages < kMaxStages ? stages : kMaxStages) : C::kStreamStages;
+    p.w_blocks = t.run_tiles > 1 ? kb : p.stages;
+    const int64_t pair_runs = (int64_t)p.pair_cols * t.runs;
+    const int64_t runs = pair_runs + (twin_col ? ceil_div(p.M, 2 * (int64_t)t.block_t) : 0);
+    if (runs > 0x7FFFFFFF) return false;
+    p.pair_runs = (int)pair_runs;
+    p.num_runs = (int)runs;
     p.twin_n0 = p.pair_cols * kPairF;
-    p.oob_row = round_up(N, kPairF);  // beyond the packed rows (N rounded up) and the plain ones (N) alike
+    p.oob_row = round_up(p.N, kPairF);  // beyond the packed rows (N rounded up) and the plain ones (N) alike
     p.wait_us = g_wait_us.load(std::memory_order_relaxed);
     p.withhold = g_withhold_loads.load(std::memory_order_relaxed);
     return true;
+}
+
+// dynamic shared memory of a launch
+template <typename C>
+static int smem_bytes(const GemmParams &p)
+{
+    return kEpiBytes + p.w_blocks * C::kWBytes + p.stages * C::kBBytes + C::kCtlBytes + 2048;
 }
 
 // SM pairs that can hold one cluster of this kernel each, per device (0 = unknown yet)
@@ -917,7 +1014,7 @@ static int max_clusters(int sms)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(sms & ~1), 1, 1);
         cfg.blockDim = dim3(kThreadsGemm, 1, 1);
-        cfg.dynamicSmemBytes = Cfg<kSparse, kHalf>::kSmemBytes;
+        cfg.dynamicSmemBytes = kMaxSmem;
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, kHalf>, &cfg) != cudaSuccess || n <= 0) {
             (void)cudaGetLastError();
@@ -953,23 +1050,26 @@ static bool prepare_device(int kind)
     if (done[dev][kind] == 0) {
         bool ok = true;
         if (kind == 0) {
-            const int b = Cfg<true>::kSmemBytes;
+            const int b = kMaxSmem;
             ok = allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16>, b) && allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true>, b) &&
-                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, b);
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, false, false, true>, b);
         } else if (kind == 1) {
-            const int b = Cfg<false>::kSmemBytes;
+            const int b = kMaxSmem;
             ok = allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_F16>, b) && allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I8>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I32>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_F16, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I8, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I32, false, true>, b);
         } else {
-            const int b = Cfg<true, true>::kSmemBytes;
+            const int b = kMaxSmem;
             ok = allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, b) && allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, true, true>, b);
@@ -981,14 +1081,14 @@ static bool prepare_device(int kind)
 }
 
 template <typename Kernel>
-static int launch_on(Kernel kernel, int smem_bytes, const CUtensorMap &map_a, const CUtensorMap &map_b,
+static int launch_on(Kernel kernel, int smem, const CUtensorMap &map_a, const CUtensorMap &map_b,
                      const CUtensorMap &map_b2, const CUtensorMap &map_e, const GemmParams &p, int clusters, void *stream)
 {
-    const int grid = 2 * (p.num_tiles < clusters ? p.num_tiles : clusters);
+    const int grid = 2 * (p.num_runs < clusters ? p.num_runs : clusters);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(kThreadsGemm, 1, 1);
-    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // start while the previous kernel drains
@@ -1036,8 +1136,8 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
     p.K = K;
     p.act = act;
     p.out_type = out_type;
-    if (!set_tiling(p, M, N, K, clusters)) return GPUSQ_ERR_SHAPE;
-    const bool twin_col = p.pair_tiles < p.num_tiles;
+    if (!set_tiling<C>(p, K, clusters)) return GPUSQ_ERR_SHAPE;
+    const bool twin_col = p.pair_runs < p.num_runs;
     const bool mixed = p.block_t >= 64;      // the lower height exists
     const int Kp = round_up(K, 128), Np = round_up(N, kPairF);
 
@@ -1063,7 +1163,15 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
     if (!ok) return GPUSQ_ERR_CUDA;
 
     // launches without a twin column run the instantiation that has no trace of it
-    const int smem = C::kSmemBytes;
+    const int smem = smem_bytes<C>(p);
+    if constexpr (C::kMayStay) {
+        if (p.run_tiles > 1) {
+            if (out_type == GPUSQ_OUT_I8)
+                return launch_on(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+            return y_absmax ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
+                            : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+        }
+    }
     if (out_type == GPUSQ_OUT_F16 && y_absmax && kSparse)
         return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
                         : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
@@ -1107,8 +1215,8 @@ static int launch_gemm_f16(const void *X, const void *Wpacked, const float *bias
     p.K = K;
     p.act = act;
     p.out_type = out_type;
-    if (!set_tiling(p, M, N, 2 * K, clusters)) return GPUSQ_ERR_SHAPE;        // twice the bytes per column
-    const bool twin_col = p.pair_tiles < p.num_tiles;
+    if (!set_tiling<C>(p, 2 * K, clusters)) return GPUSQ_ERR_SHAPE;        // twice the bytes per column
+    const bool twin_col = p.pair_runs < p.num_runs;
     const bool mixed = p.block_t >= 64;
     const int Kp = round_up(K, 128), Np = round_up(N, kPairF);
 
@@ -1127,7 +1235,7 @@ static int launch_gemm_f16(const void *X, const void *Wpacked, const float *bias
                            CU_TENSOR_MAP_SWIZZLE_NONE);
     if (!ok) return GPUSQ_ERR_CUDA;
 
-    const int smem = C::kSmemBytes;
+    const int smem = smem_bytes<C>(p);
     if (out_type == GPUSQ_OUT_F16)
         return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
                         : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
