@@ -558,16 +558,23 @@ patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, floa
 }
 
 // ---- one-launch activation quantisation (scale computed from the tensor) ----
-// A cooperative grid of one 1024-thread CTA per SM.  Each CTA owns a contiguous slice of X:
-//   1. bulk-asynchronous copies bring as much of the slice as fits into shared memory (sixteen-KB
-//      pieces, each completing on its own mbarrier, all in flight at once); what does not fit is
-//      read with plain loads, last, so that it is still in L2 in step 3.  The threads take the
-//      maximum |x| of every piece as it lands;
+// A cooperative grid of one 1024-thread CTA per SM:
+//   1. bulk-asynchronous copies bring what the CTAs' shared memory holds (sixteen-KB pieces, each
+//      completing on its own mbarrier, all in flight at once); the rest of the tensor is read with plain
+//      loads, last chunk first.  The threads take the maximum |x| of every piece as it lands;
 //   2. grid-wide maximum: the CTA merges its maximum into a word of the workspace, counts itself in
 //      and polls, with a bounded wait, until every CTA has been counted;
-//   3. quantises the slice, from shared memory where it was kept, and writes the codes.
-// So X crosses HBM once when a slice fits (up to 192 KB per SM, 28 MB per tensor) and there is one
-// launch instead of two.
+//   3. quantises its chunks in ascending order, then what it kept, and writes the codes.
+// So X crosses HBM once when it fits (192 KB per SM, 29 MB) and there is one launch instead of two.
+// Bound by HBM beyond that; what the caches cannot hold is read twice.  The chunks of all CTAs lie next to
+// each other, so that every CTA is in L2 or in HBM at the same time: step 1 meets first what the producer
+// of X wrote last, step 3 what step 1 read last, and the CTAs finish together (a contiguous slice per CTA
+// left 10% of them waiting).  Taking pieces between the loads, the count of step 2's end behind the
+// barriers of find_single_product instead of in front, and the chunks, back to back on cold tensors, before
+// -> after: 5.3 MB 6.9 -> 6.3 us, 19.4 MB 9.0 -> 8.3, 51.6 MB 23.8 -> 20.9, 77.5 MB 30.8 -> 26.8, 168 MB
+// 66.3 -> 61.4, 674 MB 266 -> 251.  Slower, each measured: 224 KB kept (the loads lose their L1: 168 MB
+// 76.6 us); the whole tensor through a ring of pieces (51.6 MB 29.8: 70 instructions per vector instead of
+// 44); a word per CTA that every CTA polls instead of one counter (+3 us).
 // All or nothing: block 0 sets *x_scale to NaN on entry; the CTA that is last to finish step 2 (a
 // counter, off the critical path) writes the real scale and puts the control words back to zero.  A
 // CTA whose wait expires records GPUSQ_ERR_TIMEOUT in the status word and returns without
@@ -577,6 +584,7 @@ constexpr int kPieceVecs = 1024;                                 // 16-byte vect
 constexpr int kMaxPieces = 12;
 constexpr int kFusedCacheVecs = kPieceVecs * kMaxPieces;         // vectors kept per CTA (192 KB)
 constexpr int kFusedSmemBytes = kFusedCacheVecs * 16;
+constexpr int kStreamLoads = 4;                                  // loads in flight per thread outside the cache
 constexpr int kSingleMinVecs = 2 * kFusedThreads;                // slices below this are not worth the test of quant8_single
 constexpr int kWsDone = kMaxPartials;                            // workspace words: CTAs past the barrier ...
 constexpr int kWsStatus = kMaxPartials + 1;                      // ... status (0 or GPUSQ_ERR_TIMEOUT) ...
@@ -606,46 +614,68 @@ __device__ __forceinline__ bool mbar_try_wait_parity0(uint32_t bar)
     return ok != 0;
 }
 
-// A CTA's slice of n vectors, the first n_kept of them in shared memory.  The others are taken from the
-// end backwards: the maximum pass read them forwards, so the last ones are the ones still in L2.
+__device__ __forceinline__ bool mbar_test_parity0(uint32_t bar)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred P;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 P, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, P;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar)
+        : "memory");
+    return ok != 0;
+}
+
+// How a tensor is shared out.  Vectors [0, kept) are read once: CTA b keeps `per` of them from b per on.
+// The others, chunks x gridDim x chunk_len or a little less, are taken in equal chunks of at most kStreamLoads
+// vectors per thread, all CTAs next to each other: chunk j of CTA b begins at kept + (j gridDim + b) chunk_len.
+struct QuantShare {
+    int64_t vec8, kept;
+    int per, chunks, chunk_len;
+};
+
+// Step 3 of one CTA: the chunks, in order, then the n_kept vectors in shared memory.
 // kSingle: one product per value is known to give the codes (find_single_product).
 template <bool kSingle>
-__device__ __forceinline__ void quantise_slice(const uint4 *cache, const uint4 *__restrict__ Xs, uint2 *__restrict__ Xqs,
-                                               int n_kept, int n, const QuantScale &a, int regroup)
+__device__ __forceinline__ void quantise_share(const uint4 *cache, const uint4 *__restrict__ X, uint2 *__restrict__ Xq,
+                                               const QuantShare &sh, int64_t lo, int n_kept, const QuantScale &a, int regroup)
 {
     auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<false>(v, a) : quant8_f16<false>(v, a), regroup); };
-    int i = n - 1 - (int)threadIdx.x;
-    for (; i - 3 * kFusedThreads >= n_kept; i -= 4 * kFusedThreads) {
-        uint4 v[4];
+    for (int j = 0; j < sh.chunks; ++j) {
+        const int64_t at = sh.kept + ((int64_t)j * gridDim.x + blockIdx.x) * sh.chunk_len;
+        const int left = (int)min((int64_t)sh.chunk_len, sh.vec8 - at) - (int)threadIdx.x;
+        const uint4 *Xc = X + at + threadIdx.x;
+        uint2 *Xqc = Xq + at + threadIdx.x;
+        uint4 v[kStreamLoads];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(Xs + i - u * kFusedThreads);
+        for (int u = 0; u < kStreamLoads; ++u)
+            if (u * kFusedThreads < left) v[u] = __ldg(Xc + u * kFusedThreads);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) __stcs(Xqs + i - u * kFusedThreads, codes(v[u]));
+        for (int u = 0; u < kStreamLoads; ++u)
+            if (u * kFusedThreads < left) __stcs(Xqc + u * kFusedThreads, codes(v[u]));
     }
-    for (; i >= n_kept; i -= kFusedThreads) __stcs(Xqs + i, codes(__ldg(Xs + i)));
+    uint2 *Xqs = Xq + lo;
 #pragma unroll 2
-    for (i = threadIdx.x; i < n_kept; i += kFusedThreads) __stcs(Xqs + i, codes(cache[i]));
+    for (int i = threadIdx.x; i < n_kept; i += kFusedThreads) __stcs(Xqs + i, codes(cache[i]));
 }
 
 __global__ void __launch_bounds__(kFusedThreads, 1)
 act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
-                       uint32_t *ws, int64_t vec8, unsigned long long wait_ns, int withhold, float qmax, int regroup)
+                       uint32_t *ws, const __grid_constant__ QuantShare sh, unsigned long long wait_ns, int withhold, float qmax, int regroup)
 {
     extern __shared__ __align__(128) uint4 cache[];
     __shared__ uint32_t red[kFusedThreads / 32];
     __shared__ __align__(8) uint64_t piece_bar[kMaxPieces];
     __shared__ uint32_t gave_up, grid_max;
-    const int64_t per = (vec8 + gridDim.x - 1) / gridDim.x;
-    const int64_t lo = (int64_t)blockIdx.x * per;
-    const int64_t hi = lo + per < vec8 ? lo + per : vec8;
     const int tid = threadIdx.x;
 
-    // The slice in 32-bit terms: n vectors from Xs; the first n_kept of them stay in shared memory.
-    const int n = hi > lo ? (int)(hi - lo) : 0;             // host side: per < 2^31
-    const int n_kept = n < kFusedCacheVecs ? n : kFusedCacheVecs;
+    const int64_t lo = (int64_t)blockIdx.x * sh.per;
+    const int n_kept = lo < sh.kept ? (int)min(sh.kept - lo, (int64_t)sh.per) : 0;
     const int pieces = (n_kept + kPieceVecs - 1) / kPieceVecs;
     const uint4 *Xs = X + lo;
-    uint2 *Xqs = Xq + lo;
 
     if (tid == 0) {
         for (int c = 0; c < pieces; ++c)
@@ -673,30 +703,34 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
                          : "memory");
         }
     }
-    // what does not fit: maximum only, plain loads that leave the lines in L2 for step 3
+    // What does not fit: maximum only, plain loads that leave the lines in L2 for step 3.  Behind every batch
+    // of them the pieces that have landed by then: thread t looks at vector t of each.
     uint32_t m = 0;
-    int i = n_kept + tid;
-    for (; i + 3 * kFusedThreads < n; i += 4 * kFusedThreads) {
-        uint4 v[4];
+    int c = 0;
+    auto piece = [&] {
+        const int v = c * kPieceVecs + tid;
+        if (v < n_kept) m = max(m, absmax_bits8(cache[v]));
+        ++c;
+    };
+    for (int j = sh.chunks - 1; j >= 0; --j) {
+        const int64_t at = sh.kept + ((int64_t)j * gridDim.x + blockIdx.x) * sh.chunk_len;
+        const int left = (int)min((int64_t)sh.chunk_len, sh.vec8 - at) - tid;
+        const uint4 *Xc = X + at + tid;
+        uint4 v[kStreamLoads];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(Xs + i + u * kFusedThreads);
+        for (int u = 0; u < kStreamLoads; ++u)
+            v[u] = u * kFusedThreads < left ? __ldg(Xc + u * kFusedThreads) : make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < 4 && c < pieces && mbar_test_parity0((uint32_t)__cvta_generic_to_shared(&piece_bar[c])); ++k) piece();
 #pragma unroll
-        for (int u = 0; u < 4; ++u) m = max(m, absmax_bits8(v[u]));
+        for (int u = 0; u < kStreamLoads; ++u) m = max(m, absmax_bits8(v[u]));
     }
-    for (; i < n; i += kFusedThreads) m = max(m, absmax_bits8(__ldg(Xs + i)));
-    // the pieces as they land: thread t looks at vector t of each
     const uint64_t t0 = globaltimer_now();
     bool ok = true;
-    for (int c = 0; c < pieces && ok; ++c) {
+    while (c < pieces) {
         const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&piece_bar[c]);
-        while (!mbar_try_wait_parity0(bar)) {
-            if (globaltimer_now() - t0 > wait_ns) {
-                ok = false;
-                break;
-            }
-        }
-        const int v = c * kPieceVecs + tid;
-        if (ok && v < n_kept) m = max(m, absmax_bits8(cache[v]));
+        while (ok && !mbar_try_wait_parity0(bar)) ok = globaltimer_now() - t0 <= wait_ns;
+        if (!ok) break;
+        piece();
     }
     if (!ok) gave_up = 1;                                    // benign race: every writer writes 1
     m = __reduce_max_sync(0xffffffffu, m);
@@ -744,6 +778,10 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         __syncthreads();
         return;
     }
+    const float s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
+    QuantScale a = make_quant_scale(s, qmax);
+
+    const bool single = n_kept >= kSingleMinVecs && find_single_product<false>(a);
     if (tid == 0) {
         // the last CTA past the barrier: nobody polls any more, so the workspace goes back to zero and
         // the scale, which tells the caller that every CTA came through, is written
@@ -751,17 +789,15 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         if (atomicAdd(ws + kWsDone, 1u) == gridDim.x - 1) {
             __stcg(reinterpret_cast<uint2 *>(bar_word), make_uint2(0u, 0u));
             __stcg(ws + kWsDone, 0u);
-            *x_scale = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
+            *x_scale = s;
         }
     }
-    const float s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
-    QuantScale a = make_quant_scale(s, qmax);
 
-    // 3. quantise the slice: what was kept, from shared memory; the rest, from L2 / HBM
-    if (n >= kSingleMinVecs && find_single_product<false>(a))
-        quantise_slice<true>(cache, Xs, Xqs, n_kept, n, a, regroup);
+    // 3. quantise the share
+    if (single)
+        quantise_share<true>(cache, X, Xq, sh, lo, n_kept, a, regroup);
     else
-        quantise_slice<false>(cache, Xs, Xqs, n_kept, n, a, regroup);
+        quantise_share<false>(cache, X, Xq, sh, lo, n_kept, a, regroup);
 }
 
 // ---- one-launch activation quantisation of small tensors ----
@@ -1053,7 +1089,16 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         // small tensors: no more CTAs than give every thread two vectors (fewer arrivals at the barrier)
         const int64_t want = ceil_div(vec8, 2 * kFusedThreads);
         if ((int64_t)grid > want) grid = (int)(want < 1 ? 1 : want);
-        if (ceil_div(vec8, grid) > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;      // a CTA's slice is indexed with 32 bits
+        QuantShare sh = {};
+        sh.vec8 = vec8;
+        sh.kept = vec8 < (int64_t)grid * kFusedCacheVecs ? vec8 : (int64_t)grid * kFusedCacheVecs;
+        sh.per = (int)ceil_div(sh.kept, grid);
+        if (const int64_t rest = vec8 - sh.kept) {
+            const int64_t chunks = ceil_div(rest, (int64_t)grid * kStreamLoads * kFusedThreads);
+            if (chunks > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
+            sh.chunks = (int)chunks;
+            sh.chunk_len = (int)ceil_div(rest, chunks * grid);
+        }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid, 1, 1);
         cfg.blockDim = dim3(kFusedThreads, 1, 1);
@@ -1069,7 +1114,7 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         const unsigned long long wait_ns = g_grid_wait_ns.load(std::memory_order_relaxed);
         const int withhold = g_withhold_slot.load(std::memory_order_relaxed);
         if (cudaLaunchKernelEx(&cfg, act_quant_fused_kernel, reinterpret_cast<const uint4 *>(X),
-                               reinterpret_cast<uint2 *>(Xq), x_scale, reinterpret_cast<uint32_t *>(workspace), vec8,
+                               reinterpret_cast<uint2 *>(Xq), x_scale, reinterpret_cast<uint32_t *>(workspace), sh,
                                wait_ns, withhold, qmax, regroup) != cudaSuccess) {
             (void)cudaGetLastError();
             return GPUSQ_ERR_CUDA;

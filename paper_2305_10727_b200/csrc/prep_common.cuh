@@ -165,11 +165,10 @@ __device__ __forceinline__ bool find_single_product(QuantScale &a)
         ok1 = ok1 && __fmaf_rn(x, c1, kRoundMagic) == exact;
         return exact;
     };
-    for (int k = threadIdx.x; k < (int)a.qmax; k += blockDim.x) {
-        const int h = __half_as_ushort(__float2half_rn(__fmul_rn((float)k + 0.5f, a.s)));
-#pragma unroll
-        for (int d = -1; d <= 1; ++d)
-            if (h + d >= 0 && h + d < 0x7C00) look(h + d);
+    // one neighbour of one threshold, one division, per thread and step
+    for (int t = threadIdx.x; t < 3 * (int)a.qmax; t += blockDim.x) {
+        const int k = t / 3, h = __half_as_ushort(__float2half_rn(__fmul_rn((float)k + 0.5f, a.s))) + t - 3 * k - 1;
+        if (h >= 0 && h < 0x7C00) look(h);
     }
     if (kClamp) {
         const int b = __half_as_ushort(__float2half_rn(a.x_max));

@@ -118,9 +118,11 @@ def test_quant_weight_row_lengths(B, N, K):
 
 
 # vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2, 4 and 6 vectors per thread, the first size
-# beyond it, and slices that just do and just do not fit the one-launch kernel's shared memory
+# beyond it, tensors that just do and just do not fit the one-launch kernel's shared memory, and what does not
+# fit being one vector, one and two full rounds of chunks, one vector more, and an odd part of the third
 @pytest.mark.parametrize("vecs", [1, 1023, 1024, 1025, 8193, 16384, 16385, 32769, 65537, 98304, 98305, 300001,
-                                  148 * 12288, 148 * 12288 + 4097])
+                                  148 * 12288, 148 * 12288 + 1, 148 * 12288 + 4097, 148 * 16384,
+                                  148 * 16384 + 1, 148 * 20480, 148 * 20480 + 150001])
 def test_quant_act_sizes(B, vecs):
     g = np.random.default_rng(vecs)
     X = g.standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
