@@ -367,35 +367,44 @@ __device__ __forceinline__ uint2 regrouped(uint2 q, int regroup)
     return regroup ? make_uint2(__byte_perm(q.x, q.y, 0x6420), __byte_perm(q.x, q.y, 0x7531)) : q;
 }
 
-// One pass over a tensor whose scale is known, four vectors in flight per thread.
+// One pass over a tensor whose scale is known, four vectors in flight per thread.  Every thread has `rounds`
+// vectors, one less where the last round does not reach; backwards: from the last one on.
 // kSingle: one product per value is known to give the codes (find_single_product).
 template <bool kSingle>
-__device__ __forceinline__ void quantise_strided(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, int64_t vec8,
-                                                 const QuantScale &a, int regroup)
+__device__ __forceinline__ void quantise_strided(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, int64_t vec8, int rounds,
+                                                 bool backwards, const QuantScale &a, int regroup)
 {
     auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<true>(v, a) : quant8_f16<true>(v, a), regroup); };
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 3 * stride < vec8; i += 4 * stride) {
+    int left = i + (rounds - 1) * stride < vec8 ? rounds : rounds - 1;
+    if (backwards) {
+        i += (left - 1) * stride;
+        stride = -stride;
+    }
+    for (; left >= 4; left -= 4, i += 4 * stride) {
         uint4 v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = __ldg(X + i + u * stride);
 #pragma unroll
         for (int u = 0; u < 4; ++u) Xq[i + u * stride] = codes(v[u]);
     }
-    for (; i < vec8; i += stride) Xq[i] = codes(__ldg(X + i));
+    for (; left > 0; --left, i += stride) Xq[i] = codes(__ldg(X + i));
 }
 
 // n_partials > 0: the scale is derived from the partial maxima and written to
 // *x_scale by block 0; absmax != NULL: it is derived from *absmax (the tensor's maximum magnitude,
 // left there by the kernel that produced X) and written; otherwise *x_scale is read.
+// With absmax, X was written just before, front to back, and what was written last is still in L2: it is
+// read backwards (205 MB behind the GEMM that wrote them: 5 us less; a tensor from HBM with a supplied
+// scale in front of its GEMM: up to 0.3 us more, hence forwards).
 // Bound by HBM: back to back on cold tensors 51.6 MB take 14.6 us (17.1 with two loads in flight, two
 // waves of blocks and the bracketing products), 11.8 being what the bytes need; in front of a GEMM
 // 19.4 MB add 7.3 us (8.3), 0.65 MB 1.6 (2.7).
 constexpr int kQuantBlocksPerSm = 4;      // what 64 registers a thread leave room for: one wave
 __global__ void __launch_bounds__(kThreads, kQuantBlocksPerSm)
 act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
-                 const uint32_t *__restrict__ partial, int n_partials, int64_t vec8,
+                 const uint32_t *__restrict__ partial, int n_partials, int64_t vec8, int rounds,
                  const float *__restrict__ absmax, float qmax, int regroup)
 {
     __shared__ float red[kThreads / 32];
@@ -417,17 +426,19 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
     QuantScale a = make_quant_scale(s, qmax);
     // the test of the single product pays from four vectors per thread on
     if (vec8 >= 4 * (int64_t)gridDim.x * blockDim.x && find_single_product<true>(a))
-        quantise_strided<true>(X, Xq, vec8, a, regroup);
+        quantise_strided<true>(X, Xq, vec8, rounds, absmax != nullptr, a, regroup);
     else
-        quantise_strided<false>(X, Xq, vec8, a, regroup);
+        quantise_strided<false>(X, Xq, vec8, rounds, absmax != nullptr, a, regroup);
 }
 
 static int launch_act_quant(const void *X, int8_t *Xq, float *x_scale, const uint32_t *partial, int n_partials, int64_t vec8,
                             const float *absmax, float qmax, int regroup, cudaStream_t stream)
 {
-    return launch_behind(act_quant_kernel, grid_for(vec8, kQuantBlocksPerSm), kThreads, stream,
-                         reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, partial, n_partials,
-                         vec8, absmax, qmax, regroup);
+    const int grid = grid_for(vec8, kQuantBlocksPerSm);
+    const int64_t rounds = ceil_div(vec8, (int64_t)grid * kThreads);
+    if (rounds > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
+    return launch_behind(act_quant_kernel, grid, kThreads, stream, reinterpret_cast<const uint4 *>(X),
+                         reinterpret_cast<uint2 *>(Xq), x_scale, partial, n_partials, vec8, (int)rounds, absmax, qmax, regroup);
 }
 
 // ---- patch embedding (Sec. 3.3): quantise an image batch and lay it out as the GEMM's rows ----

@@ -131,6 +131,11 @@ def test_quant_act_sizes(B, vecs):
     Xq, s = B.quant_act(cu(X))
     assert s.cpu().numpy()[0] == s_o
     assert np.array_equal(Xq.cpu().numpy(), Xq_o)
+    # the one-pass kernels: backwards with the maximum known, forwards with the scale supplied
+    Xq, s = B.quant_act_absmax(cu(X), cu(np.array([np.abs(X).max()], np.float32)))
+    assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq.cpu().numpy(), Xq_o)
+    Xq, _ = B.quant_act(cu(X), x_scale=cu(np.array([s_o], np.float32)), scale_mode=B.SCALE_GIVEN)
+    assert np.array_equal(Xq.cpu().numpy(), Xq_o)
 
 
 @pytest.mark.parametrize("amax", [7.0, 3.75, 5.87890625, 6.1e-5, 65504.0, 4.87, 2.2578125])
