@@ -127,9 +127,9 @@ int gpusq_pack24(const int8_t *vals, const uint8_t *meta, void *Wpacked, int N, 
  *     right after allocation); every call leaves it usable by the next call,
  *     of any size, so one buffer serves a whole stream of calls.  Calls that
  *     can overlap on the GPU need separate workspaces.
- *   GPUSQ_SCALE_COMPUTE runs as one launch: tensors of up to 1.5 MB on one
- *   thread-block cluster, larger ones as a cooperative launch whose CTAs meet at
- *   a grid-wide barrier.  Its waits are bounded (2 s), and the outcome is all or
+ *   GPUSQ_SCALE_COMPUTE runs as one launch: tensors of up to 1 MB on one
+ *   thread-block cluster, larger ones as a grid whose CTAs meet at a grid-wide
+ *   barrier (no CTA waits for one that has not started).  Its waits are bounded (2 s), and the outcome is all or
  *   nothing as far as the scale goes: *x_scale is set to NaN when the kernel
  *   starts and receives the real scale only after EVERY CTA has passed the
  *   barrier.  If a wait ever expires, the int32 at byte offset

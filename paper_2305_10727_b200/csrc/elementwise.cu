@@ -569,37 +569,47 @@ patch_quant_kernel(const __half *__restrict__ img, int8_t *__restrict__ Xq, floa
 }
 
 // ---- one-launch activation quantisation (scale computed from the tensor) ----
-// A cooperative grid of one 1024-thread CTA per SM:
-//   1. bulk-asynchronous copies bring what the CTAs' shared memory holds (sixteen-KB pieces, each
-//      completing on its own mbarrier, all in flight at once); the rest of the tensor is read with plain
-//      loads, last chunk first.  The threads take the maximum |x| of every piece as it lands;
+// A grid of one 1024-thread CTA per SM, each with a share of X:
+//   1. bulk-asynchronous copies bring what is to stay in the CTA's shared memory (sixteen-KB pieces, each
+//      completing on its own mbarrier, all in flight at once); the rest passes through a ring in shared
+//      memory, last vectors first.  The threads take the maximum |x| of everything as it lands;
 //   2. grid-wide maximum: the CTA merges its maximum into a word of the workspace, counts itself in
-//      and polls, with a bounded wait, until every CTA has been counted;
-//   3. quantises its chunks in ascending order, then what it kept, and writes the codes.
-// So X crosses HBM once when it fits (192 KB per SM, 29 MB) and there is one launch instead of two.
-// Bound by HBM beyond that; what the caches cannot hold is read twice.  The chunks of all CTAs lie next to
-// each other, so that every CTA is in L2 or in HBM at the same time: step 1 meets first what the producer
-// of X wrote last, step 3 what step 1 read last, and the CTAs finish together (a contiguous slice per CTA
-// left 10% of them waiting).  Taking pieces between the loads, the count of step 2's end behind the
-// barriers of find_single_product instead of in front, and the chunks, back to back on cold tensors, before
-// -> after: 5.3 MB 6.9 -> 6.3 us, 19.4 MB 9.0 -> 8.3, 51.6 MB 23.8 -> 20.9, 77.5 MB 30.8 -> 26.8, 168 MB
-// 66.3 -> 61.4, 674 MB 266 -> 251.  Slower, each measured: 224 KB kept (the loads lose their L1: 168 MB
-// 76.6 us); the whole tensor through a ring of pieces (51.6 MB 29.8: 70 instructions per vector instead of
-// 44); a word per CTA that every CTA polls instead of one counter (+3 us).
+//      and polls, with a bounded wait, until every share has been counted;
+//   3. quantises the rest of its share in ascending order, then what it kept, and writes the codes.
+// So X crosses HBM once when it fits (160 KB per SM, 24 MB; with the ring 33 MB) and there is one launch
+// instead of two.
+// The launch is an ordinary one, not a cooperative one, which in a stream starts 2.4 us later (2.6 to 19 MB,
+// back to back: 8.3 -> 5.9 us, 10.3 -> 7.9).  In its place CTAs claim their shares when they start, and a
+// CTA that has waited for 20 us claims shares that nobody has and does them too.  So whatever is waited for
+// is in the hands of a CTA that runs, and a CTA that starts late finds its share taken and leaves: no wait
+// depends on a CTA that has no SM.
+// Bound by HBM from some 20 MB on; what the caches cannot hold is read twice.  The vectors of the rest go to
+// all CTAs in turn, so that every CTA is in L2 or in HBM at the same time: step 1 meets first what the
+// producer of X wrote last, step 3 what step 1 read last, and the CTAs finish together (with a contiguous
+// slice per CTA 10% of them waited).  Back to back on cold tensors, against contiguous slices, plain loads
+// four at a time and a cooperative launch: 5.3 MB 8.3 -> 5.6 us, 19.4 MB 10.3 -> 7.9, 51.6 MB 25 -> 19.7,
+// 77.5 MB 31 -> 26.4, 168 MB 66.3 -> 59.0, 674 MB 266 -> 251.  Slower, each measured: plain loads for the rest
+// (a CTA that starts on an SM as a GEMM leaves it finds 28 KB of L1: 168 MB 84 us); the whole tensor through
+// a ring of bulk copies (51.6 MB 29.8: 70 instructions per vector instead of 44); a word per CTA that
+// every CTA polls instead of one counter (+3 us).
 // All or nothing: block 0 sets *x_scale to NaN on entry; the CTA that is last to finish step 2 (a
 // counter, off the critical path) writes the real scale and puts the control words back to zero.  A
 // CTA whose wait expires records GPUSQ_ERR_TIMEOUT in the status word and returns without
 // quantising; the scale then stays NaN and the workspace has to be zero-filled again.
 constexpr int kFusedThreads = 1024;
 constexpr int kPieceVecs = 1024;                                 // 16-byte vectors per bulk copy (16 KB): one per thread
-constexpr int kMaxPieces = 12;
-constexpr int kFusedCacheVecs = kPieceVecs * kMaxPieces;         // vectors kept per CTA (192 KB)
-constexpr int kFusedSmemBytes = kFusedCacheVecs * 16;
-constexpr int kStreamLoads = 4;                                  // loads in flight per thread outside the cache
+constexpr int kMaxPieces = 10;
+constexpr int kFusedCacheVecs = kPieceVecs * kMaxPieces;         // vectors kept per CTA (160 KB)
+constexpr int kRing = 4;                                         // copies in flight per thread for the rest
+constexpr int kFusedSmemBytes = (kFusedCacheVecs + kRing * kFusedThreads) * 16;
 constexpr int kSingleMinVecs = 2 * kFusedThreads;                // slices below this are not worth the test of quant8_single
 constexpr int kWsDone = kMaxPartials;                            // workspace words: CTAs past the barrier ...
 constexpr int kWsStatus = kMaxPartials + 1;                      // ... status (0 or GPUSQ_ERR_TIMEOUT) ...
-constexpr int kWsBarrier = kMaxPartials + 2;                     // ... and the 8-byte word {arrivals, maximum}
+constexpr int kWsBarrier = kMaxPartials + 2;                     // ... the 8-byte word {arrivals, maximum} ...
+constexpr int kWsClaims = kMaxPartials + 4;                      // ... and a bit per share: some CTA has it
+constexpr int kMaxQuantCtas = 512;
+static_assert(kWsClaims + kMaxQuantCtas / 32 <= kMaxPartials + kWorkspaceExtra, "the control words fit");
+constexpr unsigned long long kTakeOverNs = 20000;                // wait before the shares of CTAs that have not started are taken over
 static std::atomic<unsigned long long> g_grid_wait_ns{2000000000ull};    // bound of the waits below (2 s)
 static std::atomic<int> g_withhold_slot{0};                      // test hook: the last CTA does not publish
 
@@ -641,36 +651,139 @@ __device__ __forceinline__ bool mbar_test_parity0(uint32_t bar)
 }
 
 // How a tensor is shared out.  Vectors [0, kept) are read once: CTA b keeps `per` of them from b per on.
-// The others, chunks x gridDim x chunk_len or a little less, are taken in equal chunks of at most kStreamLoads
-// vectors per thread, all CTAs next to each other: chunk j of CTA b begins at kept + (j gridDim + b) chunk_len.
+// The rest goes to all threads in turn, `full` rounds of one vector per thread and one of rest_last vectors.
 struct QuantShare {
-    int64_t vec8, kept;
-    int per, chunks, chunk_len;
+    int64_t kept, rest_last;
+    int per, full;
 };
 
-// Step 3 of one CTA: the chunks, in order, then the n_kept vectors in shared memory.
+// A thread's vectors of the rest pass through its own kRing places in shared memory, which asynchronous
+// copies fill: only this thread reads them, so the copies' own counting is all the synchronisation.
+// Unlike loads they need no L1, of which a CTA that starts beside a GEMM's last ones has 28 KB.
+struct VecRing {
+    uint32_t first, at;         // shared-memory address of place 0 and of the next vector's place
+
+    __device__ __forceinline__ VecRing(const uint4 *places)
+        : first((uint32_t)__cvta_generic_to_shared(places + threadIdx.x)), at(first) {}
+    __device__ __forceinline__ void copy(const uint4 *x) const
+    {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(x) : "memory");
+    }
+    __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+    template <int kPending>
+    __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
+    __device__ __forceinline__ uint4 read() const
+    {
+        uint4 v;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+        return v;
+    }
+    __device__ __forceinline__ void up() { at = at == first + (kRing - 1) * kFusedThreads * 16 ? first : at + kFusedThreads * 16; }
+    __device__ __forceinline__ void down() { at = at == first ? first + (kRing - 1) * kFusedThreads * 16 : at - kFusedThreads * 16; }
+};
+
+// Step 3 of one CTA: the thread's vectors of the rest, in order, the first kRing of which are still in the
+// ring; then the n_kept vectors in shared memory.
 // kSingle: one product per value is known to give the codes (find_single_product).
 template <bool kSingle>
-__device__ __forceinline__ void quantise_share(const uint4 *cache, const uint4 *__restrict__ X, uint2 *__restrict__ Xq,
-                                               const QuantShare &sh, int64_t lo, int n_kept, const QuantScale &a, int regroup)
+__device__ __forceinline__ void quantise_share(const uint4 *cache, VecRing ring, const uint4 *__restrict__ Xr, uint2 *__restrict__ Xqr,
+                                               int64_t step, int rest, uint2 *__restrict__ Xqs, int n_kept, const QuantScale &a,
+                                               int regroup)
 {
     auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<false>(v, a) : quant8_f16<false>(v, a), regroup); };
-    for (int j = 0; j < sh.chunks; ++j) {
-        const int64_t at = sh.kept + ((int64_t)j * gridDim.x + blockIdx.x) * sh.chunk_len;
-        const int left = (int)min((int64_t)sh.chunk_len, sh.vec8 - at) - (int)threadIdx.x;
-        const uint4 *Xc = X + at + threadIdx.x;
-        uint2 *Xqc = Xq + at + threadIdx.x;
-        uint4 v[kStreamLoads];
-#pragma unroll
-        for (int u = 0; u < kStreamLoads; ++u)
-            if (u * kFusedThreads < left) v[u] = __ldg(Xc + u * kFusedThreads);
-#pragma unroll
-        for (int u = 0; u < kStreamLoads; ++u)
-            if (u * kFusedThreads < left) __stcs(Xqc + u * kFusedThreads, codes(v[u]));
+    Xr += kRing * step;
+    for (int r = 0; r < rest; ++r) {
+        VecRing::wait<kRing - 1>();
+        const uint2 c = codes(ring.read());
+        if (r + kRing < rest) ring.copy(Xr);
+        VecRing::commit();
+        __stcs(Xqr, c);
+        ring.down();
+        Xr += step;
+        Xqr += step;
     }
-    uint2 *Xqs = Xq + lo;
 #pragma unroll 2
     for (int i = threadIdx.x; i < n_kept; i += kFusedThreads) __stcs(Xqs + i, codes(cache[i]));
+}
+
+// Share v, vector by vector, for a CTA that takes it over: its maximum and its codes.  Inlined: as calls, never
+// made in the usual case, they cost 0.5 us through the stack frame.
+template <typename F>
+__device__ __forceinline__ void for_share(const QuantShare &sh, int v, F f)
+{
+    const int64_t lo = (int64_t)v * sh.per, hi = min(lo + sh.per, sh.kept);
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kFusedThreads) f(i);
+    const int64_t r0 = (int64_t)v * kFusedThreads + threadIdx.x, step = (int64_t)gridDim.x * kFusedThreads;
+    const int rest = sh.full + (r0 < sh.rest_last ? 1 : 0);
+    for (int r = 0; r < rest; ++r) f(sh.kept + r0 + r * step);
+}
+
+__device__ __forceinline__ uint32_t share_max(const uint4 *X, const QuantShare &sh, int v)
+{
+    uint32_t m = 0;
+    for_share(sh, v, [&](int64_t i) { m = max(m, absmax_bits8(__ldg(X + i))); });
+    return m;
+}
+
+__device__ __forceinline__ void share_codes(const uint4 *X, uint2 *Xq, const QuantShare &sh, int v, const QuantScale &a, int regroup)
+{
+    for_share(sh, v, [&](int64_t i) { Xq[i] = regrouped(quant8_f16<false>(__ldg(X + i), a), regroup); });
+}
+
+// One thread counts its CTA as past the barrier; the result, for count_out(), takes a while to come.  The last
+// one (nobody polls any more) puts the workspace back to zero and writes the scale, which tells the caller
+// that every share is done.
+__device__ __forceinline__ uint32_t count_past(uint32_t *ws)
+{
+    __threadfence();
+    return atomicAdd(ws + kWsDone, 1u);
+}
+
+__device__ __forceinline__ void count_out(uint32_t *ws, uint32_t before, float *x_scale, uint32_t all, float qmax)
+{
+    if (before != gridDim.x - 1) return;
+    __stcg(reinterpret_cast<uint2 *>(ws + kWsBarrier), make_uint2(0u, 0u));
+    for (int w = 0; w < kMaxQuantCtas / 32; w += 4) __stcg(reinterpret_cast<uint4 *>(ws + kWsClaims + w), make_uint4(0u, 0u, 0u, 0u));
+    __stcg(ws + kWsDone, 0u);
+    *x_scale = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
+}
+
+// What a CTA does after its wait: everybody has arrived, its wait ran out, somebody else has its share, or
+// kTakeOver + v: it has claimed share v.
+enum : uint32_t { kAllArrived, kGaveUp, kTooLate, kTakeOver };
+
+// One thread: counts the share just looked at in, with its maximum, and waits for the others.  Everything
+// waited for is in the hands of a CTA that runs: shares that nobody has claimed after kTakeOverNs, because
+// their CTAs have no SM yet, are claimed here, one per call.
+__device__ __forceinline__ uint32_t arrive_and_wait(uint32_t *ws, uint32_t mine, bool publish, uint64_t t0, uint64_t wait_ns,
+                                                    uint32_t *taken, uint32_t &all)
+{
+    uint32_t *bar_word = ws + kWsBarrier;
+    if (publish) {
+        atomicMax(bar_word + 1, mine);
+        __threadfence();
+        atomicAdd(bar_word, 1u);
+    }
+    for (uint32_t it = 1;; ++it) {
+        const uint2 word = __ldcv(reinterpret_cast<const uint2 *>(bar_word));
+        if (word.x >= gridDim.x) {
+            all = word.y;
+            return kAllArrived;
+        }
+        if ((it & 15u) != 0u) continue;
+        const uint64_t now = globaltimer_now();
+        if (now - t0 > wait_ns) return kGaveUp;
+        if (now - t0 < kTakeOverNs) continue;
+        for (uint32_t v = 0; v < gridDim.x; v += 32) {
+            const uint32_t shares = gridDim.x - v >= 32 ? 0xffffffffu : (1u << (gridDim.x - v)) - 1u;
+            const uint32_t open = ~__ldcv(ws + kWsClaims + v / 32) & shares;
+            if (open == 0u) continue;
+            const uint32_t bit = open & (0u - open);
+            if (atomicOr(ws + kWsClaims + v / 32, bit) & bit) continue;
+            taken[v / 32] |= bit;
+            return kTakeOver + v + (uint32_t)__ffs((int)bit) - 1u;
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kFusedThreads, 1)
@@ -680,13 +793,17 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
     extern __shared__ __align__(128) uint4 cache[];
     __shared__ uint32_t red[kFusedThreads / 32];
     __shared__ __align__(8) uint64_t piece_bar[kMaxPieces];
-    __shared__ uint32_t gave_up, grid_max;
+    __shared__ uint32_t gave_up, grid_max, next, taken[kMaxQuantCtas / 32];
     const int tid = threadIdx.x;
 
     const int64_t lo = (int64_t)blockIdx.x * sh.per;
     const int n_kept = lo < sh.kept ? (int)min(sh.kept - lo, (int64_t)sh.per) : 0;
     const int pieces = (n_kept + kPieceVecs - 1) / kPieceVecs;
     const uint4 *Xs = X + lo;
+    const int64_t step = (int64_t)gridDim.x * kFusedThreads, r0 = (int64_t)blockIdx.x * kFusedThreads + tid;
+    const int rest = sh.full + (r0 < sh.rest_last ? 1 : 0);
+    const uint4 *Xr = X + sh.kept + r0;
+    VecRing ring(cache + kFusedCacheVecs);
 
     if (tid == 0) {
         for (int c = 0; c < pieces; ++c)
@@ -694,6 +811,7 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         gave_up = 0;
     }
+    if (tid < kMaxQuantCtas / 32) taken[tid] = 0;
     __syncthreads();
     // the previous kernel of the stream (a producer of X, or a user of the workspace) is complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -702,6 +820,7 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
     if (blockIdx.x == 0 && tid == 0) *x_scale = __int_as_float(0x7FC00000);
 
     // 1. the slice into shared memory, all pieces in flight at once
+    uint32_t claimed = 0;                                    // thread 0: not 0 if another CTA has this one's share
     if (tid == 0) {
         for (int c = 0; c < pieces; ++c) {
             const int v0 = c * kPieceVecs;
@@ -713,9 +832,10 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
                          "l"(Xs + v0), "r"(bytes), "r"(bar)
                          : "memory");
         }
+        claimed = atomicOr(ws + kWsClaims + blockIdx.x / 32, 1u << (blockIdx.x & 31));
     }
-    // What does not fit: maximum only, plain loads that leave the lines in L2 for step 3.  Behind every batch
-    // of them the pieces that have landed by then: thread t looks at vector t of each.
+    // What does not fit: maximum only, from the last vector to the first.  In between the pieces that have
+    // landed by then: thread t looks at vector t of each.
     uint32_t m = 0;
     int c = 0;
     auto piece = [&] {
@@ -723,17 +843,24 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         if (v < n_kept) m = max(m, absmax_bits8(cache[v]));
         ++c;
     };
-    for (int j = sh.chunks - 1; j >= 0; --j) {
-        const int64_t at = sh.kept + ((int64_t)j * gridDim.x + blockIdx.x) * sh.chunk_len;
-        const int left = (int)min((int64_t)sh.chunk_len, sh.vec8 - at) - tid;
-        const uint4 *Xc = X + at + tid;
-        uint4 v[kStreamLoads];
-#pragma unroll
-        for (int u = 0; u < kStreamLoads; ++u)
-            v[u] = u * kFusedThreads < left ? __ldg(Xc + u * kFusedThreads) : make_uint4(0u, 0u, 0u, 0u);
-        for (int k = 0; k < 4 && c < pieces && mbar_test_parity0((uint32_t)__cvta_generic_to_shared(&piece_bar[c])); ++k) piece();
-#pragma unroll
-        for (int u = 0; u < kStreamLoads; ++u) m = max(m, absmax_bits8(v[u]));
+    if (rest > 0) {
+        const uint4 *Xd = Xr + (int64_t)(rest - 1) * step;
+        for (int k = 0; k < kRing; ++k) {
+            if (k < rest) ring.copy(Xd);
+            VecRing::commit();
+            ring.up();
+            Xd -= step;
+        }
+        for (int r = rest - 1; r >= 0; --r) {
+            VecRing::wait<kRing - 1>();
+            m = max(m, absmax_bits8(ring.read()));
+            if (r >= kRing) ring.copy(Xd);
+            VecRing::commit();
+            ring.up();
+            Xd -= step;
+            if (c < pieces && mbar_test_parity0((uint32_t)__cvta_generic_to_shared(&piece_bar[c]))) piece();
+        }
+        ring.down();                                         // place of vector 0, the last one read
     }
     const uint64_t t0 = globaltimer_now();
     bool ok = true;
@@ -744,38 +871,38 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         piece();
     }
     if (!ok) gave_up = 1;                                    // benign race: every writer writes 1
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((tid & 31) == 0) red[tid >> 5] = m;
-    __syncthreads();
-
     // 2. grid-wide maximum.  One 8-byte word holds {arrivals, maximum}: a CTA first merges its maximum,
     // then counts itself in, so a single 8-byte read that sees every arrival also sees the final
     // maximum; each CTA has one poll in flight at a time, all on one line.
-    uint32_t *bar_word = ws + kWsBarrier;
-    if (tid < 32 && !gave_up) {
-        const uint32_t mine = __reduce_max_sync(0xffffffffu, red[tid]);
-        if (tid == 0) {
-            if (!(withhold && blockIdx.x == gridDim.x - 1)) {
-                atomicMax(bar_word + 1, mine);
-                __threadfence();
-                atomicAdd(bar_word, 1u);
-            }
-            for (uint32_t it = 1;; ++it) {
-                const uint2 word = __ldcv(reinterpret_cast<const uint2 *>(bar_word));
-                if (word.x >= gridDim.x) {
-                    grid_max = word.y;
-                    break;
-                }
-                if ((it & 63u) == 0u && globaltimer_now() - t0 > wait_ns) {
-                    gave_up = 1;
-                    break;
-                }
+    bool any = false;
+    for (bool own = true;; own = false) {
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((tid & 31) == 0) red[tid >> 5] = m;
+        __syncthreads();
+        if (tid < 32) {
+            const uint32_t mine = __reduce_max_sync(0xffffffffu, red[tid]);
+            if (tid == 0) {
+                const bool publish = !(withhold && own && blockIdx.x == gridDim.x - 1);
+                uint32_t all = 0;
+                next = gave_up ? kGaveUp : own && (claimed >> (blockIdx.x & 31) & 1u) ? kTooLate : arrive_and_wait(ws, mine, publish, t0, wait_ns, taken, all);
+                grid_max = all;
             }
         }
+        __syncthreads();
+        if (next < kTakeOver) break;
+        any = true;
+        m = share_max(X, sh, (int)(next - kTakeOver));
     }
-    __syncthreads();
     const uint32_t all = grid_max;
-    if (gave_up) {
+    if (next != kAllArrived) VecRing::wait<0>();
+    if (next == kTooLate) {
+        if (tid == 0) {
+            const uint32_t word = __ldcv(ws + kWsBarrier + 1);              // final if this CTA is the last one
+            count_out(ws, count_past(ws), x_scale, word, qmax);
+        }
+        return;
+    }
+    if (next == kGaveUp) {
         if (tid == 0) atomicExch(ws + kWsStatus, (uint32_t)GPUSQ_ERR_TIMEOUT);
         // bulk copies that may still be in flight write into this CTA's shared memory: wait for them (bounded)
         if (tid == 0) {
@@ -793,35 +920,32 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
     QuantScale a = make_quant_scale(s, qmax);
 
     const bool single = n_kept >= kSingleMinVecs && find_single_product<false>(a);
-    if (tid == 0) {
-        // the last CTA past the barrier: nobody polls any more, so the workspace goes back to zero and
-        // the scale, which tells the caller that every CTA came through, is written
-        __threadfence();
-        if (atomicAdd(ws + kWsDone, 1u) == gridDim.x - 1) {
-            __stcg(reinterpret_cast<uint2 *>(bar_word), make_uint2(0u, 0u));
-            __stcg(ws + kWsDone, 0u);
-            *x_scale = s;
-        }
-    }
+    uint32_t before = 0;
+    if (tid == 0) before = count_past(ws);
 
     // 3. quantise the share
+    uint2 *Xqr = Xq + sh.kept + r0;
     if (single)
-        quantise_share<true>(cache, X, Xq, sh, lo, n_kept, a, regroup);
+        quantise_share<true>(cache, ring, Xr, Xqr, step, rest, Xq + lo, n_kept, a, regroup);
     else
-        quantise_share<false>(cache, X, Xq, sh, lo, n_kept, a, regroup);
+        quantise_share<false>(cache, ring, Xr, Xqr, step, rest, Xq + lo, n_kept, a, regroup);
+    if (tid == 0) count_out(ws, before, x_scale, all, qmax);
+    if (any) for (int v = 0; v < (int)gridDim.x; v += 32)             // shares taken over
+        for (uint32_t bits = taken[v / 32]; bits; bits &= bits - 1)
+            share_codes(X, Xq, sh, v + __ffs((int)bits) - 1, a, regroup);
 }
 
 // ---- one-launch activation quantisation of small tensors ----
 // One cluster of up to sixteen CTAs keeps the tensor in registers and exchanges its warps' maxima
 // through distributed shared memory: every warp writes its maximum into each CTA, one cluster barrier,
 // and every warp reduces them all.  Bound by latencies (launch, one load, the barrier, one store), of
-// which the grid-wide barrier through L2 of the kernel above is the longest.  Microseconds that a call
-// adds in front of a GEMM (kernel above -> this one): 9 KB 3.6 -> 1.6, 0.65 MB 5.4 -> 3.4, 1.5 MB
-// 6.0 -> 4.7; at 2.4 MB sixteen SMs are too few to load and store it (8.1 against 5.1): hence the limit
-// of six vectors per thread.
+// which the grid-wide barrier through L2 of the kernel above is the longest.  Back to back, kernel above ->
+// this one: 0.3 MB 5.0 -> 3.6 us, 0.65 MB 5.0 -> 4.1, 0.9 MB 4.9 -> 4.5; at 1.2 MB both take 4.9 and at
+// 1.5 MB sixteen SMs are too few to load and store it (5.0 against 5.3): hence the limit of four vectors
+// per thread, 1 MB.
 constexpr int kClusterThreads = 1024;
 constexpr int kMaxCluster = 16;
-constexpr int kClusterMaxPerThread = 6;
+constexpr int kClusterMaxPerThread = 4;
 
 template <int kPer>
 __global__ void __launch_bounds__(kClusterThreads, 1)
@@ -1050,7 +1174,7 @@ static int launch_cluster_quant(const void *X, int8_t *Xq, float *x_scale, int v
     cfg.attrs = at;
     cfg.numAttrs = 2;
     auto kernel = per <= 1 ? act_quant_cluster_kernel<1> : per <= 2 ? act_quant_cluster_kernel<2>
-                : per <= 4 ? act_quant_cluster_kernel<4> : act_quant_cluster_kernel<kClusterMaxPerThread>;
+                : act_quant_cluster_kernel<kClusterMaxPerThread>;
     if (cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, vec8,
                            qmax, regroup) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -1079,7 +1203,7 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         const int cluster_max = max_quant_cluster();
         if (cluster_max > 0 && vec8 <= (int64_t)cluster_max * kClusterThreads * kClusterMaxPerThread)
             return launch_cluster_quant(X, Xq, x_scale, (int)vec8, cluster_max, qmax, regroup, s);
-        // one cooperative launch: every CTA must be resident for the grid-wide barrier.  The opt-in to
+        // The opt-in to
         // large dynamic shared memory is per device.
         static std::mutex mu;
         static uint8_t attr_state[kMaxDevices] = {};          // 1 = set, 2 = failed
@@ -1096,32 +1220,27 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
             if (attr_state[dev] != 1) return GPUSQ_ERR_CUDA;
         }
         int grid = num_sms();
-        if (grid > kMaxPartials) grid = kMaxPartials;
+        if (grid > kMaxQuantCtas) grid = kMaxQuantCtas;
         // small tensors: no more CTAs than give every thread two vectors (fewer arrivals at the barrier)
         const int64_t want = ceil_div(vec8, 2 * kFusedThreads);
         if ((int64_t)grid > want) grid = (int)(want < 1 ? 1 : want);
         QuantShare sh = {};
-        sh.vec8 = vec8;
         sh.kept = vec8 < (int64_t)grid * kFusedCacheVecs ? vec8 : (int64_t)grid * kFusedCacheVecs;
         sh.per = (int)ceil_div(sh.kept, grid);
-        if (const int64_t rest = vec8 - sh.kept) {
-            const int64_t chunks = ceil_div(rest, (int64_t)grid * kStreamLoads * kFusedThreads);
-            if (chunks > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
-            sh.chunks = (int)chunks;
-            sh.chunk_len = (int)ceil_div(rest, chunks * grid);
-        }
+        const int64_t round = (int64_t)grid * kFusedThreads, rest = vec8 - sh.kept;
+        if (rest / round > 0x7FFFFFF0) return GPUSQ_ERR_SHAPE;
+        sh.full = (int)(rest / round);
+        sh.rest_last = rest % round;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)grid, 1, 1);
         cfg.blockDim = dim3(kFusedThreads, 1, 1);
         cfg.dynamicSmemBytes = kFusedSmemBytes;
         cfg.stream = s;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // set up while the previous kernel drains
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // set up while the previous kernel drains
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 2;
+        cfg.numAttrs = 1;
         const unsigned long long wait_ns = g_grid_wait_ns.load(std::memory_order_relaxed);
         const int withhold = g_withhold_slot.load(std::memory_order_relaxed);
         if (cudaLaunchKernelEx(&cfg, act_quant_fused_kernel, reinterpret_cast<const uint4 *>(X),

@@ -117,12 +117,12 @@ def test_quant_weight_row_lengths(B, N, K):
     assert np.array_equal(ws.cpu().numpy(), ws_o) and np.array_equal(Wq.cpu().numpy(), Wq_o)
 
 
-# vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2, 4 and 6 vectors per thread, the first size
-# beyond it, tensors that just do and just do not fit the one-launch kernel's shared memory, and what does not
-# fit being one vector, one and two full rounds of chunks, one vector more, and an odd part of the third
+# vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2 and 4 vectors per thread, the first size beyond
+# it, tensors that just do and just do not fit the one-launch kernel's shared memory, and the rest being one
+# vector, one round, as many as the ring has places, one vector more, and an odd part of a later round
 @pytest.mark.parametrize("vecs", [1, 1023, 1024, 1025, 8193, 16384, 16385, 32769, 65537, 98304, 98305, 300001,
-                                  148 * 12288, 148 * 12288 + 1, 148 * 12288 + 4097, 148 * 16384,
-                                  148 * 16384 + 1, 148 * 20480, 148 * 20480 + 150001])
+                                  148 * 10240, 148 * 10240 + 1, 148 * 11264, 148 * 14336, 148 * 14336 + 1,
+                                  148 * 20480 + 75001])
 def test_quant_act_sizes(B, vecs):
     g = np.random.default_rng(vecs)
     X = g.standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
@@ -136,6 +136,29 @@ def test_quant_act_sizes(B, vecs):
     assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq.cpu().numpy(), Xq_o)
     Xq, _ = B.quant_act(cu(X), x_scale=cu(np.array([s_o], np.float32)), scale_mode=B.SCALE_GIVEN)
     assert np.array_equal(Xq.cpu().numpy(), Xq_o)
+
+
+def test_quant_act_beside_other_kernels(B):
+    # CTAs that find no SM at first: a matrix product of many waves in another stream, and two calls at a time.
+    # Shares are then taken over by CTAs that run; scale and codes have to be the same.
+    Xs = [np.random.default_rng(i).standard_normal((rows, 1024), dtype=np.float32).astype(np.float16) for i, rows in ((0, 4001), (1, 16003))]
+    want = [oracle.quant_act(X) for X in Xs]
+    Xd = [cu(X) for X in Xs]
+    ws = [torch.zeros((B.quant_act_workspace(*X.shape),), dtype=torch.uint8, device="cuda") for X in Xs]
+    big = torch.ones((8192, 8192), dtype=torch.float16, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    torch.cuda.synchronize()
+    got = []
+    for _ in range(6):
+        with torch.cuda.stream(streams[2]):
+            torch.mm(big, big)
+        for X, w, s in zip(Xd, ws, streams):
+            with torch.cuda.stream(s):
+                got.append(B.quant_act(X, workspace=w))
+    torch.cuda.synchronize()
+    for k, (Xq, s) in enumerate(got):
+        assert s.cpu().numpy()[0] == want[k % 2][1] and np.array_equal(Xq.cpu().numpy(), want[k % 2][0])
+    assert [B.quant_act_status(w) for w in ws] == [0, 0] and not any(w.any() for w in ws)
 
 
 @pytest.mark.parametrize("amax", [7.0, 3.75, 5.87890625, 6.1e-5, 65504.0, 4.87, 2.2578125])
