@@ -48,7 +48,7 @@ def build_binding(force: bool = False) -> str:
            "-I" + os.path.join(t, "include", "torch", "csrc", "api", "include"),
            "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(cuda, "include"),
            "-o", tmp, os.path.join(CSRC, "torch_binding.cpp"), "-L" + HERE, "-l:libgpusq.so",
-           "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+           "-L" + os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
     subprocess.run(cmd, check=True)
     os.replace(tmp, BINDING)
     return BINDING
