@@ -413,6 +413,41 @@ def test_int8_output_writes_its_rows_and_nothing_else(B, M, N):
     assert (buf[:2048] == 77).all() and (buf[2048 + M * N:] == 77).all()
 
 
+# Weights that stay in shared memory for a run of token tiles: few CTA pairs, so that each has runs of several tiles,
+# the last ones shorter.  K from one k block (fewer than the pipeline's stages) to thirteen, the most that leaves
+# room (more than the stages), a last k block that is not whole; one and two columns, the second one of 144 features.
+@pytest.mark.parametrize("M,N,K,clusters", [(2033, 256, 64, 3), (1345, 240, 640, 1), (1360, 400, 1040, 2), (2017, 256, 1280, 3),
+                                            (1409, 256, 1664, 2), (1409, 256, 1680, 2)])
+@pytest.mark.parametrize("block_t", [0, 64])
+def test_weights_that_stay(B, M, N, K, clusters, block_t):
+    d, prep, Xq, xs = _prep(M + K, M, N, K)
+    acc_o = oracle.spgemm_acc(Xq, prep["vals"], prep["meta"])
+    Wp, sc, x1, bi = B.pack24(cu(prep["vals"]), cu(prep["meta"])), cu(prep["w_scale"]), cu(np.array([xs], np.float32)), cu(d["bias"])
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    buf = torch.full((M * N + 4096,), 77, dtype=torch.float16, device="cuda")
+    Y = buf[2048:2048 + M * N].view(M, N)
+    B.set_block_tokens(block_t)
+    B.set_max_clusters(clusters)
+    try:
+        for act in (0, 1):
+            Y_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=act, out_type=0)
+            out_scale = np.float32(np.abs(Y_o.astype(np.float32)).max() / 127.0)
+            Q_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=act, out_type=1, out_scale=out_scale)
+            B.spgemm_i8(cu(Xq), Wp, N, sc, x1, bi, act=act, out_type=B.OUT_F16, Y=Y.fill_(0), status_buf=status)
+            assert f16_ulp_distance(Y.cpu().numpy(), Y_o).max() <= (F16_ULP_TOL if act else 0)
+            Q = B.spgemm_i8(cu(Xq), Wp, N, sc, x1, bi, act=act, out_type=B.OUT_I8, out_scale=cu(np.array([out_scale], np.float32)),
+                            status_buf=status).cpu().numpy()
+            # codes of a fixed IEEE sequence; with GELU one step at most, where the approximation meets a tie
+            assert np.abs(Q.astype(np.int32) - Q_o).max() <= act
+            Ya, amax = B.spgemm_i8_absmax(cu(Xq), Wp, N, sc, x1, bi, act=act, status_buf=status)
+            assert torch.equal(Ya, Y) and amax.item() == Y.float().abs().max().item()
+    finally:
+        B.set_block_tokens(0)
+        B.set_max_clusters(0)
+    assert status.cpu().tolist() == [0, 0, 0, 0]
+    assert (buf[:2048] == 77).all() and (buf[2048 + M * N:] == 77).all()
+
+
 @pytest.mark.parametrize("M,N,K,block_t", [(514, 256, 1280, 0), (197, 128, 192, 0), (1000, 384, 256, 96),
                                            (33, 128, 64, 32), (1576, 768, 192, 224), (394, 96, 48, 0),
                                            (500, 288, 96, 64), (333, 576, 192, 0), (70, 16, 16, 0)])
