@@ -283,7 +283,7 @@ def run_gpusq(args, cfg):
             layer_quant(s)
             layer_gemm(s)
 
-    launches_per_step = 2 * len(state)        # quant_act (one cooperative launch) + GEMM per layer
+    launches_per_step = 2 * len(state)        # quant_act (one launch) + GEMM per layer
 
     def barrier():
         if world > 1:
