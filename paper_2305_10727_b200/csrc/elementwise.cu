@@ -51,6 +51,14 @@ prune24_kernel(const float4 *__restrict__ W, float4 *Wp, uint8_t *mask, int64_t 
 }
 
 // ------------------------------------------------------------- quant_weight
+// Four codes by the division, in one word (lowest byte first).  A quotient that is no number (a NaN weight, an
+// infinite one, a zero of a row whose maximum / qmax is too small for binary32) has code 0.
+__device__ __forceinline__ uint32_t quant_codes4(float4 v, float s, int qmax)
+{
+    return (uint32_t)(quant_code(v.x, s, qmax) & 0xFF) | ((uint32_t)(quant_code(v.y, s, qmax) & 0xFF) << 8) |
+           ((uint32_t)(quant_code(v.z, s, qmax) & 0xFF) << 16) | ((uint32_t)(quant_code(v.w, s, qmax) & 0xFF) << 24);
+}
+
 // Symmetric per-row quantisation.  A row sits in the registers of one warp (kBlockRow = false, rows of
 // up to 1024) or of one block (up to 8192), kPer float4 per thread: one pass over the weights, no barrier
 // in the warp form, and the codes by the bracketing products instead of a division per weight.  Bound by
@@ -88,12 +96,12 @@ quant_weight_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ Wq, fl
     for (int u = 0; u < kPer; ++u) {
         const float2 f0 = make_float2(v[u].x, v[u].y), f1 = make_float2(v[u].z, v[u].w);
         uint32_t differ = 0;
-        float2 m0 = quant2_sums<false>(f0, a, differ), m1 = quant2_sums<false>(f1, a, differ);
-        if (differ != 0u || a.always_divide) {
-            m0 = quant2_exact<true>(f0, a);
-            m1 = quant2_exact<true>(f1, a);
-        }
-        if (t + u * T < K4) out[t + u * T] = pack4_low_bytes(m0, m1);
+        const float2 m0 = quant2_sums<false>(f0, a, differ), m1 = quant2_sums<false>(f1, a, differ);
+        // a NaN's sums agree, but have the exponent bit that 1.5 * 2^23 +- 127 have not
+        differ |= (__float_as_uint(m0.x) | __float_as_uint(m0.y) | __float_as_uint(m1.x) | __float_as_uint(m1.y)) & 0x00800000u;
+        uint32_t codes = pack4_low_bytes(m0, m1);
+        if (differ != 0u || a.always_divide) codes = quant_codes4(v[u], s, (int)qmax);
+        if (t + u * T < K4) out[t + u * T] = codes;
     }
 }
 
@@ -115,11 +123,7 @@ quant_weight_long_kernel(const float4 *__restrict__ Wp, uint32_t *__restrict__ W
         if (threadIdx.x == 0) w_scale[n] = s;
         uint32_t *out = Wq + (int64_t)n * K4;
         const int q = (int)qmax;
-        for (int k = threadIdx.x; k < K4; k += blockDim.x) {
-            const float4 v = __ldg(row + k);
-            out[k] = (uint32_t)(quant_code(v.x, s, q) & 0xFF) | ((uint32_t)(quant_code(v.y, s, q) & 0xFF) << 8) |
-                     ((uint32_t)(quant_code(v.z, s, q) & 0xFF) << 16) | ((uint32_t)(quant_code(v.w, s, q) & 0xFF) << 24);
-        }
+        for (int k = threadIdx.x; k < K4; k += blockDim.x) out[k] = quant_codes4(__ldg(row + k), s, q);
     }
 }
 

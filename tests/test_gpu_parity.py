@@ -117,6 +117,29 @@ def test_quant_weight_row_lengths(B, N, K):
     assert np.array_equal(ws.cpu().numpy(), ws_o) and np.array_equal(Wq.cpu().numpy(), Wq_o)
 
 
+# quotients that are no number have code 0, in registers of a warp, of a block and in longer rows alike
+@pytest.mark.parametrize("K", [64, 1024, 1028, 4100, 8192, 8196])
+@pytest.mark.parametrize("q", [127, 7])
+def test_quant_weight_degenerate_rows(B, K, q):
+    W = (np.random.default_rng(K).standard_normal((4, K)) * 0.02).astype(np.float32)
+    W[:, 2::4] = 0.0                                        # pruned positions
+    W[:, 3::4] = 0.0
+    plain, quant = (oracle.quant_weight, B.quant_weight) if q == 127 else (oracle.quant_weight4, B.quant_weight4)
+    want, ws_o = plain(W)
+    tiny = np.float32(1.4e-45)                              # the smallest subnormal: tiny / q is 0, zeros are 0 / 0
+    W[1] = np.sign(W[1]) * tiny
+    W[1, 4:8] = 0.0
+    want[1], ws_o[1] = np.sign(W[1]) * q, 0.0
+    W[2, K - 4] = -np.inf                                   # the scale is infinite: all others are 0
+    want[2], ws_o[2] = 0, np.inf
+    W[3, K - 3] = np.nan                                    # does not count for the maximum
+    clean = np.where(np.isnan(W[3:]), 0, W[3:])
+    want[3:], ws_o[3:] = plain(clean)
+    Wq, ws = quant(cu(W))
+    assert np.array_equal(ws.cpu().numpy(), ws_o)
+    assert np.array_equal(Wq.cpu().numpy(), want)
+
+
 # vectors of eight values: cluster kernel of 1 to 16 CTAs with 1, 2 and 4 vectors per thread, the first size beyond
 # it, tensors that just do and just do not fit the one-launch kernel's shared memory, and the rest being one
 # vector, one round, as many as the ring has places, one vector more, and an odd part of a later round
