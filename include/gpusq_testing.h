@@ -33,7 +33,19 @@ int gpusq_set_tile_mix(int block_t, int n_big);
  * faults or hangs: the waits end at the bound. */
 int gpusq_set_quant_act_wait(unsigned long long limit_ns, int withhold_last_cta);
 
-/* The same for the GEMM kernels: bound of every device-side wait in microseconds
+/* CTAs [first, first + count) of gpusq_quant_act's one-launch kernel (tensors
+ * above 1 MB) wait for ns nanoseconds (at most 1 ms; 0 or count 0: none) before
+ * they claim their shares, as if no SM had been free for them, and as long
+ * again, if the share is gone by then, before they count themselves out.
+ * CTAs that run take over shares that nobody has claimed after 20 us. */
+int gpusq_set_quant_act_late(int first, int count, unsigned ns);
+
+/* Shares taken over on the current device since the library was loaded.
+ * Synchronises. */
+int gpusq_quant_act_shares_taken(unsigned *shares);
+
+/* As gpusq_set_quant_act_wait, for the GEMM kernels: bound of every device-side
+ * wait in microseconds
  * (default 2 s) and, with withhold_loads != 0, a planted failure in an allowed
  * form: the producers of the first CTA pair stop before the last k block of
  * their first tile, so the MMA issuer's bounded wait for that block runs out;

@@ -616,6 +616,16 @@ static_assert(kWsClaims + kMaxQuantCtas / 32 <= kMaxPartials + kWorkspaceExtra, 
 constexpr unsigned long long kTakeOverNs = 20000;                // wait before the shares of CTAs that have not started are taken over
 static std::atomic<unsigned long long> g_grid_wait_ns{2000000000ull};    // bound of the waits below (2 s)
 static std::atomic<int> g_withhold_slot{0};                      // test hook: the last CTA does not publish
+static std::atomic<int> g_late_first{0}, g_late_count{0};        // test hook: CTAs that start late ...
+static std::atomic<unsigned> g_late_ns{0};                       // ... and by how much
+constexpr unsigned kMaxLateNs = 1000000;
+static __device__ uint32_t g_shares_taken;                       // shares taken over since the library was loaded (tests)
+
+// The test hooks of a launch (gpusq_testing.h).
+struct QuantTest {
+    int withhold, late_first, late_count;
+    uint32_t late_ns;
+};
 
 __device__ __forceinline__ uint64_t globaltimer_now()
 {
@@ -734,6 +744,14 @@ __device__ __forceinline__ void share_codes(const uint4 *X, uint2 *Xq, const Qua
     for_share(sh, v, [&](int64_t i) { Xq[i] = regrouped(quant8_f16<false>(__ldg(X + i), a), regroup); });
 }
 
+// One thread of a CTA that a test makes late.
+__device__ __forceinline__ void be_late(uint32_t ns)
+{
+    const uint64_t t0 = globaltimer_now();
+    while (globaltimer_now() - t0 < ns) {
+    }
+}
+
 // One thread counts its CTA as past the barrier; the result, for count_out(), takes a while to come.  The last
 // one (nobody polls any more) puts the workspace back to zero and writes the scale, which tells the caller
 // that every share is done.
@@ -785,6 +803,7 @@ __device__ __forceinline__ uint32_t arrive_and_wait(uint32_t *ws, uint32_t mine,
             const uint32_t bit = open & (0u - open);
             if (atomicOr(ws + kWsClaims + v / 32, bit) & bit) continue;
             taken[v / 32] |= bit;
+            atomicAdd(&g_shares_taken, 1u);
             return kTakeOver + v + (uint32_t)__ffs((int)bit) - 1u;
         }
     }
@@ -792,7 +811,7 @@ __device__ __forceinline__ uint32_t arrive_and_wait(uint32_t *ws, uint32_t mine,
 
 __global__ void __launch_bounds__(kFusedThreads, 1)
 act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
-                       uint32_t *ws, const __grid_constant__ QuantShare sh, unsigned long long wait_ns, int withhold, float qmax, int regroup)
+                       uint32_t *ws, const __grid_constant__ QuantShare sh, unsigned long long wait_ns, const __grid_constant__ QuantTest test, float qmax, int regroup)
 {
     extern __shared__ __align__(128) uint4 cache[];
     __shared__ uint32_t red[kFusedThreads / 32];
@@ -816,11 +835,15 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         gave_up = 0;
     }
     if (tid < kMaxQuantCtas / 32) taken[tid] = 0;
+    // test hook; looked at here, while the previous kernel drains: behind the wait it cost 0.1 us
+    uint32_t late_ns = tid == 0 && blockIdx.x - (uint32_t)test.late_first < (uint32_t)test.late_count ? test.late_ns : 0u;
+    asm volatile("" : "+r"(late_ns));
     __syncthreads();
     // the previous kernel of the stream (a producer of X, or a user of the workspace) is complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the next kernel of the stream may be scheduled as soon as CTAs of this grid make room
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (late_ns) be_late(late_ns);
     if (blockIdx.x == 0 && tid == 0) *x_scale = __int_as_float(0x7FC00000);
 
     // 1. the slice into shared memory, all pieces in flight at once
@@ -886,7 +909,7 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         if (tid < 32) {
             const uint32_t mine = __reduce_max_sync(0xffffffffu, red[tid]);
             if (tid == 0) {
-                const bool publish = !(withhold && own && blockIdx.x == gridDim.x - 1);
+                const bool publish = !(test.withhold && own && blockIdx.x == gridDim.x - 1);
                 uint32_t all = 0;
                 next = gave_up ? kGaveUp : own && (claimed >> (blockIdx.x & 31) & 1u) ? kTooLate : arrive_and_wait(ws, mine, publish, t0, wait_ns, taken, all);
                 grid_max = all;
@@ -901,8 +924,15 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
     if (next != kAllArrived) VecRing::wait<0>();
     if (next == kTooLate) {
         if (tid == 0) {
-            const uint32_t word = __ldcv(ws + kWsBarrier + 1);              // final if this CTA is the last one
-            count_out(ws, count_past(ws), x_scale, word, qmax);
+            // This CTA has not waited, so all it knows of the maximum is that it is final once every CTA has counted
+            // itself past the barrier (whoever took a share over does so after the last arrival).  As the last one
+            // it is to be read after the count, never before.
+            if (late_ns) be_late(late_ns);
+            const uint32_t before = count_past(ws);
+            if (before == gridDim.x - 1) {
+                __threadfence();
+                count_out(ws, before, x_scale, __ldcv(ws + kWsBarrier + 1), qmax);
+            }
         }
         return;
     }
@@ -1246,10 +1276,11 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         const unsigned long long wait_ns = g_grid_wait_ns.load(std::memory_order_relaxed);
-        const int withhold = g_withhold_slot.load(std::memory_order_relaxed);
+        const QuantTest test = {g_withhold_slot.load(std::memory_order_relaxed), g_late_first.load(std::memory_order_relaxed),
+                                g_late_count.load(std::memory_order_relaxed), g_late_ns.load(std::memory_order_relaxed)};
         if (cudaLaunchKernelEx(&cfg, act_quant_fused_kernel, reinterpret_cast<const uint4 *>(X),
                                reinterpret_cast<uint2 *>(Xq), x_scale, reinterpret_cast<uint32_t *>(workspace), sh,
-                               wait_ns, withhold, qmax, regroup) != cudaSuccess) {
+                               wait_ns, test, qmax, regroup) != cudaSuccess) {
             (void)cudaGetLastError();
             return GPUSQ_ERR_CUDA;
         }
@@ -1287,6 +1318,25 @@ int gpusq_set_quant_act_wait(unsigned long long limit_ns, int withhold_last_cta)
     if (limit_ns == 0) return GPUSQ_ERR_ARG;
     g_grid_wait_ns.store(limit_ns, std::memory_order_relaxed);
     g_withhold_slot.store(withhold_last_cta ? 1 : 0, std::memory_order_relaxed);
+    return GPUSQ_OK;
+}
+
+int gpusq_set_quant_act_late(int first, int count, unsigned ns)
+{
+    if (first < 0 || count < 0 || ns > kMaxLateNs) return GPUSQ_ERR_ARG;
+    g_late_first.store(first, std::memory_order_relaxed);
+    g_late_count.store(count, std::memory_order_relaxed);
+    g_late_ns.store(ns, std::memory_order_relaxed);
+    return GPUSQ_OK;
+}
+
+int gpusq_quant_act_shares_taken(unsigned *shares)
+{
+    if (!shares) return GPUSQ_ERR_NULL;
+    if (cudaMemcpyFromSymbol(shares, g_shares_taken, sizeof(*shares)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return GPUSQ_ERR_CUDA;
+    }
     return GPUSQ_OK;
 }
 

@@ -184,6 +184,43 @@ def test_quant_act_beside_other_kernels(B):
     assert [B.quant_act_status(w) for w in ws] == [0, 0] and not any(w.any() for w in ws)
 
 
+# CTAs that get an SM late, so that others take their shares over: the last one, the first (which writes the NaN),
+# several, all but one.  The tensor's maximum lies in a late CTA's share.  100 us is certain to be too late; around
+# the 20 us after which shares are taken over, a late CTA may find its share gone before its maximum is known, and is
+# then held back until it is the last one out, the one that writes the scale.
+@pytest.mark.parametrize("extra", [4096, 14336])            # vectors per CTA: all kept in shared memory; with a rest
+@pytest.mark.parametrize("which", ["last", "first", "several", "all_but_one"])
+@pytest.mark.parametrize("q", [127, 7])
+def test_quant_act_shares_taken_over(B, extra, which, q):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    first, count = {"last": (sms - 1, 1), "first": (0, 1), "several": (10, 12), "all_but_one": (1, sms - 1)}[which]
+    vecs = sms * extra + 501
+    X = np.random.default_rng(extra + first).standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
+    per = -(-vecs // sms) if extra <= 10240 else 10240
+    X[first * per + 5, 3] = -9.5
+    call, plain = (B.quant_act, oracle.quant_act) if q == 127 else (B.quant_act4, oracle.quant_act4)
+    Xq_o, s_o = plain(X)
+    if q == 7:                                              # the oracle's codes are in the order of the columns
+        Xq_o = Xq_o[:, [0, 2, 4, 6, 1, 3, 5, 7]]
+    Xd, want = cu(X), cu(Xq_o)
+    ws = torch.zeros((B.quant_act_workspace(*X.shape),), dtype=torch.uint8, device="cuda")
+    try:
+        for ns in [100_000] + list(range(18_000, 50_000, 1_000)):
+            B.set_quant_act_late(first, count, ns)
+            before = B.quant_act_shares_taken()
+            Xq, s = call(Xd, workspace=ws)
+            taken = B.quant_act_shares_taken() - before
+            assert s.cpu().numpy()[0] == s_o and torch.equal(Xq, want), ns
+            assert not ws.any()                             # control words back at zero, no status
+            # CTA 0 takes over what it can of 147 shares in 80 us, the others all of the late ones
+            assert ns != 100_000 or (taken > 0 if which == "all_but_one" else taken == count)
+    finally:
+        B.set_quant_act_late(0, 0, 0)
+    before = B.quant_act_shares_taken()
+    Xq, s = call(Xd, workspace=ws)
+    assert s.cpu().numpy()[0] == s_o and torch.equal(Xq, want) and not ws.any()
+
+
 @pytest.mark.parametrize("amax", [7.0, 3.75, 5.87890625, 6.1e-5, 65504.0, 4.87, 2.2578125])
 def test_quant_act_every_binary16_value(B, amax):
     # large enough that the kernels look for a single product that gives all codes; every value they can meet
