@@ -35,6 +35,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -260,7 +261,8 @@ __device__ __forceinline__ float2 gelu_pair(float2 y)
 // output had it, took for DeiT-Base at batch 64 (M = 12608): 768 -> 2304 19.7 us, 768 -> 3072 with GELU
 // 32.5, 3072 -> 768 21.5; this takes 19.0, 29.6, 20.0, part of it by the eighth pipeline stage for which
 // the staging tiles left no room.  Per-warp bulk stores instead of the plain ones: 19.3, 31.0, 19.8.
-template <bool kAccFloat, bool kI8, bool kTwin, bool kRuns>
+// kWide: the bytes of a tile's rows of Y do not fit 32 bits (wide_rows); the type of row_bytes is all that changes.
+template <bool kAccFloat, bool kI8, bool kTwin, bool kRuns, bool kWide>
 struct Epilogue {
     const GemmParams *p;
     Ctl *ctl;
@@ -270,7 +272,8 @@ struct Epilogue {
 
     uint32_t stm_addr, lds_addr;   // this lane's matrix-store and read address in the current buffer
     uint8_t *y0, *y1;              // where this lane stores the first and (FP16) second eight tokens of the chunk
-    uint32_t row_bytes;            // of Y
+    using Bytes = std::conditional_t<kWide, uint64_t, uint32_t>;
+    Bytes row_bytes;               // of Y; products with up to kMaxBlockT rows are taken in this type
     int rows;                      // rows of Y from y0's on that exist (<= 0: this lane stores nothing)
     float sc[4], bi[4];            // scale and bias of this thread's four features
     int left;                      // tokens of the tile, from the chunk on, that exist
@@ -385,7 +388,7 @@ struct Epilogue {
         const int row_l = kI8 ? lane >> 1 : lane >> 2, col_l = kI8 ? (lane & 1) * 16 : (lane & 3) * 8;
         lds_addr = kI8 ? buf0 + (uint32_t)(row_l * 32 + (((lane & 1) ^ ((row_l >> 2) & 1)) << 4))
                        : buf0 + (uint32_t)(row_l * 64 + (((lane & 3) ^ ((row_l >> 1) & 3)) << 4));
-        row_bytes = (uint32_t)N * (kI8 ? 1u : 2u);
+        row_bytes = (Bytes)(uint32_t)N * (kI8 ? 1u : 2u);
         // this thread's first feature, relative to the CTA's 128
         const int nofs = quarter * 32 + (lane >> 2);
         const float *w_scale = p->w_scale + nofs, *bias = p->bias + nofs;
@@ -480,7 +483,7 @@ struct Epilogue {
 // own register allocation
 // kAmax: the FP16 epilogue also merges max |Y| into a device word (its own instantiation, so that the
 // ordinary kernel's register allocation is untouched)
-template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false, bool kRuns = false>
+template <bool kSparse, int kOut, bool kHalf = false, bool kTwin = false, bool kAmax = false, bool kRuns = false, bool kWide = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsGemm, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_e, const GemmParams p)
@@ -721,7 +724,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t tmem_empty0 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[0]), 0);
         const uint32_t tmem_empty1 = ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[1]), 0);
         if (kOut == GPUSQ_OUT_F16 || kOut == GPUSQ_OUT_I8) {
-            Epilogue<kHalf, kOut == GPUSQ_OUT_I8, kTwin, kRuns> e;
+            Epilogue<kHalf, kOut == GPUSQ_OUT_I8, kTwin, kRuns, kWide> e;
             e.p = &p;
             e.ctl = ctl;
             e.buf0 = ptx::smem_u32(smem + (warp - 2) * 2 * kEpiBufBytes);
@@ -953,13 +956,24 @@ static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters
     return best;
 }
 
+// Rows of Y so long that the epilogue's 32-bit byte counts (up to the rows of a tile) overflow: FP16 output from
+// 9.6 million features on.  They have instantiations of their own: 64-bit counts for all cost 65792 x 1280 ->
+// 5120 with GELU 3 % (255 -> 263 us) and others up to 1.4 %.  Those stream, without twin tiles (the last of
+// 37,450 feature columns and more is not worth a second set), as does the tiling.
+static bool wide_rows(const GemmParams &p)
+{
+    const uint64_t row = (uint64_t)p.N * (p.out_type == GPUSQ_OUT_I8 ? 1 : 2);
+    return p.out_type != GPUSQ_OUT_I32 && row * kMaxBlockT > 0xFFFFFFFFull;
+}
+
 // Fills the tiling fields of the parameters; false when the number of runs does not fit 31 bits.
 template <typename C>
 static bool set_tiling(GemmParams &p, int K_cost, int clusters)
 {
     const int tiles_n = (p.N + kPairF - 1) / kPairF;
     // a last feature column of at most 128 features is worked on in twin tiles (see RunWalk)
-    const bool twin_col = p.N - (tiles_n - 1) * kPairF <= kBlockF && p.M < 0x7FFFFFFF - 4 * kMaxBlockT;
+    const bool wide = wide_rows(p);
+    const bool twin_col = !wide && p.N - (tiles_n - 1) * kPairF <= kBlockF && p.M < 0x7FFFFFFF - 4 * kMaxBlockT;
     p.pair_cols = twin_col ? tiles_n - 1 : tiles_n;
     // The weights of a column can stay when they leave room for kMinResidentStages activation stages.  (The
     // FP16 model's leave three at K = 768, with which it is slower: 27.5 us streaming, 31.7 resident.)  The
@@ -967,7 +981,7 @@ static bool set_tiling(GemmParams &p, int K_cost, int clusters)
     const int kb = (p.K + kBlockK - 1) / kBlockK;
     const int stages = kb <= kMaxWeightBlocks ? (C::kRoom - kb * C::kWBytes) / C::kBBytes : 0;
     // With fewer than three waves of tiles there is nothing to keep them for.
-    const bool may_stay = C::kMayStay && p.out_type != GPUSQ_OUT_I32 && !twin_col && stages >= C::kMinResidentStages &&
+    const bool may_stay = C::kMayStay && p.out_type != GPUSQ_OUT_I32 && !twin_col && !wide && stages >= C::kMinResidentStages &&
                           ceil_div(p.M, kMaxBlockT) * p.pair_cols >= 3 * (int64_t)clusters;
     TilePlan t;
     if (p.pair_cols == 0) {
@@ -1060,19 +1074,25 @@ static bool prepare_device(int kind)
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true, true>, b) &&
-                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, false, false, true>, b);
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, false, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, false, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I8, false, false, false, false, true>, b);
         } else if (kind == 1) {
             const int b = kMaxSmem;
             ok = allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_F16>, b) && allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I8>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I32>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_F16, false, true>, b) &&
                  allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I8, false, true>, b) &&
-                 allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I32, false, true>, b);
+                 allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I32, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_F16, false, false, false, false, true>, b) &&
+                 allow_smem(gemm_i8_kernel<false, GPUSQ_OUT_I8, false, false, false, false, true>, b);
         } else {
             const int b = kMaxSmem;
             ok = allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, b) && allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, true>, b) &&
                  allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, b) &&
-                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, true, true>, b);
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_I32, true, true>, b) &&
+                 allow_smem(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, false, false, false, true>, b);
         }
         if (!ok) (void)cudaGetLastError();
         done[dev][kind] = ok ? 1 : 2;
@@ -1172,6 +1192,13 @@ static int launch_gemm(const int8_t *Xq, const void *Wsrc, const float *w_scale,
                             : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
         }
     }
+    if (wide_rows(p)) {
+        if (out_type == GPUSQ_OUT_I8)
+            return launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_I8, false, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+        if (y_absmax)
+            return launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+        return launch_on(gemm_i8_kernel<kSparse, GPUSQ_OUT_F16, false, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
+    }
     if (out_type == GPUSQ_OUT_F16 && y_absmax && kSparse)
         return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
                         : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
@@ -1236,6 +1263,8 @@ static int launch_gemm_f16(const void *X, const void *Wpacked, const float *bias
     if (!ok) return GPUSQ_ERR_CUDA;
 
     const int smem = smem_bytes<C>(p);
+    if (wide_rows(p))
+        return launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, false, false, false, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);
     if (out_type == GPUSQ_OUT_F16)
         return twin_col ? launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream)
                         : launch_on(gemm_i8_kernel<true, GPUSQ_OUT_F16, true>, smem, map_a, map_b, map_b2, map_e, p, clusters, stream);

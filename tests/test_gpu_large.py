@@ -105,3 +105,42 @@ def test_gemm_more_than_2_31_outputs(B, out):
         Q_o = oracle.epilogue(acc_o, prep["w_scale"], xs, bias, act=0, out_type=1, out_scale=out_scale)
         assert np.array_equal(Y[cu(rows)].cpu().numpy(), Q_o)
     assert status.cpu().tolist() == [0, 0, 0, 0]
+
+
+# Rows of Y so long that the bytes of the 48 rows between a warp's chunks, or of the 224 of a tile in a run, no longer
+# fit 32 bits.  A sentinel shows outputs that were never written; slices of the features are compared with a call on
+# those features alone, which the parity tests hold to the oracle.
+@pytest.mark.parametrize("M,N,out", [(65, 44_800_064, "f16"), (65, 89_600_000, "i8"), (1000, 9_600_000, "f16"),
+                                     (1000, 9_600_000, "absmax"), (1000, 19_200_000, "i8"), (65, 44_800_000, "dense"),
+                                     (65, 89_600_000, "dense_i8"), (65, 44_800_000, "half")])
+def test_gemm_very_long_output_rows(B, M, N, out):
+    K = 16
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    W = torch.randint(-127, 128, (N, K if "dense" in out else K // 2), generator=gen, device="cuda", dtype=torch.int8)
+    nibble = torch.tensor([0x4, 0x8, 0xC, 0x9, 0xD, 0xE], dtype=torch.uint8, device="cuda")
+    meta = nibble[torch.randint(0, 6, (N, K // 8), generator=gen, device="cuda")] * 17
+    ws = torch.rand((N,), generator=gen, device="cuda") * 1e-3 + 1e-3
+    bias = torch.rand((N,), generator=gen, device="cuda")
+    Xq = torch.randint(-127, 128, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    xs = torch.full((1,), 0.01, device="cuda")
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    i8 = out in ("i8", "dense_i8")
+    kind = dict(out_type=B.OUT_I8, out_scale=torch.full((1,), 0.01, device="cuda")) if i8 else {}
+    sentinel = -128 if i8 else float("nan")                            # no code, no finite output
+    Y = torch.full((M, N), sentinel, dtype=torch.int8 if i8 else torch.float16, device="cuda")
+
+    def layer(lo, hi, Y=None):
+        w, n, common = W[lo:hi], hi - lo, dict(Y=Y, status_buf=status)
+        if out == "half":
+            return B.spgemm_f16(Xq.half(), B.pack24_f16(w.half(), meta[lo:hi]), n, bias[lo:hi], **common)
+        if "dense" in out:
+            return B.gemm_i8_dense(Xq, w, ws[lo:hi], xs, bias[lo:hi], **kind, **common)
+        args = (Xq, B.pack24(w, meta[lo:hi]), n, ws[lo:hi], xs, bias[lo:hi])
+        return B.spgemm_i8_absmax(*args, **common)[0] if out == "absmax" else B.spgemm_i8(*args, **kind, **common)
+
+    layer(0, N, Y)
+    for i in range(M):
+        assert not ((Y[i] == sentinel) if i8 else Y[i].isnan()).any(), i
+    for lo in (0, 2048 * 999, N // 2 // 256 * 256, N - 2048):
+        assert torch.equal(Y[:, lo:lo + 2048], layer(lo, lo + 2048))
+    assert status.cpu().tolist() == [0, 0, 0, 0]
