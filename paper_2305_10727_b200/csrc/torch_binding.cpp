@@ -4,6 +4,8 @@
 // Python through ctypes cost 2 us more for a call that allocates nothing and 5 us for one with two outputs.
 // Outputs come from torch's caching allocator without the dispatcher: 0.4 us less for a call with two of them
 // (4.7 -> 4.25, of which the launch is 2.1).
+// The interpreter's lock is given up once per call, around allocations and library call together: the one may
+// go to the driver and synchronise, the other waits when the stream's launch queue is full.
 //
 // Functions take positional arguments only; binding.py holds the public signatures and their defaults.
 #include <Python.h>
@@ -12,6 +14,9 @@
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
+
+#include <algorithm>
+#include <initializer_list>
 
 #include "gpusq.h"
 
@@ -73,41 +78,54 @@ void *address(PyObject *o, const char *what) { return o == Py_None ? nullptr : t
 template <typename T>
 T *address_as(PyObject *o, const char *what) { return static_cast<T *>(address(o, what)); }
 
-// An output: the tensor that the caller passed, or a new one.  `obj` is a reference of its own.
-struct Out {
-    PyObject *obj;
-    void *p;
-    Out(PyObject *given, const at::Tensor &like, at::ScalarType type, at::IntArrayRef shape, const char *what)
+// An output: the tensor that the caller passed, or a new one, which make() allocates.
+class Out {
+public:
+    Out(PyObject *given, const at::Tensor &like, at::ScalarType type, std::initializer_list<int64_t> shape, const char *what)
+        : given_(given), device_(like.device()), type_(type), dims_(shape.size())
     {
-        if (given != Py_None) {
-            p = tensor(given, what).data_ptr();
-            obj = Py_NewRef(given);
-        } else {
-            // torch's allocator without its dispatcher in between
-            at::Tensor t(at::detail::empty_cuda(shape, type, like.device(), std::nullopt));
-            p = t.data_ptr();
-            obj = THPVariable_Wrap(std::move(t));
-            if (!obj) throw Failed();
-        }
+        std::copy(shape.begin(), shape.end(), shape_);
+        if (given != Py_None) p_ = tensor(given, what).data_ptr();
     }
     Out(const Out &) = delete;
-    ~Out() { Py_XDECREF(obj); }
+    // without the interpreter's lock; torch's allocator without its dispatcher in between
+    void make()
+    {
+        if (given_ != Py_None) return;
+        made_ = at::Tensor(at::detail::empty_cuda(at::IntArrayRef(shape_, dims_), type_, device_, std::nullopt));
+        p_ = made_.data_ptr();
+    }
     PyObject *take()
     {
-        PyObject *o = obj;
-        obj = nullptr;
+        PyObject *o = given_ != Py_None ? Py_NewRef(given_) : THPVariable_Wrap(std::move(made_));
+        if (!o) throw Failed();
         return o;
     }
     template <typename T>
-    T *as() const { return static_cast<T *>(p); }
+    T *as() const { return static_cast<T *>(p_); }
+    void *p() const { return p_; }
+
+private:
+    PyObject *given_;
+    at::Device device_;
+    at::ScalarType type_;
+    size_t dims_;
+    int64_t shape_[2];
+    at::Tensor made_;
+    void *p_ = nullptr;
 };
 
 PyObject *pair(Out &a, Out &b)
 {
     PyObject *t = PyTuple_New(2);
     if (!t) throw Failed();
-    PyTuple_SET_ITEM(t, 0, a.take());
-    PyTuple_SET_ITEM(t, 1, b.take());
+    try {
+        PyTuple_SET_ITEM(t, 0, a.take());
+        PyTuple_SET_ITEM(t, 1, b.take());
+    } catch (...) {
+        Py_DECREF(t);
+        throw;
+    }
     return t;
 }
 
@@ -122,6 +140,27 @@ void check(int status, const char *where)
         Py_DECREF(e);
     }
     throw Failed();
+}
+
+// The interpreter's lock, given up for as long as this object lives.
+struct Unlocked {
+    PyThreadState *state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked &) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+// Allocates the outputs and calls f(stream), which calls the library and must not touch Python.
+template <typename F, typename... O>
+void run(const char *where, F f, O &...outs)
+{
+    int status;
+    {
+        Unlocked u;
+        (outs.make(), ...);
+        status = f(stream());
+    }
+    check(status, where);
 }
 
 // C++ exceptions (out of memory, wrong tensor) become Python ones
@@ -146,13 +185,16 @@ PyObject *prune24(PyObject *const *a)
 {
     const at::Tensor &W = IN_F32(a[0], "W");
     const auto [N, K] = matrix(W, "W");
+    const int n = as_int(N), k = as_int(K);
+    const float *w = W.const_data_ptr<float>();
     Out Wp(a[1], W, at::kFloat, {N, K}, "Wp");
     if (a[3] == Py_True) {
         Out mask(a[2], W, at::kByte, {N, K / 4}, "mask");
-        check(gpusq_prune24(W.const_data_ptr<float>(), Wp.as<float>(), mask.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_prune24");
+        run("gpusq_prune24", [&](void *s) { return gpusq_prune24(w, Wp.as<float>(), mask.as<uint8_t>(), n, k, s); }, Wp, mask);
         return pair(Wp, mask);
     }
-    check(gpusq_prune24(W.const_data_ptr<float>(), Wp.as<float>(), address_as<uint8_t>(a[2], "mask"), as_int(N), as_int(K), stream()), "gpusq_prune24");
+    uint8_t *mask = address_as<uint8_t>(a[2], "mask");
+    run("gpusq_prune24", [&](void *s) { return gpusq_prune24(w, Wp.as<float>(), mask, n, k, s); }, Wp);
     return Wp.take();
 }
 
@@ -161,13 +203,15 @@ PyObject *prune48(PyObject *const *a)
 {
     const at::Tensor &W = IN_F32(a[0], "W");
     const auto [N, K] = matrix(W, "W");
+    const int n = as_int(N), k = as_int(K);
+    const float *w = W.const_data_ptr<float>();
     Out Wp(Py_None, W, at::kFloat, {N, K}, "Wp");
     if (a[1] == Py_True) {
         Out mask(Py_None, W, at::kByte, {N, K / 8}, "mask");
-        check(gpusq_prune48(W.const_data_ptr<float>(), Wp.as<float>(), mask.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_prune48");
+        run("gpusq_prune48", [&](void *s) { return gpusq_prune48(w, Wp.as<float>(), mask.as<uint8_t>(), n, k, s); }, Wp, mask);
         return pair(Wp, mask);
     }
-    check(gpusq_prune48(W.const_data_ptr<float>(), Wp.as<float>(), nullptr, as_int(N), as_int(K), stream()), "gpusq_prune48");
+    run("gpusq_prune48", [&](void *s) { return gpusq_prune48(w, Wp.as<float>(), nullptr, n, k, s); }, Wp);
     return Wp.take();
 }
 
@@ -177,8 +221,10 @@ PyObject *quantise_weight(PyObject *const *a, const char *where)
 {
     const at::Tensor &Wp = IN_F32(a[0], "Wp");
     const auto [N, K] = matrix(Wp, "Wp");
+    const int n = as_int(N), k = as_int(K);
+    const float *w = Wp.const_data_ptr<float>();
     Out Wq(a[1], Wp, at::kChar, {N, K}, "Wq"), w_scale(a[2], Wp, at::kFloat, {N}, "w_scale");
-    check(Fn(Wp.const_data_ptr<float>(), Wq.as<int8_t>(), w_scale.as<float>(), as_int(N), as_int(K), stream()), where);
+    run(where, [&](void *s) { return Fn(w, Wq.as<int8_t>(), w_scale.as<float>(), n, k, s); }, Wq, w_scale);
     return pair(Wq, w_scale);
 }
 PyObject *quant_weight(PyObject *const *a) { return quantise_weight<gpusq_quant_weight>(a, "gpusq_quant_weight"); }
@@ -189,8 +235,10 @@ PyObject *compress24(PyObject *const *a)
 {
     const at::Tensor &Wq = IN_I8(a[0], "Wq");
     const auto [N, K] = matrix(Wq, "Wq");
+    const int n = as_int(N), k = as_int(K);
+    const int8_t *w = Wq.const_data_ptr<int8_t>();
     Out vals(a[1], Wq, at::kChar, {N, K / 2}, "vals"), meta(a[2], Wq, at::kByte, {N, K / 8}, "meta");
-    check(gpusq_compress24(Wq.const_data_ptr<int8_t>(), vals.as<int8_t>(), meta.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_compress24");
+    run("gpusq_compress24", [&](void *s) { return gpusq_compress24(w, vals.as<int8_t>(), meta.as<uint8_t>(), n, k, s); }, vals, meta);
     return pair(vals, meta);
 }
 
@@ -199,8 +247,10 @@ PyObject *compress24_f16(PyObject *const *a)
 {
     const at::Tensor &Wp = IN_F32(a[0], "Wp");
     const auto [N, K] = matrix(Wp, "Wp");
+    const int n = as_int(N), k = as_int(K);
+    const float *w = Wp.const_data_ptr<float>();
     Out vals(Py_None, Wp, at::kHalf, {N, K / 2}, "vals"), meta(Py_None, Wp, at::kByte, {N, K / 8}, "meta");
-    check(gpusq_compress24_f16(Wp.const_data_ptr<float>(), vals.p, meta.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_compress24_f16");
+    run("gpusq_compress24_f16", [&](void *s) { return gpusq_compress24_f16(w, vals.p(), meta.as<uint8_t>(), n, k, s); }, vals, meta);
     return pair(vals, meta);
 }
 
@@ -209,8 +259,10 @@ PyObject *compress48(PyObject *const *a)
 {
     const at::Tensor &Wq = IN_I8(a[0], "Wq");
     const auto [N, K] = matrix(Wq, "Wq");
+    const int n = as_int(N), k = as_int(K);
+    const int8_t *w = Wq.const_data_ptr<int8_t>();
     Out vals4(Py_None, Wq, at::kByte, {N, K / 4}, "vals4"), meta4(Py_None, Wq, at::kByte, {N, K / 16}, "meta4");
-    check(gpusq_compress48(Wq.const_data_ptr<int8_t>(), vals4.as<uint8_t>(), meta4.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_compress48");
+    run("gpusq_compress48", [&](void *s) { return gpusq_compress48(w, vals4.as<uint8_t>(), meta4.as<uint8_t>(), n, k, s); }, vals4, meta4);
     return pair(vals4, meta4);
 }
 
@@ -220,8 +272,10 @@ PyObject *expand48(PyObject *const *a)
     const at::Tensor &vals4 = IN_U8(a[0], "vals4"), &meta4 = IN_U8(a[1], "meta4");
     const auto [N, K4] = matrix(vals4, "vals4");
     const int64_t K = K4 * 4;
+    const int n = as_int(N), k = as_int(K);
+    const uint8_t *v4 = vals4.const_data_ptr<uint8_t>(), *m4 = meta4.const_data_ptr<uint8_t>();
     Out vals(Py_None, vals4, at::kChar, {N, K / 2}, "vals"), meta(Py_None, vals4, at::kByte, {N, K / 8}, "meta");
-    check(gpusq_expand48(vals4.const_data_ptr<uint8_t>(), meta4.const_data_ptr<uint8_t>(), vals.as<int8_t>(), meta.as<uint8_t>(), as_int(N), as_int(K), stream()), "gpusq_expand48");
+    run("gpusq_expand48", [&](void *s) { return gpusq_expand48(v4, m4, vals.as<int8_t>(), meta.as<uint8_t>(), n, k, s); }, vals, meta);
     return pair(vals, meta);
 }
 
@@ -230,9 +284,11 @@ PyObject *pack24(PyObject *const *a)
 {
     const at::Tensor &vals = IN_I8(a[0], "vals"), &meta = IN_U8(a[1], "meta");
     const auto [N, K2] = matrix(vals, "vals");
-    const int K = as_int(K2 * 2);
-    Out packed(a[2], vals, at::kByte, {(int64_t)gpusq_packed_bytes(as_int(N), K)}, "Wpacked");
-    check(gpusq_pack24(vals.const_data_ptr<int8_t>(), meta.const_data_ptr<uint8_t>(), packed.p, as_int(N), K, stream()), "gpusq_pack24");
+    const int n = as_int(N), k = as_int(K2 * 2);
+    const int8_t *v = vals.const_data_ptr<int8_t>();
+    const uint8_t *m = meta.const_data_ptr<uint8_t>();
+    Out packed(a[2], vals, at::kByte, {(int64_t)gpusq_packed_bytes(n, k)}, "Wpacked");
+    run("gpusq_pack24", [&](void *s) { return gpusq_pack24(v, m, packed.p(), n, k, s); }, packed);
     return packed.take();
 }
 
@@ -241,9 +297,11 @@ PyObject *pack24_f16(PyObject *const *a)
 {
     const at::Tensor &vals = IN_F16(a[0], "vals"), &meta = IN_U8(a[1], "meta");
     const auto [N, K2] = matrix(vals, "vals");
-    const int K = as_int(K2 * 2);
-    Out packed(a[2], vals, at::kByte, {(int64_t)gpusq_packed_bytes_f16(as_int(N), K)}, "Wpacked");
-    check(gpusq_pack24_f16(vals.const_data_ptr(), meta.const_data_ptr<uint8_t>(), packed.p, as_int(N), K, stream()), "gpusq_pack24_f16");
+    const int n = as_int(N), k = as_int(K2 * 2);
+    const void *v = vals.const_data_ptr();
+    const uint8_t *m = meta.const_data_ptr<uint8_t>();
+    Out packed(a[2], vals, at::kByte, {(int64_t)gpusq_packed_bytes_f16(n, k)}, "Wpacked");
+    run("gpusq_pack24_f16", [&](void *s) { return gpusq_pack24_f16(v, m, packed.p(), n, k, s); }, packed);
     return packed.take();
 }
 
@@ -255,22 +313,28 @@ PyObject *quantise_act(PyObject *const *a, const char *where)
 {
     const at::Tensor &X = IN_F16(a[0], "X");
     const auto [M, K] = matrix(X, "X");
-    const int mode = int_arg(a[3]);
+    const int64_t m = M;
+    const int k = as_int(K), mode = int_arg(a[3]);
     if (mode == GPUSQ_SCALE_GIVEN && a[2] == Py_None) fail(PyExc_ValueError, "scale_mode GIVEN needs x_scale");
+    const void *x = X.const_data_ptr();
     Out Xq(a[1], X, at::kChar, {M, K}, "Xq"), x_scale(a[2], X, at::kFloat, {1}, "x_scale");
     void *ws = nullptr;
     size_t ws_bytes = 0;
-    at::Tensor own;
     if (a[4] != Py_None) {
         const at::Tensor &w = tensor(a[4], "workspace");
         ws = w.data_ptr();
         ws_bytes = (size_t)w.numel() * w.element_size();
-    } else if (mode == GPUSQ_SCALE_COMPUTE) {
-        ws_bytes = gpusq_quant_act_workspace(M, as_int(K));
-        own = at::zeros({(int64_t)ws_bytes}, at::TensorOptions().dtype(at::kByte).device(X.device()));
-        ws = own.data_ptr();
     }
-    check(Fn(X.const_data_ptr(), Xq.as<int8_t>(), x_scale.as<float>(), mode, M, as_int(K), ws, ws_bytes, stream()), where);
+    const bool needs_own = a[4] == Py_None && mode == GPUSQ_SCALE_COMPUTE;
+    at::Tensor own;
+    run(where, [&](void *s) {
+        if (needs_own) {
+            ws_bytes = gpusq_quant_act_workspace(m, k);
+            own = at::zeros({(int64_t)ws_bytes}, at::TensorOptions().dtype(at::kByte).device(X.device()));
+            ws = own.data_ptr();
+        }
+        return Fn(x, Xq.as<int8_t>(), x_scale.as<float>(), mode, m, k, ws, ws_bytes, s);
+    }, Xq, x_scale);
     return pair(Xq, x_scale);
 }
 PyObject *quant_act(PyObject *const *a) { return quantise_act<gpusq_quant_act>(a, "gpusq_quant_act"); }
@@ -281,8 +345,12 @@ PyObject *quant_act_absmax(PyObject *const *a)
 {
     const at::Tensor &X = IN_F16(a[0], "X");
     const auto [M, K] = matrix(X, "X");
+    const int64_t m = M;
+    const int k = as_int(K);
+    const void *x = X.const_data_ptr();
+    const float *absmax = address_as<float>(a[1], "absmax");
     Out Xq(a[2], X, at::kChar, {M, K}, "Xq"), x_scale(a[3], X, at::kFloat, {1}, "x_scale");
-    check(gpusq_quant_act_absmax(X.const_data_ptr(), Xq.as<int8_t>(), x_scale.as<float>(), address_as<float>(a[1], "absmax"), M, as_int(K), stream()), "gpusq_quant_act_absmax");
+    run("gpusq_quant_act_absmax", [&](void *s) { return gpusq_quant_act_absmax(x, Xq.as<int8_t>(), x_scale.as<float>(), absmax, m, k, s); }, Xq, x_scale);
     return pair(Xq, x_scale);
 }
 
@@ -294,13 +362,17 @@ PyObject *gemm(PyObject *const *a, const char *where)
 {
     const at::Tensor &Xq = IN_I8(a[0], "Xq");
     const auto [M, K] = matrix(Xq, "Xq");
-    const int N = int_arg(a[2]), act = int_arg(a[6]), out_type = int_arg(a[7]);
+    const int64_t m = M;
+    const int N = int_arg(a[2]), k = as_int(K), act = int_arg(a[6]), out_type = int_arg(a[7]);
     const at::ScalarType type = out_type == GPUSQ_OUT_F16 ? at::kHalf : out_type == GPUSQ_OUT_I8 ? at::kChar : at::kInt;
     if (a[9] == Py_None && (out_type < 0 || out_type > 2)) fail(PyExc_KeyError, "out_type");
+    const int8_t *x = Xq.const_data_ptr<int8_t>();
+    const void *w = address(a[1], "weight");
+    const float *w_scale = address_as<float>(a[3], "w_scale"), *x_scale = address_as<float>(a[4], "x_scale");
+    const float *bias = address_as<float>(a[5], "bias"), *out_scale = address_as<float>(a[8], "out_scale");
+    int32_t *status = address_as<int32_t>(a[10], "status_buf");
     Out Y(a[9], Xq, type, {M, N}, "Y");
-    check(Fn(Xq.const_data_ptr<int8_t>(), address(a[1], "weight"), address_as<float>(a[3], "w_scale"), address_as<float>(a[4], "x_scale"),
-             address_as<float>(a[5], "bias"), act, out_type, address_as<float>(a[8], "out_scale"), Y.p, M, N, as_int(K),
-             address_as<int32_t>(a[10], "status_buf"), stream()), where);
+    run(where, [&](void *s) { return Fn(x, w, w_scale, x_scale, bias, act, out_type, out_scale, Y.p(), m, N, k, status, s); }, Y);
     return Y.take();
 }
 int dense(const int8_t *Xq, const void *Wq, const float *ws, const float *xs, const float *bias, int act, int out_type,
@@ -316,11 +388,16 @@ PyObject *spgemm_i8_absmax(PyObject *const *a)
 {
     const at::Tensor &Xq = IN_I8(a[0], "Xq");
     const auto [M, K] = matrix(Xq, "Xq");
-    const int N = int_arg(a[2]), act = int_arg(a[6]);
+    const int64_t m = M;
+    const int N = int_arg(a[2]), k = as_int(K), act = int_arg(a[6]);
+    const int8_t *x = Xq.const_data_ptr<int8_t>();
+    const void *w = address(a[1], "Wpacked");
+    const float *w_scale = address_as<float>(a[3], "w_scale"), *x_scale = address_as<float>(a[4], "x_scale"), *bias = address_as<float>(a[5], "bias");
+    int32_t *status = address_as<int32_t>(a[9], "status_buf");
     Out Y(a[7], Xq, at::kHalf, {M, N}, "Y"), y_absmax(a[8], Xq, at::kFloat, {1}, "y_absmax");
-    check(gpusq_spgemm_i8_absmax(Xq.const_data_ptr<int8_t>(), address(a[1], "Wpacked"), address_as<float>(a[3], "w_scale"),
-                                 address_as<float>(a[4], "x_scale"), address_as<float>(a[5], "bias"), act, Y.p, y_absmax.as<float>(), M, N,
-                                 as_int(K), address_as<int32_t>(a[9], "status_buf"), stream()), "gpusq_spgemm_i8_absmax");
+    run("gpusq_spgemm_i8_absmax", [&](void *s) {
+        return gpusq_spgemm_i8_absmax(x, w, w_scale, x_scale, bias, act, Y.p(), y_absmax.as<float>(), m, N, k, status, s);
+    }, Y, y_absmax);
     return pair(Y, y_absmax);
 }
 
@@ -329,10 +406,13 @@ PyObject *spgemm_f16(PyObject *const *a)
 {
     const at::Tensor &X = IN_F16(a[0], "X");
     const auto [M, K] = matrix(X, "X");
-    const int N = int_arg(a[2]), act = int_arg(a[4]), out_type = int_arg(a[5]);
+    const int64_t m = M;
+    const int N = int_arg(a[2]), k = as_int(K), act = int_arg(a[4]), out_type = int_arg(a[5]);
+    const void *x = X.const_data_ptr(), *w = address(a[1], "Wpacked");
+    const float *bias = address_as<float>(a[3], "bias");
+    int32_t *status = address_as<int32_t>(a[7], "status_buf");
     Out Y(a[6], X, out_type == GPUSQ_OUT_F16 ? at::kHalf : at::kFloat, {M, N}, "Y");
-    check(gpusq_spgemm_f16(X.const_data_ptr(), address(a[1], "Wpacked"), address_as<float>(a[3], "bias"), act, out_type, Y.p, M, N, as_int(K),
-                           address_as<int32_t>(a[7], "status_buf"), stream()), "gpusq_spgemm_f16");
+    run("gpusq_spgemm_f16", [&](void *s) { return gpusq_spgemm_f16(x, w, bias, act, out_type, Y.p(), m, N, k, status, s); }, Y);
     return Y.take();
 }
 

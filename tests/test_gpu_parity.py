@@ -2,6 +2,9 @@
 through the C-ABI (ctypes binding), on seeded inputs that span several tiles
 and ragged tails.  Integer stages must be bit-exact; the FP16 epilogue must be
 within 1 binary16 ulp of the oracle's FP32 epilogue rounded to binary16."""
+import threading
+import time
+
 import numpy as np
 import pytest
 
@@ -620,6 +623,38 @@ def test_non_default_stream(B):
         Y = B.spgemm_i8(cu(Xq), Wpk, 128, out_type=B.OUT_I32)
     s.synchronize()
     assert np.array_equal(Y.cpu().numpy(), acc_o)
+
+
+def test_other_threads_run_while_a_call_waits(B):
+    # A stream whose launch queue is full makes the next launch wait on the host.  Other Python threads go on.
+    X = torch.zeros((256, 256), dtype=torch.float16, device="cuda")
+    Xq, s = B.quant_act(X)
+    ws = torch.zeros((B.quant_act_workspace(*X.shape),), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    gaps, stop = [], threading.Event()
+
+    def tick():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(1e-3)
+            now = time.perf_counter()
+            gaps.append(now - last)
+            last = now
+
+    other = threading.Thread(target=tick)
+    other.start()
+    try:
+        torch.cuda._sleep(2_000_000_000)                    # about a second; ends by itself
+        t0 = time.perf_counter()
+        for _ in range(5000):                               # more than a launch queue holds
+            B.quant_act(X, Xq, s, workspace=ws)
+        issued = time.perf_counter() - t0
+    finally:
+        stop.set()
+        other.join()
+        torch.cuda.synchronize()
+    assert issued > 0.5                                     # the calls did wait
+    assert max(gaps) < 0.25, max(gaps)
 
 
 def _random_gemm_cases(n, seed):
