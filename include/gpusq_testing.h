@@ -13,6 +13,8 @@
 #ifndef GPUSQ_TESTING_H
 #define GPUSQ_TESTING_H
 
+#include <stdint.h>
+
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -24,6 +26,11 @@ int gpusq_set_block_tokens(int block_t);
 /* Mixed heights: the first n_big token tiles block_t tokens high (block_t a
  * multiple of 32 in [64, 224]), the rest block_t - 32, as many as cover M. */
 int gpusq_set_tile_mix(int block_t, int n_big);
+
+/* How the 2:4 GEMM (half != 0: the FP16 model's) would cut its token axis on
+ * `clusters` CTA pairs, without a GPU: plan = {tokens per tile, token runs of
+ * that height, token runs in all (0: twin tiles only), token tiles per run}. */
+int gpusq_tile_plan(int64_t M, int N, int K, int half, int out_type, int clusters, int plan[4]);
 
 /* Bound of the device-side waits of gpusq_quant_act's one-launch kernel, in
  * nanoseconds (default 2 s), and, with withhold_last_cta != 0, a planted

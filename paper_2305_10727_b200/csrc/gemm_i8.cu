@@ -858,8 +858,10 @@ static double run_cost(double kb, int64_t h, int tiles)
 
 // Time until the last cluster is done when cluster c works on runs c, c + clusters, ...: the pair runs
 // (token run major, pair_cols feature columns each) first, then the twin tiles of a last narrow feature
-// column (two token tiles of block_t each, the k blocks taken twice).
-static double makespan(const TilePlan &t, int64_t M, int pair_cols, bool twin_col, int clusters, double kb)
+// column (two token tiles of block_t each, the k blocks taken twice).  Of the runs below a count n, cluster c has
+// n / clusters, and one more while c < n % clusters: the time changes with c only at the remainders of the four
+// counts, so it is looked at there.  `bound`: a plan whose mean time reaches it may be given any time that does.
+static double makespan(const TilePlan &t, int64_t M, int pair_cols, bool twin_col, int clusters, double kb, double bound)
 {
     const int h_low = t.block_t - 32;
     const double big_cost = run_cost(kb, t.block_t, t.run_tiles);
@@ -874,16 +876,28 @@ static double makespan(const TilePlan &t, int64_t M, int pair_cols, bool twin_co
         last_cost = t.run_tiles == 1 ? tile_cost(kb, left) : (double)left / (double)((int64_t)h * t.run_tiles) * (low ? low_cost : big_cost);
     }
     const int64_t pair_runs = (int64_t)t.runs * pair_cols, big = (int64_t)t.n_big * pair_cols;
-    const int64_t twins = twin_col ? ceil_div(M, 2 * (int64_t)t.block_t) : 0;
-    const double twin_cost = twin_col ? tile_cost(2.0 * kb, t.block_t) : 0.0;
+    const int64_t full = pair_runs - pair_cols > 0 ? pair_runs - pair_cols : 0;
+    // runs up to the last full-height one, the last full one, the last pair run, the last twin tile; time of each kind
+    const int64_t n[4] = {big < full ? big : full, full, pair_runs, pair_runs + (twin_col ? ceil_div(M, 2 * (int64_t)t.block_t) : 0)};
+    const double cost[4] = {big_cost, low_cost, last_cost, twin_col ? tile_cost(2.0 * kb, t.block_t) : 0.0};
+    auto load = [&](const int64_t (&m)[4]) {
+        return (double)m[0] * cost[0] + (double)(m[1] - m[0]) * cost[1] + (double)(m[2] - m[1]) * cost[2] + (double)(m[3] - m[2]) * cost[3];
+    };
+    const double mean = load(n) / clusters;
+    if (mean * (1.0 - 1e-9) > bound) return mean;
+    int64_t each[4];
+    int more[4];
+    for (int i = 0; i < 4; ++i) {
+        each[i] = n[i] / clusters;
+        more[i] = (int)(n[i] - each[i] * clusters);
+    }
     double worst = 0.0;
-    for (int c = 0; c < clusters; ++c) {
-        // how many of the first n runs are cluster c's
-        auto of = [&](int64_t n) { return n > c ? (n - c - 1) / clusters + 1 : (int64_t)0; };
-        const int64_t mine = of(pair_runs), full = of(pair_runs - pair_cols), full_big = of(big < pair_runs - pair_cols ? big : pair_runs - pair_cols);
-        const double load = (double)full_big * big_cost + (double)(full - full_big) * low_cost +
-                            (double)(mine - full) * last_cost + (double)(of(pair_runs + twins) - mine) * twin_cost;
-        worst = load > worst ? load : worst;
+    for (int i = -1; i < 4; ++i) {
+        const int c = i < 0 ? 0 : more[i];
+        int64_t mine[4];
+        for (int j = 0; j < 4; ++j) mine[j] = each[j] + (c < more[j] ? 1 : 0);
+        const double l = load(mine);
+        worst = l > worst ? l : worst;
     }
     return worst;
 }
@@ -926,7 +940,7 @@ static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters
     TilePlan best = {kMaxBlockT, 0, 0, 1};
     double best_cost = 1e300;
     auto consider = [&](const TilePlan &t) {
-        const double c = makespan(t, M, pair_cols, twin_col, clusters, kb);
+        const double c = makespan(t, M, pair_cols, twin_col, clusters, kb, best_cost);
         if (c < best_cost * 0.999) {
             best_cost = c;
             best = t;
@@ -1310,6 +1324,23 @@ int gpusq_gemm_i8_dense(const int8_t *Xq, const int8_t *Wq, const float *w_scale
 {
     return launch_gemm<false>(Xq, Wq, w_scale, x_scale, bias, act, out_type, out_scale, Y, M, N, K, status_buf,
                               stream);
+}
+
+int gpusq_tile_plan(int64_t M, int N, int K, int half, int out_type, int clusters, int plan[4])
+{
+    if (!plan) return GPUSQ_ERR_NULL;
+    if (M <= 0 || M > 0x7FFFFFFF || N <= 0 || K <= 0 || clusters <= 0) return GPUSQ_ERR_SHAPE;
+    GemmParams p = {};
+    p.M = M;
+    p.N = N;
+    p.K = K;
+    p.out_type = out_type;
+    if (!(half ? set_tiling<Cfg<true, true>>(p, 2 * K, clusters) : set_tiling<Cfg<true>>(p, K, clusters))) return GPUSQ_ERR_SHAPE;
+    plan[0] = p.block_t;
+    plan[1] = p.n_big;
+    plan[2] = p.pair_cols > 0 ? p.pair_runs / p.pair_cols : 0;
+    plan[3] = p.run_tiles;
+    return GPUSQ_OK;
 }
 
 int gpusq_set_block_tokens(int block_t)
