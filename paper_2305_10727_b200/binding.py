@@ -103,11 +103,14 @@ _native = None
 
 
 def _n():
-    """The native part of this binding; raises if it or libgpusq.so is missing."""
+    """The native part of this binding; raises if it or libgpusq.so is missing, or built for another torch or Python."""
     global _native
     if _native is None:
         load()
-        from . import _gpusq_torch
+        from . import _gpusq_torch, build
+        if _gpusq_torch.built_for != build.built_for():
+            raise RuntimeError("_gpusq_torch.so was built for %s, this is %s: build it with `python -m paper_2305_10727_b200.build`"
+                               % (_gpusq_torch.built_for, build.built_for()))
         _gpusq_torch.set_errors(GpusqError, torch.OutOfMemoryError)
         _native = _gpusq_torch
     return _native

@@ -28,9 +28,19 @@ def _deps():
     return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
 
 
+def built_for() -> str:
+    """What the native part of the binding depends on, written into it: another torch or Python needs another build."""
+    import torch
+
+    return "torch %s, Python %d.%d" % (torch.__version__, *sys.version_info[:2])
+
+
 def _binding_is_stale() -> bool:
     deps = [os.path.join(CSRC, "torch_binding.cpp"), os.path.join(ROOT, "include", "gpusq.h")]
-    return not os.path.exists(BINDING) or any(os.path.getmtime(f) > os.path.getmtime(BINDING) for f in deps)
+    if not os.path.exists(BINDING) or any(os.path.getmtime(f) > os.path.getmtime(BINDING) for f in deps):
+        return True
+    with open(BINDING, "rb") as f:
+        return built_for().encode() not in f.read()
 
 
 def build_binding(force: bool = False) -> str:
@@ -43,7 +53,7 @@ def build_binding(force: bool = False) -> str:
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = BINDING + ".%d.tmp" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DGPUSQ_BUILT_FOR="%s"' % built_for(),
            "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(t, "include"),
            "-I" + os.path.join(t, "include", "torch", "csrc", "api", "include"),
            "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(cuda, "include"),

@@ -446,4 +446,10 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_gpusq_torch", nullptr, -1, g_me
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__gpusq_torch() { return PyModule_Create(&g_module); }
+// built_for: the torch and the Python this module was compiled against (build.py)
+PyMODINIT_FUNC PyInit__gpusq_torch()
+{
+    PyObject *m = PyModule_Create(&g_module);
+    if (m && PyModule_AddStringConstant(m, "built_for", GPUSQ_BUILT_FOR) < 0) Py_CLEAR(m);
+    return m;
+}

@@ -135,3 +135,14 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         B.load()
+
+
+def test_native_binding_of_another_torch_is_rebuilt_and_refused(lib, monkeypatch):
+    import torch
+    assert not lib_build._binding_is_stale()
+    assert B._n().built_for == lib_build.built_for()
+    monkeypatch.setattr(B, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert lib_build._binding_is_stale()
+    with pytest.raises(RuntimeError, match="built for"):
+        B._n()
