@@ -218,9 +218,11 @@ int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mod
  *   x_scale device float[1];  bias [N] f32 nullable;  out_scale device
  *   float[1], GPUSQ_OUT_I8 only;  Y [M, N] out.
  *   status_buf: device int32[4], nullable.  If given it must be zero on entry;
- *     a kernel whose bounded wait expires writes {GPUSQ_ERR_TIMEOUT, tile,
+ *     a kernel whose bounded wait expires writes {GPUSQ_ERR_TIMEOUT, run,
  *     role, stage} there and stops issuing work (the output is then
- *     undefined).  The host call itself never waits for the device.
+ *     undefined).  A run is a tile, or the consecutive token tiles that one CTA
+ *     pair works on with the same weights.  The host call itself never waits
+ *     for the device.
  * Requires M > 0, K % 16 == 0, Xq / Wpacked / Y 16-byte aligned, and a row of
  * Y that is a multiple of 16 bytes: N % 8 == 0 for GPUSQ_OUT_F16, N % 16 == 0
  * for GPUSQ_OUT_I8 (any N for GPUSQ_OUT_I32).  N need not be a multiple of

@@ -27,6 +27,11 @@ int gpusq_set_block_tokens(int block_t);
  * multiple of 32 in [64, 224]), the rest block_t - 32, as many as cover M. */
 int gpusq_set_tile_mix(int block_t, int n_big);
 
+/* The same in token runs of run_tiles tiles (1 to 64), whose weights stay in
+ * shared memory, also where a launch is too small for that to pay; launches
+ * that cannot keep their weights ignore run_tiles. */
+int gpusq_set_tile_runs(int block_t, int n_big, int run_tiles);
+
 /* How the 2:4 GEMM (half != 0: the FP16 model's) would cut its token axis on
  * `clusters` CTA pairs, without a GPU: plan = {tokens per tile, token runs of
  * that height, token runs in all (0: twin tiles only), token tiles per run}. */
@@ -52,13 +57,13 @@ int gpusq_set_quant_act_late(int first, int count, unsigned ns);
 int gpusq_quant_act_shares_taken(unsigned *shares);
 
 /* As gpusq_set_quant_act_wait, for the GEMM kernels: bound of every device-side
- * wait in microseconds
- * (default 2 s) and, with withhold_loads != 0, a planted failure in an allowed
- * form: the producers of the first CTA pair stop before the last k block of
- * their first tile, so the MMA issuer's bounded wait for that block runs out;
- * it raises the pair's abort flag, writes {GPUSQ_ERR_TIMEOUT, tile, role,
- * stage} to status_buf, every role of the pair leaves its loop, and the kernel
- * returns.  The other pairs finish their tiles.  Nothing faults or hangs. */
+ * wait in microseconds (default 2 s) and, with withhold_loads != 0, a planted
+ * failure in an allowed form: the producers of the first CTA pair stop before
+ * the last k block of their first token run (of its last tile, where a run has
+ * several), so the MMA issuer's bounded wait for that block runs out; it raises
+ * the pair's abort flag, writes {GPUSQ_ERR_TIMEOUT, run, role, stage} to
+ * status_buf, every role of the pair leaves its loop, and the kernel returns.
+ * The other pairs finish their tiles.  Nothing faults or hangs. */
 int gpusq_set_gemm_wait(unsigned limit_us, int withhold_loads);
 
 /* Measurement hook: the GEMM launches use at most `clusters` CTA pairs (0 = as

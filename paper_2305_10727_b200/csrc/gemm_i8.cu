@@ -126,7 +126,7 @@ struct GemmParams {
     int twin_n0;    // first feature of the twin column (256 pair_cols)
     int oob_row;    // a row coordinate beyond the weight tensor: loads from there fill with zeros
     uint32_t wait_us;   // limit of every device-side wait, microseconds
-    int withhold;       // test hook: the first cluster's producers stop before the last k block of their first tile
+    int withhold;       // test hook: the first cluster's producers stop before the last k block of their first run
 };
 
 // Where the work sits.  It is cut into runs: run_tiles consecutive token tiles (fewer at the end) of one
@@ -196,14 +196,14 @@ struct RunWalk {
 };
 
 // A wait of this CTA expired: raise the abort flag in both CTAs of the pair and record where.
-__device__ __forceinline__ void report_timeout(const GemmParams &p, Ctl *ctl, int tile, int role, int stage)
+__device__ __forceinline__ void report_timeout(const GemmParams &p, Ctl *ctl, int run, int role, int stage)
 {
     const uint32_t flag = ptx::smem_u32(&ctl->abort_flag);
     const bool first = atomicExch(&ctl->abort_flag, 1u) == 0u;
     ptx::st_cluster_u32(ptx::map_to_cta(flag, ptx::cluster_ctarank() ^ 1u), 1u);
     if (first && p.status) {
         if (atomicCAS(p.status, 0, GPUSQ_ERR_TIMEOUT) == 0) {
-            p.status[1] = tile;
+            p.status[1] = run;
             p.status[2] = role;
             p.status[3] = stage;
         }
@@ -827,9 +827,11 @@ static bool make_map_u8(CUtensorMap *map, const void *base, uint64_t rows, uint6
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// testing hooks (gpusq_testing.h): a forced tile height, and a forced number of full-height token tiles
+// testing hooks (gpusq_testing.h): a forced tile height, a forced number of full-height token runs, and the tiles of
+// such a run
 static std::atomic<int> g_block_t_override{0};
 static std::atomic<int> g_n_big_override{-1};
+static std::atomic<int> g_run_tiles_override{1};
 static std::atomic<unsigned> g_wait_us{ptx::kDefaultWaitUs};
 static std::atomic<int> g_withhold_loads{0};
 static std::atomic<int> g_cluster_cap{0};           // CTA pairs a launch may use (0 = as many as fit)
@@ -915,10 +917,11 @@ static TilePlan plan_tiles(int64_t M, int pair_cols, bool twin_col, int clusters
     const int forced = g_block_t_override.load(std::memory_order_relaxed);
     const int forced_big = g_n_big_override.load(std::memory_order_relaxed);
     if (forced && forced_big >= 0 && forced >= 64 && pair_cols > 0) {
-        // as many full-height tiles as asked for (at most what covers M), lower ones for the rest
-        const int64_t nb = forced_big < ceil_div(M, forced) ? forced_big : ceil_div(M, forced);
-        const int64_t rest = M - nb * forced;
-        return {forced, (int)nb, (int)(nb + (rest > 0 ? ceil_div(rest, forced - 32) : 0)), 1};
+        // as many full-height runs as asked for (at most what covers M), lower ones for the rest
+        const int R = may_stay ? g_run_tiles_override.load(std::memory_order_relaxed) : 1;
+        const int64_t most = ceil_div(M, (int64_t)forced * R), nb = forced_big < most ? forced_big : most;
+        const int64_t rest = M - nb * forced * R;
+        return {forced, (int)nb, (int)(nb + (rest > 0 ? ceil_div(rest, (int64_t)(forced - 32) * R) : 0)), R};
     }
     struct Entry {
         int64_t M;
@@ -996,7 +999,8 @@ static bool set_tiling(GemmParams &p, int K_cost, int clusters)
     const int stages = kb <= kMaxWeightBlocks ? (C::kRoom - kb * C::kWBytes) / C::kBBytes : 0;
     // With fewer than three waves of tiles there is nothing to keep them for.
     const bool may_stay = C::kMayStay && p.out_type != GPUSQ_OUT_I32 && !twin_col && !wide && stages >= C::kMinResidentStages &&
-                          ceil_div(p.M, kMaxBlockT) * p.pair_cols >= 3 * (int64_t)clusters;
+                          (ceil_div(p.M, kMaxBlockT) * p.pair_cols >= 3 * (int64_t)clusters ||
+                           g_run_tiles_override.load(std::memory_order_relaxed) > 1);
     TilePlan t;
     if (p.pair_cols == 0) {
         // twin tiles only: each cluster takes two token tiles and the k blocks twice
@@ -1348,6 +1352,7 @@ int gpusq_set_block_tokens(int block_t)
     if (block_t != 0 && (block_t < 32 || block_t > kMaxBlockT || block_t % 32)) return GPUSQ_ERR_ARG;
     g_block_t_override.store(block_t, std::memory_order_relaxed);
     g_n_big_override.store(-1, std::memory_order_relaxed);
+    g_run_tiles_override.store(1, std::memory_order_relaxed);
     return GPUSQ_OK;
 }
 
@@ -1368,9 +1373,15 @@ int gpusq_set_max_clusters(int clusters)
 
 int gpusq_set_tile_mix(int block_t, int n_big)
 {
-    if (block_t < 64 || block_t > kMaxBlockT || block_t % 32 || n_big < 0) return GPUSQ_ERR_ARG;
+    return gpusq_set_tile_runs(block_t, n_big, 1);
+}
+
+int gpusq_set_tile_runs(int block_t, int n_big, int run_tiles)
+{
+    if (block_t < 64 || block_t > kMaxBlockT || block_t % 32 || n_big < 0 || run_tiles < 1 || run_tiles > 64) return GPUSQ_ERR_ARG;
     g_block_t_override.store(block_t, std::memory_order_relaxed);
     g_n_big_override.store(n_big, std::memory_order_relaxed);
+    g_run_tiles_override.store(run_tiles, std::memory_order_relaxed);
     return GPUSQ_OK;
 }
 

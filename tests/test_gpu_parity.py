@@ -410,6 +410,41 @@ def test_gemm_wait_that_runs_out_is_reported(B):
     assert np.array_equal(Y.cpu().numpy(), acc_o)
 
 
+# The same for the epilogue that writes FP16 or INT8, with weights by the tile and weights that stay (status: run 0).
+@pytest.mark.parametrize("out", ["f16", "i8", "absmax"])
+@pytest.mark.parametrize("tiling", [None, (96, 2, 3)])
+def test_gemm_wait_that_runs_out_with_each_output(B, out, tiling):
+    M, N, K = 1576, 768, 192
+    d, prep, Xq, xs = _prep(124, M, N, K)
+    args = (cu(Xq), B.pack24(cu(prep["vals"]), cu(prep["meta"])), N, cu(prep["w_scale"]), cu(np.array([xs], np.float32)), cu(d["bias"]))
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+
+    def layer():
+        if out == "absmax":
+            return B.spgemm_i8_absmax(*args, act=1, status_buf=status)[0]
+        return B.spgemm_i8(*args, act=1, out_type=B.OUT_I8 if out == "i8" else B.OUT_F16,
+                           out_scale=cu(np.array([0.02], np.float32)), status_buf=status)
+
+    want = layer()
+    assert status.cpu().tolist() == [0, 0, 0, 0]
+    if tiling:
+        B.set_tile_runs(*tiling)
+    B.set_gemm_wait(5000, withhold_loads=True)
+    try:
+        layer()
+        torch.cuda.synchronize()
+        st = status.cpu().tolist()
+        # the MMA issuer waits for the block, the epilogue for the tile it belongs to: either may be the first to give up
+        assert st[0] == 7 and st[1] == 0 and st[2] in (1, 2), st
+        B.set_gemm_wait(2_000_000, withhold_loads=False)
+        status.zero_()
+        assert torch.equal(layer(), want)
+    finally:
+        B.set_gemm_wait(2_000_000, withhold_loads=False)
+        B.set_block_tokens(0)
+    assert status.cpu().tolist() == [0, 0, 0, 0]
+
+
 def test_spgemm_extreme_codes_do_not_overflow(B):
     # every kept code and every activation at +-127, K = 5120: |acc| = 127^2 * K / 2
     M, N, K = 40, 128, 5120
@@ -492,6 +527,8 @@ def test_weights_that_stay(B, M, N, K, clusters, block_t):
     B.set_block_tokens(block_t)
     B.set_max_clusters(clusters)
     try:
+        # thirteen k blocks are the most that stay; tiles of 64 tokens with one k block are cheaper streamed
+        assert (B.tile_plan(M, N, K, clusters=clusters)[3] > 1) == (K <= 1664 and (K, block_t) != (64, 64))
         for act in (0, 1):
             Y_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=act, out_type=0)
             out_scale = np.float32(np.abs(Y_o.astype(np.float32)).max() / 127.0)
@@ -509,6 +546,44 @@ def test_weights_that_stay(B, M, N, K, clusters, block_t):
         B.set_max_clusters(0)
     assert status.cpu().tolist() == [0, 0, 0, 0]
     assert (buf[:2048] == 77).all() and (buf[2048 + M * N:] == 77).all()
+
+
+# Runs of several tiles whose heights differ from run to run, as large launches mix them.  K of fewer, as many and more k
+# blocks than the pipeline has activation stages (eight up to K = 1024, seven at 1152, five at 1664), a last one that is
+# not whole; full-height runs first, in the middle of a pair's, none; a last run of fewer tiles and a last tile of fewer tokens.
+@pytest.mark.parametrize("M,N,K,clusters", [(1501, 512, 48, 3), (1237, 400, 896, 2), (1501, 512, 1024, 3), (1777, 256, 1152, 2), (1300, 512, 1664, 2)])
+@pytest.mark.parametrize("block_t,n_big,run_tiles", [(224, 1, 2), (96, 3, 3), (64, 0, 4), (160, 1, 5), (192, 2, 2)])
+def test_weights_that_stay_with_mixed_heights(B, M, N, K, clusters, block_t, n_big, run_tiles):
+    d, prep, Xq, xs = _prep(M + K + block_t, M, N, K)
+    acc_o = oracle.spgemm_acc(Xq, prep["vals"], prep["meta"], threads=oracle.host_cores())
+    Wp, sc, x1, bi = B.pack24(cu(prep["vals"]), cu(prep["meta"])), cu(prep["w_scale"]), cu(np.array([xs], np.float32)), cu(d["bias"])
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    buf = torch.full((M * N + 4096,), 77, dtype=torch.float16, device="cuda")
+    buf8 = torch.full((M * N + 4096,), 77, dtype=torch.int8, device="cuda")
+    Y, Q = buf[2048:2048 + M * N].view(M, N), buf8[2048:2048 + M * N].view(M, N)
+    B.set_tile_runs(block_t, n_big, run_tiles)
+    B.set_max_clusters(clusters)
+    try:
+        plan = B.tile_plan(M, N, K, clusters=clusters)
+        assert plan[0] == block_t and plan[1] == n_big < plan[2] and plan[3] == run_tiles
+        for act in (0, 1):
+            Y_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=act, out_type=0, threads=oracle.host_cores())
+            out_scale = np.float32(np.abs(Y_o.astype(np.float32)).max() / 127.0)
+            Q_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=act, out_type=1, out_scale=out_scale)
+            B.spgemm_i8(cu(Xq), Wp, N, sc, x1, bi, act=act, out_type=B.OUT_F16, Y=Y.fill_(0), status_buf=status)
+            assert f16_ulp_distance(Y.cpu().numpy(), Y_o).max() <= (F16_ULP_TOL if act else 0)
+            B.spgemm_i8(cu(Xq), Wp, N, sc, x1, bi, act=act, out_type=B.OUT_I8, out_scale=cu(np.array([out_scale], np.float32)),
+                        Y=Q.fill_(0), status_buf=status)
+            # codes of a fixed IEEE sequence; with GELU one step at most, where the approximation meets a tie
+            assert np.abs(Q.cpu().numpy().astype(np.int32) - Q_o).max() <= act
+            Ya, amax = B.spgemm_i8_absmax(cu(Xq), Wp, N, sc, x1, bi, act=act, status_buf=status)
+            assert torch.equal(Ya, Y) and amax.item() == Y.float().abs().max().item()
+    finally:
+        B.set_block_tokens(0)
+        B.set_max_clusters(0)
+    assert status.cpu().tolist() == [0, 0, 0, 0]
+    for b in (buf, buf8):
+        assert (b[:2048] == 77).all() and (b[2048 + M * N:] == 77).all()
 
 
 @pytest.mark.parametrize("M,N,K,block_t", [(514, 256, 1280, 0), (197, 128, 192, 0), (1000, 384, 256, 96),
