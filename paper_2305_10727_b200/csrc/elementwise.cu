@@ -1,7 +1,8 @@
-// HBM-bound operand-preparation kernels of libgpusq: 2:4 pruning, weight and
-// activation quantisation, compression to values + metadata, decompression and
-// packing for the tensor-core kernel.  One pass of coalesced 16-byte accesses
-// per tensor; no shared-memory staging is needed (no reuse across threads).
+// Operand-preparation kernels of libgpusq: 2:4 pruning, weight and activation
+// quantisation, compression to values + metadata, decompression and packing for
+// the tensor-core kernel.  One pass of coalesced 16-byte accesses per tensor,
+// without staging, except for activations whose scale is computed from them:
+// they stay in registers or shared memory between the two looks at them.
 #include <cuda_fp16.h>
 
 #include <atomic>
@@ -1166,10 +1167,11 @@ static int max_quant_cluster()
     if (k) return k - 1;
     int best = 0;
     const void *kernels[] = {(const void *)act_quant_cluster_kernel<1>, (const void *)act_quant_cluster_kernel<2>,
-                             (const void *)act_quant_cluster_kernel<4>, (const void *)act_quant_cluster_kernel<kClusterMaxPerThread>};
+                             (const void *)act_quant_cluster_kernel<kClusterMaxPerThread>};
     bool opted = true;
     for (const void *f : kernels)
         opted = opted && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    bool failed = !opted;
     for (int size = opted ? kMaxCluster : 8; size >= 8 && !best; size /= 2) {
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1181,9 +1183,10 @@ static int max_quant_cluster()
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernels[3], &cfg) == cudaSuccess && n > 0) best = size;
+        if (cudaOccupancyMaxActiveClusters(&n, kernels[2], &cfg) != cudaSuccess) failed = true;
+        else if (n > 0) best = size;
     }
-    (void)cudaGetLastError();
+    if (failed) (void)cudaGetLastError();                     // this function's own; an earlier one is not ours to clear
     known[dev].store(best + 1, std::memory_order_relaxed);
     return best;
 }
@@ -1237,8 +1240,7 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
         const int cluster_max = max_quant_cluster();
         if (cluster_max > 0 && vec8 <= (int64_t)cluster_max * kClusterThreads * kClusterMaxPerThread)
             return launch_cluster_quant(X, Xq, x_scale, (int)vec8, cluster_max, qmax, regroup, s);
-        // The opt-in to
-        // large dynamic shared memory is per device.
+        // the opt-in to large dynamic shared memory is per device
         static std::mutex mu;
         static uint8_t attr_state[kMaxDevices] = {};          // 1 = set, 2 = failed
         int dev = 0;

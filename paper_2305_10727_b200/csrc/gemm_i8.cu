@@ -844,8 +844,10 @@ struct TilePlan {
 
 // Relative time of one tile of h tokens over kb 128-wide k blocks.  Per tile and CTA the shared memory
 // moves, per k block, 128 bytes per token (activations written and read) plus a fixed ~20 KB for the
-// weight block (as much as 160 tokens), and the epilogue's staging costs as much as four k blocks per
-// token: time per tile ~ (kb + 4) * h + 160 * kb.
+// weight block (as much as 160 tokens); what a tile costs beside its k blocks is put at four of them per
+// token: time per tile ~ (kb + 4) * h + 160 * kb.  The four was fitted to an earlier epilogue with FP16
+// output; the present one takes 4 to 9 % less of a launch, more with GELU or INT8 output, which the
+// estimate does not tell apart.
 static double tile_cost(double kb, int64_t h) { return (kb + 4.0) * (double)h + 160.0 * kb; }
 
 // The same for a run of `tiles` tiles whose weights stay: a tile is 8 % shorter, and a change of run,
