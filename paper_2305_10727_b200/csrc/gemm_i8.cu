@@ -58,7 +58,14 @@ constexpr int kTmemCols = 512;
 constexpr int kAccStride = kMaxBlockT;      // column of the second accumulator
 constexpr int kMetaCol = 2 * kMaxBlockT;    // metadata: 4 columns per weight block from here
 constexpr int kMaxWeightBlocks = (kTmemCols - kMetaCol) / 4;
-constexpr int kMaxStages = 8;
+// Stages of the operand ring: as many as fit, eight for tiles of 224 tokens, sixteen for 32.  A load out of L2 takes
+// some 1400 cycles, so eight stages cannot bring in a k block more often than every 175.
+constexpr int kMaxStages = 16;
+// k blocks per iteration of the two single-thread loops (loads, MMAs).  A k block costs the slower of the two 140
+// cycles, and coming back to the start of the loop another 110, whatever the tile's height: few tokens and long K
+// were bound by that.  Per k block of 256 features x 32 tokens: 264 cycles not unrolled, 199 by two, 165 by four,
+// 170 by eight.
+constexpr int kUnrollK = 4;
 constexpr int kMaxSmem = 232448;            // dynamic shared memory that a CTA may have
 constexpr int kEpiBufBytes = kChunkT * 64;            // [16 tokens][32 features] f16 (INT8 output uses half of it)
 constexpr int kEpiBytes = kEpiWarps * 2 * kEpiBufBytes;     // two buffers per epilogue warp
@@ -71,7 +78,8 @@ struct Cfg {
     static_assert(kSparse || !kHalf, "the FP16 model exists only in the 2:4 sparse form");
     static constexpr int kABytes = kHalf ? kBlockF * 128 : kSparse ? kBlockF * 64 : kBlockF * 128;
     static constexpr int kBAtoms = kHalf ? 2 : 1;                // 128-byte-wide activation tiles per stage
-    static constexpr int kBBytes = kBAtoms * (kMaxBlockT / 2) * 128;   // this CTA's half of the token rows
+    // activation bytes of a stage: this CTA's half of the rows of a tile of block_t tokens
+    static __host__ __device__ constexpr int b_bytes(int block_t) { return kBAtoms * (block_t / 2) * 128; }
     static constexpr int kMetaBytes = kSparse ? 2048 : 0;
     static constexpr int kCtlBytes = 1024;
     // Shared memory for operands: weight blocks (values and metadata of 128 features x one k block) and
@@ -79,7 +87,9 @@ struct Cfg {
     // feature column stay for a run of tiles and the rest of the room holds activation stages.
     static constexpr int kWBytes = kABytes + kMetaBytes;
     static constexpr int kRoom = kMaxSmem - kEpiBytes - kCtlBytes - 2048 /* alignment slack */;
-    static constexpr int kStreamStages = kRoom / (kWBytes + kBBytes) < kMaxStages ? kRoom / (kWBytes + kBBytes) : kMaxStages;
+    static __host__ constexpr int most(int stages) { return stages < kMaxStages ? stages : kMaxStages; }
+    static __host__ constexpr int stream_stages(int block_t) { return most(kRoom / (kWBytes + b_bytes(block_t))); }
+    static __host__ constexpr int resident_stages(int block_t, int k_blocks) { return most((kRoom - k_blocks * kWBytes) / b_bytes(block_t)); }
     static constexpr bool kMayStay = kSparse && !kHalf;     // instantiations with resident weights exist
     static constexpr int kMinResidentStages = 5;
     static constexpr int kMmasPerStage = kHalf ? 4 : kSparse ? 2 : 4;
@@ -87,8 +97,8 @@ struct Cfg {
     static constexpr int kBStepBytes = kHalf ? 64 : kSparse ? 64 : 32;
     static constexpr int kASwizzle = kHalf ? 128 : kSparse ? 64 : 128;
     static constexpr int kMetaColsPerMma = kHalf ? 1 : 2;     // 32-bit tensor-memory columns of metadata per MMA
-    static_assert(kABytes % 1024 == 0 && kMetaBytes % 1024 == 0 && kBBytes % 1024 == 0, "alignment of the swizzled tiles");
-    static_assert(kStreamStages <= kMaxWeightBlocks, "metadata columns");
+    static_assert(kABytes % 1024 == 0 && kMetaBytes % 1024 == 0 && b_bytes(32) % 1024 == 0, "alignment of the swizzled tiles");
+    static_assert(kMaxStages <= kMaxWeightBlocks, "metadata columns");
 };
 
 struct Ctl {
@@ -121,8 +131,8 @@ struct GemmParams {
     int pair_cols;  // feature columns of 256 that are worked on as ordinary pair tiles
     int pair_runs;  // pair_cols x token runs: runs from here on are twin tiles of the last 128 features
     int num_runs;
-    int stages;     // kRuns: activation stages
-    int w_blocks;   // kRuns: weight blocks in shared memory, one per k block
+    int stages;     // activation stages
+    int w_blocks;   // weight blocks in shared memory: one per stage; kRuns: one per k block
     int twin_n0;    // first feature of the twin column (256 pair_cols)
     int oob_row;    // a row coordinate beyond the weight tensor: loads from there fill with zeros
     uint32_t wait_us;   // limit of every device-side wait, microseconds
@@ -436,9 +446,8 @@ struct Epilogue {
                 y1 = y0 + (uint64_t)(8u * row_bytes);
                 y_tile += (uint64_t)((uint32_t)h * row_bytes);
                 uint32_t taddr = lane_taddr + (uint32_t)(acc * kAccStride + first * kChunkT);
-                bool to;
-                if (!ptx::mbar_wait_bounded(full0 + 8u * acc, acc_phase, &ctl->abort_flag, to)) {
-                    if (to && lane == 0) report_timeout(*p, ctl, walk.run, 2, 100 + acc);
+                if (const int fail = ptx::mbar_wait(full0 + 8u * acc, acc_phase, &ctl->abort_flag)) {
+                    if (fail == 2 && lane == 0) report_timeout(*p, ctl, walk.run, 2, 100 + acc);
                     ok = false;
                     break;
                 }
@@ -493,12 +502,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // operand tiles need 1024-byte alignment for the 128-byte swizzle, the pairs of staging buffers 2048 (the
     // second is reached by flipping an address bit); both CTAs of a pair get the same offsets
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 2047) & ~uintptr_t(2047));
-    // staging buffers, weight values, weight metadata, activation stages, control block
-    uint8_t *a_smem = smem + kEpiBytes;
-    const int stages = kRuns ? p.stages : C::kStreamStages, w_blocks = kRuns ? p.w_blocks : C::kStreamStages;
-    uint8_t *m_smem = a_smem + w_blocks * C::kABytes;
-    uint8_t *b_smem = m_smem + w_blocks * C::kMetaBytes;
-    Ctl *ctl = reinterpret_cast<Ctl *>(b_smem + stages * C::kBBytes);
+    // staging buffers, control block, weight values, weight metadata, activation stages
+    Ctl *ctl = reinterpret_cast<Ctl *>(smem + kEpiBytes);
+    uint8_t *a_smem = smem + kEpiBytes + C::kCtlBytes;
+    const int stages = p.stages, b_bytes = C::b_bytes(p.block_t);
+    uint8_t *m_smem = a_smem + p.w_blocks * C::kABytes;
+    uint8_t *b_smem = m_smem + p.w_blocks * C::kMetaBytes;
     volatile uint32_t *abort_flag = &ctl->abort_flag;
 
     const int warp = threadIdx.x >> 5;
@@ -550,8 +559,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             const uint32_t full0 = ptx::map_to_cta(full_own, 0);    // all bytes of a stage are counted on CTA 0's barrier
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued = 0;            // bit s: a load into stage s was issued
-            uint32_t last_parity = 0;       // bit s: parity of the last phase issued into stage s
+            bool wrapped = false;           // every stage has been loaded
+            int fail = 0;
+            const bool withhold = p.withhold != 0;
             bool ok = true, first_run = true;
             for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); ok && walk.run < num_runs; walk.next(p, num_clusters)) {
                 const bool twin = walk.twin(p);
@@ -570,31 +580,23 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const int passes = twin ? 2 : tiles;                              // over the k blocks
                 bool weights = true;                                              // this pass brings the weight blocks
                 for (int pass = 0; ok && pass < passes; ++pass) {
-                    for (int kb = 0; kb < k_blocks; ++kb) {
-                        if (p.withhold && walk.run == 0 && pass == passes - 1 && kb == k_blocks - 1) {
-                            // planted failure (test hook): these loads never come, the MMA issuer's wait runs out
-                            ok = false;
-                            break;
-                        }
-                        bool to;
-                        if (!ptx::mbar_wait_bounded(empty0 + 8u * stage, phase ^ 1u, abort_flag, to)) {
-                            if (to) report_timeout(p, ctl, walk.run, 0, stage);
-                            ok = false;
-                            break;
-                        }
+                    // planted failure (test hook): the last loads never come, the MMA issuer's wait runs out
+                    const bool withheld = withhold && walk.run == 0 && pass == passes - 1;
+                    const int kb_end = withheld ? k_blocks - 1 : k_blocks;
+#pragma unroll kUnrollK
+                    for (int kb = 0; kb < kb_end; ++kb) {
+                        fail = ptx::mbar_wait(empty0 + 8u * stage, phase ^ 1u, abort_flag);
+                        if (fail) break;
                         if (kRuns && weights && !first_run && stages > k_blocks) {
                             // the weight block's previous contents (k block kb of the run before, k_blocks uses of the
                             // ring ago) have been multiplied; with fewer stages the wait above says so already
                             const int st = stage >= k_blocks ? stage - k_blocks : stage - k_blocks + stages;
-                            if (!ptx::mbar_wait_bounded(empty0 + 8u * st, stage >= k_blocks ? phase : phase ^ 1u, abort_flag, to)) {
-                                if (to) report_timeout(p, ctl, walk.run, 0, 32 + st);
-                                ok = false;
-                                break;
-                            }
+                            fail = ptx::mbar_wait(empty0 + 8u * st, stage >= k_blocks ? phase : phase ^ 1u, abort_flag);
+                            if (fail) break;
                         }
                         const uint32_t bar = full0 + 8u * stage;
                         if (rank == 0) ptx::mbar_arrive_expect_tx(full_own + 8u * stage, weights ? tx_wx : tx_x);
-                        const uint32_t b = b0 + (uint32_t)(stage * C::kBBytes);
+                        const uint32_t b = b0 + (uint32_t)(stage * b_bytes);
                         if (kHalf) {
                             // 128 binary16 columns = two tiles of 128 bytes per token row
                             ptx::tma_load_2d_pair(b, mb, bar, kb * 256, m0);
@@ -607,13 +609,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             ptx::tma_load_2d_pair(a0 + (uint32_t)(blk * C::kABytes), &map_a, bar, kb * (kHalf ? 128 : kSparse ? 64 : 128), f0);
                             if (kSparse) ptx::tma_load_2d_pair(e0 + (uint32_t)(blk * C::kMetaBytes), &map_e, bar, 0, e_row + kb * 8);
                         }
-                        issued |= 1u << stage;
-                        last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
                         if (++stage == stages) {
                             stage = 0;
                             phase ^= 1u;
+                            wrapped = true;
                         }
                     }
+                    if (fail == 2) report_timeout(p, ctl, walk.run, 0, stage);
+                    if (fail || withheld) ok = false;
                     m0 += h;
                     f0 = twin && rank == 0 ? p.oob_row : n0;
                     weights = !kRuns;
@@ -623,10 +626,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             if (*abort_flag && rank == 0) {
                 // do not leave while bulk copies may still land in the pair's shared memory
                 for (int s = 0; s < stages; ++s) {
-                    if (issued & (1u << s)) {
+                    if (wrapped || s < stage) {
                         uint32_t none[2] = {0u, p.wait_us};
-                        bool to;
-                        (void)ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->full[s]), (last_parity >> s) & 1u, none, to);
+                        (void)ptx::mbar_wait(ptx::smem_u32(&ctl->full[s]), s < stage ? phase : phase ^ 1u, none);
                     }
                 }
             }
@@ -648,6 +650,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             int acc = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
+            int fail = 0;
             for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); ok && walk.run < num_runs; walk.next(p, num_clusters)) {
                 int n0_unused, m0_unused, h, tiles;
                 walk.origin(p, 0, n0_unused, m0_unused, h, tiles);
@@ -657,26 +660,24 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const uint32_t half_units = (uint32_t)((h >> 1) * 128) >> 4;
                 bool weights = true;                                   // this tile's stages bring weight blocks
                 for (; ok && tiles > 0; --tiles) {
-                    bool to;
-                    if (!ptx::mbar_wait_bounded(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, to)) {
-                        if (to) report_timeout(p, ctl, walk.run, 1, 100 + acc);
+                    fail = ptx::mbar_wait(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag);
+                    if (fail) {
+                        if (fail == 2) report_timeout(p, ctl, walk.run, 1, 100 + acc);
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
                     const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kAccStride);
+#pragma unroll kUnrollK
                     for (int kb = 0; kb < num_kb; ++kb) {
-                        if (!ptx::mbar_wait_bounded(full0 + 8u * stage, phase, abort_flag, to)) {
-                            if (to) report_timeout(p, ctl, walk.run, 1, stage);
-                            ok = false;
-                            break;
-                        }
+                        fail = ptx::mbar_wait(full0 + 8u * stage, phase, abort_flag);
+                        if (fail) break;
                         ptx::tc_fence_after();
                         const int blk = kRuns ? kb : stage;
                         const uint32_t meta_t = tmem_base + (uint32_t)(kMetaCol + 4 * blk);
                         if (kSparse && weights) ptx::tc_cp_128x128b_pair(meta_t, edesc0 + (uint64_t)((uint32_t)(blk * C::kMetaBytes) >> 4));
                         const uint64_t adesc = adesc0 + (uint64_t)((uint32_t)(blk * C::kABytes) >> 4);
-                        const uint64_t bdesc = bdesc0 + (uint64_t)((uint32_t)(stage * C::kBBytes) >> 4);
+                        const uint64_t bdesc = bdesc0 + (uint64_t)((uint32_t)(stage * b_bytes) >> 4);
 #pragma unroll
                         for (int k = 0; k < C::kMmasPerStage; ++k) {
                             const uint64_t ad = adesc + (uint64_t)((k * C::kAStepBytes) >> 4);
@@ -701,7 +702,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             phase ^= 1u;
                         }
                     }
-                    if (ok) ptx::tc_commit_pair(tfull0 + 8u * acc, 3);
+                    if (fail) {
+                        if (fail == 2) report_timeout(p, ctl, walk.run, 1, stage);
+                        ok = false;
+                        break;
+                    }
+                    ptx::tc_commit_pair(tfull0 + 8u * acc, 3);
                     weights = !kRuns;
                     acc ^= 1;
                     acc_phase ^= acc == 0 ? 1u : 0u;
@@ -711,8 +717,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 // let every MMA issued so far retire before tensor memory is released
                 ptx::tc_commit(ptx::smem_u32(&ctl->drain));
                 uint32_t none[2] = {0u, p.wait_us};
-                bool to;
-                (void)ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->drain), 0, none, to);
+                (void)ptx::mbar_wait(ptx::smem_u32(&ctl->drain), 0, none);
             }
         }
     } else {
@@ -753,9 +758,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 walk.origin(p, (int)rank, n0, m0, h, tiles);
                 const int n = n0 + quarter * 32 + lane;                // this thread's output feature
                 for (; tiles > 0; --tiles, m0 += h) {
-                    bool to;
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, to)) {
-                        if (to && lane == 0) report_timeout(p, ctl, walk.run, 2, 100 + acc);
+                    if (const int fail = ptx::mbar_wait(ptx::smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag)) {
+                        if (fail == 2 && lane == 0) report_timeout(p, ctl, walk.run, 2, 100 + acc);
                         ok = false;
                         break;
                     }
@@ -998,7 +1002,7 @@ static bool set_tiling(GemmParams &p, int K_cost, int clusters)
     // FP16 model's leave three at K = 768, with which it is slower: 27.5 us streaming, 31.7 resident.)  The
     // raw sums and the dense variant have no such instantiation, and twin tiles stream.
     const int kb = (p.K + kBlockK - 1) / kBlockK;
-    const int stages = kb <= kMaxWeightBlocks ? (C::kRoom - kb * C::kWBytes) / C::kBBytes : 0;
+    const int stages = kb <= kMaxWeightBlocks ? C::resident_stages(kMaxBlockT, kb) : 0;
     // With fewer than three waves of tiles there is nothing to keep them for.
     const bool may_stay = C::kMayStay && p.out_type != GPUSQ_OUT_I32 && !twin_col && !wide && stages >= C::kMinResidentStages &&
                           (ceil_div(p.M, kMaxBlockT) * p.pair_cols >= 3 * (int64_t)clusters ||
@@ -1014,7 +1018,7 @@ static bool set_tiling(GemmParams &p, int K_cost, int clusters)
     p.block_t = t.block_t;
     p.n_big = t.n_big;
     p.run_tiles = t.run_tiles;
-    p.stages = t.run_tiles > 1 ? (stages < kMaxStages ? stages : kMaxStages) : C::kStreamStages;
+    p.stages = t.run_tiles > 1 ? C::resident_stages(t.block_t, kb) : C::stream_stages(t.block_t);
     p.w_blocks = t.run_tiles > 1 ? kb : p.stages;
     const int64_t pair_runs = (int64_t)p.pair_cols * t.runs;
     const int64_t runs = pair_runs + (twin_col ? ceil_div(p.M, 2 * (int64_t)t.block_t) : 0);
@@ -1032,7 +1036,7 @@ static bool set_tiling(GemmParams &p, int K_cost, int clusters)
 template <typename C>
 static int smem_bytes(const GemmParams &p)
 {
-    return kEpiBytes + p.w_blocks * C::kWBytes + p.stages * C::kBBytes + C::kCtlBytes + 2048;
+    return kEpiBytes + p.w_blocks * C::kWBytes + p.stages * C::b_bytes(p.block_t) + C::kCtlBytes + 2048;
 }
 
 // SM pairs that can hold one cluster of this kernel each, per device (0 = unknown yet)

@@ -67,8 +67,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 
 // Bounded wait: gives up after the time limit, or as soon as another thread of the CTA has raised
 // *abort_flag.  The limit, in microseconds, is the word behind the flag (abort_flag[1]; 2 s unless the
-// test hook shortens it).  Returns false on either; the
-// caller that timed out raises the flag itself.  The common case (the phase
+// test hook shortens it).  The caller whose wait timed out raises the flag itself.  The common case (the phase
 // is complete already) costs one try and one branch; the retry loop is kept
 // out of line so that it does not bloat the callers' instruction streams.
 // A retry parks the thread in hardware until the phase completes or the hint
@@ -100,7 +99,6 @@ __device__ __forceinline__ bool mbar_try_wait_32(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// returns 0 = phase complete, 1 = abort flag seen, 2 = time limit reached
 __device__ __noinline__ int mbar_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag)
 {
     const uint64_t t0 = globaltimer_ns();
@@ -110,14 +108,11 @@ __device__ __noinline__ int mbar_wait_slow(uint32_t bar, uint32_t parity, volati
         if (globaltimer_ns() - t0 > (uint64_t)abort_flag[1] * 1000ull) return 2;
     }
 }
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
-                                                  volatile uint32_t *abort_flag, bool &timed_out)
+// 0 = phase complete, 1 = abort flag seen, 2 = time limit reached
+__device__ __forceinline__ int mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag)
 {
-    timed_out = false;
-    if (mbar_try_wait(bar, parity)) return true;
-    const int r = mbar_wait_slow(bar, parity, abort_flag);
-    timed_out = r == 2;
-    return r == 0;
+    if (__builtin_expect(mbar_try_wait(bar, parity), 1)) return 0;
+    return mbar_wait_slow(bar, parity, abort_flag);
 }
 
 // ---- TMA ----

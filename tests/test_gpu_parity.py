@@ -331,6 +331,35 @@ def test_spgemm_int32_bit_exact(B, M, N, K, block_t):
     assert np.array_equal(Yd.cpu().numpy(), acc_o)       # same C as the dense GEMM (Fig. 1)
 
 
+# The ring of operand stages has as many places as fit (sixteen at 32 tokens, eight at 224); k blocks that fill it not
+# quite, exactly, more than once and more than twice, over tiles of full and lower height, whose last k block is whole or not.
+@pytest.mark.parametrize("block_t", [32, 64, 96, 128, 160, 192, 224])
+@pytest.mark.parametrize("k_blocks", [3, 7, 8, 9, 13, 16, 17, 35])
+def test_operand_ring_lengths(B, block_t, k_blocks):
+    M, N, K = 2 * block_t + 45, 300, 128 * k_blocks - (16 if k_blocks % 2 else 0)
+    d, prep, Xq, xs = _prep(block_t + K, M, N, K)
+    acc_o = oracle.spgemm_acc(Xq, prep["vals"], prep["meta"], threads=oracle.host_cores())
+    Y_o = oracle.epilogue(acc_o, prep["w_scale"], xs, d["bias"], act=0, out_type=0)
+    Wpk, status = B.pack24(cu(prep["vals"]), cu(prep["meta"])), torch.zeros(4, dtype=torch.int32, device="cuda")
+    N8 = N // 8 * 8
+    try:
+        B.set_max_clusters(2)
+        for n_big in (None, 1) if block_t > 32 else (None,):
+            if n_big is None:
+                B.set_block_tokens(block_t)
+            else:
+                B.set_tile_mix(block_t, n_big)
+            acc = B.spgemm_i8(cu(Xq), Wpk, N, out_type=B.OUT_I32, status_buf=status).cpu().numpy()
+            accd = B.gemm_i8_dense(cu(Xq), cu(prep["Wq"]), out_type=B.OUT_I32, status_buf=status).cpu().numpy()
+            assert np.array_equal(acc, acc_o) and np.array_equal(accd, acc_o)
+        Y = B.spgemm_i8(cu(Xq), Wpk, N8, cu(prep["w_scale"][:N8]), cu(np.array([xs], np.float32)), cu(d["bias"][:N8]), status_buf=status)
+    finally:
+        B.set_block_tokens(0)
+        B.set_max_clusters(0)
+    assert status.cpu().tolist() == [0, 0, 0, 0]
+    assert np.array_equal(Y.cpu().numpy(), Y_o[:, :N8])
+
+
 @pytest.mark.parametrize("M,N,K,block_t,n_big", [
     (1000, 512, 256, 96, 3), (1576, 768, 192, 224, 2), (700, 256, 128, 64, 0), (2000, 384, 320, 160, 5),
     (333, 576, 192, 128, 1), (900, 1024, 64, 192, 100), (12608, 768, 256, 192, 24), (5000, 96, 48, 128, 7)])
