@@ -34,6 +34,7 @@
 #include <cuda_fp16.h>
 
 #include <atomic>
+#include <cstddef>
 #include <mutex>
 #include <type_traits>
 
@@ -111,6 +112,8 @@ struct Ctl {
     uint32_t abort_flag;
     uint32_t wait_us;       // directly behind the flag: the bounded waits read their limit from here
 };
+constexpr int kTmemEmptyBar = 2 * kMaxStages + 2, kBarriers = kTmemEmptyBar + 3;      // barriers are numbered from full[0] on
+static_assert(offsetof(Ctl, tmem_empty) == 8 * kTmemEmptyBar && offsetof(Ctl, tmem_base) == 8 * kBarriers, "numbering of the barriers");
 
 struct GemmParams {
     const float *w_scale;
@@ -518,19 +521,17 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int num_runs = p.num_runs;
     const int k_blocks = (p.K + kBlockK - 1) / kBlockK;        // k blocks of the layer; a twin tile takes them twice
 
+    // Set-up, exposed wherever the previous kernel held the SM to its end: 0.73 us when one thread initialised all
+    // barriers (some 20 cycles each) and both cluster barriers had release semantics, 0.5 now.
+    if (warp >= 2 && lane == 0) {
+        const uint32_t first = ptx::smem_u32(&ctl->full[0]);
+        for (int b = warp - 2; b < kBarriers; b += kEpiWarps)
+            ptx::mbar_init(first + 8u * b, b >= kTmemEmptyBar && b < kTmemEmptyBar + 2 ? 2 * kEpiWarps : 1);     // the epilogue warps of both CTAs
+        ptx::fence_barrier_init();
+    }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&ctl->empty[s]), 1);
-        }
-        for (int a = 0; a < 2; ++a) {
-            ptx::mbar_init(ptx::smem_u32(&ctl->tmem_full[a]), 1);
-            ptx::mbar_init(ptx::smem_u32(&ctl->tmem_empty[a]), 2 * kEpiWarps);   // the epilogue warps of both CTAs
-        }
-        ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
         ctl->abort_flag = 0;
         ctl->wait_us = p.wait_us;
-        ptx::fence_barrier_init();
         ptx::prefetch_tensormap(&map_a);
         ptx::prefetch_tensormap(&map_b);
         if (p.n_big * p.pair_cols < p.pair_runs) ptx::prefetch_tensormap(&map_b2);
@@ -542,7 +543,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
     ptx::tc_fence_before();
     __syncthreads();
-    ptx::cluster_sync();            // the other CTA's barriers exist before anything is signalled on them
+    ptx::cluster_arrive_relaxed();  // the other CTA's barriers exist before anything is signalled on them
+    ptx::cluster_wait();
     ptx::tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     // Programmatic dependent launch: everything above ran while the previous kernel in the stream was
@@ -628,10 +630,23 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 for (int s = 0; s < stages; ++s) {
                     if (wrapped || s < stage) {
                         uint32_t none[2] = {0u, p.wait_us};
-                        (void)ptx::mbar_wait(ptx::smem_u32(&ctl->full[s]), s < stage ? phase : phase ^ 1u, none);
+                        if (ptx::mbar_wait(ptx::smem_u32(&ctl->full[s]), s < stage ? phase : phase ^ 1u, none) == 2) break;
                     }
                 }
             }
+        }
+        __syncwarp();
+        // Nor while the release of a stage is under way to this CTA: the last one of each is waited for, lane by stage.
+        // (Counted anew: kept for this, the loop's own state made the loop above slower, 165 -> 260 cycles per k block.)
+        int uses = 0;
+        for (RunWalk<kTwin, kRuns> walk(p, cluster_id, num_clusters); walk.run < num_runs; walk.next(p, num_clusters)) {
+            int n0_unused, m0_unused, h_unused, tiles;
+            walk.origin(p, 0, n0_unused, m0_unused, h_unused, tiles);
+            uses += k_blocks * (walk.twin(p) ? 2 : tiles);
+        }
+        if (lane < stages && lane < uses) {
+            const int last = uses - 1 - (uses - 1 - lane) % stages;
+            (void)ptx::mbar_wait(ptx::smem_u32(&ctl->empty[lane]), (uint32_t)(last / stages) & 1u, abort_flag);
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
@@ -713,6 +728,13 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     acc_phase ^= acc == 0 ? 1u : 0u;
                 }
             }
+            // both CTAs' epilogue warps have given back the last two accumulators: none of their signals is under way
+            // when this CTA leaves
+            for (int i = 0; ok && i < 2; ++i) {
+                (void)ptx::mbar_wait(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag);
+                acc ^= 1;
+                acc_phase ^= acc == 0 ? 1u : 0u;
+            }
             if (*abort_flag) {
                 // let every MMA issued so far retire before tensor memory is released
                 ptx::tc_commit(ptx::smem_u32(&ctl->drain));
@@ -786,10 +808,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     }
 
-    // neither CTA leaves while the other may still signal its barriers or read its shared memory
+    // Neither CTA leaves while the other may still signal its barriers or read its shared memory.  Relaxed: all such
+    // signals have been waited for above, and a release would first drain the stores of Y (0.5 us), which the end of
+    // the kernel does anyway.  After an abort signals may be under way that nobody waits for: they get time to land.
+    if (*abort_flag) __nanosleep(20000);
     ptx::tc_fence_before();
-    __syncthreads();
-    ptx::cluster_sync();
+    __syncwarp();
+    ptx::cluster_arrive_relaxed();
+    ptx::cluster_wait();
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
