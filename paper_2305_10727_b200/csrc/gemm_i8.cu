@@ -306,6 +306,8 @@ struct Epilogue {
         ptx::tmem_ld_16x256b_x2(taddr + (16u << 16), v, 8);
     }
 
+    __device__ __forceinline__ static __half2 half2_of(uint32_t h2) { return *reinterpret_cast<const __half2 *>(&h2); }
+
     // value pair e of the chunk: features f + 8 (e % 2) + 16 (e / 4), tokens 8 (e / 2 % 2) + 2 (lane % 4), + 1
     template <bool kGelu>
     __device__ __forceinline__ float2 value(const uint32_t (&v)[16], int e) const
@@ -345,14 +347,20 @@ struct Epilogue {
                 const float2 y = value<kGelu>(v, e);
                 const __half2 hh = __floats2half2_rn(y.x, y.y);   // low = token 2(t%4), high = +1
                 pk[e] = *reinterpret_cast<const uint32_t *>(&hh);
-                if (kAmax) {
-                    __half2 a = hh;
-                    if (left < kChunkT) {                          // tokens past the end hold the bias only
+            }
+            if (kAmax) {
+                // one maximum per pair; only the tensor's last chunk of tokens, past whose end there is only the bias,
+                // takes the selections (taken with every pair they made 50176 x 512 -> 2048 a fifth slower)
+                if (left < kChunkT) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
                         const int tok = 8 * ((e >> 1) & 1) + 2 * (lane & 3);
-                        a = make_half2(tok < left ? __low2half(hh) : __ushort_as_half(0),
-                                       tok + 1 < left ? __high2half(hh) : __ushort_as_half(0));
+                        const uint32_t keep = (tok < left ? 0xFFFFu : 0u) | (tok + 1 < left ? 0xFFFF0000u : 0u);
+                        amax2 = __hmax2(amax2, __habs2(half2_of(pk[e] & keep)));
                     }
-                    amax2 = __hmax2(amax2, __habs2(a));
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) amax2 = __hmax2(amax2, __habs2(half2_of(pk[e])));
                 }
             }
         }
