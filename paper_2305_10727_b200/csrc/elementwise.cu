@@ -390,29 +390,56 @@ __device__ __forceinline__ uint2 regrouped(uint2 q, int regroup)
     return regroup ? make_uint2(__byte_perm(q.x, q.y, 0x6420), __byte_perm(q.x, q.y, 0x7531)) : q;
 }
 
-// One pass over a tensor whose scale is known, four vectors in flight per thread.  Every thread has `rounds`
-// vectors, one less where the last round does not reach; backwards: from the last one on.
+// A thread's vectors pass through its own kPlaces places in shared memory, one in kT threads' rows, which asynchronous
+// copies fill: only this thread reads them, so the copies' own counting is all the synchronisation.
+// Unlike loads they need no L1, of which a CTA that starts beside a GEMM's last ones has 28 KB.
+template <int kT, int kPlaces>
+struct VecRing {
+    uint32_t first, at;         // shared-memory address of place 0 and of the next vector's place
+
+    __device__ __forceinline__ VecRing(const uint4 *places)
+        : first((uint32_t)__cvta_generic_to_shared(places + threadIdx.x)), at(first) {}
+    __device__ __forceinline__ void copy(const uint4 *x) const
+    {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(x) : "memory");
+    }
+    __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+    template <int kPending>
+    __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
+    __device__ __forceinline__ uint4 read() const
+    {
+        uint4 v;
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+        return v;
+    }
+    __device__ __forceinline__ void up() { at = at == first + (kPlaces - 1) * kT * 16 ? first : at + kT * 16; }
+    __device__ __forceinline__ void down() { at = at == first ? first + (kPlaces - 1) * kT * 16 : at - kT * 16; }
+};
+
+// One pass over a tensor whose scale is known: the `left` vectors of this thread, `stride` apart, the first
+// kQuantPlaces of which are on their way into the ring; they are taken in pairs, a pair being a group of copies.
 // kSingle: one product per value is known to give the codes (find_single_product).
+constexpr int kQuantPlaces = 4;
+using QuantRing = VecRing<kThreads, kQuantPlaces>;
+
 template <bool kSingle>
-__device__ __forceinline__ void quantise_strided(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, int64_t vec8, int rounds,
-                                                 bool backwards, const QuantScale &a, int regroup)
+__device__ __forceinline__ void quantise_strided(QuantRing ring, const uint4 *__restrict__ X, uint2 *__restrict__ Xq, int64_t stride,
+                                                 int left, const QuantScale &a, int regroup)
 {
     auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<true>(v, a) : quant8_f16<true>(v, a), regroup); };
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int left = i + (rounds - 1) * stride < vec8 ? rounds : rounds - 1;
-    if (backwards) {
-        i += (left - 1) * stride;
-        stride = -stride;
-    }
-    for (; left >= 4; left -= 4, i += 4 * stride) {
-        uint4 v[4];
+    X += kQuantPlaces * stride;
+    for (; left > 0; left -= 2, X += 2 * stride, Xq += 2 * stride) {
+        QuantRing::wait<kQuantPlaces / 2 - 1>();
+        uint4 v[2];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(X + i + u * stride);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) Xq[i + u * stride] = codes(v[u]);
+        for (int u = 0; u < 2; ++u, ring.up()) {
+            v[u] = ring.read();                            // not a copied one where left is 1: not used
+            if (left - u > kQuantPlaces) ring.copy(X + u * stride);
+        }
+        QuantRing::commit();
+        Xq[0] = codes(v[0]);
+        if (left > 1) Xq[stride] = codes(v[1]);
     }
-    for (; left > 0; --left, i += stride) Xq[i] = codes(__ldg(X + i));
 }
 
 // n_partials > 0: the scale is derived from the partial maxima and written to
@@ -421,9 +448,12 @@ __device__ __forceinline__ void quantise_strided(const uint4 *__restrict__ X, ui
 // With absmax, X was written just before, front to back, and what was written last is still in L2: it is
 // read backwards (205 MB behind the GEMM that wrote them: 5 us less; a tensor from HBM with a supplied
 // scale in front of its GEMM: up to 0.3 us more, hence forwards).
-// Bound by HBM: back to back on cold tensors 51.6 MB take 14.6 us (17.1 with two loads in flight, two
-// waves of blocks and the bracketing products), 11.8 being what the bytes need; in front of a GEMM
-// 19.4 MB add 7.3 us (8.3), 0.65 MB 1.6 (2.7).
+// Bound by HBM.  The tensor comes through asynchronous copies, which start before the scale is looked at, and the kernel
+// asks for L1 (prefer_carveout): behind a GEMM, whose shared memory leaves 28 KB of L1, plain loads had to queue
+// for it.  Four loads per thread in registers -> this, us: 19.4 MB cold 6.9 -> 6.2, with the GEMM behind it 15.0 -> 13.8;
+// 51.6 MB 14.3 -> 13.6 and 35.4 -> 31.6 (11.8 being what the bytes need); 205 MB behind the GEMM that wrote them 57 -> 49;
+// 3.1 MB 3.4 -> 3.1.  Copies one by one take 53.5 for the last but one, four places without preference 42.3
+// where 37.2 is right (100352 x 96 and its GEMM).
 constexpr int kQuantBlocksPerSm = 4;      // what 64 registers a thread leave room for: one wave
 __global__ void __launch_bounds__(kThreads, kQuantBlocksPerSm)
 act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale,
@@ -431,7 +461,22 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
                  const float *__restrict__ absmax, float qmax, int regroup)
 {
     __shared__ float red[kThreads / 32];
+    __shared__ uint4 places[kQuantPlaces * kThreads];
     begin_behind();
+    // every thread has `rounds` vectors, one less where the last round does not reach
+    int64_t stride = (int64_t)gridDim.x * blockDim.x, at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int left = at + (rounds - 1) * stride < vec8 ? rounds : rounds - 1;
+    if (absmax) {
+        at += (left - 1) * stride;
+        stride = -stride;
+    }
+    const QuantRing ring(places);
+    QuantRing filled = ring;
+#pragma unroll
+    for (int k = 0; k < kQuantPlaces; ++k, filled.up()) {
+        if (k < left) filled.copy(X + at + k * stride);
+        if (k % 2) QuantRing::commit();
+    }
     float s;
     if (absmax) {
         s = scale_from_amax(__ldg(absmax), qmax);
@@ -449,9 +494,9 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
     QuantScale a = make_quant_scale(s, qmax);
     // the test of the single product pays from four vectors per thread on
     if (vec8 >= 4 * (int64_t)gridDim.x * blockDim.x && find_single_product<true>(a))
-        quantise_strided<true>(X, Xq, vec8, rounds, absmax != nullptr, a, regroup);
+        quantise_strided<true>(ring, X + at, Xq + at, stride, left, a, regroup);
     else
-        quantise_strided<false>(X, Xq, vec8, rounds, absmax != nullptr, a, regroup);
+        quantise_strided<false>(ring, X + at, Xq + at, stride, left, a, regroup);
 }
 
 static int launch_act_quant(const void *X, int8_t *Xq, float *x_scale, const uint32_t *partial, int n_partials, int64_t vec8,
@@ -460,6 +505,7 @@ static int launch_act_quant(const void *X, int8_t *Xq, float *x_scale, const uin
     const int grid = grid_for(vec8, kQuantBlocksPerSm);
     const int64_t rounds = ceil_div(vec8, (int64_t)grid * kThreads);
     if (rounds > 0x7FFFFFFF) return GPUSQ_ERR_SHAPE;
+    prefer_carveout<act_quant_kernel>(50);         // four blocks' rings take 64 KB
     return launch_behind(act_quant_kernel, grid, kThreads, stream, reinterpret_cast<const uint4 *>(X),
                          reinterpret_cast<uint2 *>(Xq), x_scale, partial, n_partials, vec8, (int)rounds, absmax, qmax, regroup);
 }
@@ -690,46 +736,23 @@ struct QuantShare {
     int per, full;
 };
 
-// A thread's vectors of the rest pass through its own kRing places in shared memory, which asynchronous
-// copies fill: only this thread reads them, so the copies' own counting is all the synchronisation.
-// Unlike loads they need no L1, of which a CTA that starts beside a GEMM's last ones has 28 KB.
-struct VecRing {
-    uint32_t first, at;         // shared-memory address of place 0 and of the next vector's place
-
-    __device__ __forceinline__ VecRing(const uint4 *places)
-        : first((uint32_t)__cvta_generic_to_shared(places + threadIdx.x)), at(first) {}
-    __device__ __forceinline__ void copy(const uint4 *x) const
-    {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(x) : "memory");
-    }
-    __device__ __forceinline__ static void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-    template <int kPending>
-    __device__ __forceinline__ static void wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
-    __device__ __forceinline__ uint4 read() const
-    {
-        uint4 v;
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
-        return v;
-    }
-    __device__ __forceinline__ void up() { at = at == first + (kRing - 1) * kFusedThreads * 16 ? first : at + kFusedThreads * 16; }
-    __device__ __forceinline__ void down() { at = at == first ? first + (kRing - 1) * kFusedThreads * 16 : at - kFusedThreads * 16; }
-};
+using FusedRing = VecRing<kFusedThreads, kRing>;
 
 // Step 3 of one CTA: the thread's vectors of the rest, in order, the first kRing of which are still in the
 // ring; then the n_kept vectors in shared memory.
 // kSingle: one product per value is known to give the codes (find_single_product).
 template <bool kSingle>
-__device__ __forceinline__ void quantise_share(const uint4 *cache, VecRing ring, const uint4 *__restrict__ Xr, uint2 *__restrict__ Xqr,
+__device__ __forceinline__ void quantise_share(const uint4 *cache, FusedRing ring, const uint4 *__restrict__ Xr, uint2 *__restrict__ Xqr,
                                                int64_t step, int rest, uint2 *__restrict__ Xqs, int n_kept, const QuantScale &a,
                                                int regroup)
 {
     auto codes = [&](uint4 v) { return regrouped(kSingle ? quant8_single<false>(v, a) : quant8_f16<false>(v, a), regroup); };
     Xr += kRing * step;
     for (int r = 0; r < rest; ++r) {
-        VecRing::wait<kRing - 1>();
+        FusedRing::wait<kRing - 1>();
         const uint2 c = codes(ring.read());
         if (r + kRing < rest) ring.copy(Xr);
-        VecRing::commit();
+        FusedRing::commit();
         __stcs(Xqr, c);
         ring.down();
         Xr += step;
@@ -845,7 +868,7 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
     const int64_t step = (int64_t)gridDim.x * kFusedThreads, r0 = (int64_t)blockIdx.x * kFusedThreads + tid;
     const int rest = sh.full + (r0 < sh.rest_last ? 1 : 0);
     const uint4 *Xr = X + sh.kept + r0;
-    VecRing ring(cache + kFusedCacheVecs);
+    FusedRing ring(cache + kFusedCacheVecs);
 
     if (tid == 0) {
         for (int c = 0; c < pieces; ++c)
@@ -893,15 +916,15 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         const uint4 *Xd = Xr + (int64_t)(rest - 1) * step;
         for (int k = 0; k < kRing; ++k) {
             if (k < rest) ring.copy(Xd);
-            VecRing::commit();
+            FusedRing::commit();
             ring.up();
             Xd -= step;
         }
         for (int r = rest - 1; r >= 0; --r) {
-            VecRing::wait<kRing - 1>();
+            FusedRing::wait<kRing - 1>();
             m = max(m, absmax_bits8(ring.read()));
             if (r >= kRing) ring.copy(Xd);
-            VecRing::commit();
+            FusedRing::commit();
             ring.up();
             Xd -= step;
             if (c < pieces && mbar_test_parity0((uint32_t)__cvta_generic_to_shared(&piece_bar[c]))) piece();
@@ -940,7 +963,7 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
         m = share_max(X, sh, (int)(next - kTakeOver));
     }
     const uint32_t all = grid_max;
-    if (next != kAllArrived) VecRing::wait<0>();
+    if (next != kAllArrived) FusedRing::wait<0>();
     if (next == kTooLate) {
         if (tid == 0) {
             // This CTA has not waited, so all it knows of the maximum is that it is final once every CTA has counted

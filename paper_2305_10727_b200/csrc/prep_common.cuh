@@ -3,6 +3,8 @@
 
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "quant_math.cuh"
 
@@ -185,6 +187,19 @@ inline int grid_for(int64_t items, int per_sm)
     int64_t blocks = ceil_div(items, kThreads);
     int64_t cap = (int64_t)num_sms() * per_sm;
     return (int)(blocks < cap ? (blocks < 1 ? 1 : blocks) : cap);
+}
+
+// Asks for a split of an SM's 228 KB between shared memory (percent) and L1, once per device.  Without it a kernel that is
+// set up while a GEMM drains gets the GEMM's split, 28 KB of L1, through which all its loads have to pass.
+template <auto kKernel>
+inline void prefer_carveout(int percent)
+{
+    static std::atomic<uint64_t> asked{0};
+    static_assert(kMaxDevices == 64, "a bit per device");
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || asked.load(std::memory_order_relaxed) >> dev & 1) return;
+    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent) != cudaSuccess) (void)cudaGetLastError();
+    asked.fetch_or((uint64_t)1 << dev, std::memory_order_relaxed);
 }
 
 // Launch that may be set up while the previous kernel of the stream drains; the kernel itself waits

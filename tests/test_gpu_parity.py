@@ -164,6 +164,23 @@ def test_quant_act_sizes(B, vecs):
     assert np.array_equal(Xq.cpu().numpy(), Xq_o)
 
 
+# The one-pass kernel: its threads' vectors come through a ring of four places, two at a time.  Tensors that end between
+# two rounds, one vector before and one behind, with fewer rounds than places, as many, and more, odd and even.
+@pytest.mark.parametrize("rounds", [1, 2, 3, 4, 5, 6, 7, 9])
+@pytest.mark.parametrize("more", [-1, 0, 1, 70000])
+def test_one_pass_quantisation_rounds(B, rounds, more):
+    vecs = rounds * 4 * 256 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    X = np.random.default_rng(rounds).standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
+    for scale in (np.float32(4.5 / 127), None):             # supplied, clamping; of the known maximum
+        Xq_o, s_o = oracle.quant_act(X, scale)
+        if scale is None:
+            Xq, s = B.quant_act_absmax(cu(X), cu(np.array([np.abs(X).max()], np.float32)))
+            assert s.cpu().numpy()[0] == s_o
+        else:
+            Xq, _ = B.quant_act(cu(X), x_scale=cu(np.array([scale], np.float32)), scale_mode=B.SCALE_GIVEN)
+        assert np.array_equal(Xq.cpu().numpy(), Xq_o)
+
+
 def test_quant_act_beside_other_kernels(B):
     # CTAs that find no SM at first: a matrix product of many waves in another stream, and two calls at a time.
     # Shares are then taken over by CTAs that run; scale and codes have to be the same.
