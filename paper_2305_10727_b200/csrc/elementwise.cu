@@ -1400,6 +1400,7 @@ int gpusq_quant_act_static(const void *X, int8_t *Xq, float *x_scale, int scale_
     if (scale_mode == GPUSQ_SCALE_COMPUTE) {
         // every slot that is read below is written here first, so stale contents do not matter
         n_partials = absmax_blocks(vec8);
+        prefer_carveout<act_absmax_kernel>(0);
         if (int st = launch_behind(act_absmax_kernel, n_partials, kAbsmaxThreads, s, reinterpret_cast<const uint4 *>(X),
                                    scratch, vec8))
             return st;
@@ -1435,6 +1436,7 @@ int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mod
         // read; the words behind them (gpusq_quant_act's barrier) are not touched
         const int64_t vec8 = elems / 8;
         n_partials = absmax_blocks(vec8);
+        prefer_carveout<act_absmax_kernel>(0);
         if (int st = launch_behind(act_absmax_kernel, n_partials, kAbsmaxThreads, s, reinterpret_cast<const uint4 *>(img),
                                    partial, vec8))
             return st;
@@ -1448,6 +1450,11 @@ int gpusq_patch_quant(const void *img, int8_t *Xq, float *x_scale, int scale_mod
     g.by_p = make_fast_div((uint32_t)P);
     g.by_t = make_fast_div((uint32_t)g.T);
     g.by_tx = make_fast_div((uint32_t)g.Tx);
+    // all of the SM's memory as L1, for the loads in flight; 128 images of 224 x 224, 16 x 16 patches, and their GEMM, behind
+    // each other: 46.0 -> 38.4 us, with a supplied scale 40.3 -> 31.4
+    if (vec == 8) prefer_carveout<patch_quant_kernel<8>>(0);
+    else if (vec == 4) prefer_carveout<patch_quant_kernel<4>>(0);
+    else prefer_carveout<patch_quant_kernel<2>>(0);
     const auto kernel = vec == 8 ? patch_quant_kernel<8> : vec == 4 ? patch_quant_kernel<4> : patch_quant_kernel<2>;
     return launch_behind(kernel, grid_for(items, kQuantBlocksPerSm), kThreads, s, reinterpret_cast<const __half *>(img), Xq,
                          x_scale, (const uint32_t *)partial, n_partials, g, (uint32_t)items);
