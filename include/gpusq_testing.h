@@ -40,13 +40,13 @@ int gpusq_tile_plan(int64_t M, int N, int K, int half, int out_type, int cluster
 /* Bound of the device-side waits of gpusq_quant_act's one-launch kernel, in
  * nanoseconds (default 2 s), and, with withhold_last_cta != 0, a planted
  * failure made on purpose in an allowed form: the last CTA never publishes its
- * maximum, so every CTA's bounded wait runs out, the kernel returns, and the
+ * maximum, so the bounded wait of every CTA (of its cluster, for small tensors) runs out, the kernel returns, and the
  * status word and the NaN scale described in gpusq.h can be observed.  Nothing
  * faults or hangs: the waits end at the bound. */
 int gpusq_set_quant_act_wait(unsigned long long limit_ns, int withhold_last_cta);
 
 /* CTAs [first, first + count) of gpusq_quant_act's one-launch kernel (tensors
- * above 1 MB) wait for ns nanoseconds (at most 1 ms; 0 or count 0: none) before
+ * above 2.9 MB) wait for ns nanoseconds (at most 1 ms; 0 or count 0: none) before
  * they claim their shares, as if no SM had been free for them, and as long
  * again, if the share is gone by then, before they count themselves out.
  * CTAs that run take over shares that nobody has claimed after 20 us. */

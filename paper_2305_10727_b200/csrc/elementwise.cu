@@ -1012,57 +1012,84 @@ act_quant_fused_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, floa
 }
 
 // ---- one-launch activation quantisation of small tensors ----
-// One cluster of up to sixteen CTAs keeps the tensor in registers and exchanges its warps' maxima
-// through distributed shared memory: every warp writes its maximum into each CTA, one cluster barrier,
-// and every warp reduces them all.  Bound by latencies (launch, one load, the barrier, one store), of
-// which the grid-wide barrier through L2 of the kernel above is the longest.  Back to back, kernel above ->
-// this one: 0.3 MB 5.0 -> 3.6 us, 0.65 MB 5.0 -> 4.1, 0.9 MB 4.9 -> 4.5; at 1.2 MB both take 4.9 and at
-// 1.5 MB sixteen SMs are too few to load and store it (5.0 against 5.3): hence the limit of four vectors
-// per thread, 1 MB.
+// Clusters of up to sixteen CTAs.  Each reads the whole tensor for its maximum, and quantises kOwn of every thread's
+// vectors, which it still has in registers: so sixteen SMs, which is as many as can exchange a number without going
+// through L2, suffice for the maximum (the tensor comes out of L2 that often), and the codes, bound by issue, are shared
+// by more.  The CTAs exchange their maxima with asynchronous stores into each other's shared memory, which complete on
+// the receiver's mbarrier.  Bound by latencies: launch, one round of loads, the exchange (0.4 us), one store.
+// Back to back, us, one cluster that also made all codes, its warps' maxima exchanged behind a cluster barrier -> this:
+// 0.1 MB 2.5 -> 2.2, 0.4 MB 3.5 -> 2.5, 0.65 MB 3.9 -> 2.7, 1 MB 4.45 -> 2.8; the kernel above -> this: 1.5 MB 4.6 -> 3.4,
+// 1.9 MB 4.7 -> 4.1, 2.4 MB 4.7 -> 4.4, 2.6 MB 4.85 -> 4.6; at 3 MB both take 4.9.  Two vectors per cluster take 0.3 us more than
+// one, so they are for tensors that need more clusters than run at a time (seven).
 constexpr int kClusterThreads = 1024;
 constexpr int kMaxCluster = 16;
-constexpr int kClusterMaxPerThread = 4;
+constexpr int kClusterMaxPerThread = 11;
 
-template <int kPer>
+// per: vectors per thread, at most kPer; cluster c owns those from c kOwn on
+template <int kPer, int kOwn>
 __global__ void __launch_bounds__(kClusterThreads, 1)
-act_quant_cluster_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale, int vec8, float qmax, int regroup)
+act_quant_cluster_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_scale, uint32_t *ws, int vec8, int size, int per,
+                         unsigned long long wait_ns, int withhold, float qmax, int regroup)
 {
-    __shared__ uint32_t maxima[kMaxCluster * (kClusterThreads / 32)];
-    uint32_t rank, size;
+    __shared__ uint32_t warp_max[kClusterThreads / 32], cta_max[kMaxCluster];
+    __shared__ __align__(8) uint64_t arrived;
+    uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // every CTA of the cluster has started before its shared memory is written (waited for below)
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&arrived);
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(4 * size) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    // every CTA of the cluster has started, and has its barrier, before its shared memory is written (waited for below)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");                  // the producer of X is complete
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int stride = (int)size * kClusterThreads;
-    const int i0 = (int)rank * kClusterThreads + (int)threadIdx.x;
-    uint4 v[kPer];
-    uint32_t m = 0;
+    const int first = (int)blockIdx.x / size * kOwn;
+    const int stride = size * kClusterThreads, i0 = (int)rank * kClusterThreads + (int)threadIdx.x;
+    uint4 v[kPer];                                                      // from vector `first` on, round the end
 #pragma unroll
-    for (int u = 0; u < kPer; ++u) v[u] = i0 + u * stride < vec8 ? __ldg(X + i0 + u * stride) : make_uint4(0u, 0u, 0u, 0u);
+    for (int u = 0; u < kPer; ++u) {
+        const int k = first + u < per ? first + u : first + u - per;
+        v[u] = u < per && i0 + k * stride < vec8 ? __ldg(X + i0 + k * stride) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    uint32_t m = 0;
 #pragma unroll
     for (int u = 0; u < kPer; ++u) m = max(m, absmax_bits8(v[u]));
     m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) warp_max[warp] = m;
+    __syncthreads();
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-    if (lane < (int)size) {
-        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&maxima[rank * (kClusterThreads / 32) + warp]);
-        uint32_t theirs;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(lane));
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(theirs), "r"(m) : "memory");
+    if (warp == 0) {
+        m = __reduce_max_sync(0xffffffffu, warp_max[lane]);
+        if (lane < size && !(withhold && blockIdx.x == gridDim.x - 1)) {
+            uint32_t theirs, their_bar;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"((uint32_t)__cvta_generic_to_shared(&cta_max[rank])), "r"(lane));
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(their_bar) : "r"(bar), "r"(lane));
+            asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(theirs), "r"(m), "r"(their_bar) : "memory");
+        }
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    uint32_t all = 0;
-    for (int i = lane; i < (int)size * (kClusterThreads / 32); i += 32) all = max(all, maxima[i]);
-    all = __reduce_max_sync(0xffffffffu, all);
+    // Everything sent here has arrived when the barrier completes, so nothing is under way to a CTA that leaves.
+    const uint64_t t0 = globaltimer_now();
+    while (!mbar_try_wait_parity0(bar)) {
+        if (globaltimer_now() - t0 <= wait_ns) continue;
+        if (threadIdx.x == 0) {
+            atomicExch(ws + kWsStatus, (uint32_t)GPUSQ_ERR_TIMEOUT);
+            *x_scale = __int_as_float(0x7FC00000);
+        }
+        return;
+    }
+    const uint32_t all = __reduce_max_sync(0xffffffffu, lane < size ? cta_max[lane] : 0u);
     const float s = scale_from_amax(__half2float(__ushort_as_half((unsigned short)all)), qmax);
-    if (rank == 0 && threadIdx.x == 0) *x_scale = s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *x_scale = s;
     const QuantScale a = make_quant_scale(s, qmax);
 #pragma unroll
-    for (int u = 0; u < kPer; ++u)
-        if (i0 + u * stride < vec8) Xq[i0 + u * stride] = regrouped(quant8_f16<false>(v[u], a), regroup);
+    for (int u = 0; u < kOwn; ++u) {
+        const int i = i0 + (first + u) * stride;
+        if (first + u < per && i < vec8) Xq[i] = regrouped(quant8_f16<false>(v[u], a), regroup);
+    }
 }
 
 // ---- library-owned scratch for gpusq_quant_act_static ----
@@ -1197,23 +1224,28 @@ size_t gpusq_quant_act_workspace(int64_t M, int K)
     return (size_t)(kMaxPartials + kWorkspaceExtra) * sizeof(uint32_t);
 }
 
-// Largest cluster act_quant_cluster_kernel can be launched with on the current device (sixteen is not
-// portable), 0 if none; looked up once per device.
-static int max_quant_cluster()
+// Largest cluster act_quant_cluster_kernel can be launched with on the current device (sixteen is not portable), 0 if
+// none, and how many of them run at a time; looked up once per device.
+struct QuantClusters {
+    int size, active;
+};
+
+static QuantClusters quant_clusters()
 {
-    static std::atomic<int> known[kMaxDevices];               // size + 1, 0 = not looked up yet
+    static std::atomic<int> known[kMaxDevices];               // size + 32 active + 1, 0 = not looked up yet
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return {0, 0};
     const int k = known[dev].load(std::memory_order_relaxed);
-    if (k) return k - 1;
-    int best = 0;
-    const void *kernels[] = {(const void *)act_quant_cluster_kernel<1>, (const void *)act_quant_cluster_kernel<2>,
-                             (const void *)act_quant_cluster_kernel<kClusterMaxPerThread>};
+    if (k) return {(k - 1) % 32, (k - 1) / 32};
+    QuantClusters best = {0, 0};
+    const void *kernels[] = {(const void *)act_quant_cluster_kernel<1, 1>, (const void *)act_quant_cluster_kernel<2, 1>,
+                             (const void *)act_quant_cluster_kernel<4, 1>, (const void *)act_quant_cluster_kernel<7, 1>,
+                             (const void *)act_quant_cluster_kernel<8, 2>, (const void *)act_quant_cluster_kernel<kClusterMaxPerThread, 2>};
     bool opted = true;
     for (const void *f : kernels)
         opted = opted && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     bool failed = !opted;
-    for (int size = opted ? kMaxCluster : 8; size >= 8 && !best; size /= 2) {
+    for (int size = opted ? kMaxCluster : 8; size >= 8 && !best.size; size /= 2) {
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)size;
@@ -1224,21 +1256,28 @@ static int max_quant_cluster()
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernels[2], &cfg) != cudaSuccess) failed = true;
-        else if (n > 0) best = size;
+        if (cudaOccupancyMaxActiveClusters(&n, kernels[5], &cfg) != cudaSuccess) failed = true;
+        else if (n > 0) best = {size, n < 1000 ? n : 1000};
     }
     if (failed) (void)cudaGetLastError();                     // this function's own; an earlier one is not ours to clear
-    known[dev].store(best + 1, std::memory_order_relaxed);
+    known[dev].store(best.size + 32 * best.active + 1, std::memory_order_relaxed);
     return best;
 }
 
-static int launch_cluster_quant(const void *X, int8_t *Xq, float *x_scale, int vec8, int cluster_max, float qmax,
-                                int regroup, cudaStream_t stream)
+// What a tensor takes on clusters of `size` CTAs: vectors per thread, and vectors per cluster (0: too large).
+static int vectors_per_cluster(int64_t vec8, const QuantClusters &c, int &per)
 {
-    // as many CTAs (a power of two) as give every thread one vector, at most cluster_max
-    int size = 1;
-    while (size < cluster_max && size * kClusterThreads < vec8) size *= 2;
-    const int per = (int)ceil_div(vec8, size * kClusterThreads);
+    if (c.size == 0 || vec8 > (int64_t)c.size * kClusterThreads * kClusterMaxPerThread) return 0;
+    per = (int)ceil_div(vec8, (int64_t)c.size * kClusterThreads);
+    return per <= (c.active < 7 ? c.active : 7) ? 1 : per <= 2 * c.active ? 2 : 0;
+}
+
+static int launch_cluster_quant(const void *X, int8_t *Xq, float *x_scale, uint32_t *ws, int vec8, int size, int per, int own,
+                                float qmax, int regroup, cudaStream_t stream)
+{
+    // as many CTAs (a power of two) as give every thread one vector, where one cluster does
+    if (per == 1)
+        while (size > 1 && size / 2 * kClusterThreads >= vec8) size /= 2;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1246,15 +1285,17 @@ static int launch_cluster_quant(const void *X, int8_t *Xq, float *x_scale, int v
     at[1].val.clusterDim.x = (unsigned)size;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)size, 1, 1);
+    cfg.gridDim = dim3((unsigned)(size * ceil_div(per, own)), 1, 1);
     cfg.blockDim = dim3(kClusterThreads, 1, 1);
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    auto kernel = per <= 1 ? act_quant_cluster_kernel<1> : per <= 2 ? act_quant_cluster_kernel<2>
-                : act_quant_cluster_kernel<kClusterMaxPerThread>;
-    if (cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, vec8,
-                           qmax, regroup) != cudaSuccess) {
+    auto kernel = own == 2 ? (per <= 8 ? act_quant_cluster_kernel<8, 2> : act_quant_cluster_kernel<kClusterMaxPerThread, 2>)
+                : per <= 1 ? act_quant_cluster_kernel<1, 1> : per <= 2 ? act_quant_cluster_kernel<2, 1>
+                : per <= 4 ? act_quant_cluster_kernel<4, 1> : act_quant_cluster_kernel<7, 1>;
+    if (cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const uint4 *>(X), reinterpret_cast<uint2 *>(Xq), x_scale, ws, vec8, size,
+                           per, g_grid_wait_ns.load(std::memory_order_relaxed), g_withhold_slot.load(std::memory_order_relaxed), qmax,
+                           regroup) != cudaSuccess) {
         (void)cudaGetLastError();
         return GPUSQ_ERR_CUDA;
     }
@@ -1278,9 +1319,10 @@ static int quant_act_common(const void *X, int8_t *Xq, float *x_scale, int scale
     const int64_t vec8 = M * (int64_t)K / 8;
     cudaStream_t s = (cudaStream_t)stream;
     if (scale_mode == GPUSQ_SCALE_COMPUTE) {
-        const int cluster_max = max_quant_cluster();
-        if (cluster_max > 0 && vec8 <= (int64_t)cluster_max * kClusterThreads * kClusterMaxPerThread)
-            return launch_cluster_quant(X, Xq, x_scale, (int)vec8, cluster_max, qmax, regroup, s);
+        const QuantClusters c = quant_clusters();
+        int per = 0;
+        if (const int own = vectors_per_cluster(vec8, c, per))
+            return launch_cluster_quant(X, Xq, x_scale, reinterpret_cast<uint32_t *>(workspace), (int)vec8, c.size, per, own, qmax, regroup, s);
         // the opt-in to large dynamic shared memory is per device
         static std::mutex mu;
         static uint8_t attr_state[kMaxDevices] = {};          // 1 = set, 2 = failed

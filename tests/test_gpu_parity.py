@@ -164,6 +164,25 @@ def test_quant_act_sizes(B, vecs):
     assert np.array_equal(Xq.cpu().numpy(), Xq_o)
 
 
+# Small tensors: clusters of sixteen CTAs of 1024 threads with 1 to 7 vectors per thread, one per cluster, and 8 to 11, two per
+# cluster; one vector fewer, as many, one more, and the first size beyond, on the one-launch grid.
+@pytest.mark.parametrize("per", range(1, 13))
+@pytest.mark.parametrize("more", [-1, 0, 1])
+def test_quant_act_clusters(B, per, more):
+    vecs = per * 16384 + more
+    X = np.random.default_rng(vecs).standard_normal((vecs, 8), dtype=np.float32).astype(np.float16)
+    for at in (0, vecs // 2, vecs - 1):                     # the maximum in the first, a middle and the last CTA's part
+        Z = X.copy()
+        Z[at, at % 8] = -9.25
+        Xq_o, s_o = oracle.quant_act(Z)
+        ws = torch.zeros((B.quant_act_workspace(*Z.shape),), dtype=torch.uint8, device="cuda")
+        Xq, s = B.quant_act(cu(Z), workspace=ws)
+        assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq.cpu().numpy(), Xq_o) and not ws.any()
+    Xq_o, s_o = oracle.quant_act4(Z)
+    Xq, s = B.quant_act4(cu(Z))
+    assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq.cpu().numpy(), Xq_o[:, [0, 2, 4, 6, 1, 3, 5, 7]])
+
+
 # The one-pass kernel: its threads' vectors come through a ring of four places, two at a time.  Tensors that end between
 # two rounds, one vector before and one behind, with fewer rounds than places, as many, and more, odd and even.
 @pytest.mark.parametrize("rounds", [1, 2, 3, 4, 5, 6, 7, 9])
