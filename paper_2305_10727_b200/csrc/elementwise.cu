@@ -462,7 +462,6 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
 {
     __shared__ float red[kThreads / 32];
     __shared__ uint4 places[kQuantPlaces * kThreads];
-    begin_behind();
     // every thread has `rounds` vectors, one less where the last round does not reach
     int64_t stride = (int64_t)gridDim.x * blockDim.x, at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int left = at + (rounds - 1) * stride < vec8 ? rounds : rounds - 1;
@@ -472,9 +471,12 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
     }
     const QuantRing ring(places);
     QuantRing filled = ring;
+    const uint4 *from = X + at;
+    asm volatile("" : "+l"(from), "+l"(stride));           // worked out before the wait
+    begin_behind();
 #pragma unroll
     for (int k = 0; k < kQuantPlaces; ++k, filled.up()) {
-        if (k < left) filled.copy(X + at + k * stride);
+        if (k < left) filled.copy(from + k * stride);
         if (k % 2) QuantRing::commit();
     }
     float s;
@@ -494,9 +496,9 @@ act_quant_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, float *x_s
     QuantScale a = make_quant_scale(s, qmax);
     // the test of the single product pays from four vectors per thread on
     if (vec8 >= 4 * (int64_t)gridDim.x * blockDim.x && find_single_product<true>(a))
-        quantise_strided<true>(ring, X + at, Xq + at, stride, left, a, regroup);
+        quantise_strided<true>(ring, from, Xq + at, stride, left, a, regroup);
     else
-        quantise_strided<false>(ring, X + at, Xq + at, stride, left, a, regroup);
+        quantise_strided<false>(ring, from, Xq + at, stride, left, a, regroup);
 }
 
 static int launch_act_quant(const void *X, int8_t *Xq, float *x_scale, const uint32_t *partial, int n_partials, int64_t vec8,
@@ -1045,16 +1047,20 @@ act_quant_cluster_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, fl
     __syncwarp();
     // every CTA of the cluster has started, and has its barrier, before its shared memory is written (waited for below)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");                  // the producer of X is complete
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int first = (int)blockIdx.x / size * kOwn;
     const int stride = size * kClusterThreads, i0 = (int)rank * kClusterThreads + (int)threadIdx.x;
-    uint4 v[kPer];                                                      // from vector `first` on, round the end
+    int at[kPer];                                                       // the thread's vectors, from `first` on, round the end
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
         const int k = first + u < per ? first + u : first + u - per;
-        v[u] = u < per && i0 + k * stride < vec8 ? __ldg(X + i0 + k * stride) : make_uint4(0u, 0u, 0u, 0u);
+        at[u] = u < per && i0 + k * stride < vec8 ? i0 + k * stride : -1;
+        asm volatile("" : "+r"(at[u]));                                 // worked out before the wait
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // the producer of X is complete
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint4 v[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) v[u] = at[u] >= 0 ? __ldg(X + at[u]) : make_uint4(0u, 0u, 0u, 0u);
     uint32_t m = 0;
 #pragma unroll
     for (int u = 0; u < kPer; ++u) m = max(m, absmax_bits8(v[u]));
@@ -1087,8 +1093,7 @@ act_quant_cluster_kernel(const uint4 *__restrict__ X, uint2 *__restrict__ Xq, fl
     const QuantScale a = make_quant_scale(s, qmax);
 #pragma unroll
     for (int u = 0; u < kOwn; ++u) {
-        const int i = i0 + (first + u) * stride;
-        if (first + u < per && i < vec8) Xq[i] = regrouped(quant8_f16<false>(v[u], a), regroup);
+        if (first + u < per && at[u] >= 0) Xq[at[u]] = regrouped(quant8_f16<false>(v[u], a), regroup);
     }
 }
 
