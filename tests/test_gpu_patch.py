@@ -78,6 +78,25 @@ def test_patch_quant_and_embedding_small(B, Bn, C, H, W, P, D, given):
     assert f16_ulp_distance(Y, r["Y"]).max() == 0
 
 
+# A thread stays in its column of Xq and takes token rows as far apart as the grid's threads fill rows at a time: one row
+# fewer than a multiple of that, as many, one more, four times it and more; rows longer than one wave of threads; padding
+# columns; each vector width.  The codes are the image's, rearranged.
+@pytest.mark.parametrize("Bn,C,H,W,P,Kp", [
+    (1578, 3, 16, 16, 16, 768), (1579, 3, 16, 16, 16, 784), (1, 3, 640, 640, 4, 48), (1, 3, 640, 640, 8, 208),
+    (6315, 3, 16, 16, 16, 768), (6316, 3, 16, 16, 16, 768), (6317, 3, 16, 16, 16, 768), (2, 1, 1600, 1600, 1600, 2560000),
+    (2, 1, 804, 804, 804, 646416), (3, 3, 420, 420, 14, 592), (2, 3, 36, 36, 12, 448)])
+def test_patch_rows(B, Bn, C, H, W, P, Kp):
+    img = np.random.default_rng(Bn + Kp).standard_normal((Bn, C, H, W), dtype=np.float32).astype(np.float16)
+    for scale in (None, np.float32(0.02)):
+        codes, s_o = oracle.quant_act(img.reshape(-1, 8), scale)
+        rows = codes.reshape(Bn, C, H // P, P, W // P, P).transpose(0, 2, 4, 1, 3, 5).reshape(-1, C * P * P)
+        xs = None if scale is None else cu(np.array([scale], np.float32))
+        Xq, s = B.patch_quant(cu(img), P, Kp, Xq=torch.full((len(rows), Kp), 9, dtype=torch.int8, device="cuda"), x_scale=xs,
+                              scale_mode=B.SCALE_COMPUTE if scale is None else B.SCALE_GIVEN)
+        Xq = Xq.cpu().numpy()
+        assert s.cpu().numpy()[0] == s_o and np.array_equal(Xq[:, :rows.shape[1]], rows) and not Xq[:, rows.shape[1]:].any()
+
+
 def test_patch_quant_reuses_the_quant_act_workspace(B):
     # one zero-filled workspace serves gpusq_quant_act and gpusq_patch_quant in any order
     d = inputs.random_patch(7, 2, 3, 32, 32, 16, 128)
